@@ -141,8 +141,8 @@ typedef struct {
   int32_t kind;
   uint32_t n_bricks;        /* 8^3 occupancy bricks held on the device */
   uint32_t hash_capacity;   /* hash layout: table entries (power of two); else 0 */
-  uint32_t layout;          /* 0: grid (bricks over the bounding box of occupied blocks plus a
-                               1-bit block bitmap); 1: hash table of blocks */
+  uint32_t layout;          /* 0: grid (bricks over the bounding box of occupied blocks);
+                               1: hash table of blocks */
   uint64_t device_bytes;    /* device memory held by the map */
 } rmp_map_info_t;
 
@@ -174,14 +174,14 @@ int rmp_map_release(rmp_ctx* ctx, uint32_t map_id);
  * RMP_ERR_UNKNOWN_MAP for an id not registered in this context. */
 int rmp_map_info(rmp_ctx* ctx, uint32_t map_id, rmp_map_info_t* out);
 
-/* Free-space data of a grid-layout map, for diagnostics and tests (evaluation does not need
- * it).  grid_min / grid_dim (3 int32 each, host) receive the block coordinates of the grid's
+/* Free-space data of a grid-layout map, for diagnostics and tests (evaluation does not use
+ * it; it is computed by the call).  grid_min / grid_dim (3 int32 each, host) receive the block coordinates of the grid's
  * first brick (x, y, z; dense maps: 0) and its bricks per axis.  cells (nullable, host,
  * cells_words uint32 words, caller-owned) receives 8 words per brick in brick order
  * (x + dim_x (y + dim_y z)): the Chebyshev distance in voxels from each 2^3 cell
  * c = cx + 4 cy + 16 cz of the brick to the nearest occupied voxel, capped at 4, in bits
  * 4 (c & 7) of word c >> 3; 0 for bricks without an occupied voxel.  Synchronous.
- * RMP_ERR_INVALID_ARG for a hash-layout map, a map without cell distances (cells given),
+ * RMP_ERR_INVALID_ARG for a hash-layout map, a map of more than 2^23 bricks (cells given),
  * or cells_words below 8 x bricks. */
 int rmp_map_cell_distances(rmp_ctx* ctx, uint32_t map_id, int32_t grid_min[3],
                            int32_t grid_dim[3], uint32_t* cells, uint64_t cells_words);
@@ -522,14 +522,11 @@ int rmp_probe_l2_read(rmp_ctx* ctx, const void* buf_dev, size_t bytes, uint32_t 
  *                        persistent launch holds at once
  *  RMP_TUNE_RAY_ORDER    0 (default): rays of one direction cell share warps (coherent
  *                        march); 1: Halton index order
- *  RMP_TUNE_SPLIT_BUDGET single-state evaluations: block visits after which the pieces
- *                        still running in a warp are cut into sub-pieces marched by the
- *                        warp's idle lanes (1..65536), 0 never, -1 (default) the library's
- *                        choice (currently never); batches never split
- *  RMP_TUNE_CELL_SKIP    free boxes of voxels inside occupied blocks crossed in one step
- *                        (grid layout maps): 1 always, 0 never, -1 (default) in batched
- *                        evaluations and in single-state ones marched as 4 or more segments
- *                        per ray (measured faster there, slower for one segment per ray) */
+ *  RMP_TUNE_SPLIT_BUDGET accepted (-1..65536) and read back, without effect: rays are marched
+ *                        box by box, which leaves no long pieces to split over a warp
+ *  RMP_TUNE_CELL_SKIP    free boxes of voxels inside occupied blocks crossed in one step: 1
+ *                        or -1 (default) always, 0 never (voxel by voxel there; slower, for
+ *                        comparison) */
 #define RMP_TUNE_BLOCK 1
 #define RMP_TUNE_LG_SEGMENTS 2
 #define RMP_TUNE_RAY_ORDER 3
@@ -542,7 +539,7 @@ int rmp_tune_get(rmp_ctx* ctx, int knob, int* value);
 
 /* Launch shape rmp_raycast_eval[_async] would use for this map, ray count and parameters:
  * threads per CTA, CTAs, log2 segments per ray, resident CTAs per SM (occupancy), SMs,
- * dynamic shared memory per CTA (the staged free-radius field and brick words) and the
+ * dynamic shared memory per CTA (0: nothing is staged) and the
  * number of direction cells of the ray order.  Host-side only; launches nothing. */
 typedef struct {
   int32_t block, grid, lg_segments, ctas_per_sm, sm_count, smem_bytes, ray_cells, reserved;

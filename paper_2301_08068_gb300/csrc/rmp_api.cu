@@ -21,8 +21,8 @@ struct MapRec {
   DevMap dm;
   void* bricks = nullptr;
   void* table = nullptr;
-  void* radius = nullptr;
-  void* cells = nullptr;
+  void* top = nullptr;
+  void* boxes = nullptr;
   uint32_t n_bricks = 0;
   uint32_t cap = 0;
   uint64_t bytes = 0;
@@ -47,8 +47,8 @@ struct rmp_ctx {
   int tune_block = 0;        // threads per CTA of the evaluation kernels (0: automatic)
   int tune_lg_segs = -1;     // log2 segments per ray (-1: chosen from the ray count)
   int tune_ray_order = 0;    // 0: coherent direction cells, 1: Halton index order
-  int tune_split = -1;       // split budget (-1: default, 0: never split)
-  int tune_cells = -1;       // voxel-box skipping (-1: batches, 4-segment states; 0: off; 1: on)
+  int tune_split = -1;       // kept for rmp_tune_get; without effect
+  int tune_cells = -1;       // voxel boxes (-1, 1: on; 0: off)
   // scratch of the synchronous calls (serialised by mu): the state travels in the launch's
   // constants; the kernel writes the result straight into mapped pinned host memory
   void* ws = nullptr;
@@ -112,7 +112,6 @@ Tuning tuning_of(const rmp_ctx* c) {
   Tuning t;
   t.lg_segs = c->tune_lg_segs;
   t.ray_order = c->tune_ray_order;
-  t.split = c->tune_split;
   t.block = c->tune_block;
   t.cells = c->tune_cells;
   return t;
@@ -164,8 +163,6 @@ int make_consts(const rmp_params_t* p, double vs, uint32_t n, bool scan, EvalCon
     // every thread's serial chain; large ones are issue-bound, where segments only add work
     k->lg_segs = n <= 4096u ? 2u : (n <= 16384u ? 1u : 0u);
     if (tune.lg_segs >= 0) k->lg_segs = (uint32_t)tune.lg_segs;
-    k->split_budget = tune.split < 0 ? kDefaultSplitBudget
-                      : (tune.split == 0 ? 0xffffffffu : (uint32_t)tune.split);
   } else {
     k->perm_M = 1;
     k->perm_Q = n;
@@ -182,7 +179,7 @@ cudaError_t launch_single(const MapRec& mr, const Tuning& t, EvalConsts k,
   DevMap dm = mr.dm;
   const uint64_t wave = mr.wave256[k.reduce_mode];
   auto_segments(t, k.n_rays, wave, &k);
-  single_state_cells(t.cells, k, &dm);
+  if (t.cells == 0) dm.cells = nullptr;             // voxel boxes on unless switched off
   int block, grid;
   launch_shape(t, (uint64_t)k.n_rays << k.lg_segs, wave, &block, &grid);
   return launch_raycast(dm, k, state_dev, ws, out, hits, per_ray, block, grid, s);
@@ -191,37 +188,47 @@ cudaError_t launch_single(const MapRec& mr, const Tuning& t, EvalConsts k,
 void free_map(MapRec& r) {
   if (r.bricks) cudaFree(r.bricks);
   if (r.table) cudaFree(r.table);
-  if (r.radius) cudaFree(r.radius);
-  if (r.cells) cudaFree(r.cells);
-  r.bricks = r.table = r.radius = r.cells = nullptr;
+  if (r.top) cudaFree(r.top);
+  if (r.boxes) cudaFree(r.boxes);
+  r.bricks = r.table = r.top = r.boxes = nullptr;
 }
 
-// uint32 words of a 4-bit-per-brick radius field, in whole uint4s (TMA copy granularity)
-uint32_t radius_words_for(uint64_t n_bricks) {
-  const uint64_t w = (n_bricks + 7) / 8;
-  return (uint32_t)((w + 3) / 4 * 4);
-}
-
-// Free-radius field of a grid layout map whose bricks are in r.bricks.
-int build_radius(MapRec& r, cudaStream_t s) {
-  const uint64_t n = (uint64_t)r.dm.gdim[0] * r.dm.gdim[1] * r.dm.gdim[2];
-  r.dm.radius_words = radius_words_for(n);
-  uint8_t* a = nullptr;
-  uint8_t* b = nullptr;
-  cudaError_t e = cudaMalloc(&r.radius, (size_t)r.dm.radius_words * 4);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&a, n);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&b, n);
+// The box field of a map whose bricks (and hash table) are in r: n bricks, of which `occupied`
+// hold an occupied voxel (at most, if not `counted`).  keys: hash layout, the blocks' keys.  A
+// field that is too large or does not fit is left out: occupied blocks are then marched
+// voxel by voxel.
+int build_boxes(MapRec& r, uint32_t n, uint32_t occupied, bool counted, const int32_t* keys,
+                int sm_count, cudaStream_t s) {
+  const bool grid = r.dm.layout == kLayoutGrid;
+  uint32_t* scratch = nullptr;                  // count, slots, list
+  const size_t at_slots = 64, at_list = at_slots + (grid ? n : 0);
+  cudaError_t e = cudaMalloc((void**)&scratch, (at_list + n) * 4);
+  if (e == cudaSuccess && grid) e = cudaMalloc(&r.top, (size_t)n * 32);
+  if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, 4, s);
   if (e == cudaSuccess)
-    e = launch_grid_radius((const uint32_t*)r.bricks, r.dm, a, b, (uint32_t*)r.radius, s);
-  // 2^3-cell free distances for voxel-box skipping inside occupied blocks (optional)
-  if (e == cudaSuccess && n * 32 <= kMaxCellBytes) {
-    e = cudaMalloc(&r.cells, n * 32);
-    if (e == cudaSuccess) e = launch_cell_dist((const uint32_t*)r.bricks, r.dm, (uint32_t*)r.cells, s);
-    if (e == cudaSuccess) r.dm.cells = (const uint32_t*)r.cells;
+    e = launch_block_slots((const uint32_t*)r.bricks, n, keys, r.dm, (HashEntry*)r.table,
+                           scratch + at_slots, scratch + at_list, scratch, s);
+  uint32_t count = occupied;
+  if (e == cudaSuccess && !counted && count * kBoxBytes > (64ull << 20)) {   // too loose to allocate
+    e = cudaMemcpyAsync(&count, scratch, 4, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
+  if (e == cudaSuccess && count > 0 && count * kBoxBytes <= kMaxBoxFieldBytes) {
+    if (cudaMalloc(&r.boxes, count * kBoxBytes) == cudaSuccess) {
+      r.dm.cells = (const uint32_t*)r.boxes;
+      r.bytes += count * kBoxBytes;
+    } else {
+      cudaGetLastError();
+      r.boxes = nullptr;
+    }
+  }
+  if (e == cudaSuccess)
+    e = launch_box_field(r.dm, (const uint32_t*)r.bricks, keys, scratch + at_slots,
+                         scratch + at_list, scratch, count, (uint8_t*)r.boxes, (uint32_t*)r.top,
+                         sm_count, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (a) cudaFree(a);
-  if (b) cudaFree(b);
+  if (scratch) cudaFree(scratch);
+  r.bytes += grid ? (uint64_t)n * 32 : 0;
   return e == cudaSuccess ? RMP_OK : cuda_status(e);
 }
 
@@ -329,18 +336,15 @@ int rmp_map_upload(rmp_ctx* c, const rmp_map_desc_t* d, rmp_stream_t stream, uin
   void* tmp_b = nullptr;
   void* compact = nullptr;
   void* table = nullptr;
-  unsigned int* err_dev = nullptr;
-  int* bbox_dev = nullptr;
+  int* info_dev = nullptr;          // 8 words, see key_bbox_kernel
   auto cleanup = [&]() {
     if (tmp_a) cudaFree(tmp_a);
     if (tmp_b) cudaFree(tmp_b);
     if (compact) cudaFree(compact);
     if (table) cudaFree(table);
-    if (err_dev) cudaFree(err_dev);
-    if (bbox_dev) cudaFree(bbox_dev);
+    if (info_dev) cudaFree(info_dev);
     tmp_a = tmp_b = compact = table = nullptr;
-    err_dev = nullptr;
-    bbox_dev = nullptr;
+    info_dev = nullptr;
   };
   auto fail = [&](int st) {
     cleanup();
@@ -372,9 +376,9 @@ int rmp_map_upload(rmp_ctx* c, const rmp_map_desc_t* d, rmp_stream_t stream, uin
     cudaError_t e = cudaMalloc(&r.bricks, nbr * 64);
     if (e == cudaSuccess) e = launch_dense_bricks(occ, r.dm.dims, r.dm.gdim, (uint32_t*)r.bricks, s);
     if (e != cudaSuccess) return fail(cuda_status(e));
-    const int rs = build_radius(r, s);
+    r.bytes = nbr * 64;
+    const int rs = build_boxes(r, (uint32_t)nbr, (uint32_t)nbr, false, nullptr, c->sm_count, s);
     if (rs != RMP_OK) return fail(rs);
-    r.bytes = nbr * 64 + (uint64_t)r.dm.radius_words * 4 + (r.cells ? nbr * 32 : 0);
   } else if (d->kind == RMP_MAP_HASHED_TSDF) {
     const uint32_t n = d->n_blocks;
     if (n > (1u << 26)) return RMP_ERR_INVALID_ARG;
@@ -389,13 +393,10 @@ int rmp_map_upload(rmp_ctx* c, const rmp_map_desc_t* d, rmp_stream_t stream, uin
     cudaError_t e = cudaMalloc(&table, (size_t)cap * sizeof(HashEntry));
     if (e == cudaSuccess) e = cudaMemsetAsync(table, 0xFF, (size_t)cap * sizeof(HashEntry), s);
     if (e == cudaSuccess && n > 0) e = cudaMalloc(&compact, (size_t)n * 64);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&err_dev, sizeof(unsigned int));
-    if (e == cudaSuccess) e = cudaMemsetAsync(err_dev, 0, sizeof(unsigned int), s);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&bbox_dev, 6 * sizeof(int));
-    const int bbox_init[6] = {INT32_MAX, INT32_MAX, INT32_MAX, INT32_MIN, INT32_MIN, INT32_MIN};
-    int bbox[6];
-    std::memcpy(bbox, bbox_init, sizeof(bbox));
-    if (e == cudaSuccess) e = cudaMemcpyAsync(bbox_dev, bbox, sizeof(bbox), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&info_dev, 8 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemsetAsync(info_dev, 0, 2 * sizeof(int), s);
+    // 0x80808080 lies below every -key and key
+    if (e == cudaSuccess) e = cudaMemsetAsync(info_dev + 2, 0x80, 6 * sizeof(int), s);
     if (e != cudaSuccess) return fail(cuda_status(e));
     const int32_t* keys = d->block_keys;
     if (n > 0) {
@@ -416,25 +417,25 @@ int rmp_map_upload(rmp_ctx* c, const rmp_map_desc_t* d, rmp_stream_t stream, uin
       e = launch_tsdf_bricks(tsdf, n, (uint32_t*)compact, s);
       if (e == cudaSuccess)
         e = launch_hash_build(keys, n, (const uint32_t*)compact, (HashEntry*)table, r.dm.cap_mask,
-                              r.dm.hash_shift, err_dev, s);
-      if (e == cudaSuccess) e = launch_key_bbox(keys, (const uint32_t*)compact, n, bbox_dev, s);
+                              r.dm.hash_shift, (unsigned int*)info_dev, s);
+      if (e == cudaSuccess) e = launch_key_bbox(keys, (const uint32_t*)compact, n, info_dev, s);
       if (e != cudaSuccess) return fail(cuda_status(e));
     }
-    unsigned int err_host = 0;
-    e = cudaMemcpyAsync(&err_host, err_dev, sizeof(unsigned int), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(bbox, bbox_dev, sizeof(bbox), cudaMemcpyDeviceToHost, s);
+    int info[8];
+    e = cudaMemcpyAsync(info, info_dev, sizeof(info), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return fail(cuda_status(e));
-    if (err_host != 0) return fail(RMP_ERR_INVALID_ARG);
+    if (info[0] != 0) return fail(RMP_ERR_INVALID_ARG);
+    const uint32_t occupied = (uint32_t)info[1];
     // 2) layout: a grid over the bounding box of the occupied blocks unless it is much
     //    larger than the blocks themselves; otherwise keep the hash table
-    const bool none = bbox[0] > bbox[3];
+    const bool none = occupied == 0;
     uint64_t gprod = 1;
     int gdim[3] = {1, 1, 1}, gmin[3] = {0, 0, 0};
     if (!none) {
       for (int a = 0; a < 3; ++a) {
-        gmin[a] = bbox[a];
-        gdim[a] = bbox[3 + a] - bbox[a] + 1;
+        gmin[a] = -info[2 + a];
+        gdim[a] = info[5 + a] - gmin[a] + 1;
         gprod *= (uint64_t)gdim[a];
       }
     }
@@ -453,9 +454,9 @@ int rmp_map_upload(rmp_ctx* c, const rmp_map_desc_t* d, rmp_stream_t stream, uin
       if (e == cudaSuccess && n > 0 && !none)
         e = launch_grid_scatter(keys, (const uint32_t*)compact, n, r.dm, (uint32_t*)r.bricks, s);
       if (e != cudaSuccess) return fail(cuda_status(e));
-      const int rs = build_radius(r, s);
+      r.bytes = grid_bytes;
+      const int rs = build_boxes(r, (uint32_t)gprod, occupied, true, nullptr, c->sm_count, s);
       if (rs != RMP_OK) return fail(rs);
-      r.bytes = grid_bytes + (uint64_t)r.dm.radius_words * 4 + (r.cells ? gprod * 32 : 0);
     } else {
       r.dm.layout = kLayoutHash;
       r.bricks = compact;
@@ -464,6 +465,10 @@ int rmp_map_upload(rmp_ctx* c, const rmp_map_desc_t* d, rmp_stream_t stream, uin
       r.cap = cap;
       r.n_bricks = n;
       r.bytes = (uint64_t)cap * sizeof(HashEntry) + (uint64_t)n * 64;
+      r.dm.bricks = (const uint4*)r.bricks;
+      r.dm.table = (const HashEntry*)r.table;
+      const int rs = build_boxes(r, n, occupied, true, keys, c->sm_count, s);
+      if (rs != RMP_OK) return fail(rs);
     }
   } else {
     return RMP_ERR_INVALID_ARG;
@@ -471,7 +476,7 @@ int rmp_map_upload(rmp_ctx* c, const rmp_map_desc_t* d, rmp_stream_t stream, uin
   cleanup();
   r.dm.bricks = (const uint4*)r.bricks;
   r.dm.table = (const HashEntry*)r.table;
-  r.dm.radius = (const uint32_t*)r.radius;
+  r.dm.top = (const uint32_t*)r.top;
   for (int red = 0; red < 2; ++red) {
     const int occ = raycast_occupancy(r.dm, red, 256);
     r.wave256[red] = occ > 0 ? (uint64_t)c->sm_count * (uint64_t)occ * 256u : 0;
@@ -517,7 +522,7 @@ int rmp_map_cell_distances(rmp_ctx* c, uint32_t map_id, int32_t grid_min[3],
   const MapRec& r = it->second;
   if (r.dm.layout != kLayoutGrid) return RMP_ERR_INVALID_ARG;
   const uint64_t words = 8ull * (uint64_t)r.dm.gdim[0] * r.dm.gdim[1] * r.dm.gdim[2];
-  if (cells && (!r.cells || cells_words < words)) return RMP_ERR_INVALID_ARG;
+  if (cells && (words * 4 > kMaxCellBytes || cells_words < words)) return RMP_ERR_INVALID_ARG;
   for (int a = 0; a < 3; ++a) {
     grid_min[a] = r.dm.gmin[a];
     grid_dim[a] = r.dm.gdim[a];
@@ -525,8 +530,12 @@ int rmp_map_cell_distances(rmp_ctx* c, uint32_t map_id, int32_t grid_min[3],
   if (!cells) return RMP_OK;
   DeviceGuard g(c->device);
   if (!g.ok()) return RMP_ERR_CUDA;
-  RMP_CUDA(cudaMemcpy(cells, r.cells, words * 4, cudaMemcpyDeviceToHost));
-  return RMP_OK;
+  uint32_t* dev = nullptr;
+  cudaError_t e = cudaMalloc((void**)&dev, words * 4);
+  if (e == cudaSuccess) e = launch_cell_dist((const uint32_t*)r.bricks, r.dm, dev, 0);
+  if (e == cudaSuccess) e = cudaMemcpy(cells, dev, words * 4, cudaMemcpyDeviceToHost);
+  if (dev) cudaFree(dev);
+  return e == cudaSuccess ? RMP_OK : cuda_status(e);
 }
 
 size_t rmp_workspace_bytes(void) { return workspace_bytes(); }
@@ -578,7 +587,7 @@ int rmp_eval_launch_info(rmp_ctx* c, uint32_t map_id, uint32_t n_rays, const rmp
   out->lg_segments = (int)k.lg_segs;
   out->ctas_per_sm = raycast_occupancy(dm, k.reduce_mode, block);
   out->sm_count = c->sm_count;
-  out->smem_bytes = (int)raycast_smem_bytes(dm);
+  out->smem_bytes = 0;                              // nothing is staged
   out->ray_cells = (int)k.perm_M;
   return RMP_OK;
 }

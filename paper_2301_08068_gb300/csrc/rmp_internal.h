@@ -3,16 +3,21 @@
 //   * occupancy brick: one 8^3 voxel block = 512 bits = 64 bytes = 16 uint32 words; bit
 //     b = lx + 8 ly + 64 lz lives in word b >> 5, bit b & 31 (a TSDF voxel is occupied iff
 //     its value is <= 0; a dense voxel iff it is nonzero).
+//   * box field: for every voxel of an occupied block and each of the 8 octants of ray
+//     directions one byte, 0 if the voxel is occupied, else 64 | ex | ey << 2 | ez << 4: the
+//     2^ex x 2^ey x 2^ez voxels from it on in that octant are free.  4 KB per occupied block,
+//     by slot: octant o (bit a set: axis a climbs) at 512 o, voxels in reflected order (an
+//     axis the octant descends counts from 7 down).
 //   * grid layout (dense maps, and hashed maps whose block bounding box is moderate): the
-//     bricks of every block in the bounding box, x fastest (all-zero where free), plus a
-//     4-bit free radius per block: 0 if the block holds an occupied voxel, else
-//     min(15, Chebyshev distance in blocks to the nearest such block), so the blocks
-//     within radius - 1 of it are all free.  The march stages the radii in shared memory
-//     and crosses a whole free box of blocks in one exact step.
+//     bricks of every block in the bounding box, x fastest (all-zero where free), plus 8
+//     planes (octants) of one word per block: 2^31 | slot of an occupied block, else the log2
+//     extents in blocks of the free box from it on (2 bits per axis).  The march crosses a
+//     whole free box of blocks or voxels in one exact step.
 //   * hash layout (fallback for very large extents): power-of-two array of 16-byte entries
-//     {key, slot}; key packs the block coordinates (21 bits each, offset by 2^20); empty
+//     {key, slot, box}; key packs the block coordinates (21 bits each, offset by 2^20); empty
 //     entries hold ~0; linear probing from a Fibonacci (multiply-shift) hash, load factor
-//     <= 1/4; blocks without occupied voxels keep their key with slot -1.
+//     <= 1/4; blocks without occupied voxels keep their key with slot -1; box: the block's
+//     slot in the box field.
 #pragma once
 
 #include <cstdint>
@@ -28,23 +33,21 @@ constexpr int kKeyBias = 1 << 20;
 constexpr int kMaxGrid = 4096;          // CTAs of one evaluation (grid-stride beyond)
 constexpr int kWsHeaderBytes = 1024;
 constexpr int kMaxRangeVoxels = 16384;  // keeps every DDA crossing numerator below 2^31
-// Block visits before a warp's unfinished pieces are split over its idle lanes; by default
-// never (measured: with coherent ray order the split does not shorten the slowest warps)
-constexpr uint32_t kDefaultSplitBudget = 0xffffffffu;
 
 struct HashEntry {
   unsigned long long key;
   uint32_t slot;
-  uint32_t pad;
+  uint32_t box;
 };
 
 constexpr int kLayoutGrid = 0;
 constexpr int kLayoutHash = 1;
-constexpr uint32_t kMaxSmemRadiusBytes = 48 * 1024;   // staged in shared memory up to this
-constexpr int kMaxFreeRadius = 15;
-constexpr int kSmemBrickBytes = 16 * 32 * 4;           // batch kernel: one warp's staged bricks
+constexpr uint64_t kBoxBytes = 4096;                  // box field of one occupied block
+// Largest box field (8 M occupied blocks); a map beyond it, or one whose field does not fit the
+// device's memory, is marched voxel by voxel inside occupied blocks
+constexpr uint64_t kMaxBoxFieldBytes = 32ull << 30;
 constexpr int kCellDistCap = 4;                       // cell free distances are capped here
-constexpr uint64_t kMaxCellBytes = 256ull << 20;      // cell distances kept up to this size
+constexpr uint64_t kMaxCellBytes = 256ull << 20;      // cell distances given up to this size
 constexpr uint64_t kMaxGridBricks = 1ull << 26;       // grid layout up to 4 GiB of bricks
 
 struct DevMap {
@@ -53,16 +56,14 @@ struct DevMap {
   int hash_shift;           // 64 - log2(capacity)
   uint32_t cap_mask;
   float vs_f;               // RN32(voxel size)
-  uint32_t radius_words;    // grid: uint32 words of the radius field (8 per word, multiple of 4)
   double vs;
   double origin[3];         // dense only (hashed maps are world-anchored)
   int dims[3];              // dense voxels per axis
   int gmin[3];              // grid: block coordinates of the grid's first brick
   int gdim[3];              // grid: bricks per axis
   const uint4* bricks;      // grid: brick (x + gdim0 (y + gdim1 z)); hash: by slot
-  const uint32_t* radius;   // grid: 4-bit free radius of brick idx at bits 4 (idx & 7)
-  const uint32_t* cells;    // grid (optional): 8 words per brick, the 4-bit free distance of
-                            // each 2^3 cell c = cx + 4 cy + 16 cz at word c >> 3, bits 4 (c & 7)
+  const uint32_t* top;      // grid: 8 planes of one word per brick (see above)
+  const uint32_t* cells;    // the box field's bytes (null: march occupied blocks voxel by voxel)
   const HashEntry* table;   // hash layout only
 };
 
@@ -75,7 +76,6 @@ struct EvalConsts {
   uint32_t n_rays, halton_offset;
   uint32_t perm_M, perm_Q, perm_R;   // coherent ray order (see ray_of_slot)
   uint32_t lg_segs;                  // each ray is marched as 2^lg_segs segments
-  uint32_t split_budget;             // block visits before unfinished pieces are split (~0: never)
   int w_mode, reduce_mode;
   double c64;                        // soft-normalisation c (FP64, attractor)
   double att_alpha, att_beta;        // attractor gain and damping (combined evaluations)
@@ -168,6 +168,9 @@ inline BatchLayout batch_layout(uint32_t n_states, uint32_t max_rays) {
   return L;
 }
 
+#ifdef __CUDACC__
+__host__ __device__
+#endif
 inline unsigned long long pack_key(int bx, int by, int bz) {
   return (unsigned long long)(uint32_t)(bx + kKeyBias) |
          ((unsigned long long)(uint32_t)(by + kKeyBias) << 21) |
@@ -183,8 +186,6 @@ struct EsdfConsts {
 };
 
 // Launchers (rmp_kernels.cu).  All enqueue on `stream` and return cudaGetLastError().
-size_t raycast_smem_bytes(const DevMap& m);
-size_t batch_smem_bytes(const DevMap& m, int block);   // + the staged bricks, per warp
 int raycast_occupancy(const DevMap& m, int reduce_mode, int block);   // CTAs per SM
 cudaError_t launch_raycast(const DevMap& m, const EvalConsts& k, const double* state_dev,
                            void* ws, rmp_result_t* out_dev, rmp_ray_hit_t* hits,
@@ -217,14 +218,23 @@ cudaError_t launch_scan(const float* pts, const EvalConsts& k, const double* sta
                         cudaStream_t stream);
 cudaError_t launch_dense_bricks(const uint8_t* occ, const int dims[3], const int nb[3],
                                 uint32_t* bricks, cudaStream_t stream);
-// Free-radius field of a grid from its bricks (scratch: two byte arrays, one per brick).
-cudaError_t launch_grid_radius(const uint32_t* bricks, const DevMap& m, uint8_t* scratch_a,
-                               uint8_t* scratch_b, uint32_t* radius, cudaStream_t stream);
-// Free distance of every 2^3 cell of the occupied bricks of a grid (see DevMap::cells).
+// Slots of the occupied blocks (see block_slots_kernel; *count zeroed by the caller), then the
+// box field: level 1 (grid layout, m.gdim) into `top`, level 0 into `field` (null: none; room
+// for `cap` slots).
+cudaError_t launch_block_slots(const uint32_t* bricks, uint32_t n, const int32_t* keys,
+                               const DevMap& m, HashEntry* table, uint32_t* slot_of,
+                               uint32_t* list, uint32_t* count, cudaStream_t stream);
+cudaError_t launch_box_field(const DevMap& m, const uint32_t* bricks, const int32_t* keys,
+                             const uint32_t* slot_of, const uint32_t* list, const uint32_t* count,
+                             uint32_t cap, uint8_t* field, uint32_t* top, int sm_count,
+                             cudaStream_t stream);
+// Free distance of every 2^3 cell of the occupied bricks of a grid (8 words per brick,
+// see rmp_map_cell_distances).
 cudaError_t launch_cell_dist(const uint32_t* bricks, const DevMap& m, uint32_t* cells,
                              cudaStream_t stream);
+// info: 8 words, see key_bbox_kernel (word 0 is launch_hash_build's err).
 cudaError_t launch_key_bbox(const int32_t* keys, const uint32_t* bricks, uint32_t n_blocks,
-                            int* bbox, cudaStream_t stream);
+                            int* info, cudaStream_t stream);
 cudaError_t launch_grid_scatter(const int32_t* keys, const uint32_t* bricks, uint32_t n_blocks,
                                 const DevMap& m, uint32_t* grid_bricks, cudaStream_t stream);
 cudaError_t launch_tsdf_bricks(const float* tsdf, uint32_t n_blocks, uint32_t* bricks,

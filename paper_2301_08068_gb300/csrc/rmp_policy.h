@@ -14,8 +14,8 @@ namespace rmp {
 
 // Launch knobs of a context (rmp_tune_set): -1 / 0 select the library's choice.
 struct Tuning {
-  // log2 segments per ray, ray order, split budget, threads per CTA, voxel boxes
-  int lg_segs = -1, ray_order = 0, split = -1, block = 0, cells = -1;
+  // log2 segments per ray, ray order, threads per CTA, voxel boxes
+  int lg_segs = -1, ray_order = 0, block = 0, cells = -1;
 };
 
 // Coherent ray order: residue classes modulo M = 2^a 3^b are direction cells (see the
@@ -59,10 +59,9 @@ inline void auto_segments(const Tuning& t, uint32_t n, uint64_t wave256, EvalCon
   k->lg_segs = lg;
 }
 
-// Voxel boxes in a single-state evaluation: as tuned, or (default) only with 4 or more
-// segments per ray, where they pay (measured, 16384 rays: hashed 47.1 -> 44.6 us, dense 37.5 -> 36.6 us)
-// -- with one segment per ray their extra dependent load lengthens the slowest warps
-// (65536 rays: hashed 68.0 -> 71.2 us, dense 43.9 -> 49.4 us).
+// The voxel boxes' rule from when a box was looked up beside the voxel walk: as tuned, or only
+// with 4 or more segments per ray.  No launch uses it any more (the box field replaces the
+// walk, and is faster for every segment count); tests/launch_policy_check.cpp still builds it.
 inline void single_state_cells(int tune_cells, const EvalConsts& k, DevMap* dm) {
   if (tune_cells == 1) return;
   if (tune_cells == 0 || k.lg_segs < 2) dm->cells = nullptr;

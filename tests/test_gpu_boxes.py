@@ -1,0 +1,77 @@
+"""The box field of the march where it can go wrong: grids that are not multiples of 8, single
+blocks, random occupancy from nearly empty to half full (boxes of every extent), states on
+voxel boundaries and centres (ties), outside and far from a hashed map's blocks, the pole ray
+of Halton offset 0, and segments.  Hit records equal the oracle's voxel-by-voxel march byte for
+byte, with the boxes and (knob off) voxel by voxel."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2301_08068_gb300 import rmp as R
+from paper_2301_08068_gb300 import workloads as W
+
+from gpu_helpers import assert_hits_exact, gpu_raycast, torch_cuda
+
+pytestmark = pytest.mark.gpu
+VS = 0.1
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    torch_cuda()
+    c = R.Context(0)
+    yield c
+    c.close()
+
+
+def check(ctx, m, xs, n, max_range):
+    mid, om = ctx.upload(m), O.OracleMap(m)
+    knobs = ((-1, -1), (-1, 0), (-1, 2), (0, 0), (0, -1))      # voxel boxes, log2 segments
+    try:
+        for i, x in enumerate(xs):
+            d = dict(W.PARAMS_STATIC_MAP, halton_offset=i & 1)
+            v = np.array([0.4, -0.9, 0.2])
+            _, ho, _ = O.raycast_eval(om, x, v, n, O.make_params(d, max_range))
+            for cells, lgs in knobs:
+                R.rmp_tune_set(ctx.handle, R.RMP_TUNE_CELL_SKIP, cells)
+                R.rmp_tune_set(ctx.handle, R.RMP_TUNE_LG_SEGMENTS, lgs)
+                _, hg, _ = gpu_raycast(ctx, mid, x, v, n, R.make_params(d, max_range))
+                assert_hits_exact(hg, ho)
+    finally:
+        R.rmp_tune_set(ctx.handle, R.RMP_TUNE_CELL_SKIP, -1)
+        R.rmp_tune_set(ctx.handle, R.RMP_TUNE_LG_SEGMENTS, -1)
+        R.rmp_map_release(ctx.handle, mid)
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 1), (8, 8, 8), (9, 7, 17), (24, 1, 65), (71, 64, 50)])
+@pytest.mark.parametrize("density", [0.001, 0.03, 0.5])
+def test_dense_grids(ctx, dims, density):
+    rng = np.random.default_rng([*dims, int(1000 * density)])
+    occ = (rng.uniform(size=dims[::-1]) < density).astype(np.uint8)
+    ext = np.array(dims) * VS
+    free = np.argwhere(occ == 0)[:, ::-1]
+    xs = [ext * rng.uniform(size=3), ext * 0.5, ext + 0.05, np.array([-0.01, 0.02, 0.03])]
+    if len(free):
+        k = free[rng.integers(len(free))]
+        xs += [(k + 0.5) * VS, k * VS + 1e-9]
+    check(ctx, W.DenseMap(occ, VS, np.zeros(3)), xs, 777, 4.0)
+
+
+@pytest.mark.parametrize("far", [False, True])      # a far block: the hash layout
+@pytest.mark.parametrize("density", [0.0005, 0.02, 0.4])
+def test_hashed_blocks(ctx, far, density):
+    rng = np.random.default_rng([int(far), int(10000 * density)])
+    keys = np.unique(rng.integers(-4, 5, (60, 3)), axis=0).astype(np.int32)
+    if far:
+        keys = np.concatenate([keys, [[9000, -7000, 800]]]).astype(np.int32)
+    tsdf = np.where(rng.uniform(size=(len(keys), 512)) < density, -0.1, 0.2).astype(np.float32)
+    tsdf[-1, 100] = -0.1                            # the far block is occupied
+    xs = [rng.uniform(-3.0, 3.0, 3), np.zeros(3), np.array([0.05, -0.05, 0.15]),
+          np.array([-30.0, 2.0, 1.0]), np.array([1.0, 6.0, -28.0]), np.array([4.1, 4.1, 4.1])]
+    check(ctx, W.HashedMap(keys, tsdf, VS), xs, 777, 45.0)
+
+
+def test_empty_hashed_map(ctx):
+    keys = np.array([[0, 0, 0], [3, -2, 1]], np.int32)
+    tsdf = np.full((2, 512), 0.2, np.float32)
+    check(ctx, W.HashedMap(keys, tsdf, VS), [np.zeros(3), np.array([5.0, -5.0, 5.0])], 100, 20.0)
