@@ -505,13 +505,6 @@ __device__ __forceinline__ void acc_add(Acc32& acc, const float v[9]) {
   }
 }
 
-__device__ __forceinline__ void acc_merge(Acc32& acc, float s2, float c2, int q) {
-  float s, e;
-  two_sum(acc.s[q], s2, s, e);
-  acc.s[q] = s;
-  acc.c[q] = __fadd_rn(__fadd_rn(acc.c[q], c2), e);
-}
-
 struct Acc64 {
   double s[9];
 };
@@ -533,7 +526,71 @@ __device__ __forceinline__ void merge1(float& s, float& c, float s2, float c2) {
   c = __fadd_rn(__fadd_rn(c, c2), e);
 }
 
-// Block-level reduction of the per-thread accumulators and counts: a shuffle tree per warp,
+__device__ __forceinline__ void merge1(double& s, double s2) { s += s2; }
+
+// Sums of the 9 terms over each group of W = 32 >> lgW lanes by the tree of a shuffle-down
+// reduction (lane i takes lane i + W/2, then W/4, ...), but with the terms shared out: at each
+// level a lane and its partner keep half of their terms each and merge only those, 12 merges a
+// lane instead of 45 (the merges commute bit for bit, so the tree's results are the same).
+// Afterwards slot j (j < WarpTerms::n) of a lane holds term first + j; n is 0 where the lane
+// holds none.  Lanes 0, W, 2 W, ... hold term 0.
+struct WarpTerms {
+  int first, n;
+};
+
+// terms a lane holds before level j
+__host__ __device__ constexpr int term_split(int j) {
+  return j == 0 ? 9 : (j == 1 ? 5 : (j == 2 ? 3 : (j == 3 ? 2 : 1)));
+}
+
+__device__ __forceinline__ WarpTerms warp_terms(uint32_t lgW) {
+  const uint32_t lane = threadIdx.x & 31;
+  WarpTerms t{0, 9};
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    const uint32_t off = 16u >> (lgW + j);
+    const int h = term_split(j + 1);
+    if (off == 0) continue;
+    if (lane & off) {
+      t.first += h;
+      t.n -= h;
+    } else {
+      t.n = t.n < h ? t.n : h;
+    }
+    if (t.n < 0) t.n = 0;
+  }
+  return t;
+}
+
+// FP32 pairs (s, c), or FP64 values (c unused); slots 0 .. of s (and c) are left as above.
+template <typename T, bool PAIR>
+__device__ __forceinline__ void warp_reduce_terms(T (&s)[9], T (&c)[9], uint32_t lgW) {
+  const uint32_t lane = threadIdx.x & 31;
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    const uint32_t off = 16u >> (lgW + j);
+    if (off == 0) continue;
+    const int m = term_split(j), h = term_split(j + 1);
+    const bool upper = (lane & off) != 0;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+      if (i >= h) continue;
+      const T s1 = h + i < m ? s[h + i < 9 ? h + i : 8] : T(0), s0 = s[i];
+      const T rs = __shfl_xor_sync(0xffffffffu, upper ? s0 : s1, off);
+      s[i] = upper ? s1 : s0;
+      if constexpr (PAIR) {
+        const T c1 = h + i < m ? c[h + i < 9 ? h + i : 8] : T(0), c0 = c[i];
+        const T rc = __shfl_xor_sync(0xffffffffu, upper ? c0 : c1, off);
+        c[i] = upper ? c1 : c0;
+        merge1(s[i], c[i], rs, rc);
+      } else {
+        merge1(s[i], rs);
+      }
+    }
+  }
+}
+
+// Block-level reduction of the per-thread accumulators and counts: the shared-out tree per warp,
 // then lane q of warp 0 merges term q of the warps in warp order (all terms at once, not one
 // thread walking them).  Called by every thread.
 template <int RED>
@@ -551,23 +608,15 @@ struct BlockReduce<RMP_REDUCE_KAHAN32> {
     __shared__ float sh[32][18];
     __shared__ unsigned shu[32][2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-      for (int q = 0; q < 9; ++q) {
-        const float s2 = __shfl_down_sync(0xffffffffu, a.s[q], off);
-        const float c2 = __shfl_down_sync(0xffffffffu, a.c[q], off);
-        acc_merge(a, s2, c2, q);
-      }
-    }
+    const WarpTerms t = warp_terms(0);
+    warp_reduce_terms<float, true>(a.s, a.c, 0);
     nh = __reduce_add_sync(0xffffffffu, nh);
     na = __reduce_add_sync(0xffffffffu, na);
+    if (t.n > 0) {
+      sh[warp][t.first] = a.s[0];
+      sh[warp][9 + t.first] = a.c[0];
+    }
     if (lane == 0) {
-#pragma unroll
-      for (int q = 0; q < 9; ++q) {
-        sh[warp][q] = a.s[q];
-        sh[warp][9 + q] = a.c[q];
-      }
       shu[warp][0] = nh;
       shu[warp][1] = na;
     }
@@ -603,15 +652,12 @@ struct BlockReduce<RMP_REDUCE_FP64> {
     __shared__ double sh[32][9];
     __shared__ unsigned shu[32][2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-      for (int q = 0; q < 9; ++q) a.s[q] += __shfl_down_sync(0xffffffffu, a.s[q], off);
+    const WarpTerms t = warp_terms(0);
+    warp_reduce_terms<double, false>(a.s, a.s, 0);
     nh = __reduce_add_sync(0xffffffffu, nh);
     na = __reduce_add_sync(0xffffffffu, na);
+    if (t.n > 0) sh[warp][t.first] = a.s[0];
     if (lane == 0) {
-#pragma unroll
-      for (int q = 0; q < 9; ++q) sh[warp][q] = a.s[q];
       shu[warp][0] = nh;
       shu[warp][1] = na;
     }
@@ -1557,23 +1603,50 @@ __global__ void __launch_bounds__(1024) batch_prep_kernel(
   }
 }
 
-// Sum of a partial over the lanes of a warp (lane i holds p_i; lanes without one hold 0):
-// FP64 shuffle tree in a fixed order, result in lane 0.
-__device__ __forceinline__ void warp_sum_partial(double v[9], unsigned& h, unsigned& a) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-    for (int q = 0; q < 9; ++q) v[q] += __shfl_down_sync(0xffffffffu, v[q], off);
-  h = __reduce_add_sync(0xffffffffu, h);
-  a = __reduce_add_sync(0xffffffffu, a);
-}
-
+// Lane i's terms and counts of a chunk partial (FP32 pairs for the compensated reduction, as
+// CtaPartial32) or of a group partial (FP64), read past L1: another SM wrote it.
+template <bool PAIR>
 __device__ __forceinline__ void load_partial(const CtaPartial* p, double v[9], unsigned& h,
                                              unsigned& a) {
+  if (PAIR) {
+    const uint4* q = reinterpret_cast<const uint4*>(p);
+    uint32_t w[20];
 #pragma unroll
-  for (int q = 0; q < 9; ++q) v[q] = __ldcg(&p->v[q]);
-  h = __ldcg(&p->n_hits);
-  a = __ldcg(&p->n_active);
+    for (int i = 0; i < 5; ++i) {
+      const uint4 x = __ldcg(q + i);
+      w[4 * i] = x.x;
+      w[4 * i + 1] = x.y;
+      w[4 * i + 2] = x.z;
+      w[4 * i + 3] = x.w;
+    }
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+      v[i] = (double)__uint_as_float(w[i]) + (double)__uint_as_float(w[9 + i]);
+    h = w[18];
+    a = w[19];
+  } else {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) v[i] = __ldcg(&p->v[i]);
+    h = __ldcg(&p->n_hits);
+    a = __ldcg(&p->n_active);
+  }
+}
+
+// Sum of 32 lanes' FP64 terms into *p (or the lanes' slot 0, p null), counts into h, a.
+__device__ __forceinline__ WarpTerms warp_sum_partial(double (&v)[9], unsigned& h, unsigned& a,
+                                                      CtaPartial* p) {
+  const WarpTerms t = warp_terms(0);
+  warp_reduce_terms<double, false>(v, v, 0);
+  h = __reduce_add_sync(0xffffffffu, h);
+  a = __reduce_add_sync(0xffffffffu, a);
+  if (p) {
+    if (t.n > 0) p->v[t.first] = v[0];
+    if ((threadIdx.x & 31) == 0) {
+      p->n_hits = h;
+      p->n_active = a;
+    }
+  }
+  return t;
 }
 
 // Attractor policy (Sec. III-B, Eq. attractorPolicy) combined by Eq. (1): its metric I is
@@ -1704,7 +1777,11 @@ __global__ void rollout_step_kernel(DevMap m, RolloutConsts rc, const rmp_result
 // group of a state sums the state's groups, adds the attractor (combined evaluations) and
 // resolves.  Called by all 32 lanes of the warp whose chunk completed the group.  Kept
 // out of line: it runs once per 32 chunks, and inlined it would sit between the march
-// loops in the instruction stream.
+// loops in the instruction stream.  A chunk partial's FP32 pairs become FP64 here, one chunk
+// per lane, not where they are stored: an FP64 instruction holds a scheduler's pipe about 64
+// cycles whatever the active lanes (256 states: 17.2 M -> 1.3 M FP64 warp instructions; with the
+// shared-out trees 1289 -> 1000 us).
+template <int RED>
 __device__ __noinline__ void batch_group_finish(const EvalConsts& k, CtaPartial* cparts,
                                                 CtaPartial* gparts, uint32_t* sticket,
                                                 uint32_t chunk0, uint32_t gi, uint32_t gsz,
@@ -1712,58 +1789,58 @@ __device__ __noinline__ void batch_group_finish(const EvalConsts& k, CtaPartial*
                                                 uint32_t n_b, const double* states,
                                                 const double* goals, rmp_result_t* out) {
   const uint32_t lane = threadIdx.x & 31;
-  uint32_t stage = 0;
   // last chunk of its group: sum the group's chunk partials (lane i: chunk i)
   __threadfence();
   double gv[9] = {0., 0., 0., 0., 0., 0., 0., 0., 0.};
   unsigned gh = 0, ga = 0;
-  if (lane < gsz) load_partial(cparts + chunk0 + gi * kBatchGroup + lane, gv, gh, ga);
-  warp_sum_partial(gv, gh, ga);
+  if (lane < gsz)
+    load_partial<RED == RMP_REDUCE_KAHAN32>(cparts + chunk0 + gi * kBatchGroup + lane, gv, gh, ga);
+  warp_sum_partial(gv, gh, ga, gparts + group0 + gi);
   const uint32_t n_groups = (n_chunks + kBatchGroup - 1) / kBatchGroup;
-  if (lane == 0) {
-    CtaPartial p;
+  __threadfence();
+  __syncwarp();
+  uint32_t last = 0;
+  if (lane == 0) last = atomicAdd(&sticket[b], 1u) == n_groups - 1 ? 1u : 0u;
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
+  // last group of the state: lane i sums groups i, i + 32, ... in order, then the tree
+  __threadfence();
+  double tv[9] = {0., 0., 0., 0., 0., 0., 0., 0., 0.};
+  unsigned th = 0, ta = 0;
+  for (uint32_t j = lane; j < n_groups; j += 32) {
+    double pv2[9];
+    unsigned h2, a2;
+    load_partial<false>(gparts + group0 + j, pv2, h2, a2);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) p.v[i] = gv[i];
-    p.n_hits = gh;
-    p.n_active = ga;
-    gparts[group0 + gi] = p;
-    __threadfence();
-    stage = atomicAdd(&sticket[b], 1u) == n_groups - 1 ? 2u : 0u;
+    for (int i = 0; i < 9; ++i) tv[i] += pv2[i];
+    th += h2;
+    ta += a2;
   }
-  stage = __shfl_sync(0xffffffffu, stage, 0);
-  if (stage == 2) {
-    // last group of the state: lane i sums groups i, i + 32, ... in order, then the tree
-    __threadfence();
-    double tv[9] = {0., 0., 0., 0., 0., 0., 0., 0., 0.};
-    unsigned th = 0, ta = 0;
-    for (uint32_t j = lane; j < n_groups; j += 32) {
-      double pv2[9];
-      unsigned h2, a2;
-      load_partial(gparts + group0 + j, pv2, h2, a2);
+  const WarpTerms t = warp_sum_partial(tv, th, ta, nullptr);
+  // every lane gets all terms back from the lanes that hold them
+  const double mine = tv[0];
 #pragma unroll
-      for (int i = 0; i < 9; ++i) tv[i] += pv2[i];
-      th += h2;
-      ta += a2;
-    }
-    warp_sum_partial(tv, th, ta);
-    if (goals && lane == 0)
-      add_attractor(k, states + 6 * (size_t)b, goals + 3 * (size_t)b, n_b, tv);
+  for (int i = 0; i < 9; ++i) {
+    const uint32_t at = __ballot_sync(0xffffffffu, t.n > 0 && t.first == i);
+    tv[i] = __shfl_sync(0xffffffffu, mine, __ffs(at) - 1);
+  }
+  if (goals) {
+    if (lane == 0) add_attractor(k, states + 6 * (size_t)b, goals + 3 * (size_t)b, n_b, tv);
 #pragma unroll
     for (int i = 0; i < 9; ++i) tv[i] = __shfl_sync(0xffffffffu, tv[i], 0);
-    rmp_result_t r;
-    resolve_pinv(tv, tv + 6, r);
-    if (lane == 0) {
+  }
+  rmp_result_t r;
+  resolve_pinv(tv, tv + 6, r);
+  if (lane == 0) {
 #pragma unroll
-      for (int i = 0; i < 6; ++i) r.A[i] = tv[i];
+    for (int i = 0; i < 6; ++i) r.A[i] = tv[i];
 #pragma unroll
-      for (int i = 0; i < 3; ++i) r.Af[i] = tv[6 + i];
-      r.n_rays = n_b;
-      r.n_hits = th;
-      r.n_active = ta;
-      r.status = RMP_OK;
-      r.reserved = 0;
-      out[b] = r;
-    }
+    for (int i = 0; i < 3; ++i) r.Af[i] = tv[6 + i];
+    r.n_rays = n_b;
+    r.n_hits = th;
+    r.n_active = ta;
+    r.status = RMP_OK;
+    r.reserved = 0;
+    out[b] = r;
   }
 }
 
@@ -1828,48 +1905,38 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
                   na);
     }
     // chunk partial
-    double pv[9];
+    CtaPartial* part = cparts + chunk0 + q;
     if (RED == RMP_REDUCE_FP64) {
+      double pv[9];
 #pragma unroll
       for (int i = 0; i < 9; ++i) pv[i] = (double)vals[i];
-      warp_sum_partial(pv, nh, na);
+      warp_sum_partial(pv, nh, na, part);
     } else {
-      Acc32 acc;
-#pragma unroll
-      for (int i = 0; i < 9; ++i) {
-        acc.s[i] = vals[i];
-        acc.c[i] = 0.0f;
-      }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-          const float s2 = __shfl_down_sync(0xffffffffu, acc.s[i], off);
-          const float c2 = __shfl_down_sync(0xffffffffu, acc.c[i], off);
-          acc_merge(acc, s2, c2, i);
-        }
-#pragma unroll
-      for (int i = 0; i < 9; ++i) pv[i] = (double)acc.s[i] + (double)acc.c[i];
+      const WarpTerms t = warp_terms(0);
+      float cv[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      warp_reduce_terms<float, true>(vals, cv, 0);
       nh = __reduce_add_sync(0xffffffffu, nh);
       na = __reduce_add_sync(0xffffffffu, na);
+      CtaPartial32* p = reinterpret_cast<CtaPartial32*>(part);
+      if (t.n > 0) {
+        p->s[t.first] = vals[0];
+        p->c[t.first] = cv[0];
+      }
+      if (lane == 0) {
+        p->n_hits = nh;
+        p->n_active = na;
+      }
     }
     const uint32_t gi = q / kBatchGroup;
     const uint32_t gsz = min(kBatchGroup, n_chunks - gi * kBatchGroup);
     uint32_t stage = 0;
-    if (lane == 0) {
-      CtaPartial p;
-#pragma unroll
-      for (int i = 0; i < 9; ++i) p.v[i] = pv[i];
-      p.n_hits = nh;
-      p.n_active = na;
-      cparts[chunk0 + q] = p;
-      __threadfence();
-      stage = atomicAdd(&gticket[group0 + gi], 1u) == gsz - 1 ? 1u : 0u;
-    }
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) stage = atomicAdd(&gticket[group0 + gi], 1u) == gsz - 1 ? 1u : 0u;
     stage = __shfl_sync(0xffffffffu, stage, 0);
     if (stage)
-      batch_group_finish(k, cparts, gparts, sticket, chunk0, gi, gsz, n_chunks, group0, b, n_b,
-                         states, goals, out);
+      batch_group_finish<RED>(k, cparts, gparts, sticket, chunk0, gi, gsz, n_chunks, group0, b,
+                              n_b, states, goals, out);
     c = __shfl_sync(0xffffffffu, cn, 0);
   }
 }
