@@ -1418,25 +1418,29 @@ __device__ __forceinline__ uint32_t pick_cells_warp(uint32_t n) {
   float best_score = 3.0e38f;
   uint32_t best = 1;
   const int a = (int)lane;
-  if (a <= 24 && (32ull << a) <= n) {
-    const int bk = (int)floorf((lt - (float)a) / L3);
-    const int bm = (int)floorf((lm - (float)a) / L3) + 1;
-    const int cand[4] = {0, bk, bk + 1, bm};
+  const bool fits = a <= 24 && (32ull << a) <= n;
+  int b_max = 0;                                    // largest b with 32 2^a 3^b <= n (< 2^25)
+  uint32_t m = 32u << (fits ? a : 0), pow3 = 1;     // pow3: 3^lane (lanes 0-15)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      int bb = cand[i] < 0 ? 0 : (cand[i] > 15 ? 15 : cand[i]);
-      unsigned long long mm = 1ull << a;
-      for (int j = 0; j < bb; ++j) mm *= 3ull;
-      while (bb > 0 && mm * 32ull > n) {          // largest feasible b <= the candidate
-        mm /= 3ull;
-        --bb;
-      }
-      const float score = fabsf((float)a + (float)bb * L3 - lt) +
-                          0.5f * fabsf((float)bb * L3 - LPI - (float)a);
-      if (score < best_score) {
-        best_score = score;
-        best = (uint32_t)mm;
-      }
+  for (int i = 0; i < 15; ++i) {
+    m *= 3u;
+    if (m > n) m = 0x40000000u;                     // past it for good
+    b_max += m <= n ? 1 : 0;
+    pow3 *= i < (int)(lane & 15u) ? 3u : 1u;
+    m = m > n ? 0x15555555u : m;
+  }
+  const int bk = (int)floorf((lt - (float)a) / L3);
+  const int bm = (int)floorf((lm - (float)a) / L3) + 1;
+  const int cand[4] = {0, bk, bk + 1, bm};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int bb = min(max(cand[i], 0), b_max);
+    const uint32_t mm = __shfl_sync(0xffffffffu, pow3, bb) << (fits ? a : 0);
+    const float score = fabsf((float)a + (float)bb * L3 - lt) +
+                        0.5f * fabsf((float)bb * L3 - LPI - (float)a);
+    if (fits && score < best_score) {
+      best_score = score;
+      best = mm;
     }
   }
 #pragma unroll
@@ -1466,82 +1470,74 @@ __device__ __forceinline__ uint32_t ray_of_slot_p(uint32_t j, uint32_t M, uint32
   return r + M * q;
 }
 
-// Per-state set-up of a batch (one CTA of 1024 threads).  Phase A, one warp per state:
-// validate the ray count, quantise the position (lanes 0-2, FP64), split the velocity
-// (lanes 3-5), choose the direction cells, count chunks and groups.  Phase B, one thread
-// per state: exclusive block scans assign consecutive chunk and group ranges.  Then the
-// tickets and the work counter are cleared and every state without chunks (no rays, or
-// invalid) gets its result here.
-__global__ void __launch_bounds__(1024) batch_prep_kernel(
+// A state's summation segments (log2): the launch's fixed choice, or the most (up to 4) whose
+// threads the persistent launch holds at once -- a function of the ray count and the launch
+// shape alone, so a state's result does not depend on the other states of the batch or their
+// order.
+__device__ __forceinline__ uint32_t state_lg_segs(const EvalConsts& k, uint32_t n) {
+  if (k.lg_segs <= 2u) return k.lg_segs;
+  if (k.seg_threads == 0u) return n <= 4096u ? 2u : (n <= 16384u ? 1u : 0u);
+  uint32_t lg = 2u;
+  while (lg > 0u && ((unsigned long long)n << lg) > k.seg_threads) --lg;
+  return lg;
+}
+
+// Sum of x over the CTA's threads (256), in every thread; sh: 8 words.
+__device__ __forceinline__ uint32_t block_sum256(uint32_t x, uint32_t* sh) {
+  x = __reduce_add_sync(0xffffffffu, x);
+  __syncthreads();                                  // sh is no longer read
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
+  __syncthreads();
+  uint32_t t = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) t += sh[w];
+  return t;
+}
+
+// Per-state set-up of a batch, CTAs of 256 threads with a run of consecutive states each.  The
+// chunks and groups before a CTA's run follow from the ray counts alone, so every CTA adds
+// them up itself (4 bytes a state) instead of waiting for the others; then, 256 states at a
+// time, one thread per state takes its ranges from a block scan and one warp per state
+// quantises the position (lanes 0-2, FP64), splits the velocity (lanes 3-5) and chooses the
+// direction cells.  The tickets and the work counter are cleared, and every state without
+// rays or with an error gets its result here (chunks of an invalid state are skipped).
+// Bound by one state's latency: 7.3 us for 256 states (one CTA with 8 states a warp, and cells
+// picked with divisions: 46 us).
+__global__ void __launch_bounds__(256) batch_prep_kernel(
     const double* __restrict__ states, const uint32_t* __restrict__ n_rays, uint32_t n_states,
     uint32_t max_rays, DevMap m, EvalConsts k, BatchHeader* hdr, BatchState* bs,
     uint32_t* sticket, uint32_t* gticket, rmp_result_t* out) {
-  __shared__ uint32_t s_chunks[1024], s_groups[1024];
-  __shared__ uint32_t wsum_c[32], wsum_g[32];
-  __shared__ uint32_t carry_c, carry_g;
-  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-  if (tid == 0) {
-    carry_c = 0;
-    carry_g = 0;
-  }
-  for (uint32_t base = 0; base < n_states; base += blockDim.x) {
-    const uint32_t tile = min(blockDim.x, n_states - base);
-    for (uint32_t j = warp; j < tile; j += nwarps) {
-      const uint32_t b = base + j;
-      const uint32_t n = n_rays[b];
-      const double* x = states + 6 * (size_t)b;
-      long long Pa = 0;
-      int bad_a = 0;
-      float va = 0.f, vla = 0.f;
-      if (lane < 3) {
-        const double o = m.kind != RMP_MAP_DENSE_U8 ? 0.0
-                         : (lane == 0 ? m.origin[0] : (lane == 1 ? m.origin[1] : m.origin[2]));
-        const double q = __dmul_rn(__ddiv_rn(__dsub_rn(x[lane], o), m.vs), 65536.0);
-        bad_a = !(fabs(q) < 274877906944.0);
-        Pa = bad_a ? 0 : __double2ll_rn(q);
-      } else if (lane < 6) {
-        const double v = x[lane];
-        va = __double2float_rn(v);
-        vla = __double2float_rn(__dsub_rn(v, (double)va));
-      }
-      const bool bad = (__ballot_sync(0xffffffffu, bad_a != 0) != 0) || n > max_rays;
-      const uint32_t M = n >= 32 ? pick_cells_warp(n) : 1u;
-      BatchState* sp = bs + b;
-      if (lane < 3) sp->P[lane] = Pa;
-      else if (lane < 6) {
-        sp->v[lane - 3] = va;
-        sp->vl[lane - 3] = vla;
-      }
-      if (lane == 0) {
-        // segments per ray: the launch's fixed choice, or the most (up to 4) whose threads
-        // the persistent launch holds at once -- either way a function of the state and
-        // the launch shape alone, so the result does not depend on the other states of
-        // the batch or their order (one state alone, measured: 8192 rays 64.2 -> 53.8 us
-        // with 4 segments instead of 2, 32768 rays 81.1 -> 63.8 us with 4 instead of 1,
-        // 65536 rays 85.4 -> 77.8 us with 2)
-        uint32_t lg = k.lg_segs;
-        if (lg > 2u) {
-          if (k.seg_threads > 0u) {
-            lg = 2u;
-            while (lg > 0u && ((unsigned long long)n << lg) > k.seg_threads) --lg;
-          } else {
-            lg = n <= 4096u ? 2u : (n <= 16384u ? 1u : 0u);
-          }
-        }
-        const uint32_t chunks = (!bad && n > 0) ? ((n << lg) + 31) / 32 : 0u;
-        sp->n_rays = n;
-        sp->status = bad ? RMP_ERR_INVALID_ARG : RMP_OK;
-        sp->n_chunks = chunks;
-        sp->perm_M = M;
-        sp->perm_Q = n / M;
-        sp->lg_segs = lg;
-        s_chunks[j] = chunks;
-        s_groups[j] = (chunks + kBatchGroup - 1) / kBatchGroup;
-      }
+  __shared__ uint32_t sh[8], scan_c[8], scan_g[8];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t per = (n_states + gridDim.x - 1) / gridDim.x;
+  const uint32_t s0 = min(blockIdx.x * per, n_states), s1 = min(s0 + per, n_states);
+  uint32_t before_c = 0, before_g = 0, all_c = 0;
+  for (uint32_t j = tid; j < n_states; j += 256) {
+    const uint32_t n = n_rays[j];
+    const uint32_t chunks = n <= max_rays ? ((n << state_lg_segs(k, n)) + 31) / 32 : 0u;
+    all_c += chunks;
+    if (j < s0) {
+      before_c += chunks;
+      before_g += (chunks + kBatchGroup - 1) / kBatchGroup;
     }
-    __syncthreads();
-    const uint32_t chunks = tid < tile ? s_chunks[tid] : 0u;
-    const uint32_t groups = tid < tile ? s_groups[tid] : 0u;
+  }
+  before_c = block_sum256(before_c, sh);
+  before_g = block_sum256(before_g, sh);
+  if (blockIdx.x == 0) {
+    all_c = block_sum256(all_c, sh);
+    if (tid == 0) {
+      hdr->next_chunk = 0;
+      hdr->total_chunks = all_c;
+      hdr->n_states = n_states;
+    }
+  }
+  const uint32_t first_g = before_g;
+  for (uint32_t base = s0; base < s1; base += 256) {
+    const uint32_t tile = min(256u, s1 - base);
+    const uint32_t n = tid < tile ? n_rays[base + tid] : 0u;
+    const uint32_t lg = state_lg_segs(k, n);
+    const uint32_t chunks = n <= max_rays ? ((n << lg) + 31) / 32 : 0u;
+    const uint32_t groups = (chunks + kBatchGroup - 1) / kBatchGroup;
     uint32_t ic = chunks, ig = groups;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -1552,55 +1548,67 @@ __global__ void __launch_bounds__(1024) batch_prep_kernel(
         ig += g2;
       }
     }
+    __syncthreads();                                // the last tile's scan is no longer read
     if (lane == 31) {
-      wsum_c[warp] = ic;
-      wsum_g[warp] = ig;
+      scan_c[warp] = ic;
+      scan_g[warp] = ig;
     }
     __syncthreads();
-    if (warp == 0) {
-      uint32_t wc = lane < nwarps ? wsum_c[lane] : 0u;
-      uint32_t wg = lane < nwarps ? wsum_g[lane] : 0u;
+    uint32_t all_tc = 0, all_tg = 0;
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const uint32_t c2 = __shfl_up_sync(0xffffffffu, wc, off);
-        const uint32_t g2 = __shfl_up_sync(0xffffffffu, wg, off);
-        if (lane >= (uint32_t)off) {
-          wc += c2;
-          wg += g2;
-        }
+    for (uint32_t w = 0; w < 8; ++w) {
+      if (w == warp) {
+        ic += all_tc;
+        ig += all_tg;
       }
-      wsum_c[lane] = wc;   // inclusive over warps
-      wsum_g[lane] = wg;
+      all_tc += scan_c[w];
+      all_tg += scan_g[w];
     }
-    __syncthreads();
-    const uint32_t pre_c = carry_c + (warp ? wsum_c[warp - 1] : 0u) + ic - chunks;
-    const uint32_t pre_g = carry_g + (warp ? wsum_g[warp - 1] : 0u) + ig - groups;
     if (tid < tile) {
-      const uint32_t b = base + tid;
-      bs[b].chunk0 = pre_c;
-      bs[b].group0 = pre_g;
-      sticket[b] = 0;
-      if (chunks == 0) {
-        rmp_result_t r;
-        memset(&r, 0, sizeof(r));
-        r.n_rays = bs[b].n_rays;
-        r.status = bs[b].status;
-        out[b] = r;
+      BatchState* sp = bs + base + tid;
+      sp->n_rays = n;
+      sp->chunk0 = before_c + ic - chunks;
+      sp->n_chunks = chunks;
+      sp->group0 = before_g + ig - groups;
+      sp->lg_segs = lg;
+      sticket[base + tid] = 0;
+    }
+    before_c += all_tc;
+    before_g += all_tg;
+    for (uint32_t j = warp; j < tile; j += 8) {
+      const uint32_t b = base + j;
+      const uint32_t nb = n_rays[b];
+      const double* x = states + 6 * (size_t)b;
+      BatchState* sp = bs + b;
+      bool bad = false;
+      if (lane < 3) {
+        const double o = m.kind != RMP_MAP_DENSE_U8 ? 0.0
+                         : (lane == 0 ? m.origin[0] : (lane == 1 ? m.origin[1] : m.origin[2]));
+        const double q = __dmul_rn(__ddiv_rn(__dsub_rn(x[lane], o), m.vs), 65536.0);
+        bad = !(fabs(q) < 274877906944.0);
+        sp->P[lane] = bad ? 0 : __double2ll_rn(q);
+      } else if (lane < 6) {
+        const double v = x[lane];
+        const float vh = __double2float_rn(v);
+        sp->v[lane - 3] = vh;
+        sp->vl[lane - 3] = __double2float_rn(__dsub_rn(v, (double)vh));
+      }
+      bad = __any_sync(0xffffffffu, bad) || nb > max_rays;
+      const uint32_t M = nb >= 32 ? pick_cells_warp(nb) : 1u;
+      if (lane == 0) {
+        sp->status = bad ? RMP_ERR_INVALID_ARG : RMP_OK;
+        sp->perm_M = M;
+        sp->perm_Q = nb / M;
+      }
+      if (bad || nb == 0) {                         // 18 8-byte words of result
+        const unsigned long long w =
+            lane == 15 ? (unsigned long long)nb
+                       : (lane == 17 && bad ? (unsigned long long)RMP_ERR_INVALID_ARG : 0ull);
+        if (lane < 18) reinterpret_cast<unsigned long long*>(out + b)[lane] = w;
       }
     }
-    __syncthreads();
-    if (tid == blockDim.x - 1) {
-      carry_c = pre_c + chunks;
-      carry_g = pre_g + groups;
-    }
-    __syncthreads();
   }
-  for (uint32_t i = tid; i < carry_g; i += blockDim.x) gticket[i] = 0;
-  if (tid == 0) {
-    hdr->next_chunk = 0;
-    hdr->total_chunks = carry_c;
-    hdr->n_states = n_states;
-  }
+  for (uint32_t i = first_g + tid; i < before_g; i += 256) gticket[i] = 0;
 }
 
 // Lane i's terms and counts of a chunk partial (FP32 pairs for the compensated reduction, as
@@ -1880,6 +1888,10 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
     }
     const uint32_t b = lo;
     const BatchState* sp = bs + b;
+    if (__ldg(&sp->status) != RMP_OK) {              // its result is the prep kernel's
+      c = __shfl_sync(0xffffffffu, cn, 0);
+      continue;
+    }
     const long long P[3] = {__ldg(&sp->P[0]), __ldg(&sp->P[1]), __ldg(&sp->P[2])};
     const uint32_t n_b = __ldg(&sp->n_rays), chunk0 = __ldg(&sp->chunk0);
     const uint32_t q = c - chunk0;
@@ -2772,7 +2784,9 @@ cudaError_t launch_batch(const DevMap& m, const EvalConsts& k, const double* sta
   uint32_t* gticket = (uint32_t*)(w + L.gticket);
   CtaPartial* cparts = (CtaPartial*)(w + L.cparts);
   CtaPartial* gparts = (CtaPartial*)(w + L.gparts);
-  batch_prep_kernel<<<1, 1024, 0, stream>>>(states_dev, n_rays_dev, n_states, max_rays, m, k, hdr,
+  // 8 states a CTA (a warp each) as far as the SMs go; longer runs beyond
+  const unsigned prep = n_states < 8u * 152u ? (n_states + 7u) / 8u : 152u;
+  batch_prep_kernel<<<prep, 256, 0, stream>>>(states_dev, n_rays_dev, n_states, max_rays, m, k, hdr,
                                             bs, sticket, gticket, out_dev);
   if (m.kind == RMP_MAP_DENSE_U8)
     launch_batch_r<RMP_MAP_DENSE_U8, kLayoutGrid>(m, k, hdr, bs, sticket, gticket, cparts, gparts,
