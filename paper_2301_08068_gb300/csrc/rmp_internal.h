@@ -125,10 +125,12 @@ inline cudaError_t workspace_reset(void* ws, cudaStream_t s) {
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // ------------------------------------------------------------------ batched evaluation
-// Work of a batch is cut into chunks of 32 threads (32 / S rays of one state, S segments
-// per ray, S chosen per state) that the warps of a persistent grid take from a counter.  Each chunk stores a
-// partial; kBatchGroup consecutive chunks of a state form a group (the last chunk of a
-// group to finish sums them), and the last group of a state sums the groups and resolves.
+// A state's rays are summed in partials of 32 / S rays (S a function of its ray count and the
+// launch shape), kBatchGroup consecutive ones a group (the warp that completes a group sums it),
+// and the last group of a state sums the groups and resolves.  Work is another cut of the same
+// rays: chunks of 32 threads (32 / s rays, s <= S segments marched per ray, s from the whole
+// batch's load) that the warps of a persistent grid take from a counter; a chunk stores S / s
+// partials.  s therefore changes no bit of a result.
 constexpr uint32_t kBatchGroup = 32;
 constexpr uint32_t kMaxBatchStates = 1u << 16;
 constexpr uint32_t kMaxBatchSegs = 4;        // workspace is sized for up to 4 segments per ray
@@ -136,15 +138,15 @@ constexpr uint32_t kMaxBatchSegs = 4;        // workspace is sized for up to 4 s
 struct BatchState {         // 80 bytes, written by the prep kernel
   long long P[3];           // quantised position (2^-16 voxels)
   float v[3], vl[3];        // velocity as an FP32 pair
-  uint32_t n_rays, chunk0, n_chunks, group0;
+  uint32_t n_rays, work0, part0, group0;   // first work chunk, partial and group
   uint32_t perm_M, perm_Q;  // direction cells (the remainder n_rays - perm_Q perm_M is derived)
-  uint32_t lg_segs;         // log2 segments per ray of this state
+  uint32_t lg_segs;         // log2 S | log2 s << 8
   int status;               // RMP_OK or RMP_ERR_INVALID_ARG
 };
 
 struct BatchHeader {        // 128 bytes
   uint32_t next_chunk;      // work counter of the persistent grid
-  uint32_t total_chunks;
+  uint32_t total_chunks;    // work chunks
   uint32_t n_states;
   uint32_t pad[29];
 };

@@ -1482,6 +1482,18 @@ __device__ __forceinline__ uint32_t state_lg_segs(const EvalConsts& k, uint32_t 
   return lg;
 }
 
+// Segments marched per ray (log2), at most the summation's: a tuned launch marches those, the
+// default the most whose threads fill half of the persistent launch over the whole batch of
+// `total` rays -- beyond that, the extra segments' set-up costs more than their shorter chains
+// save (256 states, 5.3 M rays: 1 / 2 / 4 segments 458 / 745 / 1252 us; 16 states, 50 k rays: 36 /
+// 38 / 50; one state of 16384: 44 / 37 / 35).
+__device__ __forceinline__ uint32_t march_lg_segs(const EvalConsts& k, uint32_t lg_sum,
+                                                  unsigned long long total) {
+  if (k.lg_segs <= 2u) return lg_sum;
+  while (lg_sum > 0u && (total << lg_sum) > k.seg_threads / 2) --lg_sum;
+  return lg_sum;
+}
+
 // Sum of x over the CTA's threads (256), in every thread; sh: 8 words.
 __device__ __forceinline__ uint32_t block_sum256(uint32_t x, uint32_t* sh) {
   x = __reduce_add_sync(0xffffffffu, x);
@@ -1507,27 +1519,37 @@ __global__ void __launch_bounds__(256) batch_prep_kernel(
     const double* __restrict__ states, const uint32_t* __restrict__ n_rays, uint32_t n_states,
     uint32_t max_rays, DevMap m, EvalConsts k, BatchHeader* hdr, BatchState* bs,
     uint32_t* sticket, uint32_t* gticket, rmp_result_t* out) {
-  __shared__ uint32_t sh[8], scan_c[8], scan_g[8];
+  __shared__ uint32_t sh[8], scan[3][8];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t per = (n_states + gridDim.x - 1) / gridDim.x;
   const uint32_t s0 = min(blockIdx.x * per, n_states), s1 = min(s0 + per, n_states);
-  uint32_t before_c = 0, before_g = 0, all_c = 0;
+  // rays of the batch in units of 16, rounded up per state (32 bits hold them: a workspace takes
+  // about 10 bytes a ray)
+  uint32_t load = 0;
+  for (uint32_t j = tid; j < n_states; j += 256)
+    load += n_rays[j] <= max_rays ? (n_rays[j] + 15) / 16 : 0u;
+  const unsigned long long total = 16ull * block_sum256(load, sh);
+  uint32_t before_w = 0, before_p = 0, before_g = 0, all_w = 0;
   for (uint32_t j = tid; j < n_states; j += 256) {
     const uint32_t n = n_rays[j];
-    const uint32_t chunks = n <= max_rays ? ((n << state_lg_segs(k, n)) + 31) / 32 : 0u;
-    all_c += chunks;
+    if (n > max_rays) continue;
+    const uint32_t lg = state_lg_segs(k, n), parts = ((n << lg) + 31) / 32;
+    const uint32_t work = ((n << march_lg_segs(k, lg, total)) + 31) / 32;
+    all_w += work;
     if (j < s0) {
-      before_c += chunks;
-      before_g += (chunks + kBatchGroup - 1) / kBatchGroup;
+      before_w += work;
+      before_p += parts;
+      before_g += (parts + kBatchGroup - 1) / kBatchGroup;
     }
   }
-  before_c = block_sum256(before_c, sh);
+  before_w = block_sum256(before_w, sh);
+  before_p = block_sum256(before_p, sh);
   before_g = block_sum256(before_g, sh);
   if (blockIdx.x == 0) {
-    all_c = block_sum256(all_c, sh);
+    all_w = block_sum256(all_w, sh);
     if (tid == 0) {
       hdr->next_chunk = 0;
-      hdr->total_chunks = all_c;
+      hdr->total_chunks = all_w;
       hdr->n_states = n_states;
     }
   }
@@ -1535,46 +1557,44 @@ __global__ void __launch_bounds__(256) batch_prep_kernel(
   for (uint32_t base = s0; base < s1; base += 256) {
     const uint32_t tile = min(256u, s1 - base);
     const uint32_t n = tid < tile ? n_rays[base + tid] : 0u;
-    const uint32_t lg = state_lg_segs(k, n);
-    const uint32_t chunks = n <= max_rays ? ((n << lg) + 31) / 32 : 0u;
-    const uint32_t groups = (chunks + kBatchGroup - 1) / kBatchGroup;
-    uint32_t ic = chunks, ig = groups;
+    const uint32_t lg = state_lg_segs(k, n), lgs = march_lg_segs(k, lg, total);
+    const uint32_t nv = n <= max_rays ? n : 0u;
+    // work chunks, partials and groups of this thread's state, then their inclusive scans
+    const uint32_t v[3] = {((nv << lgs) + 31) / 32, ((nv << lg) + 31) / 32,
+                           (((nv << lg) + 31) / 32 + kBatchGroup - 1) / kBatchGroup};
+    uint32_t inc[3] = {v[0], v[1], v[2]};
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const uint32_t c2 = __shfl_up_sync(0xffffffffu, ic, off);
-      const uint32_t g2 = __shfl_up_sync(0xffffffffu, ig, off);
-      if (lane >= (uint32_t)off) {
-        ic += c2;
-        ig += g2;
+    for (int off = 1; off < 32; off <<= 1)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc[i], off);
+        if (lane >= (uint32_t)off) inc[i] += y;
       }
-    }
     __syncthreads();                                // the last tile's scan is no longer read
-    if (lane == 31) {
-      scan_c[warp] = ic;
-      scan_g[warp] = ig;
-    }
-    __syncthreads();
-    uint32_t all_tc = 0, all_tg = 0;
+    if (lane == 31)
 #pragma unroll
-    for (uint32_t w = 0; w < 8; ++w) {
-      if (w == warp) {
-        ic += all_tc;
-        ig += all_tg;
+      for (int i = 0; i < 3; ++i) scan[i][warp] = inc[i];
+    __syncthreads();
+    uint32_t all[3] = {0, 0, 0};
+#pragma unroll
+    for (uint32_t w = 0; w < 8; ++w)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        if (w == warp) inc[i] += all[i];
+        all[i] += scan[i][w];
       }
-      all_tc += scan_c[w];
-      all_tg += scan_g[w];
-    }
     if (tid < tile) {
       BatchState* sp = bs + base + tid;
       sp->n_rays = n;
-      sp->chunk0 = before_c + ic - chunks;
-      sp->n_chunks = chunks;
-      sp->group0 = before_g + ig - groups;
-      sp->lg_segs = lg;
+      sp->work0 = before_w + inc[0] - v[0];
+      sp->part0 = before_p + inc[1] - v[1];
+      sp->group0 = before_g + inc[2] - v[2];
+      sp->lg_segs = lg | (lgs << 8);
       sticket[base + tid] = 0;
     }
-    before_c += all_tc;
-    before_g += all_tg;
+    before_w += all[0];
+    before_p += all[1];
+    before_g += all[2];
     for (uint32_t j = warp; j < tile; j += 8) {
       const uint32_t b = base + j;
       const uint32_t nb = n_rays[b];
@@ -1781,30 +1801,30 @@ __global__ void rollout_step_kernel(DevMap m, RolloutConsts rc, const rmp_result
   else if (running) atomicAdd(running, 1u);
 }
 
-// The last chunk of a group sums the group's chunk partials into a group partial; the last
-// group of a state sums the state's groups, adds the attractor (combined evaluations) and
+// The last chunk of a group sums the group's partials into a group partial; the last group
+// of a state sums the state's groups, adds the attractor (combined evaluations) and
 // resolves.  Called by all 32 lanes of the warp whose chunk completed the group.  Kept
-// out of line: it runs once per 32 chunks, and inlined it would sit between the march
-// loops in the instruction stream.  A chunk partial's FP32 pairs become FP64 here, one chunk
+// out of line: it runs once per 32 partials, and inlined it would sit between the march
+// loops in the instruction stream.  A partial's FP32 pairs become FP64 here, one partial
 // per lane, not where they are stored: an FP64 instruction holds a scheduler's pipe about 64
 // cycles whatever the active lanes (256 states: 17.2 M -> 1.3 M FP64 warp instructions; with the
 // shared-out trees 1289 -> 1000 us).
 template <int RED>
 __device__ __noinline__ void batch_group_finish(const EvalConsts& k, CtaPartial* cparts,
                                                 CtaPartial* gparts, uint32_t* sticket,
-                                                uint32_t chunk0, uint32_t gi, uint32_t gsz,
-                                                uint32_t n_chunks, uint32_t group0, uint32_t b,
+                                                uint32_t part0, uint32_t gi, uint32_t gsz,
+                                                uint32_t n_parts, uint32_t group0, uint32_t b,
                                                 uint32_t n_b, const double* states,
                                                 const double* goals, rmp_result_t* out) {
   const uint32_t lane = threadIdx.x & 31;
-  // last chunk of its group: sum the group's chunk partials (lane i: chunk i)
+  // the group's partials, lane i: partial i
   __threadfence();
   double gv[9] = {0., 0., 0., 0., 0., 0., 0., 0., 0.};
   unsigned gh = 0, ga = 0;
   if (lane < gsz)
-    load_partial<RED == RMP_REDUCE_KAHAN32>(cparts + chunk0 + gi * kBatchGroup + lane, gv, gh, ga);
+    load_partial<RED == RMP_REDUCE_KAHAN32>(cparts + part0 + gi * kBatchGroup + lane, gv, gh, ga);
   warp_sum_partial(gv, gh, ga, gparts + group0 + gi);
-  const uint32_t n_groups = (n_chunks + kBatchGroup - 1) / kBatchGroup;
+  const uint32_t n_groups = (n_parts + kBatchGroup - 1) / kBatchGroup;
   __threadfence();
   __syncwarp();
   uint32_t last = 0;
@@ -1852,13 +1872,13 @@ __device__ __noinline__ void batch_group_finish(const EvalConsts& k, CtaPartial*
   }
 }
 
-// Persistent batched evaluation: every warp takes chunks (its own index first, then from
-// the work counter) until none is left; a chunk is 32 / S rays of one state (coherent ray order of that state), marched
-// and evaluated as in the single-state kernel.  The chunk's 9 terms are summed over the
-// warp (compensated FP32 or FP64 tree), stored, and the chunk's group and state tickets
-// decide which warp sums a group (<= 32 chunk partials, one per lane) and which one sums
-// the state's groups and resolves it -- every sum in a fixed order, so results do not
-// depend on which warp ran which chunk.
+// Persistent batched evaluation: every warp takes work chunks (its own index first, then from
+// the work counter) until none is left; a chunk is 32 / s rays of one state (coherent ray order of
+// that state), marched and evaluated as in the single-state kernel.  Each partial's 9 terms are
+// summed over its lanes (compensated FP32 or FP64 tree), stored, and the partial's group and the
+// state's tickets decide which warp sums a group (<= 32 partials, one per lane) and which one
+// sums the state's groups and resolves it -- every sum in a fixed order, so results do not
+// depend on which warp ran which chunk, nor on s.
 // Register budget 64 (launch bounds 256 x 4): 32 warps per SM hide each other's latency; the
 // per-state values used only after the march are read after it.
 template <int KIND, int LAYOUT, int RED>
@@ -1883,7 +1903,7 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
     uint32_t lo = 0, hi = nst;
     while (hi - lo > 1) {
       const uint32_t mid = (lo + hi) >> 1;
-      if (__ldg(&bs[mid].chunk0) <= c) lo = mid;
+      if (__ldg(&bs[mid].work0) <= c) lo = mid;
       else hi = mid;
     }
     const uint32_t b = lo;
@@ -1893,62 +1913,79 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
       continue;
     }
     const long long P[3] = {__ldg(&sp->P[0]), __ldg(&sp->P[1]), __ldg(&sp->P[2])};
-    const uint32_t n_b = __ldg(&sp->n_rays), chunk0 = __ldg(&sp->chunk0);
-    const uint32_t q = c - chunk0;
-    const uint32_t lgS = __ldg(&sp->lg_segs), S = 1u << lgS;
+    const uint32_t n_b = __ldg(&sp->n_rays);
+    const uint32_t q = c - __ldg(&sp->work0);
+    const uint32_t lgs = __ldg(&sp->lg_segs) >> 8, S = 1u << lgs;
     const uint32_t g = q * 32 + lane;
-    const uint32_t slot = g >> lgS, seg = g & (S - 1);
+    const uint32_t slot = g >> lgs, seg = g & (S - 1);
     const bool active = slot < n_b;
     const uint32_t pM = __ldg(&sp->perm_M), pQ = __ldg(&sp->perm_Q);
     const uint32_t ray_idx = ray_of_slot_p(active ? slot : 0, pM, pQ, n_b - pQ * pM);
     const Ray ray = make_ray(ray_idx + k.halton_offset);
     const size_t ro = (size_t)b * max_rays + ray_idx;
     uint32_t en, ea;
-    const int mstat = march_ray<KIND, LAYOUT>(m, k, P, ray, seg, lgS, active, en, ea,
+    const int mstat = march_ray<KIND, LAYOUT>(m, k, P, ray, seg, lgs, active, en, ea,
                                               hits ? hits + ro : nullptr);
     // read after the march, so that they are not held in registers across it
     const float v[3] = {__ldg(&sp->v[0]), __ldg(&sp->v[1]), __ldg(&sp->v[2])};
     const float vl[3] = {__ldg(&sp->vl[0]), __ldg(&sp->vl[1]), __ldg(&sp->vl[2])};
-    const uint32_t n_chunks = __ldg(&sp->n_chunks), group0 = __ldg(&sp->group0);
+    const uint32_t part0 = __ldg(&sp->part0), group0 = __ldg(&sp->group0);
+    const uint32_t lg = __ldg(&sp->lg_segs) & 255u, lgW = lg - lgs;
     float vals[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     unsigned nh = 0, na = 0;
-    if (active && seg == 0) {
+    if (active && seg == 0)
       ray_outputs(m, k, ray, mstat, en, ea, v, vl, per_ray ? per_ray + 9 * ro : nullptr, vals, nh,
                   na);
+    // the chunk's 2^lgW partials, 32 >> lgW lanes each (a ray's other segments hold zeros)
+    const uint32_t n_parts = ((n_b << lg) + 31) / 32;
+    const uint32_t first = q << lgW, mine = first + (lane >> (5 - lgW));
+    uint32_t cnt = nh | (na << 16);
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      const uint32_t off = 16u >> (lgW + j);
+      if (off) cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
     }
-    // chunk partial
-    CtaPartial* part = cparts + chunk0 + q;
+    const WarpTerms t = warp_terms(lgW);
+    CtaPartial* part = cparts + part0 + mine;
     if (RED == RMP_REDUCE_FP64) {
       double pv[9];
 #pragma unroll
       for (int i = 0; i < 9; ++i) pv[i] = (double)vals[i];
-      warp_sum_partial(pv, nh, na, part);
-    } else {
-      const WarpTerms t = warp_terms(0);
-      float cv[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      warp_reduce_terms<float, true>(vals, cv, 0);
-      nh = __reduce_add_sync(0xffffffffu, nh);
-      na = __reduce_add_sync(0xffffffffu, na);
-      CtaPartial32* p = reinterpret_cast<CtaPartial32*>(part);
-      if (t.n > 0) {
-        p->s[t.first] = vals[0];
-        p->c[t.first] = cv[0];
+      warp_reduce_terms<double, false>(pv, pv, lgW);
+      if (mine < n_parts) {
+        if (t.n > 0) part->v[t.first] = pv[0];
+        if (t.n > 1) part->v[t.first + 1] = pv[1];
       }
-      if (lane == 0) {
-        p->n_hits = nh;
-        p->n_active = na;
+    } else {
+      float cv[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      warp_reduce_terms<float, true>(vals, cv, lgW);
+      CtaPartial32* p = reinterpret_cast<CtaPartial32*>(part);
+      if (mine < n_parts) {
+        if (t.n > 0) {
+          p->s[t.first] = vals[0];
+          p->c[t.first] = cv[0];
+        }
+        if (t.n > 1) {
+          p->s[t.first + 1] = vals[1];
+          p->c[t.first + 1] = cv[1];
+        }
       }
     }
-    const uint32_t gi = q / kBatchGroup;
-    const uint32_t gsz = min(kBatchGroup, n_chunks - gi * kBatchGroup);
+    if (mine < n_parts && (lane & ((32u >> lgW) - 1)) == 0) {
+      part->n_hits = cnt & 0xffffu;
+      part->n_active = cnt >> 16;
+    }
+    const uint32_t gi = first / kBatchGroup;
+    const uint32_t gsz = min(kBatchGroup, n_parts - gi * kBatchGroup);
+    const uint32_t stored = min(1u << lgW, n_parts - first);
     uint32_t stage = 0;
     __threadfence();
     __syncwarp();
-    if (lane == 0) stage = atomicAdd(&gticket[group0 + gi], 1u) == gsz - 1 ? 1u : 0u;
+    if (lane == 0) stage = atomicAdd(&gticket[group0 + gi], stored) + stored == gsz ? 1u : 0u;
     stage = __shfl_sync(0xffffffffu, stage, 0);
     if (stage)
-      batch_group_finish<RED>(k, cparts, gparts, sticket, chunk0, gi, gsz, n_chunks, group0, b,
-                              n_b, states, goals, out);
+      batch_group_finish<RED>(k, cparts, gparts, sticket, part0, gi, gsz, n_parts, group0, b, n_b,
+                              states, goals, out);
     c = __shfl_sync(0xffffffffu, cn, 0);
   }
 }
