@@ -293,27 +293,38 @@ __device__ __forceinline__ uint32_t block_entry(const DevMap& m, const uint32_t*
   return 0x80000000u | slot;
 }
 
+// 1 / x to an ulp or so; infinity for 0.
+__device__ __forceinline__ float recip_fast(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // March a piece from state st until a hit, a map exit or the limits L (returns `at_limit`; st is
 // then not the piece's end, which piece_start gives in closed form when it is wanted).
+// Called by all lanes of the warp (`work` false: nothing to march), which meet at every box:
+// left to itself, the compiler lets lanes whose paths parted (free or occupied block, a hit)
+// run on as separate groups, and a pass then costs a multiple of its ~120 instructions.
 // Bound by the chain from one box to the next (a block entry, a byte of the box field, the
-// exit axis by exact 64-bit comparisons, the crossing counts of the other two axes), about
-// 120 instructions with two dependent loads; the field's lines stay in L1, which holds all
-// of the SM's 228 KB since nothing is staged in shared memory.  Measured against a march over
-// symmetric free boxes of blocks with a voxel walk inside occupied blocks: 65536 rays on the
-// 40 m map 54 -> 31.6 us, 262144 rays on the 100 m map 101.6 -> 42.8 us, 256 states of
-// 4096-65536 rays 2677 -> 1289 us.
+// exit axis by exact 64-bit comparisons, the crossing counts of the other two axes) with two
+// dependent loads; the field's lines stay in L1, which holds all of the SM's 228 KB since
+// nothing is staged in shared memory.  Measured against a march over symmetric free boxes of
+// blocks with a voxel walk inside occupied blocks: 65536 rays on the 40 m map 54 -> 22 us,
+// 262144 rays on the 100 m map 101.6 -> 36.7 us.
 template <int KIND, int LAYOUT>
 __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const RayFx& r,
-                                         const uint32_t L[3], int at_limit) {
+                                         const uint32_t L[3], int at_limit, bool work) {
   const uint32_t* A = r.A;
   int* q = st.q;
   const bool up[3] = {(r.up & 1u) != 0, (r.up & 2u) != 0, (r.up & 4u) != 0};
-  const float rA[3] = {__frcp_rn(__uint2float_rn(A[0])) * (1.0f / 65536.0f),
-                       __frcp_rn(__uint2float_rn(A[1])) * (1.0f / 65536.0f),
-                       __frcp_rn(__uint2float_rn(A[2])) * (1.0f / 65536.0f)};
+  const float rA[3] = {recip_fast(__uint2float_rn(A[0])) * (1.0f / 65536.0f),
+                       recip_fast(__uint2float_rn(A[1])) * (1.0f / 65536.0f),
+                       recip_fast(__uint2float_rn(A[2])) * (1.0f / 65536.0f)};
   int hi[3];                                        // first voxel beyond the map / the grid
   int step[4] = {0, 0, 0, 0};                       // signed brick strides and the first brick
   const uint32_t* top = m.top;
+  int status = at_limit;
+  bool run = work;
   if (LAYOUT == kLayoutGrid) {
     const int str[3] = {1, m.gdim[0], m.gdim[0] * m.gdim[1]};
 #pragma unroll
@@ -322,20 +333,23 @@ __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const 
       step[a] = up[a] ? str[a] : -str[a];
       step[3] += up[a] ? 0 : (m.gdim[a] - 1) * str[a];
       // a dense map: a piece that starts outside has left the map
-      if (KIND == RMP_MAP_DENSE_U8 && !up[a] && q[a] < 8 * m.gdim[a] - m.dims[a])
-        return RMP_RAY_MISS_EXIT;
+      if (KIND == RMP_MAP_DENSE_U8 && !up[a] && q[a] < 8 * m.gdim[a] - m.dims[a]) {
+        status = RMP_RAY_MISS_EXIT;
+        run = false;
+      }
     }
     top += (size_t)r.up * ((size_t)str[2] * m.gdim[2]) + step[3];
   }
   const uint8_t* box = reinterpret_cast<const uint8_t*>(m.cells) + 512 * r.up;
-  // every pass advances at least one voxel
+  // every pass advances each running lane by at least one voxel
   for (uint32_t it = 0; it < 8u * (kMaxRangeVoxels + 2); ++it) {
+    if (!__any_sync(0xffffffffu, run)) break;
+    if (!run) continue;
     int end[3];                                     // first voxel beyond the free box
     bool inside = true;
     if (LAYOUT == kLayoutGrid)
       inside = (unsigned)q[0] < (unsigned)hi[0] && (unsigned)q[1] < (unsigned)hi[1] &&
                (unsigned)q[2] < (unsigned)hi[2];
-    if (KIND == RMP_MAP_DENSE_U8 && !inside) return RMP_RAY_MISS_EXIT;
     if (inside) {
       const int b[3] = {q[0] >> 3, q[1] >> 3, q[2] >> 3};
       const uint32_t* brick = nullptr;
@@ -349,7 +363,10 @@ __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const 
           const uint32_t w = p ^ ((up[0] ? 0u : 7u) | (up[1] ? 0u : 56u) | (up[2] ? 0u : 448u));
           e = (__ldg(brick + (w >> 5)) >> (w & 31u)) & 1u ? 0u : 64u;
         }
-        if (e == 0u) return RMP_RAY_HIT;
+      }
+      if (occupied && e == 0u) {
+        status = RMP_RAY_HIT;
+        run = false;
       }
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
@@ -358,9 +375,11 @@ __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const 
         if (KIND == RMP_MAP_DENSE_U8) end[a] = min(end[a], hi[a]);
       }
     } else {
-      // outside the grid of a hashed map: nothing ahead once it lies behind on any axis, else
-      // every voxel short of it is free (at most 240 at once, see crossings_before)
-      if (q[0] >= hi[0] || q[1] >= hi[1] || q[2] >= hi[2]) return at_limit;
+      // a dense map is left; outside the grid of a hashed map there is nothing ahead once it
+      // lies behind on any axis, else every voxel short of it is free (at most 240 at once,
+      // see crossings_before)
+      if (KIND == RMP_MAP_DENSE_U8) status = RMP_RAY_MISS_EXIT;
+      run = KIND != RMP_MAP_DENSE_U8 && q[0] < hi[0] && q[1] < hi[1] && q[2] < hi[2];
       const int gap = min(max(-q[0], max(-q[1], -q[2])), 240);
 #pragma unroll
       for (int a = 0; a < 3; ++a) end[a] = q[a] + gap;
@@ -373,7 +392,8 @@ __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const 
     const uint32_t Fw = y ? F[1] : F[0], Aw = y ? A[1] : A[0];
     const bool z = (unsigned long long)F[2] * Aw < (unsigned long long)Fw * A[2];
     const uint32_t Fe = z ? F[2] : Fw, Ae = z ? A[2] : Aw;
-    if (Fe > (z ? L[2] : (y ? L[1] : L[0]))) return at_limit;
+    run = run && Fe <= (z ? L[2] : (y ? L[1] : L[0]));
+    if (!run) continue;
     const float rE = z ? rA[2] : (y ? rA[1] : rA[0]);
     // the other two axes, i < j: i is x unless x exits, j is z unless z exits
     const bool x = !y && !z;
@@ -388,7 +408,7 @@ __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const 
     st.a_last = Ae;
     st.ax_last = z ? 2 : (y ? 1 : 0);
   }
-  return at_limit;
+  return status;
 }
 
 __device__ __forceinline__ bool piece_final(int status) {
@@ -1280,9 +1300,8 @@ __device__ __forceinline__ int march_ray(const DevMap& m, const EvalConsts& k, c
   ray_fx<LAYOUT>(m, P, ray.D, r);
   piece_start(r, k.R_fx, j_lo, st);
   limits_at(r, k.R_fx, j_hi, L);
-  int status = kSegContinues;
-  if (work)
-    status = march_run<KIND, LAYOUT>(m, st, r, L, seg == S - 1 ? RMP_RAY_MISS_RANGE : kSegContinues);
+  const int status = march_run<KIND, LAYOUT>(
+      m, st, r, L, seg == S - 1 ? RMP_RAY_MISS_RANGE : kSegContinues, work);
   const uint32_t ballot = __ballot_sync(0xffffffffu, work && piece_final(status));
   const uint32_t grp0 = lane & ~(S - 1);
   const uint32_t gmask = (S == 32 ? 0xffffffffu : ((1u << S) - 1u)) << grp0;
