@@ -12,6 +12,7 @@
 // ray) use explicitly rounded intrinsics (__fmul_rn, __fmaf_rn, ...) so that no
 // contraction or fast-math rewrite can change them.
 #include <climits>
+#include <type_traits>
 
 #include "rmp_internal.h"
 
@@ -155,18 +156,19 @@ __device__ __forceinline__ int hash_lookup(const DevMap& m, int bx, int by, int 
 //
 // Reflected frame.  Axes the ray descends are mirrored (k -> ~k), so every ray climbs; the
 // frame's origin is the grid's first block in that direction.  Voxel q_a, block q_a >> 3,
-// voxel in its block q_a & 7, and N_a = (q_a << 16) + C_a (mod 2^32, exact since N < 2^31).
+// voxel in its block q_a & 7; q_a and N_a grow together, one voxel and 2^16 a crossing.
 constexpr int kSegContinues = 0;   // piece ended at its upper parameter bound
 constexpr int kGridLog = 7;        // pieces of a ray are cut at multiples of R / 2^kGridLog
 
 struct RayFx {
   int q0[3];                // start voxel, reflected frame
-  uint32_t C[3], A[3];      // N_a = (q_a << 16) + C_a; |D_a|
+  uint32_t N0[3], A[3];     // its N_a; |D_a|
   uint32_t up;              // bit a: D_a > 0 (not mirrored); the octant of the box field
 };
 
 struct MarchState {
   int q[3];                 // voxel, reflected frame
+  uint32_t N[3];
   uint32_t n_last, a_last;  // entry numerator / |D| of the current voxel (0/1 at the start)
   int ax_last;              // axis of the last step (for map exits)
 };
@@ -194,9 +196,9 @@ __device__ __forceinline__ void ray_fx(const DevMap& m, const long long P[3], co
     r.up |= up ? 1u << a : 0u;
     r.q0[a] = (up ? k : ~k) - 8 * lo;
     r.A[a] = (uint32_t)abs(D[a]);
-    const uint32_t p = (uint32_t)P[a], first = ((uint32_t)(8 * lo) + 1u) << 16;
+    const uint32_t frac = (uint32_t)P[a] & 0xffffu;
     // D_a = 0 is mirrored like a descending axis; N_a >= 1 keeps it from ever winning
-    r.C[a] = (up ? first - p : first + p) + (D[a] == 0 ? 1u : 0u);
+    r.N0[a] = up ? 65536u - frac : (D[a] == 0 ? frac + 1u : frac);
   }
 }
 
@@ -226,17 +228,19 @@ __device__ __forceinline__ void piece_start(const RayFx& r, long long R_fx, uint
   st.a_last = 1;
   st.ax_last = 0;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) st.q[a] = r.q0[a];
+  for (int a = 0; a < 3; ++a) {
+    st.q[a] = r.q0[a];
+    st.N[a] = r.N0[a];
+  }
   if (j == 0) return;
   bool any = false;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const uint32_t N0 = ((uint32_t)r.q0[a] << 16) + r.C[a];
     const unsigned long long X = (unsigned long long)j * (unsigned long long)R_fx * r.A[a];
-    const unsigned long long Y = (unsigned long long)N0 << (24 + kGridLog);
+    const unsigned long long Y = (unsigned long long)r.N0[a] << (24 + kGridLog);
     if (r.A[a] != 0 && X >= Y) {
       const uint32_t cnt = (uint32_t)((X - Y) >> (40 + kGridLog)) + 1;
-      const uint32_t nl = N0 + ((cnt - 1) << 16);
+      const uint32_t nl = r.N0[a] + ((cnt - 1) << 16);
       if (!any || (unsigned long long)nl * st.a_last >= (unsigned long long)st.n_last * r.A[a]) {
         st.n_last = nl;
         st.a_last = r.A[a];
@@ -244,45 +248,39 @@ __device__ __forceinline__ void piece_start(const RayFx& r, long long R_fx, uint
       }
       any = true;
       st.q[a] += (int)cnt;
+      st.N[a] += cnt << 16;
     }
   }
 }
 
 // Crossings of axis p (numerator N, |D_p| = A) that the box step takes before the exit axis's
 // face crossing F / E: #{m >= 0 : (N + 2^16 m) E < F A} (`le`: <=, when p is the lower axis, the
-// tie order).  est = (F A - N E) / (E 2^16) from the exact 64-bit numerator (|num| < 2^48: at
-// most 2^8 crossings), converted from two exact 24-bit halves with one rounding: its error
-// is below 2^-14, so the count is floor(est) + 1 unless est lies within 2^-12 of an integer,
-// where exact comparisons decide.  rE = RN(1 / E) / 2^16.
+// tie order) = 1 + floor(num / (2^16 E)) with num = F A - N E (- 1 unless `le`), and, floors
+// nesting, = 1 + floor((num >> 16) / E).  A box extends at most 64 voxels, so the quotient is at
+// most 64 and num >> 16 below 2^30 in size; the quotient comes from an FP32 product (rE = 1 / E
+// to an ulp or two, error below 2^-15) and is set right by its exact remainder.  No crossing
+// (num >= -2^16 E, as N is at most 2^16 from the last one) gives 0; D_p = 0 is held to 0.
 __device__ __forceinline__ int crossings_before(uint32_t F, uint32_t E, float rE, uint32_t N,
                                                 uint32_t A, bool le) {
-  const unsigned long long X = (unsigned long long)F * A;
-  const long long num = (long long)X - (long long)((unsigned long long)N * E);
-  const float est = __fmaf_rn(__int2float_rn((int)(num >> 24)), 16777216.0f,
-                              __int2float_rn((int)(num & 0xFFFFFF))) * rE;
-  const float fl = floorf(est);
-  const float fr = est - fl;
-  int cnt = (int)fl + 1;
-  if (!(fr > 0.000244140625f && fr < 0.999755859375f)) {
-    cnt = cnt > 0 ? cnt : 0;
-    const unsigned long long y1 = (unsigned long long)(N + ((uint32_t)cnt << 16)) * E;
-    const unsigned long long y0 = y1 - ((unsigned long long)E << 16);   // used for cnt > 0 only
-    if (cnt > 0 && !(le ? y0 <= X : y0 < X)) cnt -= 1;
-    else if (le ? y1 <= X : y1 < X) cnt += 1;
-  }
-  return cnt;
+  const long long num = (long long)((unsigned long long)F * A) -
+                        (long long)((unsigned long long)N * E) - (le ? 0 : 1);
+  const int nh = (int)(num >> 16);
+  int c = __float2int_rd(__int2float_rn(nh) * rE);
+  const int rem = nh - c * (int)E;
+  c += rem < 0 ? 0 : (rem >= (int)E ? 2 : 1);
+  return max(c, 0);
 }
 
 // One block's entry for the ray's octant: bit 31 set = the block holds an occupied voxel (the
 // low bits: its slot in the box field), else the log2 extents of the free box of blocks
 // starting there, 2 bits per axis.  `brick`: where its occupancy bits are.
-template <int LAYOUT>
+template <int LAYOUT, bool BOXES>
 __device__ __forceinline__ uint32_t block_entry(const DevMap& m, const uint32_t* top,
-                                                const int step[3], const int b[3], uint32_t up,
+                                                const int step[4], const int b[3], uint32_t up,
                                                 const uint32_t*& brick) {
   if (LAYOUT == kLayoutGrid) {
     const int idx = b[0] * step[0] + b[1] * step[1] + b[2] * step[2];
-    brick = m.cells ? nullptr : reinterpret_cast<const uint32_t*>(m.bricks) + 16 * (size_t)(idx + step[3]);
+    if (!BOXES) brick = reinterpret_cast<const uint32_t*>(m.bricks) + 16 * (size_t)(idx + step[3]);
     return __ldg(top + idx);
   }
   uint32_t slot = 0;
@@ -309,18 +307,18 @@ __device__ __forceinline__ float recip_fast(float x) {
 // exit axis by exact 64-bit comparisons, the crossing counts of the other two axes) with two
 // dependent loads; the field's lines stay in L1, which holds all of the SM's 228 KB since
 // nothing is staged in shared memory.  Measured against a march over symmetric free boxes of
-// blocks with a voxel walk inside occupied blocks: 65536 rays on the 40 m map 54 -> 22 us,
-// 262144 rays on the 100 m map 101.6 -> 36.7 us.
-template <int KIND, int LAYOUT>
+// blocks with a voxel walk inside occupied blocks: 65536 rays on the 40 m map 54 -> 20 us,
+// 262144 rays on the 100 m map 101.6 -> 33 us.
+template <int KIND, int LAYOUT, bool BOXES>
 __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const RayFx& r,
                                          const uint32_t L[3], int at_limit, bool work) {
   const uint32_t* A = r.A;
   int* q = st.q;
-  const bool up[3] = {(r.up & 1u) != 0, (r.up & 2u) != 0, (r.up & 4u) != 0};
-  const float rA[3] = {recip_fast(__uint2float_rn(A[0])) * (1.0f / 65536.0f),
-                       recip_fast(__uint2float_rn(A[1])) * (1.0f / 65536.0f),
-                       recip_fast(__uint2float_rn(A[2])) * (1.0f / 65536.0f)};
+  uint32_t* N = st.N;
+  const float rA[3] = {recip_fast(__uint2float_rn(A[0])), recip_fast(__uint2float_rn(A[1])),
+                       recip_fast(__uint2float_rn(A[2]))};
   int hi[3];                                        // first voxel beyond the map / the grid
+  uint32_t H[3];                                    // dense: N of the map's far faces
   int step[4] = {0, 0, 0, 0};                       // signed brick strides and the first brick
   const uint32_t* top = m.top;
   int status = at_limit;
@@ -329,11 +327,13 @@ __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const 
     const int str[3] = {1, m.gdim[0], m.gdim[0] * m.gdim[1]};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      hi[a] = (KIND == RMP_MAP_DENSE_U8 && up[a]) ? m.dims[a] : 8 * m.gdim[a];
-      step[a] = up[a] ? str[a] : -str[a];
-      step[3] += up[a] ? 0 : (m.gdim[a] - 1) * str[a];
+      const bool up = (r.up >> a) & 1u;
+      hi[a] = (KIND == RMP_MAP_DENSE_U8 && up) ? m.dims[a] : 8 * m.gdim[a];
+      H[a] = N[a] + ((uint32_t)(hi[a] - 1 - q[a]) << 16);
+      step[a] = up ? str[a] : -str[a];
+      step[3] += up ? 0 : (m.gdim[a] - 1) * str[a];
       // a dense map: a piece that starts outside has left the map
-      if (KIND == RMP_MAP_DENSE_U8 && !up[a] && q[a] < 8 * m.gdim[a] - m.dims[a]) {
+      if (KIND == RMP_MAP_DENSE_U8 && (q[a] >= hi[a] || q[a] < (up ? 0 : 8 * m.gdim[a] - m.dims[a]))) {
         status = RMP_RAY_MISS_EXIT;
         run = false;
       }
@@ -345,48 +345,47 @@ __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const 
   for (uint32_t it = 0; it < 8u * (kMaxRangeVoxels + 2); ++it) {
     if (!__any_sync(0xffffffffu, run)) break;
     if (!run) continue;
-    int end[3];                                     // first voxel beyond the free box
+    uint32_t F[3];                                  // numerators of the box's far faces
     bool inside = true;
-    if (LAYOUT == kLayoutGrid)
+    if (LAYOUT == kLayoutGrid && KIND != RMP_MAP_DENSE_U8)
       inside = (unsigned)q[0] < (unsigned)hi[0] && (unsigned)q[1] < (unsigned)hi[1] &&
                (unsigned)q[2] < (unsigned)hi[2];
     if (inside) {
       const int b[3] = {q[0] >> 3, q[1] >> 3, q[2] >> 3};
+      const int l[3] = {q[0] & 7, q[1] & 7, q[2] & 7};
       const uint32_t* brick = nullptr;
-      uint32_t e = block_entry<LAYOUT>(m, top, step, b, r.up, brick);
+      uint32_t e = block_entry<LAYOUT, BOXES>(m, top, step, b, r.up, brick);
       const bool occupied = (int)e < 0;
       if (occupied) {
-        const uint32_t p = (uint32_t)((q[0] & 7) | ((q[1] & 7) << 3) | ((q[2] & 7) << 6));
-        if (m.cells) {
+        const uint32_t p = (uint32_t)(l[0] | (l[1] << 3) | (l[2] << 6));
+        if (BOXES) {
           e = __ldg(box + 4096 * (size_t)(e & 0x7fffffffu) + p);
         } else {                                    // no box field: single voxels
-          const uint32_t w = p ^ ((up[0] ? 0u : 7u) | (up[1] ? 0u : 56u) | (up[2] ? 0u : 448u));
+          const uint32_t w = p ^ ((r.up & 1u ? 0u : 7u) | (r.up & 2u ? 0u : 56u) |
+                                  (r.up & 4u ? 0u : 448u));
           e = (__ldg(brick + (w >> 5)) >> (w & 31u)) & 1u ? 0u : 64u;
         }
+        if (e == 0u) {
+          status = RMP_RAY_HIT;
+          run = false;
+        }
       }
-      if (occupied && e == 0u) {
-        status = RMP_RAY_HIT;
-        run = false;
-      }
+      // extents in voxels, a block's counted from its first voxel
+      const int sh = occupied ? 0 : 3, part = occupied ? 0 : 7;
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        const int ext = 1 << ((e >> (2 * a)) & 3u);
-        end[a] = occupied ? q[a] + ext : (b[a] + ext) << 3;
-        if (KIND == RMP_MAP_DENSE_U8) end[a] = min(end[a], hi[a]);
+        const int ahead = (1 << (((e >> (2 * a)) & 3u) + sh)) - (l[a] & part) - 1;
+        F[a] = N[a] + ((uint32_t)ahead << 16);
+        if (KIND == RMP_MAP_DENSE_U8) F[a] = min(F[a], H[a]);
       }
     } else {
-      // a dense map is left; outside the grid of a hashed map there is nothing ahead once it
-      // lies behind on any axis, else every voxel short of it is free (at most 240 at once,
-      // see crossings_before)
-      if (KIND == RMP_MAP_DENSE_U8) status = RMP_RAY_MISS_EXIT;
-      run = KIND != RMP_MAP_DENSE_U8 && q[0] < hi[0] && q[1] < hi[1] && q[2] < hi[2];
-      const int gap = min(max(-q[0], max(-q[1], -q[2])), 240);
+      // outside the grid of a hashed map: nothing ahead once it lies behind on any axis, else
+      // every voxel short of it is free (at most 64 at once, see crossings_before)
+      run = q[0] < hi[0] && q[1] < hi[1] && q[2] < hi[2];
+      const int gap = min(max(-q[0], max(-q[1], -q[2])), 64);
 #pragma unroll
-      for (int a = 0; a < 3; ++a) end[a] = q[a] + gap;
+      for (int a = 0; a < 3; ++a) F[a] = N[a] + ((uint32_t)(gap - 1) << 16);
     }
-    uint32_t F[3];                                  // numerators of the face crossings
-#pragma unroll
-    for (int a = 0; a < 3; ++a) F[a] = ((uint32_t)(end[a] - 1) << 16) + r.C[a];
     // exit axis: the first face crossing (ties: the lowest axis)
     const bool y = (unsigned long long)F[1] * A[0] < (unsigned long long)F[0] * A[1];
     const uint32_t Fw = y ? F[1] : F[0], Aw = y ? A[1] : A[0];
@@ -397,16 +396,22 @@ __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const 
     const float rE = z ? rA[2] : (y ? rA[1] : rA[0]);
     // the other two axes, i < j: i is x unless x exits, j is z unless z exits
     const bool x = !y && !z;
-    const uint32_t Ni = ((uint32_t)(x ? q[1] : q[0]) << 16) + (x ? r.C[1] : r.C[0]);
-    const uint32_t Nj = ((uint32_t)(z ? q[1] : q[2]) << 16) + (z ? r.C[1] : r.C[2]);
-    const int ci = crossings_before(Fe, Ae, rE, Ni, x ? A[1] : A[0], !x);
-    const int cj = crossings_before(Fe, Ae, rE, Nj, z ? A[1] : A[2], z);
-    q[0] = x ? end[0] : q[0] + ci;
-    q[1] = x ? q[1] + ci : (z ? q[1] + cj : end[1]);
-    q[2] = z ? end[2] : q[2] + cj;
+    const int ci = crossings_before(Fe, Ae, rE, x ? N[1] : N[0], x ? A[1] : A[0], !x);
+    const int cj = crossings_before(Fe, Ae, rE, z ? N[1] : N[2], z ? A[1] : A[2], z);
+    const int ce = (int)((Fe - (z ? N[2] : (y ? N[1] : N[0]))) >> 16) + 1;
+    const int c[3] = {x ? ce : ci, x ? ci : (z ? cj : ce), z ? ce : cj};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      q[a] += c[a];
+      N[a] += (uint32_t)c[a] << 16;
+    }
     st.n_last = Fe;
     st.a_last = Ae;
     st.ax_last = z ? 2 : (y ? 1 : 0);
+    if (KIND == RMP_MAP_DENSE_U8 && Fe == (z ? H[2] : (y ? H[1] : H[0]))) {
+      status = RMP_RAY_MISS_EXIT;                   // the exit axis stepped off the map
+      run = false;
+    }
   }
   return status;
 }
@@ -1286,7 +1291,7 @@ __device__ __forceinline__ uint32_t ray_of_slot(uint32_t j, const EvalConsts& k)
 // false for lanes without a segment).  Returns the ray's status with (n, a), the entry
 // crossing of its last voxel, in every lane of the group.  `rec` (nullable): where the lane
 // that holds the ray's end writes its hit record.
-template <int KIND, int LAYOUT>
+template <int KIND, int LAYOUT, bool BOXES>
 __device__ __forceinline__ int march_ray(const DevMap& m, const EvalConsts& k, const long long P[3],
                                          const Ray& ray, uint32_t seg, uint32_t lgS, bool work,
                                          uint32_t& n, uint32_t& a, rmp_ray_hit_t* rec) {
@@ -1300,7 +1305,7 @@ __device__ __forceinline__ int march_ray(const DevMap& m, const EvalConsts& k, c
   ray_fx<LAYOUT>(m, P, ray.D, r);
   piece_start(r, k.R_fx, j_lo, st);
   limits_at(r, k.R_fx, j_hi, L);
-  const int status = march_run<KIND, LAYOUT>(
+  const int status = march_run<KIND, LAYOUT, BOXES>(
       m, st, r, L, seg == S - 1 ? RMP_RAY_MISS_RANGE : kSegContinues, work);
   const uint32_t ballot = __ballot_sync(0xffffffffu, work && piece_final(status));
   const uint32_t grp0 = lane & ~(S - 1);
@@ -1359,7 +1364,7 @@ __device__ __forceinline__ void ray_outputs(const DevMap& m, const EvalConsts& k
 // ray sit in adjacent lanes, and the ray's result is the first segment (lowest index) that
 // hit or left the map, else the last one -- found with a warp ballot and moved to the
 // ray's first lane by shuffles.  That lane evaluates the policy and writes the outputs.
-template <int KIND, int LAYOUT, int RED>
+template <int KIND, int LAYOUT, int RED, bool BOXES>
 __global__ void __launch_bounds__(256) raycast_rmp_kernel(DevMap m, EvalConsts k,
                                                           const double* __restrict__ state,
                                                           WsHeader* ws, CtaPartial* parts,
@@ -1408,7 +1413,7 @@ __global__ void __launch_bounds__(256) raycast_rmp_kernel(DevMap m, EvalConsts k
     first = false;
     const long long P[3] = {cs.P[0], cs.P[1], cs.P[2]};
     uint32_t en, ea;
-    const int mstat = march_ray<KIND, LAYOUT>(m, k, P, ray, seg, lgS, active && !bad, en, ea,
+    const int mstat = march_ray<KIND, LAYOUT, BOXES>(m, k, P, ray, seg, lgS, active && !bad, en, ea,
                                               hits ? hits + ray_idx : nullptr);
     if (!active || bad || seg != 0) continue;
     float vals[9];
@@ -1900,7 +1905,7 @@ __device__ __noinline__ void batch_group_finish(const EvalConsts& k, CtaPartial*
 // depend on which warp ran which chunk, nor on s.
 // Register budget 64 (launch bounds 256 x 4): 32 warps per SM hide each other's latency; the
 // per-state values used only after the march are read after it.
-template <int KIND, int LAYOUT, int RED>
+template <int KIND, int LAYOUT, int RED, bool BOXES>
 __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
     DevMap m, EvalConsts k, BatchHeader* hdr, const BatchState* __restrict__ bs,
     uint32_t* sticket, uint32_t* gticket, CtaPartial* cparts, CtaPartial* gparts,
@@ -1943,7 +1948,7 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
     const Ray ray = make_ray(ray_idx + k.halton_offset);
     const size_t ro = (size_t)b * max_rays + ray_idx;
     uint32_t en, ea;
-    const int mstat = march_ray<KIND, LAYOUT>(m, k, P, ray, seg, lgs, active, en, ea,
+    const int mstat = march_ray<KIND, LAYOUT, BOXES>(m, k, P, ray, seg, lgs, active, en, ea,
                                               hits ? hits + ro : nullptr);
     // read after the march, so that they are not held in registers across it
     const float v[3] = {__ldg(&sp->v[0]), __ldg(&sp->v[1]), __ldg(&sp->v[2])};
@@ -2728,104 +2733,61 @@ __global__ void hash_build_kernel(const int32_t* __restrict__ keys, uint32_t n_b
 }  // namespace
 
 // ------------------------------------------------------------------ launchers
-template <int KIND, int LAYOUT>
-static void launch_raycast_t(const DevMap& m, const EvalConsts& k, const double* state_dev,
-                             WsHeader* hdr, CtaPartial* parts, rmp_result_t* out_dev,
-                             rmp_ray_hit_t* hits, float* per_ray, int block, int grid,
-                             cudaStream_t stream) {
-  if (k.reduce_mode == RMP_REDUCE_FP64)
-    raycast_rmp_kernel<KIND, LAYOUT, RMP_REDUCE_FP64><<<grid, block, 0, stream>>>(
-        m, k, state_dev, hdr, parts, out_dev, hits, per_ray);
-  else
-    raycast_rmp_kernel<KIND, LAYOUT, RMP_REDUCE_KAHAN32><<<grid, block, 0, stream>>>(
-        m, k, state_dev, hdr, parts, out_dev, hits, per_ray);
+// Every kernel variant of a map and reduction: f is called with <kind, layout, reduction, box
+// field present> as integral constants.
+template <int V>
+using Int = std::integral_constant<int, V>;
+
+template <int KIND, int LAYOUT, class F>
+static void for_reduction(const DevMap& m, int reduce_mode, F f) {
+  if (reduce_mode == RMP_REDUCE_FP64) {
+    if (m.cells) f(Int<KIND>(), Int<LAYOUT>(), Int<RMP_REDUCE_FP64>(), Int<1>());
+    else f(Int<KIND>(), Int<LAYOUT>(), Int<RMP_REDUCE_FP64>(), Int<0>());
+  } else {
+    if (m.cells) f(Int<KIND>(), Int<LAYOUT>(), Int<RMP_REDUCE_KAHAN32>(), Int<1>());
+    else f(Int<KIND>(), Int<LAYOUT>(), Int<RMP_REDUCE_KAHAN32>(), Int<0>());
+  }
 }
 
-template <int KIND, int LAYOUT>
-static cudaError_t raycast_occupancy_t(int* n, int reduce_mode, int block) {
-  return reduce_mode ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                           n, raycast_rmp_kernel<KIND, LAYOUT, RMP_REDUCE_FP64>, block, 0)
-                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                           n, raycast_rmp_kernel<KIND, LAYOUT, RMP_REDUCE_KAHAN32>, block, 0);
+template <class F>
+static void for_map(const DevMap& m, int reduce_mode, F f) {
+  if (m.kind == RMP_MAP_DENSE_U8) for_reduction<RMP_MAP_DENSE_U8, kLayoutGrid>(m, reduce_mode, f);
+  else if (m.layout == kLayoutGrid) for_reduction<RMP_MAP_HASHED_TSDF, kLayoutGrid>(m, reduce_mode, f);
+  else for_reduction<RMP_MAP_HASHED_TSDF, kLayoutHash>(m, reduce_mode, f);
 }
 
 int raycast_occupancy(const DevMap& m, int reduce_mode, int block) {
   int n = 0;
-  cudaError_t e;
-  if (m.kind == RMP_MAP_DENSE_U8)
-    e = raycast_occupancy_t<RMP_MAP_DENSE_U8, kLayoutGrid>(&n, reduce_mode, block);
-  else if (m.layout == kLayoutGrid)
-    e = raycast_occupancy_t<RMP_MAP_HASHED_TSDF, kLayoutGrid>(&n, reduce_mode, block);
-  else
-    e = raycast_occupancy_t<RMP_MAP_HASHED_TSDF, kLayoutHash>(&n, reduce_mode, block);
+  cudaError_t e = cudaSuccess;
+  for_map(m, reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &n, raycast_rmp_kernel<kind.value, layout.value, red.value, boxes.value != 0>, block, 0);
+  });
   return e == cudaSuccess ? n : -1;
 }
 
 cudaError_t launch_raycast(const DevMap& m, const EvalConsts& k, const double* state_dev,
                            void* ws, rmp_result_t* out_dev, rmp_ray_hit_t* hits,
                            float* per_ray, int block, int grid, cudaStream_t stream) {
-  // grid_finish needs whole warps 0 and 1 (the resolve's named barrier) and at least 64
-  // threads (each summing thread takes at most two of the up to 128 group partials)
+  // grid_finish needs whole warps 0 and 1 (the resolve's named barrier)
   if (block != 64 && block != 128 && block != 256) return cudaErrorInvalidValue;
   WsHeader* hdr = (WsHeader*)ws;
   CtaPartial* parts = (CtaPartial*)((char*)ws + kWsHeaderBytes);
-  if (m.kind == RMP_MAP_DENSE_U8)
-    launch_raycast_t<RMP_MAP_DENSE_U8, kLayoutGrid>(m, k, state_dev, hdr, parts, out_dev, hits,
-                                                    per_ray, block, grid, stream);
-  else if (m.layout == kLayoutGrid)
-    launch_raycast_t<RMP_MAP_HASHED_TSDF, kLayoutGrid>(m, k, state_dev, hdr, parts, out_dev, hits,
-                                                       per_ray, block, grid, stream);
-  else
-    launch_raycast_t<RMP_MAP_HASHED_TSDF, kLayoutHash>(m, k, state_dev, hdr, parts, out_dev, hits,
-                                                       per_ray, block, grid, stream);
+  for_map(m, k.reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
+    raycast_rmp_kernel<kind.value, layout.value, red.value, boxes.value != 0>
+        <<<grid, block, 0, stream>>>(m, k, state_dev, hdr, parts, out_dev, hits, per_ray);
+  });
   return cudaGetLastError();
 }
 
-template <int KIND, int LAYOUT, int RED>
-static int batch_occupancy_t(int block) {
-  int n = 0;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, raycast_batch_kernel<KIND, LAYOUT, RED>,
-                                                       block, 0) == cudaSuccess ? n : -1;
-}
-
 int batch_occupancy(const DevMap& m, int reduce_mode, int block) {
-  if (m.kind == RMP_MAP_DENSE_U8)
-    return reduce_mode ? batch_occupancy_t<RMP_MAP_DENSE_U8, kLayoutGrid, RMP_REDUCE_FP64>(block)
-                       : batch_occupancy_t<RMP_MAP_DENSE_U8, kLayoutGrid, RMP_REDUCE_KAHAN32>(block);
-  if (m.layout == kLayoutGrid)
-    return reduce_mode ? batch_occupancy_t<RMP_MAP_HASHED_TSDF, kLayoutGrid, RMP_REDUCE_FP64>(block)
-                       : batch_occupancy_t<RMP_MAP_HASHED_TSDF, kLayoutGrid, RMP_REDUCE_KAHAN32>(block);
-  return reduce_mode ? batch_occupancy_t<RMP_MAP_HASHED_TSDF, kLayoutHash, RMP_REDUCE_FP64>(block)
-                     : batch_occupancy_t<RMP_MAP_HASHED_TSDF, kLayoutHash, RMP_REDUCE_KAHAN32>(block);
-}
-
-template <int KIND, int LAYOUT, int RED>
-static void launch_batch_t(const DevMap& m, const EvalConsts& k, BatchHeader* hdr,
-                           const BatchState* bs, uint32_t* sticket, uint32_t* gticket,
-                           CtaPartial* cparts, CtaPartial* gparts, rmp_result_t* out,
-                           rmp_ray_hit_t* hits, float* per_ray, uint32_t max_rays, int block,
-                           int grid, cudaStream_t stream, const double* states,
-                           const double* goals) {
-  raycast_batch_kernel<KIND, LAYOUT, RED><<<grid, block, 0, stream>>>(
-      m, k, hdr, bs, sticket, gticket, cparts, gparts, out, hits, per_ray, max_rays, states,
-      goals);
-}
-
-template <int KIND, int LAYOUT>
-static void launch_batch_r(const DevMap& m, const EvalConsts& k, BatchHeader* hdr,
-                           const BatchState* bs, uint32_t* sticket, uint32_t* gticket,
-                           CtaPartial* cparts, CtaPartial* gparts, rmp_result_t* out,
-                           rmp_ray_hit_t* hits, float* per_ray, uint32_t max_rays, int block,
-                           int grid, cudaStream_t stream, const double* states,
-                           const double* goals) {
-  if (k.reduce_mode == RMP_REDUCE_FP64)
-    launch_batch_t<KIND, LAYOUT, RMP_REDUCE_FP64>(m, k, hdr, bs, sticket, gticket, cparts, gparts,
-                                                  out, hits, per_ray, max_rays, block, grid,
-                                                  stream, states, goals);
-  else
-    launch_batch_t<KIND, LAYOUT, RMP_REDUCE_KAHAN32>(m, k, hdr, bs, sticket, gticket, cparts,
-                                                     gparts, out, hits, per_ray, max_rays, block,
-                                                     grid, stream, states, goals);
+  int n = 0;
+  cudaError_t e = cudaSuccess;
+  for_map(m, reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &n, raycast_batch_kernel<kind.value, layout.value, red.value, boxes.value != 0>, block, 0);
+  });
+  return e == cudaSuccess ? n : -1;
 }
 
 cudaError_t launch_batch(const DevMap& m, const EvalConsts& k, const double* states_dev,
@@ -2843,21 +2805,12 @@ cudaError_t launch_batch(const DevMap& m, const EvalConsts& k, const double* sta
   // 8 states a CTA (a warp each) as far as the SMs go; longer runs beyond
   const unsigned prep = n_states < 8u * 152u ? (n_states + 7u) / 8u : 152u;
   batch_prep_kernel<<<prep, 256, 0, stream>>>(states_dev, n_rays_dev, n_states, max_rays, m, k, hdr,
-                                            bs, sticket, gticket, out_dev);
-  if (m.kind == RMP_MAP_DENSE_U8)
-    launch_batch_r<RMP_MAP_DENSE_U8, kLayoutGrid>(m, k, hdr, bs, sticket, gticket, cparts, gparts,
-                                                  out_dev, hits, per_ray, max_rays, block, grid,
-                                                  stream, states_dev, goals_dev);
-  else if (m.layout == kLayoutGrid)
-    launch_batch_r<RMP_MAP_HASHED_TSDF, kLayoutGrid>(m, k, hdr, bs, sticket, gticket, cparts,
-                                                     gparts, out_dev, hits, per_ray, max_rays,
-                                                     block, grid, stream, states_dev,
-                                                     goals_dev);
-  else
-    launch_batch_r<RMP_MAP_HASHED_TSDF, kLayoutHash>(m, k, hdr, bs, sticket, gticket, cparts,
-                                                     gparts, out_dev, hits, per_ray, max_rays,
-                                                     block, grid, stream, states_dev,
-                                                     goals_dev);
+                                              bs, sticket, gticket, out_dev);
+  for_map(m, k.reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
+    raycast_batch_kernel<kind.value, layout.value, red.value, boxes.value != 0>
+        <<<grid, block, 0, stream>>>(m, k, hdr, bs, sticket, gticket, cparts, gparts, out_dev, hits,
+                                     per_ray, max_rays, states_dev, goals_dev);
+  });
   return cudaGetLastError();
 }
 
