@@ -71,6 +71,7 @@ struct DevMap {
 struct EvalConsts {
   float eta_rep, inv_nu_rep, eta_damp, inv_nu_damp, eps, c, r_up, inv_r;
   float r_hi, r_lo;         // r = r_hi + r_lo (FP32 pair)
+  float quiet_v2;           // |xdot|^2 below which inactive or far hits add exact zeros
   float min_up, max_dn;     // scans: d >= min_range <=> d >= min_up; d <= max <=> d <= max_dn
   long long R_fx;           // llrint(max_range / vs * 2^16)
   uint32_t n_rays, halton_offset;

@@ -25,34 +25,66 @@ __device__ __forceinline__ float halton2(uint32_t i) {
   return __fmul_rn(__uint2float_rn(__brev(i)), 2.3283064365386963e-10f);  // * 2^-32
 }
 
-// The 20 base-3 digits of i (< 3^20) reversed: H(i,3) * 3^20.
-__device__ __forceinline__ uint32_t halton3_numerator(uint32_t i) {
+// The 16 base-3 digits of i (< 2^24 < 3^16) reversed: H(i,3) * 3^16.
+template <int DIGITS>
+__device__ __forceinline__ uint32_t reverse3(uint32_t i) {
   uint32_t num = 0;
 #pragma unroll
-  for (int k = 0; k < 20; ++k) {
-    uint32_t q = i / 3u;
+  for (int k = 0; k < DIGITS; ++k) {
+    const uint32_t q = i / 3u;
     num = num * 3u + (i - 3u * q);
     i = q;
   }
   return num;
 }
 
-// num / 3^20 correctly rounded to FP32 with integer arithmetic only (FP64 division is
-// slow on this GPU): scale num by 2^s so the quotient has exactly 24 significant bits,
-// divide, and round to nearest on the remainder (no ties: 3^20 is odd).
+// The reversed digits of every 5-digit number.
+struct Reverse5 {
+  uint8_t v[243];
+  constexpr Reverse5() : v() {
+    for (int i = 0; i < 243; ++i) {
+      int num = 0, q = i;
+      for (int k = 0; k < 5; ++k) {
+        num = num * 3 + q % 3;
+        q /= 3;
+      }
+      v[i] = (uint8_t)num;
+    }
+  }
+};
+__device__ const Reverse5 kReverse5;
+
+// TABLE: three lookups of 5 digits and the last digit (25 instructions for 75; the batch kernel,
+// which is bound by instructions and keeps the table in L1); else two halves of 8 digits whose
+// chains run side by side (one evaluation, bound by latency, would wait for the table).
+template <bool TABLE>
+__device__ __forceinline__ uint32_t halton3_numerator(uint32_t i) {
+  if (TABLE) {
+    const uint32_t q1 = i / 243u, q2 = i / 59049u, q3 = i / 14348907u;
+    return __ldg(&kReverse5.v[i - 243u * q1]) * 177147u +
+           __ldg(&kReverse5.v[q1 - 243u * q2]) * 729u +
+           __ldg(&kReverse5.v[q2 - 243u * q3]) * 3u + q3;
+  }
+  const uint32_t hi = i / 6561u;
+  return reverse3<8>(i - 6561u * hi) * 6561u + reverse3<8>(hi);
+}
+
+// num / 3^16 (num < 3^16) correctly rounded to FP32: the quotient of num 2^s, s such that it has
+// exactly 24 significant bits, from an FP32 product a few units off, set right by its exact
+// remainder (within 2^28, so 32-bit arithmetic holds it); rounded to nearest on the remainder (no
+// ties: 3^16 is odd).  FP64 division and a 64-bit integer division are slower on this GPU.
 __device__ __forceinline__ float halton3_f32(uint32_t num) {
   if (num == 0) return 0.0f;
-  constexpr unsigned long long M = 3486784401ull;
-  int s = 55 - (32 - __clz(num));
-  unsigned long long X = (unsigned long long)num << s;
-  if (X < (M << 23)) {
-    X <<= 1;
-    ++s;
-  }
-  unsigned long long q = X / M;
-  unsigned long long rem = X - q * M;
-  if (2ull * rem > M) ++q;
-  return __fmul_rn(__ull2float_rn(q), __int_as_float((127 - s) << 23));
+  constexpr uint32_t M = 43046721u;
+  constexpr float rM = 1.0f / 43046721.0f;
+  const int t = __clz(num) - 6;
+  const int s = t + ((num << t) >= M ? 23 : 24);
+  int q = __float2int_rn(__fmul_rn(__fmul_rn(__uint2float_rn(num), rM), __int_as_float((127 + s) << 23)));
+  int rem = (int)((uint32_t)((unsigned long long)num << s) - (uint32_t)q * M);
+  const int adj = __float2int_rn(__fmul_rn(__int2float_rn(rem), rM));
+  rem -= adj * (int)M;
+  q += adj + (2 * rem > (int)M ? 1 : 0) - (2 * rem < -(int)M ? 1 : 0);
+  return __fmul_rn(__int2float_rn(q), __int_as_float((127 - s) << 23));
 }
 
 // cos and sin of 2*pi*v by a fixed FP32 recipe: octant q = floor(8v), fraction t,
@@ -100,9 +132,10 @@ struct Ray {
   int D[3];
 };
 
+template <bool TABLE>
 __device__ __forceinline__ Ray make_ray(uint32_t i) {
   const float u = halton2(i);
-  const float v = halton3_f32(halton3_numerator(i));
+  const float v = halton3_f32(halton3_numerator<TABLE>(i));
   const float z = __fsub_rn(1.0f, __fmul_rn(2.0f, u));
   const float st = __fmul_rn(2.0f, __fsqrt_rn(__fmul_rn(u, __fsub_rn(1.0f, u))));
   float c, s;
@@ -114,6 +147,30 @@ __device__ __forceinline__ Ray make_ray(uint32_t i) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) r.D[a] = __float2int_rn(__fmul_rn(r.dir[a], 16777216.0f));
   return r;
+}
+
+// ------------------------------------------------------------------ small arithmetic
+// 1 / x to an ulp or so; infinity for 0.
+__device__ __forceinline__ float recip_fast(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// x / d and x % d for x < 2^24 and a quotient below 2^19 (error of the FP32 product below 1/8):
+// the product set right by its remainder.
+__device__ __forceinline__ uint32_t divide24(uint32_t x, uint32_t d, uint32_t& rem) {
+  int q = __float2int_rz(__uint2float_rn(x) * recip_fast(__uint2float_rn(d)));
+  int r = (int)x - q * (int)d;
+  if (r < 0) {
+    q -= 1;
+    r += (int)d;
+  } else if (r >= (int)d) {
+    q += 1;
+    r -= (int)d;
+  }
+  rem = (uint32_t)r;
+  return (uint32_t)q;
 }
 
 // ------------------------------------------------------------------ map access
@@ -289,13 +346,6 @@ __device__ __forceinline__ uint32_t block_entry(const DevMap& m, const uint32_t*
   if (at < 0) return 0u;                            // a missing block: free, alone
   brick = reinterpret_cast<const uint32_t*>(m.bricks) + 16 * (size_t)at;
   return 0x80000000u | slot;
-}
-
-// 1 / x to an ulp or so; infinity for 0.
-__device__ __forceinline__ float recip_fast(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
 }
 
 // March a piece from state st until a hit, a map exit or the limits L (returns `at_limit`; st is
@@ -616,8 +666,9 @@ __device__ __forceinline__ void warp_reduce_terms(T (&s)[9], T (&c)[9], uint32_t
 }
 
 // Block-level reduction of the per-thread accumulators and counts: the shared-out tree per warp,
-// then lane q of warp 0 merges term q of the warps in warp order (all terms at once, not one
-// thread walking them).  Called by every thread.
+// (where one of its lanes `added` anything; all sums are zero otherwise), then lane q of warp 0
+// merges term q of the warps in warp order (all terms at once, not one thread walking them).
+// Called by every thread.
 template <int RED>
 struct BlockReduce;
 
@@ -629,12 +680,12 @@ struct BlockReduce<RMP_REDUCE_KAHAN32> {
     for (int q = 0; q < 9; ++q) a.s[q] = a.c[q] = 0.0f;
   }
   __device__ static void add(Acc& a, const float v[9]) { acc_add(a, v); }
-  __device__ static void reduce(Acc& a, unsigned nh, unsigned na, CtaSums& out) {
+  __device__ static void reduce(Acc& a, bool added, unsigned nh, unsigned na, CtaSums& out) {
     __shared__ float sh[32][18];
     __shared__ unsigned shu[32][2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const WarpTerms t = warp_terms(0);
-    warp_reduce_terms<float, true>(a.s, a.c, 0);
+    if (__any_sync(0xffffffffu, added)) warp_reduce_terms<float, true>(a.s, a.c, 0);
     nh = __reduce_add_sync(0xffffffffu, nh);
     na = __reduce_add_sync(0xffffffffu, na);
     if (t.n > 0) {
@@ -673,12 +724,12 @@ struct BlockReduce<RMP_REDUCE_FP64> {
 #pragma unroll
     for (int q = 0; q < 9; ++q) a.s[q] += (double)v[q];
   }
-  __device__ static void reduce(Acc& a, unsigned nh, unsigned na, CtaSums& out) {
+  __device__ static void reduce(Acc& a, bool added, unsigned nh, unsigned na, CtaSums& out) {
     __shared__ double sh[32][9];
     __shared__ unsigned shu[32][2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const WarpTerms t = warp_terms(0);
-    warp_reduce_terms<double, false>(a.s, a.s, 0);
+    if (__any_sync(0xffffffffu, added)) warp_reduce_terms<double, false>(a.s, a.s, 0);
     nh = __reduce_add_sync(0xffffffffu, nh);
     na = __reduce_add_sync(0xffffffffu, na);
     if (t.n > 0) sh[warp][t.first] = a.s[0];
@@ -1209,7 +1260,7 @@ __device__ void grid_finish(const CtaSums& cta, WsHeader* ws, CtaPartial* parts,
       nh += w[18];
       na += w[19];
     }
-    BlockReduce<RED>::reduce(acc, nh, na, gsum);
+    BlockReduce<RED>::reduce(acc, true, nh, na, gsum);
     const int any_expired = __syncthreads_or(expired);
     if (poisoned || any_expired) {
       if (threadIdx.x == 0) ws->poisoned = 1;
@@ -1269,19 +1320,12 @@ __device__ __forceinline__ void split_velocity(double x, CtaState& cs, int a) {
 // digits of H(i,3), so they point into one cell of the sphere; slots enumerate residue
 // classes one after the other, so a warp covers at most two cells.  Q = n / M, R = n % M:
 // classes r < R hold Q + 1 rays, the others Q.  M = 1 is the identity.
-__device__ __forceinline__ uint32_t ray_of_slot(uint32_t j, const EvalConsts& k) {
-  const uint32_t big = k.perm_R * (k.perm_Q + 1);
-  uint32_t r, q;
-  if (j < big) {
-    r = j / (k.perm_Q + 1);
-    q = j - r * (k.perm_Q + 1);
-  } else {
-    const uint32_t jj = j - big;
-    const uint32_t t = jj / k.perm_Q;
-    r = k.perm_R + t;
-    q = jj - t * k.perm_Q;
-  }
-  return r + k.perm_M * q;
+__device__ __forceinline__ uint32_t ray_of_slot(uint32_t j, uint32_t M, uint32_t Q, uint32_t R) {
+  const uint32_t big = R * (Q + 1);
+  const bool lo = j < big;
+  uint32_t q;
+  const uint32_t r = divide24(lo ? j : j - big, lo ? Q + 1 : Q, q);   // at most M <= n / 32 classes
+  return (lo ? r : R + r) + M * q;
 }
 
 // ------------------------------------------------------------------ per-ray march and outputs
@@ -1333,20 +1377,30 @@ __device__ __forceinline__ int march_ray(const DevMap& m, const EvalConsts& k, c
   return __shfl_sync(0xffffffffu, status, src);
 }
 
+// A hit (or scan point) that the robot does not approach, or beyond the policy radius, adds
+// exact zeros to the sums whenever no intermediate of the policy overflows: bound on |v|^2
+// prepared by the host (quiet_v2).  Its policy is then evaluated for the per-ray outputs only.
+__device__ __forceinline__ bool quiet_state(const EvalConsts& k, const float v[3]) {
+  return v[0] * v[0] + v[1] * v[1] + v[2] * v[2] < k.quiet_v2;
+}
+
 // The ray's obstacle policy (Sec. III-C) from its end: vals = A_i (6) and A_i f_i (3), all zero
-// unless it hit; counts hits and active rays; writes the optional per-ray (f_i, A_i).
-__device__ __forceinline__ void ray_outputs(const DevMap& m, const EvalConsts& k, const Ray& ray,
+// unless it hit; counts hits and active rays; writes the optional per-ray (f_i, A_i).  Returns
+// whether vals is to be added.
+__device__ __forceinline__ bool ray_outputs(const DevMap& m, const EvalConsts& k, const Ray& ray,
                                             int status, uint32_t n, uint32_t a, const float v[3],
-                                            const float vl[3], float* per, float vals[9],
+                                            const float vl[3], bool quiet, float* per, float vals[9],
                                             unsigned& n_hit, unsigned& n_act) {
   float f[3] = {0.f, 0.f, 0.f}, A[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, af[3] = {0.f, 0.f, 0.f};
+  bool adds = false;
   if (status == RMP_RAY_HIT) {
     const float d = n == 0 ? 0.0f : entry_distance(n, a, m.vs_f);
     const bool act = active32(v, ray.dir);
     const bool inr = d < k.r_up;
     n_hit += 1;
     n_act += (act && inr) ? 1u : 0u;
-    obstacle_policy(k, ray.dir, d, v, vl, act, inr, f, A, af);
+    adds = (act && inr) || !quiet;
+    if (adds || per) obstacle_policy(k, ray.dir, d, v, vl, act, inr, f, A, af);
   }
 #pragma unroll
   for (int q = 0; q < 6; ++q) vals[q] = A[q];
@@ -1357,6 +1411,7 @@ __device__ __forceinline__ void ray_outputs(const DevMap& m, const EvalConsts& k
     per[0] = f[0]; per[1] = f[1]; per[2] = f[2];
     per[3] = A[0]; per[4] = A[1]; per[5] = A[2]; per[6] = A[3]; per[7] = A[4]; per[8] = A[5];
   }
+  return adds;
 }
 
 // ------------------------------------------------------------------ fused raycast kernel
@@ -1385,8 +1440,9 @@ __global__ void __launch_bounds__(256) raycast_rmp_kernel(DevMap m, EvalConsts k
   const uint32_t stride = gridDim.x * blockDim.x;
   uint32_t base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
   // the first ray is generated while the state loads are in flight
-  uint32_t ray_idx = ray_of_slot(base + lane < total ? (base + lane) >> lgS : 0, k);
-  Ray ray = make_ray(ray_idx + k.halton_offset);
+  uint32_t ray_idx = ray_of_slot(base + lane < total ? (base + lane) >> lgS : 0, k.perm_M,
+                                 k.perm_Q, k.perm_R);
+  Ray ray = make_ray<false>(ray_idx + k.halton_offset);
   if (comp >= 0 && comp < 3) {
     const double o = KIND != RMP_MAP_DENSE_U8 ? 0.0
                      : (comp == 0 ? m.origin[0] : (comp == 1 ? m.origin[1] : m.origin[2]));
@@ -1400,15 +1456,16 @@ __global__ void __launch_bounds__(256) raycast_rmp_kernel(DevMap m, EvalConsts k
   }
   __syncthreads();                                  // state ready
   const bool bad = (cs.bad[0] | cs.bad[1] | cs.bad[2]) != 0;
-  bool first = true;
+  const bool quiet = quiet_state(k, cs.v);
+  bool first = true, added = false;
   // warp-uniform trip count: every lane takes part in each ballot / shuffle
   for (; base < total; base += stride) {
     const uint32_t g = base + lane;
     const bool active = g < total;
     const uint32_t seg = g & (S - 1);
     if (!first) {
-      ray_idx = ray_of_slot(active ? (g >> lgS) : 0, k);
-      ray = make_ray(ray_idx + k.halton_offset);
+      ray_idx = ray_of_slot(active ? (g >> lgS) : 0, k.perm_M, k.perm_Q, k.perm_R);
+      ray = make_ray<false>(ray_idx + k.halton_offset);
     }
     first = false;
     const long long P[3] = {cs.P[0], cs.P[1], cs.P[2]};
@@ -1417,12 +1474,14 @@ __global__ void __launch_bounds__(256) raycast_rmp_kernel(DevMap m, EvalConsts k
                                               hits ? hits + ray_idx : nullptr);
     if (!active || bad || seg != 0) continue;
     float vals[9];
-    ray_outputs(m, k, ray, mstat, en, ea, cs.v, cs.vl,
-                per_ray ? per_ray + 9 * (size_t)ray_idx : nullptr, vals, n_hit, n_act);
-    if (mstat == RMP_RAY_HIT) BlockReduce<RED>::add(acc, vals);
+    if (ray_outputs(m, k, ray, mstat, en, ea, cs.v, cs.vl, quiet,
+                    per_ray ? per_ray + 9 * (size_t)ray_idx : nullptr, vals, n_hit, n_act)) {
+      BlockReduce<RED>::add(acc, vals);
+      added = true;
+    }
   }
   __shared__ CtaSums sums;
-  BlockReduce<RED>::reduce(acc, n_hit, n_act, sums);
+  BlockReduce<RED>::reduce(acc, added, n_hit, n_act, sums);
   grid_finish<RED>(sums, ws, parts, out, k.n_rays,
                    (cs.bad[0] | cs.bad[1] | cs.bad[2]) ? RMP_ERR_INVALID_ARG : RMP_OK);
 }
@@ -1477,21 +1536,6 @@ __device__ __forceinline__ uint32_t pick_cells_warp(uint32_t n) {
     }
   }
   return __shfl_sync(0xffffffffu, best, 0);
-}
-
-__device__ __forceinline__ uint32_t ray_of_slot_p(uint32_t j, uint32_t M, uint32_t Q, uint32_t R) {
-  const uint32_t big = R * (Q + 1);
-  uint32_t r, q;
-  if (j < big) {
-    r = j / (Q + 1);
-    q = j - r * (Q + 1);
-  } else {
-    const uint32_t jj = j - big;
-    const uint32_t t = jj / Q;
-    r = R + t;
-    q = jj - t * Q;
-  }
-  return r + M * q;
 }
 
 // A state's summation segments (log2): the launch's fixed choice, or the most (up to 4) whose
@@ -1923,12 +1967,14 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
   while (c < total) {
     uint32_t cn = 0xffffffffu;
     if (lane == 0 && total > n_warps) cn = n_warps + atomicAdd(&hdr->next_chunk, 1u);
-    // the chunk's state: the last one whose first chunk is <= c
-    uint32_t lo = 0, hi = nst;
-    while (hi - lo > 1) {
-      const uint32_t mid = (lo + hi) >> 1;
-      if (__ldg(&bs[mid].work0) <= c) lo = mid;
-      else hi = mid;
+    // the chunk's state: the last one whose first chunk is <= c, 32 places tested at a time
+    uint32_t lo = 0, len = nst;
+    while (len > 1) {
+      const uint32_t by = (len + 31) / 32, at = lo + lane * by;
+      const bool le = lane * by < len && __ldg(&bs[at].work0) <= c;   // true for lane 0
+      const uint32_t last = 31 - __clz(__ballot_sync(0xffffffffu, le));
+      lo += last * by;
+      len = min(by, len - last * by);
     }
     const uint32_t b = lo;
     const BatchState* sp = bs + b;
@@ -1944,8 +1990,8 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
     const uint32_t slot = g >> lgs, seg = g & (S - 1);
     const bool active = slot < n_b;
     const uint32_t pM = __ldg(&sp->perm_M), pQ = __ldg(&sp->perm_Q);
-    const uint32_t ray_idx = ray_of_slot_p(active ? slot : 0, pM, pQ, n_b - pQ * pM);
-    const Ray ray = make_ray(ray_idx + k.halton_offset);
+    const uint32_t ray_idx = ray_of_slot(active ? slot : 0, pM, pQ, n_b - pQ * pM);
+    const Ray ray = make_ray<true>(ray_idx + k.halton_offset);
     const size_t ro = (size_t)b * max_rays + ray_idx;
     uint32_t en, ea;
     const int mstat = march_ray<KIND, LAYOUT, BOXES>(m, k, P, ray, seg, lgs, active, en, ea,
@@ -1957,9 +2003,15 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
     const uint32_t lg = __ldg(&sp->lg_segs) & 255u, lgW = lg - lgs;
     float vals[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     unsigned nh = 0, na = 0;
+    bool adds = false;
     if (active && seg == 0)
-      ray_outputs(m, k, ray, mstat, en, ea, v, vl, per_ray ? per_ray + 9 * ro : nullptr, vals, nh,
-                  na);
+      adds = ray_outputs(m, k, ray, mstat, en, ea, v, vl, quiet_state(k, v),
+                         per_ray ? per_ray + 9 * ro : nullptr, vals, nh, na);
+    // without any, the partials are the zeros that vals holds
+    const bool any = __any_sync(0xffffffffu, adds);
+    if (!any)
+#pragma unroll
+      for (int i = 0; i < 9; ++i) vals[i] = 0.0f;
     // the chunk's 2^lgW partials, 32 >> lgW lanes each (a ray's other segments hold zeros)
     const uint32_t n_parts = ((n_b << lg) + 31) / 32;
     const uint32_t first = q << lgW, mine = first + (lane >> (5 - lgW));
@@ -1974,15 +2026,15 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
     if (RED == RMP_REDUCE_FP64) {
       double pv[9];
 #pragma unroll
-      for (int i = 0; i < 9; ++i) pv[i] = (double)vals[i];
-      warp_reduce_terms<double, false>(pv, pv, lgW);
+      for (int i = 0; i < 9; ++i) pv[i] = any ? (double)vals[i] : 0.0;
+      if (any) warp_reduce_terms<double, false>(pv, pv, lgW);
       if (mine < n_parts) {
         if (t.n > 0) part->v[t.first] = pv[0];
         if (t.n > 1) part->v[t.first + 1] = pv[1];
       }
     } else {
       float cv[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      warp_reduce_terms<float, true>(vals, cv, lgW);
+      if (any) warp_reduce_terms<float, true>(vals, cv, lgW);
       CtaPartial32* p = reinterpret_cast<CtaPartial32*>(part);
       if (mine < n_parts) {
         if (t.n > 0) {
@@ -2227,6 +2279,8 @@ __global__ void __launch_bounds__(256) scan_rmp_kernel(const float* __restrict__
   unsigned n_hit = 0, n_act = 0;
   const float v[3] = {cs.v[0], cs.v[1], cs.v[2]};
   const float vl[3] = {cs.vl[0], cs.vl[1], cs.vl[2]};
+  const bool quiet = quiet_state(k, v);
+  bool added = false;
   for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < k.n_rays;
        j += gridDim.x * blockDim.x) {
     float q[3];
@@ -2245,9 +2299,13 @@ __global__ void __launch_bounds__(256) scan_rmp_kernel(const float* __restrict__
       const bool inr = d < k.r_up;
       n_hit += 1;
       n_act += (act && inr) ? 1u : 0u;
-      obstacle_policy(k, u, d, v, vl, act, inr, f, A, af);
-      const float vals[9] = {A[0], A[1], A[2], A[3], A[4], A[5], af[0], af[1], af[2]};
-      BlockReduce<RED>::add(acc, vals);
+      const bool adds = (act && inr) || !quiet;
+      if (adds || per_ray) obstacle_policy(k, u, d, v, vl, act, inr, f, A, af);
+      if (adds) {
+        const float vals[9] = {A[0], A[1], A[2], A[3], A[4], A[5], af[0], af[1], af[2]};
+        BlockReduce<RED>::add(acc, vals);
+        added = true;
+      }
     }
     if (per_ray) {
       float* o = per_ray + 9 * (size_t)j;
@@ -2256,7 +2314,7 @@ __global__ void __launch_bounds__(256) scan_rmp_kernel(const float* __restrict__
     }
   }
   __shared__ CtaSums sums;
-  BlockReduce<RED>::reduce(acc, n_hit, n_act, sums);
+  BlockReduce<RED>::reduce(acc, added, n_hit, n_act, sums);
   grid_finish<RED>(sums, ws, parts, out, k.n_rays, RMP_OK);
 }
 
