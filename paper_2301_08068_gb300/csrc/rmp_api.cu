@@ -33,7 +33,8 @@ struct MapRec {
 
 // An ESDF of primitives on the device (rmp_esdf_upload).
 struct EsdfRec {
-  rmp_primitive_t* prims = nullptr;
+  rmp_primitive_t* prims = nullptr;   // then, 16-byte aligned, their FP32 copies
+  const float4* prims32 = nullptr;
   uint32_t n = 0;
 };
 
@@ -893,7 +894,7 @@ int rollout_impl(rmp_ctx* c, uint32_t map_id, const EsdfRec* esdf, const double*
     e = cudaMemsetAsync(d_cnt, 0, 4, s);
     for (uint32_t i = 0; i < kRound && step < rp->max_steps && e == cudaSuccess; ++i, ++step) {
       if (esdf) {
-        e = launch_esdf_eval(esdf->prims, esdf->n, ek, d_st, d_goal, n, d_res, nullptr, s);
+        e = launch_esdf_eval(esdf->prims, esdf->prims32, esdf->n, ek, d_st, d_goal, n, d_res, nullptr, s);
         if (e != cudaSuccess) break;
       } else {
         status = batch_async_impl(c, map_id, d_st, d_nr, n, rp->n_rays, params, buf + o_ws, wsb,
@@ -972,9 +973,31 @@ int rmp_esdf_upload(rmp_ctx* c, const rmp_primitive_t* prims, uint32_t n, uint32
   EsdfRec r;
   r.n = n;
   if (n > 0) {
-    RMP_CUDA(cudaMalloc((void**)&r.prims, sizeof(rmp_primitive_t) * n));
-    const cudaError_t e = cudaMemcpy(r.prims, prims, sizeof(rmp_primitive_t) * n,
-                                     cudaMemcpyHostToDevice);
+    // primitives, then their FP32 copies for the nearest-primitive search (see launch_esdf_eval)
+    const size_t at32 = align256(sizeof(rmp_primitive_t) * n), bytes = at32 + 32 * (size_t)n;
+    std::vector<char> host;
+    try {
+      host.resize(bytes);
+    } catch (...) {
+      return RMP_ERR_NO_MEMORY;
+    }
+    std::memcpy(host.data(), prims, sizeof(rmp_primitive_t) * n);
+    float* f = (float*)(host.data() + at32);
+    for (uint32_t i = 0; i < n; ++i, f += 8) {
+      const bool ball = prims[i].kind == RMP_PRIM_SPHERE;
+      double sum = 0.0;
+      for (int a = 0; a < 3; ++a) {
+        const double h = ball ? (a == 0 ? prims[i].size[0] : 0.0) : prims[i].size[a];
+        f[a] = (float)prims[i].center[a];
+        f[4 + a] = (float)h;
+        sum += std::fabs(prims[i].center[a]) + h;
+      }
+      f[3] = ball ? 1.0f : 0.0f;
+      f[7] = (float)(1.0001 * sum);
+    }
+    RMP_CUDA(cudaMalloc((void**)&r.prims, bytes));
+    r.prims32 = (const float4*)((char*)r.prims + at32);
+    const cudaError_t e = cudaMemcpy(r.prims, host.data(), bytes, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
       cudaFree(r.prims);
       return cuda_status(e);
@@ -1015,7 +1038,7 @@ int rmp_esdf_eval_async(rmp_ctx* c, uint32_t esdf_id, const double* states_dev,
   }
   DeviceGuard g(c->device);
   if (!g.ok()) return RMP_ERR_CUDA;
-  RMP_CUDA(launch_esdf_eval(r.prims, r.n, k, states_dev, goals_dev, n_states, out_dev, query_dev,
+  RMP_CUDA(launch_esdf_eval(r.prims, r.prims32, r.n, k, states_dev, goals_dev, n_states, out_dev, query_dev,
                             (cudaStream_t)stream));
   return RMP_OK;
 }

@@ -208,10 +208,12 @@ cudaError_t launch_batch(const DevMap& m, const EvalConsts& k, const double* sta
 // L2 read-bandwidth probe (see rmp_probe_l2_read): grid CTAs of 512 threads.
 cudaError_t launch_probe_l2(const uint4* buf, size_t n16, uint32_t passes, int grid,
                             uint64_t* checksum, cudaStream_t stream);
-// The ESDF policy for n states, one warp each (see rmp_esdf_eval_async).
-cudaError_t launch_esdf_eval(const rmp_primitive_t* prims, uint32_t n_prims, const EsdfConsts& k,
-                             const double* states, const double* goals, uint32_t n_states,
-                             rmp_result_t* out, double* query, cudaStream_t stream);
+// The ESDF policy for n states (see rmp_esdf_eval_async).  prims32: two float4 per primitive,
+// centre and kind (1 sphere, 0 box), size and the sum of the six magnitudes (rounded up).
+cudaError_t launch_esdf_eval(const rmp_primitive_t* prims, const float4* prims32,
+                             uint32_t n_prims, const EsdfConsts& k, const double* states,
+                             const double* goals, uint32_t n_states, rmp_result_t* out,
+                             double* query, cudaStream_t stream);
 cudaError_t launch_rollout_step(const DevMap& m, const RolloutConsts& rc, const rmp_result_t* res,
                                 double* states, const double* goals, uint32_t* n_rays,
                                 RolloutDev* rs, uint32_t n, uint32_t* running,

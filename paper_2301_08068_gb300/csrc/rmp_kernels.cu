@@ -904,43 +904,10 @@ __device__ __forceinline__ float norm2_minus_one(float v0, float v1, float v2) {
   return __fadd_rn(__fsub_rn(s2, 1.0f), __fadd_rn(__fadd_rn(r1, r2), __fadd_rn(__fadd_rn(e0, e1), e2)));
 }
 
-__device__ __forceinline__ void resolve_eigen(const double* S, const float (&W)[3][3],
-                                              rmp_result_t& r, EigenSet& es) {
-  const int t = threadIdx.x & 31;
-  float V[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) V[i][j] = __shfl_sync(0xffffffffu, W[i][j], 0);
-  // lanes 0-8: lane 3 i + c takes component c of eigenvector i (column i of V): its term
-  // v_c (S v)_c in FP64; lane 3 i adds the three terms and applies 1 / v^T v = 1 - (v^T v - 1)
-  // to first order.  Seven FP64 instructions per warp (every FP64 instruction holds the
-  // pipe about 64 cycles whatever the active lanes).
-  const int iv = t < 9 ? t / 3 : 0, c = t < 9 ? t - 3 * iv : 0;
-  const float w0 = iv == 0 ? V[0][0] : (iv == 1 ? V[0][1] : V[0][2]);
-  const float w1 = iv == 0 ? V[1][0] : (iv == 1 ? V[1][1] : V[1][2]);
-  const float w2 = iv == 0 ? V[2][0] : (iv == 1 ? V[2][1] : V[2][2]);
-  double term = 0.0;
-  if (t < 9) {
-    const double sc0 = c == 0 ? S[0] : (c == 1 ? S[1] : S[2]);
-    const double sc1 = c == 0 ? S[1] : (c == 1 ? S[3] : S[4]);
-    const double sc2 = c == 0 ? S[2] : (c == 1 ? S[4] : S[5]);
-    const double u = sc0 * widen(w0) + sc1 * widen(w1) + sc2 * widen(w2);
-    term = widen(c == 0 ? w0 : (c == 1 ? w1 : w2)) * u;
-  }
-  const double t1 = __shfl_down_sync(0xffffffffu, term, 1);
-  const double t2 = __shfl_down_sync(0xffffffffu, term, 2);
-  const float dv_t = norm2_minus_one(w0, w1, w2);
-  double lam_t = (term + t1) + t2;
-  lam_t = fma(-lam_t, widen(dv_t), lam_t);
-  double lam[3];
-  float dv[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    lam[i] = __shfl_sync(0xffffffffu, lam_t, 3 * i);
-    dv[i] = __shfl_sync(0xffffffffu, dv_t, 3 * i);
-  }
-  if (t != 0) return;
+// One thread: eig (ascending), rank and what a rank-deficient projection needs, from the
+// eigenvalues, their vectors (columns of V) and v^T v - 1.
+__device__ __forceinline__ void rank_eigen(const double lam[3], const float dv[3],
+                                           const float V[3][3], rmp_result_t& r, EigenSet& es) {
   // ascending eigenpairs by a 3-element sorting network on the values' integer keys
   double e0 = lam[0], e1 = lam[1], e2 = lam[2];
   float d0 = dv[0], d1 = dv[1], d2 = dv[2];
@@ -984,6 +951,45 @@ __device__ __forceinline__ void resolve_eigen(const double* S, const float (&W)[
     es.c[1][i] = c1[i];
     es.c[2][i] = c2[i];
   }
+}
+
+__device__ __forceinline__ void resolve_eigen(const double* S, const float (&W)[3][3],
+                                              rmp_result_t& r, EigenSet& es) {
+  const int t = threadIdx.x & 31;
+  float V[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) V[i][j] = __shfl_sync(0xffffffffu, W[i][j], 0);
+  // lanes 0-8: lane 3 i + c takes component c of eigenvector i (column i of V): its term
+  // v_c (S v)_c in FP64; lane 3 i adds the three terms and applies 1 / v^T v = 1 - (v^T v - 1)
+  // to first order.  Seven FP64 instructions per warp (every FP64 instruction holds the
+  // pipe about 64 cycles whatever the active lanes).
+  const int iv = t < 9 ? t / 3 : 0, c = t < 9 ? t - 3 * iv : 0;
+  const float w0 = iv == 0 ? V[0][0] : (iv == 1 ? V[0][1] : V[0][2]);
+  const float w1 = iv == 0 ? V[1][0] : (iv == 1 ? V[1][1] : V[1][2]);
+  const float w2 = iv == 0 ? V[2][0] : (iv == 1 ? V[2][1] : V[2][2]);
+  double term = 0.0;
+  if (t < 9) {
+    const double sc0 = c == 0 ? S[0] : (c == 1 ? S[1] : S[2]);
+    const double sc1 = c == 0 ? S[1] : (c == 1 ? S[3] : S[4]);
+    const double sc2 = c == 0 ? S[2] : (c == 1 ? S[4] : S[5]);
+    const double u = sc0 * widen(w0) + sc1 * widen(w1) + sc2 * widen(w2);
+    term = widen(c == 0 ? w0 : (c == 1 ? w1 : w2)) * u;
+  }
+  const double t1 = __shfl_down_sync(0xffffffffu, term, 1);
+  const double t2 = __shfl_down_sync(0xffffffffu, term, 2);
+  const float dv_t = norm2_minus_one(w0, w1, w2);
+  double lam_t = (term + t1) + t2;
+  lam_t = fma(-lam_t, widen(dv_t), lam_t);
+  double lam[3];
+  float dv[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    lam[i] = __shfl_sync(0xffffffffu, lam_t, 3 * i);
+    dv[i] = __shfl_sync(0xffffffffu, dv_t, 3 * i);
+  }
+  if (t == 0) rank_eigen(lam, dv, V, r, es);
 }
 
 // f into r from the rank (resolve_eigen) and the adjugate solution: full rank takes the
@@ -2119,130 +2125,281 @@ __device__ __forceinline__ double esdf_prim_sdf(const rmp_primitive_t& p, const 
   return __dadd_rn(out, in);
 }
 
-// Gradient of one primitive's distance at x (unit, pointing away from the primitive).
-__device__ __forceinline__ void esdf_prim_grad(const rmp_primitive_t& p, const double x[3],
-                                               double g[3]) {
-  const double q[3] = {__dsub_rn(x[0], p.center[0]), __dsub_rn(x[1], p.center[1]),
-                       __dsub_rn(x[2], p.center[2])};
-  if (p.kind == RMP_PRIM_SPHERE) {
-    const double L = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(q[0], q[0]), __dmul_rn(q[1], q[1])),
-                                          __dmul_rn(q[2], q[2])));
-    for (int a = 0; a < 3; ++a) g[a] = L > 0.0 ? __ddiv_rn(q[a], L) : 0.0;
-    return;
+// The same distance and, if wanted, its gradient (unit, pointing away from the primitive),
+// spheres and boxes in one instruction stream: both are the length of a vector o (the offset
+// from the centre; its part outside the box) less a constant, and the gradient is o / |o| (the
+// centre of a sphere: 0; inside a box the normal of the nearest face).
+__device__ __forceinline__ double esdf_nearest(const rmp_primitive_t& p, const double x[3],
+                                               double* g) {
+  const bool ball = p.kind == RMP_PRIM_SPHERE;
+  double q[3], a[3], o[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    q[i] = __dsub_rn(x[i], p.center[i]);
+    a[i] = __dsub_rn(fabs(q[i]), p.size[i]);
+    o[i] = ball ? fabs(q[i]) : (a[i] > 0.0 ? a[i] : 0.0);
   }
-  double ai[3], o[3];
-  for (int a = 0; a < 3; ++a) {
-    ai[a] = __dsub_rn(fabs(q[a]), p.size[a]);
-    o[a] = ai[a] > 0.0 ? ai[a] : 0.0;
+  const double L = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(o[0], o[0]), __dmul_rn(o[1], o[1])),
+                                        __dmul_rn(o[2], o[2])));
+  if (g) {
+    const int k = (a[0] >= a[1] && a[0] >= a[2]) ? 0 : (a[1] >= a[2] ? 1 : 2);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double n = L > 0.0 ? __ddiv_rn(o[i], L) : ((!ball && i == k) ? 1.0 : 0.0);
+      g[i] = q[i] < 0.0 ? -n : n;
+    }
   }
-  const double out = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(o[0], o[0]), __dmul_rn(o[1], o[1])),
-                                          __dmul_rn(o[2], o[2])));
-  if (out > 0.0) {
-    for (int a = 0; a < 3; ++a) g[a] = __ddiv_rn(q[a] < 0.0 ? -o[a] : o[a], out);
-    return;
-  }
-  const int k = (ai[0] >= ai[1] && ai[0] >= ai[2]) ? 0 : (ai[1] >= ai[2] ? 1 : 2);
-  for (int a = 0; a < 3; ++a) g[a] = a == k ? (q[a] < 0.0 ? -1.0 : 1.0) : 0.0;
+  double in = a[0] > a[1] ? a[0] : a[1];
+  in = in > a[2] ? in : a[2];
+  in = in < 0.0 ? in : 0.0;
+  return __dadd_rn(L, ball ? -p.size[0] : in);
 }
 
-// One warp per state: the lanes scan the primitives (lane i: i, i + 32, ...), the warp keeps
-// the smallest distance (lowest index on ties: the first minimum of a sequential scan);
-// lane 0 evaluates the obstacle policy of Sec. III-C on (d, gradient) in FP64 and adds the
-// attractor; the warp resolves Eq. (1).
+// Signed distance of primitive i to FP32 precision, with a bound on its error: S adds up the
+// sizes of everything the distance is formed from, and the roundings of the operands, the
+// differences, the squares and the root stay below 2^-20.5 S (2^-19 is used) beside an absolute
+// term for squares that underflow.  p: centre and kind (1 sphere), size and the primitive's share
+// of S, infinite where FP32 squares could overflow: the bound is then infinite too.
+__device__ __forceinline__ float esdf_prim_sdf32(const float4 c, const float4 h, const float x[3],
+                                                 float x_sum, float& err) {
+  const float q0 = x[0] - c.x, q1 = x[1] - c.y, q2 = x[2] - c.z;
+  const bool ball = c.w != 0.0f;
+  const float a0 = fabsf(q0) - h.x, a1 = fabsf(q1) - h.y, a2 = fabsf(q2) - h.z;
+  const float o0 = ball ? q0 : fmaxf(a0, 0.0f), o1 = ball ? q1 : fmaxf(a1, 0.0f),
+              o2 = ball ? q2 : fmaxf(a2, 0.0f);
+  const float L = __fsqrt_rn(o0 * o0 + o1 * o1 + o2 * o2);
+  const float S = x_sum + h.w;
+  err = S < 1e18f ? 1.9073486328125e-6f * S + 1e-18f : INFINITY;
+  return L + (ball ? -h.x : fminf(fmaxf(fmaxf(a0, a1), a2), 0.0f));
+}
+
+// Order-preserving unsigned key of a float that is not NaN, and back.
+__device__ __forceinline__ uint32_t float_key(float f) {
+  const uint32_t b = __float_as_uint(f);
+  return b ^ ((b >> 31) ? 0xffffffffu : 0x80000000u);
+}
+__device__ __forceinline__ float key_float(uint32_t k) {
+  return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xffffffffu));
+}
+
+// The ESDF policy, G states (8 or 32) a CTA.  An FP64 instruction holds a scheduler's pipe about
+// 64 cycles whatever its active lanes, so the exact arithmetic runs with a state per lane:
+//   1. a warp per state finds the nearest primitive (lane i: i, i + 32, ...) from FP32 distances
+//      and their error bounds: it is decided when only one primitive's lower bound lies below
+//      the smallest upper bound; otherwise (ties, or closer than FP32 can tell) those primitives
+//      are compared by their FP64 distances, the first minimum of a sequential scan winning;
+//   2. one warp evaluates the damping part of the obstacle policy of Sec. III-C on (d, gradient),
+//      one its repulsion and weight, one the attractor;
+//   3. one warp runs the Jacobi sweeps, another the adjugate solve; three warps take one
+//      Rayleigh quotient each; the first sorts, decides the rank and writes the results.
+// The warps of the serial parts rotate with the CTA and with its turn on an SM (152 of them), so
+// that an SM's CTAs use different schedulers' pipes.  Bound by the FP64 chain of steps 2 and 3.  16384 states, 200 primitives:
+// 51 us (one warp per state, every distance in FP64, policy in one lane: 638 us); 128 states 18.5 (51).
 __global__ void __launch_bounds__(256) esdf_eval_kernel(const rmp_primitive_t* __restrict__ prims,
+                                                        const float4* __restrict__ prims32,
                                                         uint32_t n_prims, EsdfConsts k,
                                                         const double* __restrict__ states,
                                                         const double* __restrict__ goals,
-                                                        uint32_t n_states, rmp_result_t* out,
-                                                        double* query) {
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t n_warps = gridDim.x * (blockDim.x >> 5);
-  for (uint32_t b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); b < n_states;
-       b += n_warps) {
-    const double* st = states + 6 * (size_t)b;
-    const double x[3] = {st[0], st[1], st[2]};
-    const double v[3] = {st[3], st[4], st[5]};
-    bool bad = false;
-    for (int a = 0; a < 6; ++a) bad = bad || !isfinite(st[a]);
-    double best = INFINITY;
-    uint32_t bi = 0xffffffffu;
-    if (!bad)
-      for (uint32_t i = lane; i < n_prims; i += 32) {
-        const double sd = esdf_prim_sdf(prims[i], x);
-        if (sd < best) {                  // strict: a lane's earlier primitive wins ties
-          best = sd;
-          bi = i;
+                                                        uint32_t n_states, uint32_t G,
+                                                        rmp_result_t* out, double* query) {
+  __shared__ uint32_t near_sh[32], act_sh[32];
+  __shared__ bool bad_sh[32];
+  __shared__ double P[7][32], att[3][32], fa[3][32], lam_sh[3][32];
+  __shared__ float W[9][32], dv_sh[3][32];
+  __shared__ int ok_sh[32];
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t role = (warp + blockIdx.x + blockIdx.x / 152u) & 7u;
+  constexpr uint32_t kNone = 0xffffffffu;
+  for (uint32_t base = blockIdx.x * G; base < n_states; base += gridDim.x * G) {
+    for (uint32_t s = warp; s < G && base + s < n_states; s += 8) {
+      const double* st = states + 6 * (size_t)(base + s);
+      const bool bad = __any_sync(0xffffffffu, lane < 6 && !isfinite(st[lane < 6 ? lane : 0]));
+      uint32_t bi = kNone;
+      if (!bad) {
+        const double x[3] = {st[0], st[1], st[2]};
+        const float xf[3] = {__double2float_rn(x[0]), __double2float_rn(x[1]),
+                             __double2float_rn(x[2])};
+        const float x_sum = fabsf(xf[0]) + fabsf(xf[1]) + fabsf(xf[2]);
+        // smallest upper bound; the two smallest lower bounds and the first one's primitive
+        float up = INFINITY, lo1 = INFINITY, lo2 = INFINITY;
+        uint32_t i1 = kNone;
+        for (uint32_t i = lane; i < n_prims; i += 32) {
+          float err;
+          const float sd = esdf_prim_sdf32(__ldg(prims32 + 2 * i), __ldg(prims32 + 2 * i + 1), xf,
+                                           x_sum, err);
+          const bool known = err < INFINITY;
+          up = fminf(up, known ? sd + err : INFINITY);
+          const float lo = known ? sd - err : -INFINITY;
+          if (lo < lo1 || i1 == kNone) {
+            lo2 = lo1;
+            lo1 = lo;
+            i1 = i;
+          } else {
+            lo2 = fminf(lo2, lo);
+          }
+        }
+        const float cut = key_float(__reduce_min_sync(0xffffffffu, float_key(up)));
+        const bool mine = i1 != kNone && lo1 <= cut;
+        const uint32_t cand = __ballot_sync(0xffffffffu, mine);
+        const bool more = __any_sync(0xffffffffu, mine && lo2 <= cut);
+        if (__popc(cand) == 1 && !more) {
+          bi = __shfl_sync(0xffffffffu, i1, __ffs(cand) - 1);
+        } else {
+          double best = INFINITY;
+          for (uint32_t i = lane; i < n_prims; i += 32) {
+            float err;
+            const float sd = esdf_prim_sdf32(__ldg(prims32 + 2 * i), __ldg(prims32 + 2 * i + 1), xf,
+                                             x_sum, err);
+            if (err < INFINITY && !(sd - err <= cut)) continue;
+            const double e = esdf_prim_sdf(prims[i], x);
+            if (e < best) {                   // strict: a lane's earlier primitive wins ties
+              best = e;
+              bi = i;
+            }
+          }
+#pragma unroll
+          for (int off = 16; off > 0; off >>= 1) {
+            const double b2 = __shfl_down_sync(0xffffffffu, best, off);
+            const uint32_t i2 = __shfl_down_sync(0xffffffffu, bi, off);
+            if (b2 < best || (b2 == best && i2 < bi)) {
+              best = b2;
+              bi = i2;
+            }
+          }
         }
       }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const double b2 = __shfl_down_sync(0xffffffffu, best, off);
-      const uint32_t i2 = __shfl_down_sync(0xffffffffu, bi, off);
-      if (b2 < best || (b2 == best && i2 < bi)) {
-        best = b2;
-        bi = i2;
+      if (lane == 0) {
+        near_sh[s] = bi;
+        bad_sh[s] = bad;
       }
     }
-    double tv[9] = {0., 0., 0., 0., 0., 0., 0., 0., 0.};
-    double d = INFINITY, g[3] = {0.0, 0.0, 0.0};
-    unsigned hit = 0, act = 0;
-    if (lane == 0 && !bad) {
-      if (bi != 0xffffffffu) {
-        d = best > 0.0 ? best : 0.0;
-        esdf_prim_grad(prims[bi], x, g);
-        hit = 1;
-        // obstacle policy (Sec. III-C) on the single pair (d, r = g), FP64
-        const double xr = __dadd_rn(__dadd_rn(__dmul_rn(v[0], g[0]), __dmul_rn(v[1], g[1])),
-                                    __dmul_rn(v[2], g[2]));
-        const bool active = xr < 0.0, in_r = d < k.r;
-        act = (active && in_r) ? 1u : 0u;
-        const double frep = k.eta_rep * exp(-d / k.nu_rep);
-        const double m = active ? xr * xr : 0.0;
-        const double kd = k.eta_damp / (d / k.nu_damp + k.eps);
-        const double z = kd * m;                          // |f_damp|
-        double w = 0.0;
-        if (in_r) {
+    __syncthreads();
+    // a state per lane from here on
+    const uint32_t b = base + lane;
+    const bool mine = lane < G && b < n_states;
+    const double* st = states + 6 * (size_t)(mine ? b : base);
+    if ((role == 0 || role == 2) && mine) {
+      const double x[3] = {st[0], st[1], st[2]};
+      const uint32_t bi = near_sh[lane];
+      double d = INFINITY, g[3] = {0.0, 0.0, 0.0};
+      if (bi != kNone) {
+        const double sd = esdf_nearest(prims[bi], x, role == 0 ? g : nullptr);
+        d = sd > 0.0 ? sd : 0.0;
+      }
+      // obstacle policy (Sec. III-C) on the single pair (d, r = g), FP64
+      if (role == 2) {
+        double frep = 0.0, w = 0.0;
+        if (bi != kNone) frep = k.eta_rep * exp(-d / k.nu_rep);
+        if (d < k.r) {
           const double y = (k.r - d) / k.r;               // 1 - d / r, exact difference
           w = k.w_mode == 0 ? y * y : y * y * (1.0 + 2.0 * (d / k.r));
         }
-        const double h = z + k.c * log1p(exp(-2.0 * k.c * z));
-        const double sc = h > 0.0 ? z / h : 0.0;
-        const double alpha_m = w * sc * sc;               // A = alpha_m r r^T
-        const double fr = frep + z;                       // f = fr r
-        tv[0] = alpha_m * g[0] * g[0];
-        tv[1] = alpha_m * g[0] * g[1];
-        tv[2] = alpha_m * g[0] * g[2];
-        tv[3] = alpha_m * g[1] * g[1];
-        tv[4] = alpha_m * g[1] * g[2];
-        tv[5] = alpha_m * g[2] * g[2];
-        const double rf = fr * ((g[0] * g[0] + g[1] * g[1]) + g[2] * g[2]);
-        for (int a = 0; a < 3; ++a) tv[6 + a] = alpha_m * rf * g[a];
+        P[3][lane] = frep;
+        P[4][lane] = w;
+      } else {
+        double z = 0.0, sc = 0.0;
+        uint32_t act = 0;
+        if (bi != kNone) {
+          const double xr = __dadd_rn(__dadd_rn(__dmul_rn(st[3], g[0]), __dmul_rn(st[4], g[1])),
+                                      __dmul_rn(st[5], g[2]));
+          const bool active = xr < 0.0;
+          act = (active && d < k.r) ? 1u : 0u;
+          const double m = active ? xr * xr : 0.0;
+          const double kd = k.eta_damp / (d / k.nu_damp + k.eps);
+          z = kd * m;                                     // |f_damp|
+          const double h = z + k.c * log1p(exp(-2.0 * k.c * z));
+          sc = h > 0.0 ? z / h : 0.0;
+        }
+        P[0][lane] = g[0];
+        P[1][lane] = g[1];
+        P[2][lane] = g[2];
+        P[5][lane] = z;
+        P[6][lane] = sc;
+        act_sh[lane] = act;
+        if (query) {
+          double* qd = query + 4 * (size_t)b;
+          qd[0] = d;
+          qd[1] = g[0];
+          qd[2] = g[1];
+          qd[3] = g[2];
+        }
       }
-      if (goals) {                                         // attractor, metric I (Eq. 1)
-        const double* gl = goals + 3 * (size_t)b;
-        const double e0 = gl[0] - x[0], e1 = gl[1] - x[1], e2 = gl[2] - x[2];
-        const double zz = sqrt(e0 * e0 + e1 * e1 + e2 * e2);
-        const double hh = zz + k.c * log1p(exp(-2.0 * k.c * zz));
+    } else if (role == 1 && mine && goals) {               // attractor, metric I (Eq. 1)
+      const double* gl = goals + 3 * (size_t)b;
+      const double e0 = gl[0] - st[0], e1 = gl[1] - st[1], e2 = gl[2] - st[2];
+      const double zz = sqrt(e0 * e0 + e1 * e1 + e2 * e2);
+      const double hh = zz + k.c * log1p(exp(-2.0 * k.c * zz));
+      att[0][lane] = k.alpha * (e0 / hh) - k.beta * st[3];
+      att[1][lane] = k.alpha * (e1 / hh) - k.beta * st[4];
+      att[2][lane] = k.alpha * (e2 / hh) - k.beta * st[5];
+    }
+    __syncthreads();
+    // the sums, in the warps that need them: A = w sc^2 r r^T, f = (f_rep + z) r
+    double tv[9];
+    const bool bad = mine && bad_sh[lane];
+    if (role < 3 && mine) {
+      const double g[3] = {P[0][lane], P[1][lane], P[2][lane]};
+      const double alpha_m = P[4][lane] * P[6][lane] * P[6][lane], fr = P[3][lane] + P[5][lane];
+      tv[0] = alpha_m * g[0] * g[0];
+      tv[1] = alpha_m * g[0] * g[1];
+      tv[2] = alpha_m * g[0] * g[2];
+      tv[3] = alpha_m * g[1] * g[1];
+      tv[4] = alpha_m * g[1] * g[2];
+      tv[5] = alpha_m * g[2] * g[2];
+      const double rf = fr * ((g[0] * g[0] + g[1] * g[1]) + g[2] * g[2]);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) tv[6 + a] = alpha_m * rf * g[a];
+      if (goals && !bad) {
         tv[0] += 1.0;
         tv[3] += 1.0;
         tv[5] += 1.0;
-        tv[6] += k.alpha * (e0 / hh) - k.beta * v[0];
-        tv[7] += k.alpha * (e1 / hh) - k.beta * v[1];
-        tv[8] += k.alpha * (e2 / hh) - k.beta * v[2];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) tv[6 + a] += att[a][lane];
       }
     }
+    if (role == 0 && mine) {
+      float V[3][3] = {{1.f, 0.f, 0.f}, {0.f, 1.f, 0.f}, {0.f, 0.f, 1.f}};
+      jacobi_f32(tv, V);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) tv[i] = __shfl_sync(0xffffffffu, tv[i], 0);
-    rmp_result_t r;
-    resolve_pinv(tv, tv + 6, r);
-    if (lane == 0) {
+      for (int i = 0; i < 9; ++i) W[i][lane] = V[i / 3][i % 3];
+    } else if (role == 1 && mine) {
+      double f0 = 0.0, f1 = 0.0, f2 = 0.0;
+      int ok = 0;
+      adjugate_solve(tv, tv + 6, f0, f1, f2, ok);
+      fa[0][lane] = f0;
+      fa[1][lane] = f1;
+      fa[2][lane] = f2;
+      ok_sh[lane] = ok;
+    }
+    __syncthreads();
+    if (role < 3 && mine) {                                // eigenvalue `role`: its quotient
+      const float w0 = W[role][lane], w1 = W[3 + role][lane], w2 = W[6 + role][lane];
+      const double t0 = widen(w0) * (tv[0] * widen(w0) + tv[1] * widen(w1) + tv[2] * widen(w2));
+      const double t1 = widen(w1) * (tv[1] * widen(w0) + tv[3] * widen(w1) + tv[4] * widen(w2));
+      const double t2 = widen(w2) * (tv[2] * widen(w0) + tv[4] * widen(w1) + tv[5] * widen(w2));
+      const float dv = norm2_minus_one(w0, w1, w2);
+      const double l = __dadd_rn(__dadd_rn(t0, t1), t2);
+      lam_sh[role][lane] = fma(-l, widen(dv), l);
+      dv_sh[role][lane] = dv;
+    }
+    __syncthreads();
+    if (role == 0 && mine) {
+      rmp_result_t r;
+      const double lam[3] = {lam_sh[0][lane], lam_sh[1][lane], lam_sh[2][lane]};
+      const float dv[3] = {dv_sh[0][lane], dv_sh[1][lane], dv_sh[2][lane]};
+      float V[3][3];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) V[i / 3][i % 3] = W[i][lane];
+      EigenSet es;
+      rank_eigen(lam, dv, V, r, es);
+      resolve_f(tv + 6, es, fa[0][lane], fa[1][lane], fa[2][lane], ok_sh[lane], r);
 #pragma unroll
       for (int i = 0; i < 6; ++i) r.A[i] = tv[i];
 #pragma unroll
       for (int i = 0; i < 3; ++i) r.Af[i] = tv[6 + i];
       r.n_rays = 1;
-      r.n_hits = hit;
-      r.n_active = act;
+      r.n_hits = near_sh[lane] != kNone ? 1u : 0u;
+      r.n_active = act_sh[lane];
       r.status = bad ? RMP_ERR_INVALID_ARG : RMP_OK;
       r.reserved = 0;
       if (bad) {
@@ -2251,14 +2408,8 @@ __global__ void __launch_bounds__(256) esdf_eval_kernel(const rmp_primitive_t* _
         r.rank = 0;
       }
       out[b] = r;
-      if (query) {
-        double* qd = query + 4 * (size_t)b;
-        qd[0] = d;
-        qd[1] = g[0];
-        qd[2] = g[1];
-        qd[3] = g[2];
-      }
     }
+    __syncthreads();                                       // the next tile reuses the arrays
   }
 }
 
@@ -2896,15 +3047,18 @@ cudaError_t launch_probe_l2(const uint4* buf, size_t n16, uint32_t passes, int g
   return cudaGetLastError();
 }
 
-cudaError_t launch_esdf_eval(const rmp_primitive_t* prims, uint32_t n_prims, const EsdfConsts& k,
-                             const double* states, const double* goals, uint32_t n_states,
-                             rmp_result_t* out, double* query, cudaStream_t stream) {
+cudaError_t launch_esdf_eval(const rmp_primitive_t* prims, const float4* prims32,
+                             uint32_t n_prims, const EsdfConsts& k, const double* states,
+                             const double* goals, uint32_t n_states, rmp_result_t* out,
+                             double* query, cudaStream_t stream) {
   if (n_states == 0) return cudaSuccess;
-  const uint32_t warps = 8;                         // states per 256-thread CTA
-  uint32_t grid = (n_states + warps - 1) / warps;
-  if (grid > 65535) grid = 65535;                   // warp-stride beyond
-  esdf_eval_kernel<<<grid, 32 * warps, 0, stream>>>(prims, n_prims, k, states, goals, n_states,
-                                                     out, query);
+  // 8 states a CTA (a warp each for the search) while that leaves no more than two CTAs an SM:
+  // few states wait for latency; 32 beyond, where the FP64 steps should fill their lanes
+  const uint32_t G = n_states <= 8u * 304u ? 8u : 32u;
+  uint32_t grid = (n_states + G - 1) / G;
+  if (grid > 65535) grid = 65535;                   // CTA-stride beyond
+  esdf_eval_kernel<<<grid, 256, 0, stream>>>(prims, prims32, n_prims, k, states, goals, n_states, G,
+                                             out, query);
   return cudaGetLastError();
 }
 
