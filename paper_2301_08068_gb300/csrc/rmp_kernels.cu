@@ -274,10 +274,6 @@ __device__ __forceinline__ void ray_fx(const DevMap& m, const long long P[3], co
   }
 }
 
-__device__ __forceinline__ uint32_t sel3(const uint32_t v[3], int i) {
-  return i == 0 ? v[0] : (i == 1 ? v[1] : v[2]);
-}
-
 // Pieces of a ray.  The parameter range (0, R], R = R_fx / 2^24 voxel units, is cut at the
 // points T_j = j R / 2^kGridLog; a piece covers (T_lo, T_hi] between two of them.  A crossing
 // numerator n of axis a satisfies n / |D_a| <= T_j iff n 2^(24 + kGridLog) <= j R_fx |D_a|, so
@@ -881,20 +877,54 @@ __device__ __forceinline__ double recip_pos(double x) {
   return __longlong_as_double((br & 0x000FFFFFFFFFFFFFll) | ((long long)er << 52));
 }
 
-// FP64 solve adj(S) b / det(S); ok = det > 0.  One thread.
+// FP64 solve adj(S) b / det(S); ok = det > 0.  The roundings are spelled out, so that one thread
+// and a warp give the same bits: a cofactor p q - r u as fma(p, q, -(r u)), the determinant as
+// fma(S2, c02, fma(S1, c01, S0 c00)), a row as fma(z, b2, fma(x, b0, y b1)).
+__device__ __forceinline__ double cofactor(double p, double q, double r, double u) {
+  return __fma_rn(p, q, -__dmul_rn(r, u));
+}
+__device__ __forceinline__ double determinant(const double* S, double c00, double c01, double c02) {
+  return __fma_rn(S[2], c02, __fma_rn(S[1], c01, __dmul_rn(S[0], c00)));
+}
+__device__ __forceinline__ double adjugate_row(double x, double y, double z, const double* b,
+                                               double inv) {
+  return __dmul_rn(__fma_rn(z, b[2], __fma_rn(x, b[0], __dmul_rn(y, b[1]))), inv);
+}
+
+// One thread.
 __device__ __forceinline__ void adjugate_solve(const double* S, const double* b, double& fa0,
                                                double& fa1, double& fa2, int& ok) {
-  const double c00 = S[3] * S[5] - S[4] * S[4], c01 = S[2] * S[4] - S[1] * S[5],
-               c02 = S[1] * S[4] - S[2] * S[3], c11 = S[0] * S[5] - S[2] * S[2],
-               c12 = S[1] * S[2] - S[0] * S[4], c22 = S[0] * S[3] - S[1] * S[1];
-  const double det = S[0] * c00 + S[1] * c01 + S[2] * c02;
+  const double c00 = cofactor(S[3], S[5], S[4], S[4]), c01 = cofactor(S[2], S[4], S[1], S[5]),
+               c02 = cofactor(S[1], S[4], S[2], S[3]), c11 = cofactor(S[0], S[5], S[2], S[2]),
+               c12 = cofactor(S[1], S[2], S[0], S[4]), c22 = cofactor(S[0], S[3], S[1], S[1]);
+  const double det = determinant(S, c00, c01, c02);
   ok = det > 0.0;
   if (det > 0.0) {
     const double inv = recip_pos(det);
-    fa0 = (c00 * b[0] + c01 * b[1] + c02 * b[2]) * inv;
-    fa1 = (c01 * b[0] + c11 * b[1] + c12 * b[2]) * inv;
-    fa2 = (c02 * b[0] + c12 * b[1] + c22 * b[2]) * inv;
+    fa0 = adjugate_row(c00, c01, c02, b, inv);
+    fa1 = adjugate_row(c01, c11, c12, b, inv);
+    fa2 = adjugate_row(c02, c12, c22, b, inv);
   }
+}
+
+// A whole warp, S and b in every lane: the cofactors on lanes 0-5, the determinant and its
+// reciprocal in all of them, component i of the solution in lane i (0-2): 17 FP64 instructions
+// one after the other instead of 38.
+__device__ __forceinline__ double adjugate_solve_warp(const double* S, const double* b, int& ok) {
+  const uint32_t t = threadIdx.x & 31;
+  const double p = t == 0 ? S[3] : (t == 1 ? S[2] : (t == 2 || t == 4 ? S[1] : S[0]));
+  const double q = t == 0 || t == 3 ? S[5] : (t == 1 || t == 2 ? S[4] : (t == 4 ? S[2] : S[3]));
+  const double r = t == 0 ? S[4] : (t == 1 || t == 5 ? S[1] : (t == 4 ? S[0] : S[2]));
+  const double u = t == 0 || t == 4 ? S[4] : (t == 1 ? S[5] : (t == 2 ? S[3] : (t == 3 ? S[2] : S[1])));
+  const double c = cofactor(p, q, r, u);
+  const double c00 = __shfl_sync(0xffffffffu, c, 0), c01 = __shfl_sync(0xffffffffu, c, 1),
+               c02 = __shfl_sync(0xffffffffu, c, 2), c11 = __shfl_sync(0xffffffffu, c, 3),
+               c12 = __shfl_sync(0xffffffffu, c, 4), c22 = __shfl_sync(0xffffffffu, c, 5);
+  const double det = determinant(S, c00, c01, c02);
+  ok = det > 0.0;
+  if (!ok) return 0.0;
+  return adjugate_row(t == 0 ? c00 : (t == 1 ? c01 : c02), t == 0 ? c01 : (t == 1 ? c11 : c12),
+                      t == 0 ? c02 : (t == 1 ? c12 : c22), b, recip_pos(det));
 }
 
 // Sorted eigenpairs and rank from the FP32 eigenvectors W (valid in lane 0): lanes 0-2 take
@@ -1030,22 +1060,18 @@ __device__ __forceinline__ void resolve_f(const double* b, const EigenSet& es, d
   }
 }
 
-// One warp: lane 0 runs the Jacobi sweeps, lane 1 the adjugate solve (the two branches
-// of one warp run one after the other).  Called by all 32 lanes of one warp.
+// One warp, S and b in every lane: the adjugate solve across the lanes, then lane 0's Jacobi
+// sweeps and the Rayleigh quotients.  Only lane 0's r is set.
 __device__ void resolve_pinv(const double* S, const double* b, rmp_result_t& r) {
-  const int t = threadIdx.x & 31;
   float W[3][3] = {{1.f, 0.f, 0.f}, {0.f, 1.f, 0.f}, {0.f, 0.f, 1.f}};
-  double fa0 = 0.0, fa1 = 0.0, fa2 = 0.0;
-  int ok = 0;
-  if (t == 0) jacobi_f32(S, W);
-  else if (t == 1) adjugate_solve(S, b, fa0, fa1, fa2, ok);
-  fa0 = __shfl_sync(0xffffffffu, fa0, 1);
-  fa1 = __shfl_sync(0xffffffffu, fa1, 1);
-  fa2 = __shfl_sync(0xffffffffu, fa2, 1);
-  ok = __shfl_sync(0xffffffffu, ok, 1);
+  int ok;
+  const double f = adjugate_solve_warp(S, b, ok);
+  const double fa0 = __shfl_sync(0xffffffffu, f, 0), fa1 = __shfl_sync(0xffffffffu, f, 1),
+               fa2 = __shfl_sync(0xffffffffu, f, 2);
+  if ((threadIdx.x & 31) == 0) jacobi_f32(S, W);
   EigenSet es;
   resolve_eigen(S, W, r, es);
-  if (t == 0) resolve_f(b, es, fa0, fa1, fa2, ok, r);
+  if ((threadIdx.x & 31) == 0) resolve_f(b, es, fa0, fa1, fa2, ok, r);
 }
 
 // Two warps of a CTA (threads 0-63): warp 0 runs the Jacobi sweeps and the Rayleigh
@@ -1057,15 +1083,10 @@ __device__ void resolve_pinv_cta(const double* S, const double* b, rmp_result_t&
   __shared__ int ok_sh;
   const int t = threadIdx.x;
   if (t >= 32) {
-    if (t == 32) {
-      double fa0 = 0.0, fa1 = 0.0, fa2 = 0.0;
-      int ok = 0;
-      adjugate_solve(S, b, fa0, fa1, fa2, ok);
-      fa_sh[0] = fa0;
-      fa_sh[1] = fa1;
-      fa_sh[2] = fa2;
-      ok_sh = ok;
-    }
+    int ok;
+    const double f = adjugate_solve_warp(S, b, ok);
+    if (t < 35) fa_sh[t - 32] = f;
+    if (t == 32) ok_sh = ok;
     __syncwarp();
     asm volatile("bar.sync 1, 64;" ::: "memory");
     return;
@@ -1754,8 +1775,8 @@ __device__ __forceinline__ void load_partial(const CtaPartial* p, double v[9], u
 }
 
 // Sum of 32 lanes' FP64 terms into *p (or the lanes' slot 0, p null), counts into h, a.
-__device__ __forceinline__ WarpTerms warp_sum_partial(double (&v)[9], unsigned& h, unsigned& a,
-                                                      CtaPartial* p) {
+__device__ __forceinline__ void warp_sum_partial(double (&v)[9], unsigned& h, unsigned& a,
+                                                 CtaPartial* p) {
   const WarpTerms t = warp_terms(0);
   warp_reduce_terms<double, false>(v, v, 0);
   h = __reduce_add_sync(0xffffffffu, h);
@@ -1767,26 +1788,21 @@ __device__ __forceinline__ WarpTerms warp_sum_partial(double (&v)[9], unsigned& 
       p->n_active = a;
     }
   }
-  return t;
 }
 
-// Attractor policy (Sec. III-B, Eq. attractorPolicy) combined by Eq. (1): its metric I is
-// added to sum A and f_a = alpha s(goal - x) - beta xdot to sum A f, in FP64 -- after
-// dividing the ray sums by the ray count when the ray policies' mean is asked for.
-__device__ __forceinline__ void add_attractor(const EvalConsts& k, const double* st,
-                                              const double* goal, uint32_t n_rays, double tv[9]) {
-  if (k.att_mean && n_rays > 0)
-#pragma unroll
-    for (int i = 0; i < 9; ++i) tv[i] = tv[i] / (double)n_rays;
-  const double v0 = goal[0] - st[0], v1 = goal[1] - st[1], v2 = goal[2] - st[2];
+// Attractor policy (Sec. III-B, Eq. attractorPolicy): f_a = alpha s(goal - x) - beta xdot in FP64,
+// component a in lane a (0-2).  Called by all lanes of a warp, so that the root, the exponential
+// and the division are one warp instruction stream (an FP64 instruction holds the pipe about
+// 64 cycles whatever the lanes).
+__device__ __forceinline__ double attractor(const EvalConsts& k, const double* st,
+                                            const double* goal) {
+  const uint32_t lane = threadIdx.x & 31, a = lane < 3 ? lane : 0;
+  const double va = goal[a] - st[a];
+  const double v0 = __shfl_sync(0xffffffffu, va, 0), v1 = __shfl_sync(0xffffffffu, va, 1),
+               v2 = __shfl_sync(0xffffffffu, va, 2);
   const double z = sqrt(v0 * v0 + v1 * v1 + v2 * v2);
   const double h = z + k.c64 * log1p(exp(-2.0 * k.c64 * z));
-  tv[0] += 1.0;
-  tv[3] += 1.0;
-  tv[5] += 1.0;
-  tv[6] += k.att_alpha * (v0 / h) - k.att_beta * st[3];
-  tv[7] += k.att_alpha * (v1 / h) - k.att_beta * st[4];
-  tv[8] += k.att_alpha * (v2 / h) - k.att_beta * st[5];
+  return k.att_alpha * (va / h) - k.att_beta * st[3 + a];
 }
 
 template <int KIND>
@@ -1914,42 +1930,53 @@ __device__ __noinline__ void batch_group_finish(const EvalConsts& k, CtaPartial*
   const uint32_t lane = threadIdx.x & 31;
   // the group's partials, lane i: partial i
   __threadfence();
-  double gv[9] = {0., 0., 0., 0., 0., 0., 0., 0., 0.};
-  unsigned gh = 0, ga = 0;
-  if (lane < gsz)
-    load_partial<RED == RMP_REDUCE_KAHAN32>(cparts + part0 + gi * kBatchGroup + lane, gv, gh, ga);
-  warp_sum_partial(gv, gh, ga, gparts + group0 + gi);
-  const uint32_t n_groups = (n_parts + kBatchGroup - 1) / kBatchGroup;
-  __threadfence();
-  __syncwarp();
-  uint32_t last = 0;
-  if (lane == 0) last = atomicAdd(&sticket[b], 1u) == n_groups - 1 ? 1u : 0u;
-  if (!__shfl_sync(0xffffffffu, last, 0)) return;
-  // last group of the state: lane i sums groups i, i + 32, ... in order, then the tree
-  __threadfence();
-  double tv[9] = {0., 0., 0., 0., 0., 0., 0., 0., 0.};
+  double v[9] = {0., 0., 0., 0., 0., 0., 0., 0., 0.};
   unsigned th = 0, ta = 0;
-  for (uint32_t j = lane; j < n_groups; j += 32) {
-    double pv2[9];
-    unsigned h2, a2;
-    load_partial<false>(gparts + group0 + j, pv2, h2, a2);
+  if (lane < gsz)
+    load_partial<RED == RMP_REDUCE_KAHAN32>(cparts + part0 + gi * kBatchGroup + lane, v, th, ta);
+  const uint32_t n_groups = (n_parts + kBatchGroup - 1) / kBatchGroup;
+  warp_sum_partial(v, th, ta, n_groups > 1 ? gparts + group0 + gi : nullptr);
+  if (n_groups > 1) {                               // (a single group's sums are the state's)
+    __threadfence();
+    __syncwarp();
+    uint32_t last = 0;
+    if (lane == 0) last = atomicAdd(&sticket[b], 1u) == n_groups - 1 ? 1u : 0u;
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    // last group of the state: lane i sums groups i, i + 32, ... in order, then the tree
+    __threadfence();
 #pragma unroll
-    for (int i = 0; i < 9; ++i) tv[i] += pv2[i];
-    th += h2;
-    ta += a2;
-  }
-  const WarpTerms t = warp_sum_partial(tv, th, ta, nullptr);
-  // every lane gets all terms back from the lanes that hold them
-  const double mine = tv[0];
+    for (int i = 0; i < 9; ++i) v[i] = 0.0;
+    th = ta = 0;
+    for (uint32_t j = lane; j < n_groups; j += 32) {
+      double pv2[9];
+      unsigned h2, a2;
+      load_partial<false>(gparts + group0 + j, pv2, h2, a2);
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const uint32_t at = __ballot_sync(0xffffffffu, t.n > 0 && t.first == i);
-    tv[i] = __shfl_sync(0xffffffffu, mine, __ffs(at) - 1);
+      for (int i = 0; i < 9; ++i) v[i] += pv2[i];
+      th += h2;
+      ta += a2;
+    }
+    warp_sum_partial(v, th, ta, nullptr);
   }
+  // combined with the attractor (Eq. 1, metric I): the ray sums (or their mean, divided in the
+  // lanes that hold them) plus its terms
+  double mine = v[0];
+  double att = 0.0;
   if (goals) {
-    if (lane == 0) add_attractor(k, states + 6 * (size_t)b, goals + 3 * (size_t)b, n_b, tv);
+    if (k.att_mean) mine = mine / (double)n_b;
+    att = attractor(k, states + 6 * (size_t)b, goals + 3 * (size_t)b);
+  }
+  // every lane gets all terms back from the lanes that hold them (warp_terms(0))
+  constexpr int kHolder[9] = {0, 2, 4, 8, 10, 16, 18, 20, 24};
+  double tv[9];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) tv[i] = __shfl_sync(0xffffffffu, tv[i], 0);
+  for (int i = 0; i < 9; ++i) tv[i] = __shfl_sync(0xffffffffu, mine, kHolder[i]);
+  if (goals) {
+    tv[0] += 1.0;
+    tv[3] += 1.0;
+    tv[5] += 1.0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) tv[6 + i] += __shfl_sync(0xffffffffu, att, i);
   }
   rmp_result_t r;
   resolve_pinv(tv, tv + 6, r);
