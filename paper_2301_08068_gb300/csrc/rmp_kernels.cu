@@ -1426,6 +1426,28 @@ __device__ __forceinline__ bool quiet_state(const EvalConsts& k, const float v[3
   return v[0] * v[0] + v[1] * v[1] + v[2] * v[2] < k.quiet_v2;
 }
 
+// The rows of (f_i, A_i), 9 floats each, of 32 consecutive points (`count` of them exist) written
+// together: through `sh` (288 floats of the warp) element l + 32 i goes to lane l, so that a
+// store covers whole lines, not four bytes of 32 rows (262144 points: 15.0 -> 10.2 us; the ray
+// kernels, whose rows lie apart, would hold more registers for it and be slower without rows).
+// Called by all lanes of the warp.
+__device__ __forceinline__ void store_rows(float* rows, uint32_t count, const float f[3],
+                                           const float A[6], float* sh) {
+  const uint32_t lane = threadIdx.x & 31;
+  float* mine = sh + 9 * lane;
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < 3; ++i) mine[i] = f[i];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) mine[3 + i] = A[i];
+  __syncwarp();
+#pragma unroll
+  for (uint32_t i = 0; i < 9; ++i) {
+    const uint32_t e = lane + 32 * i;
+    if (e < 9 * count) rows[e] = sh[e];
+  }
+}
+
 // The ray's obstacle policy (Sec. III-C) from its end: vals = A_i (6) and A_i f_i (3), all zero
 // unless it hit; counts hits and active rays; writes the optional per-ray (f_i, A_i).  Returns
 // whether vals is to be added.
@@ -2473,6 +2495,7 @@ __global__ void __launch_bounds__(256) scan_rmp_kernel(const float* __restrict__
                                                        WsHeader* ws, CtaPartial* parts,
                                                        rmp_result_t* out, float* per_ray) {
   __shared__ CtaState cs;
+  __shared__ float rows[8][288];
   const int comp = state_component(threadIdx.x);
   wait_previous();
   launch_next();                                    // two CTAs an SM, with room for two more
@@ -2486,17 +2509,20 @@ __global__ void __launch_bounds__(256) scan_rmp_kernel(const float* __restrict__
   const float vl[3] = {cs.vl[0], cs.vl[1], cs.vl[2]};
   const bool quiet = quiet_state(k, v);
   bool added = false;
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < k.n_rays;
-       j += gridDim.x * blockDim.x) {
+  // warp-uniform trip count: the lanes write their rows together
+  for (uint32_t base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < k.n_rays;
+       base += gridDim.x * blockDim.x) {
+    const uint32_t j = base + (threadIdx.x & 31);
+    const bool in = j < k.n_rays;
     float q[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) q[a] = __fsub_rn(__ldg(pts + 3 * (size_t)j + a), cs.xf[a]);
-    float f[3] = {0.f, 0.f, 0.f}, A[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, af[3];
+    for (int a = 0; a < 3; ++a) q[a] = in ? __fsub_rn(__ldg(pts + 3 * (size_t)j + a), cs.xf[a]) : 0.0f;
+    float f[3] = {0.f, 0.f, 0.f}, vals[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     bool valid = isfinite(q[0]) && isfinite(q[1]) && isfinite(q[2]);
     float d = 0.0f;
     if (valid) {
       d = __fsqrt_rn(__fmaf_rn(q[2], q[2], __fmaf_rn(q[1], q[1], __fmul_rn(q[0], q[0]))));
-      valid = d > 0.0f && d >= k.min_up && d <= k.max_dn;
+      valid = in && d > 0.0f && d >= k.min_up && d <= k.max_dn;
     }
     if (valid) {
       const float u[3] = {__fdiv_rn(q[0], d), __fdiv_rn(q[1], d), __fdiv_rn(q[2], d)};
@@ -2505,18 +2531,15 @@ __global__ void __launch_bounds__(256) scan_rmp_kernel(const float* __restrict__
       n_hit += 1;
       n_act += (act && inr) ? 1u : 0u;
       const bool adds = (act && inr) || !quiet;
-      if (adds || per_ray) obstacle_policy(k, u, d, v, vl, act, inr, f, A, af);
+      if (adds || per_ray) obstacle_policy(k, u, d, v, vl, act, inr, f, vals, vals + 6);
       if (adds) {
-        const float vals[9] = {A[0], A[1], A[2], A[3], A[4], A[5], af[0], af[1], af[2]};
         BlockReduce<RED>::add(acc, vals);
         added = true;
       }
     }
-    if (per_ray) {
-      float* o = per_ray + 9 * (size_t)j;
-      o[0] = f[0]; o[1] = f[1]; o[2] = f[2];
-      o[3] = A[0]; o[4] = A[1]; o[5] = A[2]; o[6] = A[3]; o[7] = A[4]; o[8] = A[5];
-    }
+    if (per_ray)
+      store_rows(per_ray + 9 * (size_t)base, min(32u, k.n_rays - base), f, vals,
+                 rows[threadIdx.x >> 5]);
   }
   __shared__ CtaSums sums;
   BlockReduce<RED>::reduce(acc, added, n_hit, n_act, sums);
