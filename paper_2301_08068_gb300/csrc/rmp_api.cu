@@ -765,7 +765,8 @@ int batch_async_impl(rmp_ctx* c, uint32_t map_id, const double* states_dev,
                      const uint32_t* n_rays_dev, uint32_t n_states, uint32_t max_rays,
                      const rmp_params_t* params, void* ws, size_t ws_bytes, rmp_stream_t stream,
                      rmp_result_t* out_dev, rmp_ray_hit_t* hits_dev, float* per_ray_dev,
-                     const double* goals_dev, double alpha, double beta, int metric_mean = 0) {
+                     const double* goals_dev, double alpha, double beta, int metric_mean = 0,
+                     const RolloutArgs& step = RolloutArgs()) {
   if (!c || !states_dev || !n_rays_dev || !ws || !out_dev) return RMP_ERR_INVALID_ARG;
   if (n_states == 0 || n_states > kMaxBatchStates || max_rays == 0 ||
       ws_bytes < batch_layout(n_states, max_rays).total)
@@ -783,7 +784,7 @@ int batch_async_impl(rmp_ctx* c, uint32_t map_id, const double* states_dev,
   k.att_beta = beta;
   k.att_mean = metric_mean ? 1 : 0;
   RMP_CUDA(launch_batch(dm, k, states_dev, n_rays_dev, n_states, max_rays, ws, out_dev, hits_dev,
-                        per_ray_dev, block, grid, (cudaStream_t)stream, goals_dev));
+                        per_ray_dev, block, grid, (cudaStream_t)stream, goals_dev, step));
   return RMP_OK;
 }
 
@@ -873,13 +874,17 @@ int rollout_impl(rmp_ctx* c, uint32_t map_id, const EsdfRec* esdf, const double*
   rmp_result_t* d_res = (rmp_result_t*)(buf + o_res);
   RolloutDev* d_rs = (RolloutDev*)(buf + o_rs);
   uint32_t* d_cnt = (uint32_t*)(buf + o_cnt);
-  RolloutConsts rc;
-  rc.dt = rp->dt;
-  rc.goal_tol = rp->goal_tol;
-  rc.max_steps = rp->max_steps;
-  rc.seg_steps = rp->seg_steps;
-  rc.n_rays = rp->n_rays;
-  rc.pad = 0;
+  RolloutArgs args;
+  args.rc.dt = rp->dt;
+  args.rc.goal_tol = rp->goal_tol;
+  args.rc.max_steps = rp->max_steps;
+  args.rc.seg_steps = rp->seg_steps;
+  args.rc.n_rays = rp->n_rays;
+  args.rc.pad = 0;
+  args.rs = d_rs;
+  args.states = d_st;
+  args.goals = d_goal;
+  args.n_rays = d_nr;
   int status = RMP_OK;
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_st, st.data(), 48 * (size_t)n, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_goal, goal.data(), 24 * (size_t)n, cudaMemcpyHostToDevice, s);
@@ -893,17 +898,17 @@ int rollout_impl(rmp_ctx* c, uint32_t map_id, const EsdfRec* esdf, const double*
                           step < rp->max_steps;) {
     e = cudaMemsetAsync(d_cnt, 0, 4, s);
     for (uint32_t i = 0; i < kRound && step < rp->max_steps && e == cudaSuccess; ++i, ++step) {
+      args.running = i + 1 == kRound || step + 1 == rp->max_steps ? d_cnt : nullptr;
       if (esdf) {
-        e = launch_esdf_eval(esdf->prims, esdf->prims32, esdf->n, ek, d_st, d_goal, n, d_res, nullptr, s);
-        if (e != cudaSuccess) break;
-      } else {
+        e = launch_esdf_eval(esdf->prims, esdf->prims32, esdf->n, ek, d_st, d_goal, n, d_res, nullptr,
+                             s);
+        if (e == cudaSuccess) e = launch_rollout_step(dm, args, d_res, n, s);
+      } else {                                      // the evaluation takes the step as well
         status = batch_async_impl(c, map_id, d_st, d_nr, n, rp->n_rays, params, buf + o_ws, wsb,
                                   stream, d_res, nullptr, nullptr, d_goal, rp->alpha, rp->beta,
-                                  (int)rp->metric_mean);
+                                  (int)rp->metric_mean, args);
         if (status != RMP_OK) break;
       }
-      e = launch_rollout_step(dm, rc, d_res, d_st, d_goal, d_nr, d_rs, n,
-                              i + 1 == kRound || step + 1 == rp->max_steps ? d_cnt : nullptr, s);
     }
     if (e == cudaSuccess && status == RMP_OK) {
       e = cudaMemcpyAsync(&running, d_cnt, 4, cudaMemcpyDeviceToHost, s);

@@ -98,6 +98,17 @@ struct RolloutConsts {
   uint32_t max_steps, seg_steps, n_rays, pad;
 };
 
+// What the control step after an evaluation works on (rollouts): the robots' records, states and
+// ray counts; `running` (nullable) counts the robots that go on.
+struct RolloutArgs {
+  RolloutConsts rc;
+  RolloutDev* rs;           // null: no control step
+  double* states;
+  const double* goals;
+  uint32_t* n_rays;
+  uint32_t* running;
+};
+
 // Workspace of one single-state evaluation: a header, then one partial slot per CTA.  A
 // slot is empty when every byte is 0xFF; CTA i > 0 fills slot i, CTA 0 waits for the
 // slots, reads them and empties them again (see grid_finish).
@@ -197,14 +208,14 @@ cudaError_t launch_raycast(const DevMap& m, const EvalConsts& k, const double* s
 int ctx_device(const rmp_ctx* ctx);                                  // CUDA device of a context
 int batch_occupancy(const DevMap& m, int reduce_mode, int block);     // CTAs per SM
 // Prep kernel + persistent batch kernel; n_rays_dev / states_dev on the device.  With
-// goals_dev (3 doubles per state) each state's rays are combined with its attractor.
+// goals_dev (3 doubles per state) each state's rays are combined with its attractor, and with
+// step.rs each robot then takes its control step (see rollout_step).
 cudaError_t launch_batch(const DevMap& m, const EvalConsts& k, const double* states_dev,
                          const uint32_t* n_rays_dev, uint32_t n_states, uint32_t max_rays,
                          void* ws, rmp_result_t* out_dev, rmp_ray_hit_t* hits, float* per_ray,
                          int block, int grid, cudaStream_t stream,
-                         const double* goals_dev = nullptr);
-// One control step of every robot (see rollout_step_kernel); counts running robots into
-// *running (which the caller zeroes) when running is not null.
+                         const double* goals_dev = nullptr,
+                         const RolloutArgs& step = RolloutArgs());
 // L2 read-bandwidth probe (see rmp_probe_l2_read): grid CTAs of 512 threads.
 cudaError_t launch_probe_l2(const uint4* buf, size_t n16, uint32_t passes, int grid,
                             uint64_t* checksum, cudaStream_t stream);
@@ -214,10 +225,9 @@ cudaError_t launch_esdf_eval(const rmp_primitive_t* prims, const float4* prims32
                              uint32_t n_prims, const EsdfConsts& k, const double* states,
                              const double* goals, uint32_t n_states, rmp_result_t* out,
                              double* query, cudaStream_t stream);
-cudaError_t launch_rollout_step(const DevMap& m, const RolloutConsts& rc, const rmp_result_t* res,
-                                double* states, const double* goals, uint32_t* n_rays,
-                                RolloutDev* rs, uint32_t n, uint32_t* running,
-                                cudaStream_t stream);
+// One control step of every robot from its evaluation in res.
+cudaError_t launch_rollout_step(const DevMap& m, const RolloutArgs& step, const rmp_result_t* res,
+                                uint32_t n, cudaStream_t stream);
 cudaError_t launch_scan(const float* pts, const EvalConsts& k, const double* state_dev,
                         void* ws, rmp_result_t* out_dev, float* per_ray, int block, int grid,
                         cudaStream_t stream);

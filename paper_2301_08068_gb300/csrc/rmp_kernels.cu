@@ -1855,83 +1855,101 @@ __device__ __forceinline__ bool voxel_occupied(const DevMap& m, int kx, int ky, 
 }
 
 // One control step of point robot b (Sec. IV-A closed loop): the combined policy's
-// acceleration f (res[b]) is integrated by semi-implicit Euler in FP64,
-// xdot' = xdot + f dt, x' = x + xdot' dt; then, in this order: outside a dense grid ->
-// LEFT_MAP; the voxel of x' occupied -> COLLIDED; |x' - goal| < goal_tol -> REACHED;
-// steps == max_steps -> TIMEOUT.  Every seg_steps steps the displacement since the last
-// segment end is a segment, and consecutive segments A, B add 1 - acos(cos(A, B)) / pi to
-// the smoothness sum.  A robot that stops running gets 0 rays from then on.
+// acceleration f is integrated by semi-implicit Euler in FP64, xdot' = xdot + f dt,
+// x' = x + xdot' dt; then, in this order: outside a dense grid -> LEFT_MAP; the voxel of x'
+// occupied -> COLLIDED; |x' - goal| < goal_tol -> REACHED; steps == max_steps -> TIMEOUT.  Every
+// seg_steps steps the displacement since the last segment end is a segment, and consecutive
+// segments A, B add 1 - acos(cos(A, B)) / pi to the smoothness sum.  A robot that stops running
+// gets 0 rays from then on.  Called by a warp for a running robot, axis a in lane a (0-2; an FP64
+// instruction costs the same for one lane or three), f_a in those lanes.
 template <int KIND, int LAYOUT>
-__global__ void rollout_step_kernel(DevMap m, RolloutConsts rc, const rmp_result_t* __restrict__ res,
-                                    double* states, const double* __restrict__ goals,
-                                    uint32_t* n_rays, RolloutDev* rs, uint32_t n,
-                                    uint32_t* running) {
-  const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-  wait_previous();
-  launch_next();
-  if (b >= n) return;
-  RolloutDev& r = rs[b];
-  if (r.status != RMP_ROLLOUT_RUNNING) {
-    n_rays[b] = 0;
-    return;
-  }
-  double* st = states + 6 * (size_t)b;
-  const rmp_result_t& e = res[b];
-  if (e.status != RMP_OK) {
-    r.status = RMP_ROLLOUT_FAILED;
-    n_rays[b] = 0;
-    return;
-  }
-  double dl = 0.0;
-  for (int a = 0; a < 3; ++a) {
-    const double vd = st[3 + a] + e.f[a] * rc.dt;
-    const double xn = st[a] + vd * rc.dt;
-    dl += (xn - st[a]) * (xn - st[a]);
+__device__ __noinline__ void rollout_step(const DevMap& m, const RolloutArgs& g, uint32_t b,
+                                          double f) {
+  const uint32_t lane = threadIdx.x & 31, a = lane < 3 ? lane : 0;
+  auto of = [](double v, int i) { return __shfl_sync(0xffffffffu, v, i); };
+  // (v0 w0 + v1 w1) + v2 w2 of two vectors that lie across the lanes, in every lane
+  auto dot3 = [&](double v, double w) {
+    const double p = __dmul_rn(of(v, 0), of(w, 0));
+    return __fma_rn(of(v, 2), of(w, 2), __fma_rn(of(v, 1), of(w, 1), p));
+  };
+  RolloutDev& r = g.rs[b];
+  double* st = g.states + 6 * (size_t)b;
+  const double x = st[a], goal = g.goals[3 * (size_t)b + a];
+  const double path = r.path_length;
+  const uint32_t steps = r.steps + 1;
+  const double vd = __fma_rn(f, g.rc.dt, st[3 + a]);
+  const double xn = __fma_rn(vd, g.rc.dt, x);
+  const double dl = dot3(xn - x, xn - x);
+  if (lane < 3) {
     st[3 + a] = vd;
     st[a] = xn;
   }
-  r.path_length += sqrt(dl);
-  r.steps += 1;
-  if (rc.seg_steps && r.steps % rc.seg_steps == 0) {
-    double seg[3];
-    for (int a = 0; a < 3; ++a) {
-      seg[a] = st[a] - r.seg_start[a];
-      r.seg_start[a] = st[a];
-    }
-    if (r.have_prev) {
-      double dot = 0.0, na = 0.0, nb = 0.0;
-      for (int a = 0; a < 3; ++a) {
-        dot += r.prev_seg[a] * seg[a];
-        na += r.prev_seg[a] * r.prev_seg[a];
-        nb += seg[a] * seg[a];
-      }
+  if (g.rc.seg_steps && steps % g.rc.seg_steps == 0) {
+    const double seg = xn - r.seg_start[a], prev = r.prev_seg[a];
+    const bool have = r.have_prev != 0;
+    if (have) {
+      const double dot = dot3(prev, seg), na = dot3(prev, prev), nb = dot3(seg, seg);
       if (na > 0.0 && nb > 0.0) {
         double cs = dot / (sqrt(na) * sqrt(nb));
         cs = cs > 1.0 ? 1.0 : (cs < -1.0 ? -1.0 : cs);
-        r.smooth_sum += 1.0 - acos(cs) / 3.14159265358979323846;
-        r.smooth_n += 1;
+        const double add = 1.0 - acos(cs) / 3.14159265358979323846;
+        if (lane == 0) {
+          r.smooth_sum += add;
+          r.smooth_n += 1;
+        }
       }
     }
-    for (int a = 0; a < 3; ++a) r.prev_seg[a] = seg[a];
-    r.have_prev = 1;
+    if (lane < 3) {
+      r.seg_start[a] = xn;
+      r.prev_seg[a] = seg;
+    }
+    if (lane == 0) r.have_prev = 1;
   }
-  int k[3];
-  bool far = false;
-  for (int a = 0; a < 3; ++a) {
-    const double o = KIND == RMP_MAP_DENSE_U8 ? (a == 0 ? m.origin[0] : (a == 1 ? m.origin[1] : m.origin[2]))
-                                              : 0.0;
-    const double q = __dmul_rn(__ddiv_rn(__dsub_rn(st[a], o), m.vs), 65536.0);
-    far = far || !(fabs(q) < 274877906944.0);
-    k[a] = far ? 0 : (int)(__double2ll_rn(q) >> 16);
+  const double o = KIND == RMP_MAP_DENSE_U8 ? (a == 0 ? m.origin[0] : (a == 1 ? m.origin[1] : m.origin[2]))
+                                            : 0.0;
+  const double q = __dmul_rn(__ddiv_rn(__dsub_rn(xn, o), m.vs), 65536.0);
+  const bool far = __any_sync(0xffffffffu, !(fabs(q) < 274877906944.0));
+  const int ka = far ? 0 : (int)(__double2ll_rn(q) >> 16);
+  const int k[3] = {__shfl_sync(0xffffffffu, ka, 0), __shfl_sync(0xffffffffu, ka, 1),
+                    __shfl_sync(0xffffffffu, ka, 2)};
+  const double dg = dot3(xn - goal, xn - goal);
+  const double len = sqrt(lane == 1 ? dg : dl);    // lane 0: the step's, lane 1: to the goal
+  const double to_goal = of(len, 1);
+  if (lane != 0) return;
+  uint32_t status = RMP_ROLLOUT_RUNNING;
+  if (far || (KIND == RMP_MAP_DENSE_U8 && outside<KIND>(m, k))) status = RMP_ROLLOUT_LEFT_MAP;
+  else if (voxel_occupied<LAYOUT>(m, k[0], k[1], k[2])) status = RMP_ROLLOUT_COLLIDED;
+  else if (to_goal < g.rc.goal_tol) status = RMP_ROLLOUT_REACHED;
+  else if (steps >= g.rc.max_steps) status = RMP_ROLLOUT_TIMEOUT;
+  r.path_length = path + len;
+  r.steps = steps;
+  r.status = status;
+  if (status != RMP_ROLLOUT_RUNNING) g.n_rays[b] = 0;
+  else if (g.running) atomicAdd(g.running, 1u);
+}
+
+// A robot whose evaluation failed stops.
+__device__ __forceinline__ void rollout_fail(const RolloutArgs& g, uint32_t b) {
+  g.rs[b].status = RMP_ROLLOUT_FAILED;
+  g.n_rays[b] = 0;
+}
+
+// The control steps as a launch of their own (the ESDF policy's closed loop), a warp per robot.
+template <int KIND, int LAYOUT>
+__global__ void __launch_bounds__(256) rollout_step_kernel(
+    const __grid_constant__ DevMap m, const __grid_constant__ RolloutArgs g,
+    const rmp_result_t* __restrict__ res, uint32_t n) {
+  const uint32_t b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  wait_previous();
+  launch_next();
+  if (b >= n) return;
+  if (g.rs[b].status != RMP_ROLLOUT_RUNNING) {
+    if (lane == 0) g.n_rays[b] = 0;
+  } else if (res[b].status != RMP_OK) {
+    if (lane == 0) rollout_fail(g, b);
+  } else {
+    rollout_step<KIND, LAYOUT>(m, g, b, res[b].f[lane < 3 ? lane : 0]);
   }
-  double dg = 0.0;
-  for (int a = 0; a < 3; ++a) dg += (st[a] - goals[3 * (size_t)b + a]) * (st[a] - goals[3 * (size_t)b + a]);
-  if (far || (KIND == RMP_MAP_DENSE_U8 && outside<KIND>(m, k))) r.status = RMP_ROLLOUT_LEFT_MAP;
-  else if (voxel_occupied<LAYOUT>(m, k[0], k[1], k[2])) r.status = RMP_ROLLOUT_COLLIDED;
-  else if (sqrt(dg) < rc.goal_tol) r.status = RMP_ROLLOUT_REACHED;
-  else if (r.steps >= rc.max_steps) r.status = RMP_ROLLOUT_TIMEOUT;
-  if (r.status != RMP_ROLLOUT_RUNNING) n_rays[b] = 0;
-  else if (running) atomicAdd(running, 1u);
 }
 
 // The last chunk of a group sums the group's partials into a group partial; the last group
@@ -1942,8 +1960,9 @@ __global__ void rollout_step_kernel(DevMap m, RolloutConsts rc, const rmp_result
 // per lane, not where they are stored: an FP64 instruction holds a scheduler's pipe about 64
 // cycles whatever the active lanes (256 states: 17.2 M -> 1.3 M FP64 warp instructions; with the
 // shared-out trees 1289 -> 1000 us).
-template <int RED>
-__device__ __noinline__ void batch_group_finish(const EvalConsts& k, CtaPartial* cparts,
+template <int KIND, int LAYOUT, int RED>
+__device__ __noinline__ void batch_group_finish(const DevMap& m, const EvalConsts& k,
+                                                const RolloutArgs& step, CtaPartial* cparts,
                                                 CtaPartial* gparts, uint32_t* sticket,
                                                 uint32_t part0, uint32_t gi, uint32_t gsz,
                                                 uint32_t n_parts, uint32_t group0, uint32_t b,
@@ -2014,6 +2033,11 @@ __device__ __noinline__ void batch_group_finish(const EvalConsts& k, CtaPartial*
     r.reserved = 0;
     out[b] = r;
   }
+  if (step.rs) {                                    // a rollout: the robot's control step follows
+    const double f0 = __shfl_sync(0xffffffffu, r.f[0], 0), f1 = __shfl_sync(0xffffffffu, r.f[1], 0),
+                 f2 = __shfl_sync(0xffffffffu, r.f[2], 0);
+    rollout_step<KIND, LAYOUT>(m, step, b, lane == 1 ? f1 : (lane == 2 ? f2 : f0));
+  }
 }
 
 // Persistent batched evaluation: every warp takes work chunks (its own index first, then from
@@ -2027,10 +2051,10 @@ __device__ __noinline__ void batch_group_finish(const EvalConsts& k, CtaPartial*
 // per-state values used only after the march are read after it.
 template <int KIND, int LAYOUT, int RED, bool BOXES>
 __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
-    DevMap m, EvalConsts k, BatchHeader* hdr, const BatchState* __restrict__ bs,
+    const __grid_constant__ DevMap m, const __grid_constant__ EvalConsts k, BatchHeader* hdr, const BatchState* __restrict__ bs,
     uint32_t* sticket, uint32_t* gticket, CtaPartial* cparts, CtaPartial* gparts,
     rmp_result_t* out, rmp_ray_hit_t* hits, float* per_ray, uint32_t max_rays,
-    const double* __restrict__ states, const double* __restrict__ goals) {
+    const double* states, const double* goals, const __grid_constant__ RolloutArgs step) {
   const uint32_t lane = threadIdx.x & 31;
   wait_previous();
   launch_next();
@@ -2057,6 +2081,7 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
     const uint32_t b = lo;
     const BatchState* sp = bs + b;
     if (__ldg(&sp->status) != RMP_OK) {              // its result is the prep kernel's
+      if (step.rs && lane == 0 && c == __ldg(&sp->work0)) rollout_fail(step, b);
       c = __shfl_sync(0xffffffffu, cn, 0);
       continue;
     }
@@ -2138,7 +2163,7 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
     if (lane == 0) stage = atomicAdd(&gticket[group0 + gi], stored) + stored == gsz ? 1u : 0u;
     stage = __shfl_sync(0xffffffffu, stage, 0);
     if (stage)
-      batch_group_finish<RED>(k, cparts, gparts, sticket, part0, gi, gsz, n_parts, group0, b, n_b,
+      batch_group_finish<KIND, LAYOUT, RED>(m, k, step, cparts, gparts, sticket, part0, gi, gsz, n_parts, group0, b, n_b,
                               states, goals, out);
     c = __shfl_sync(0xffffffffu, cn, 0);
   }
@@ -3096,7 +3121,8 @@ int batch_occupancy(const DevMap& m, int reduce_mode, int block) {
 cudaError_t launch_batch(const DevMap& m, const EvalConsts& k, const double* states_dev,
                          const uint32_t* n_rays_dev, uint32_t n_states, uint32_t max_rays,
                          void* ws, rmp_result_t* out_dev, rmp_ray_hit_t* hits, float* per_ray,
-                         int block, int grid, cudaStream_t stream, const double* goals_dev) {
+                         int block, int grid, cudaStream_t stream, const double* goals_dev,
+                         const RolloutArgs& step) {
   const BatchLayout L = batch_layout(n_states, max_rays);
   char* w = (char*)ws;
   BatchHeader* hdr = (BatchHeader*)w;
@@ -3112,23 +3138,22 @@ cudaError_t launch_batch(const DevMap& m, const EvalConsts& k, const double* sta
   for_map(m, k.reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
     launch_after(raycast_batch_kernel<kind.value, layout.value, red.value, boxes.value != 0>, grid,
                  block, stream, m, k, hdr, bs, sticket, gticket, cparts, gparts, out_dev, hits,
-                 per_ray, max_rays, states_dev, goals_dev);
+                 per_ray, max_rays, states_dev, goals_dev, step);
   });
   return cudaGetLastError();
 }
 
-cudaError_t launch_rollout_step(const DevMap& m, const RolloutConsts& rc, const rmp_result_t* res,
-                                double* states, const double* goals, uint32_t* n_rays,
-                                RolloutDev* rs, uint32_t n, uint32_t* running,
-                                cudaStream_t stream) {
-  const int block = 128;
-  const int grid = (int)((n + block - 1) / block);
+cudaError_t launch_rollout_step(const DevMap& m, const RolloutArgs& step, const rmp_result_t* res,
+                                uint32_t n, cudaStream_t stream) {
+  const unsigned grid = (n + 7) / 8;
   if (m.kind == RMP_MAP_DENSE_U8)
-    launch_after(rollout_step_kernel<RMP_MAP_DENSE_U8, kLayoutGrid>, grid, block, stream, m, rc, res, states, goals, n_rays, rs, n, running);
+    launch_after(rollout_step_kernel<RMP_MAP_DENSE_U8, kLayoutGrid>, grid, 256, stream, m, step, res, n);
   else if (m.layout == kLayoutGrid)
-    launch_after(rollout_step_kernel<RMP_MAP_HASHED_TSDF, kLayoutGrid>, grid, block, stream, m, rc, res, states, goals, n_rays, rs, n, running);
+    launch_after(rollout_step_kernel<RMP_MAP_HASHED_TSDF, kLayoutGrid>, grid, 256, stream, m, step,
+                 res, n);
   else
-    launch_after(rollout_step_kernel<RMP_MAP_HASHED_TSDF, kLayoutHash>, grid, block, stream, m, rc, res, states, goals, n_rays, rs, n, running);
+    launch_after(rollout_step_kernel<RMP_MAP_HASHED_TSDF, kLayoutHash>, grid, 256, stream, m, step,
+                 res, n);
   return cudaGetLastError();
 }
 
