@@ -178,8 +178,24 @@ int make_consts(const rmp_params_t* p, double vs, uint32_t n, bool scan, EvalCon
   return RMP_OK;
 }
 
+// A synchronous call's state as the kernels would form it from device memory (the same IEEE
+// operations; dm null: a scan, whose points are in the frame of x).
+void host_state(const double x[3], const double xdot[3], const DevMap* dm, CtaState* cs) {
+  for (int a = 0; a < 3; ++a) {
+    if (dm) {
+      const double o = dm->kind == RMP_MAP_DENSE_U8 ? dm->origin[a] : 0.0;
+      const double q = (x[a] - o) / dm->vs * 65536.0;
+      cs->bad[a] = !(std::fabs(q) < 274877906944.0);
+      cs->P[a] = cs->bad[a] ? 0 : std::llrint(q);
+    }
+    cs->xf[a] = (float)x[a];
+    cs->v[a] = (float)xdot[a];
+    cs->vl[a] = (float)(xdot[a] - (double)cs->v[a]);
+  }
+}
+
 // Enqueue one single-state evaluation with the launch shape of the ray count and the
-// context's knobs.  k comes from make_consts; state_dev null: the state is in k.x0.
+// context's knobs.  k comes from make_consts; state_dev null: the state is in k.cs0.
 cudaError_t launch_single(const MapRec& mr, const Tuning& t, EvalConsts k,
                           const double* state_dev, void* ws, rmp_result_t* out,
                           rmp_ray_hit_t* hits, float* per_ray, cudaStream_t s) {
@@ -656,10 +672,7 @@ int rmp_raycast_eval(rmp_ctx* c, uint32_t map_id, const double x[3], const doubl
   DeviceGuard g(c->device);
   if (!g.ok()) return RMP_ERR_CUDA;
   cudaStream_t s = (cudaStream_t)stream;
-  for (int a = 0; a < 3; ++a) {        // x, xdot go to the device inside the launch
-    k.x0[a] = x[a];
-    k.x0[3 + a] = xdot[a];
-  }
+  host_state(x, xdot, &it->second.dm, &k.cs0);      // goes to the device inside the launch
   RMP_CUDA(launch_single(it->second, t, k, nullptr, c->ws, c->result_map, hits_dev, per_ray_dev,
                          s));
   RMP_CUDA(cudaStreamSynchronize(s));
@@ -701,10 +714,7 @@ int rmp_scan_eval(rmp_ctx* c, const float* points_dev, uint32_t n, const double 
   if (!g.ok()) return RMP_ERR_CUDA;
   std::lock_guard<std::mutex> lk(c->mu);
   cudaStream_t s = (cudaStream_t)stream;
-  for (int a = 0; a < 3; ++a) {
-    k.x0[a] = x[a];
-    k.x0[3 + a] = xdot[a];
-  }
+  host_state(x, xdot, nullptr, &k.cs0);
   int block, grid;
   scan_shape(tuning_of(c), c->sm_count, n, &block, &grid);
   RMP_CUDA(launch_scan(points_dev, k, nullptr, c->ws, c->result_map, per_ray_dev, block, grid,

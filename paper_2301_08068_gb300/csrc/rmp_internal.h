@@ -67,6 +67,16 @@ struct DevMap {
   const HashEntry* table;   // hash layout only
 };
 
+// One state as the kernels use it: the position quantised (2^-16 voxels) and in FP32, the
+// velocity as an FP32 pair.
+struct CtaState {
+  long long P[3];
+  float v[3];     // RN32(xdot)
+  float vl[3];    // RN32(xdot - v)
+  float xf[3];    // RN32(x) (scans)
+  int bad[3];     // the axis's position is not finite or beyond 2^22 voxels
+};
+
 // Constants of one evaluation derived on the host from rmp_params_t.
 struct EvalConsts {
   float eta_rep, inv_nu_rep, eta_damp, inv_nu_damp, eps, c, r_up, inv_r;
@@ -82,7 +92,7 @@ struct EvalConsts {
   double att_alpha, att_beta;        // attractor gain and damping (combined evaluations)
   int att_mean;                      // combined: ray sums divided by the ray count first
   uint32_t seg_threads;              // batches: threads of the persistent launch (segments)
-  double x0[6];                      // x, xdot carried in the launch itself, read when the
+  CtaState cs0;                      // the state carried in the launch itself, read when the
                                      // kernel's state pointer is null (synchronous calls)
 };
 

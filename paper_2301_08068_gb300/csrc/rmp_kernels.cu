@@ -12,6 +12,7 @@
 // ray) use explicitly rounded intrinsics (__fmul_rn, __fmaf_rn, ...) so that no
 // contraction or fast-math rewrite can change them.
 #include <climits>
+#include <cstddef>
 #include <type_traits>
 
 #include "rmp_internal.h"
@@ -679,7 +680,7 @@ __device__ __forceinline__ void warp_reduce_terms(T (&s)[9], T (&c)[9], uint32_t
 // Block-level reduction of the per-thread accumulators and counts: the shared-out tree per warp,
 // (where one of its lanes `added` anything; all sums are zero otherwise), then lane q of warp 0
 // merges term q of the warps in warp order (all terms at once, not one thread walking them).
-// Called by every thread.
+// Called by every thread of a CTA of at most 8 warps; `wide`: the FP64 values are wanted.
 template <int RED>
 struct BlockReduce;
 
@@ -691,9 +692,10 @@ struct BlockReduce<RMP_REDUCE_KAHAN32> {
     for (int q = 0; q < 9; ++q) a.s[q] = a.c[q] = 0.0f;
   }
   __device__ static void add(Acc& a, const float v[9]) { acc_add(a, v); }
-  __device__ static void reduce(Acc& a, bool added, unsigned nh, unsigned na, CtaSums& out) {
-    __shared__ float sh[32][18];
-    __shared__ unsigned shu[32][2];
+  __device__ static void reduce(Acc& a, bool added, unsigned nh, unsigned na, CtaSums& out,
+                                bool wide) {
+    __shared__ float sh[8][18];
+    __shared__ unsigned shu[8][2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const WarpTerms t = warp_terms(0);
     if (__any_sync(0xffffffffu, added)) warp_reduce_terms<float, true>(a.s, a.c, 0);
@@ -710,11 +712,19 @@ struct BlockReduce<RMP_REDUCE_KAHAN32> {
     __syncthreads();
     if (warp == 0) {
       if (lane < 9) {
-        float s = sh[0][lane], c = sh[0][9 + lane];
-        for (int w = 1; w < nw; ++w) merge1(s, c, sh[w][lane], sh[w][9 + lane]);
+        float sw[8], cw[8];                          // all loads before the serial merges
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+          sw[w] = w < nw ? sh[w][lane] : 0.0f;
+          cw[w] = w < nw ? sh[w][9 + lane] : 0.0f;
+        }
+        float s = sw[0], c = cw[0];
+#pragma unroll
+        for (int w = 1; w < 8; ++w)
+          if (w < nw) merge1(s, c, sw[w], cw[w]);
         out.s[lane] = s;
         out.c[lane] = c;
-        out.v[lane] = (double)s + (double)c;
+        if (wide) out.v[lane] = (double)s + (double)c;
       } else if (lane < 11) {
         unsigned t = 0;
         for (int w = 0; w < nw; ++w) t += shu[w][lane - 9];
@@ -735,9 +745,9 @@ struct BlockReduce<RMP_REDUCE_FP64> {
 #pragma unroll
     for (int q = 0; q < 9; ++q) a.s[q] += (double)v[q];
   }
-  __device__ static void reduce(Acc& a, bool added, unsigned nh, unsigned na, CtaSums& out) {
-    __shared__ double sh[32][9];
-    __shared__ unsigned shu[32][2];
+  __device__ static void reduce(Acc& a, bool added, unsigned nh, unsigned na, CtaSums& out, bool) {
+    __shared__ double sh[8][9];
+    __shared__ unsigned shu[8][2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const WarpTerms t = warp_terms(0);
     if (__any_sync(0xffffffffu, added)) warp_reduce_terms<double, false>(a.s, a.s, 0);
@@ -1302,7 +1312,7 @@ __device__ void grid_finish(const CtaSums& cta, WsHeader* ws, CtaPartial* parts,
       nh += w[18];
       na += w[19];
     }
-    BlockReduce<RED>::reduce(acc, true, nh, na, gsum);
+    BlockReduce<RED>::reduce(acc, true, nh, na, gsum, true);
     const int any_expired = __syncthreads_or(expired);
     if (poisoned || any_expired) {
       if (threadIdx.x == 0) ws->poisoned = 1;
@@ -1310,41 +1320,31 @@ __device__ void grid_finish(const CtaSums& cta, WsHeader* ws, CtaPartial* parts,
     }
     tot = &gsum;
   }
+  // lanes 0-8 hold the terms they reduced, lanes 9 and 10 the counts; the result leaves as 18
+  // words of 18 lanes (one thread storing the record took 800 cycles)
   __shared__ rmp_result_t r;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int q = 0; q < 6; ++q) r.A[q] = tot->v[q];
-    for (int q = 0; q < 3; ++q) r.Af[q] = tot->v[6 + q];
+  if (threadIdx.x < 9) {
+    (&r.A[0])[threadIdx.x] = tot->v[threadIdx.x];      // A, then Af
+  } else if (threadIdx.x < 11) {
+    (&r.n_hits)[threadIdx.x - 9] = tot->u[threadIdx.x - 9];
+  } else if (threadIdx.x == 11) {
     r.n_rays = n_rays;
-    r.n_hits = tot->u[0];
-    r.n_active = tot->u[1];
     r.status = st;
     r.reserved = 0;
   }
   __syncthreads();
   if (threadIdx.x < 64) resolve_pinv_cta(r.A, r.Af, r);
-  if (threadIdx.x == 0) *out = r;
+  if (threadIdx.x < 32) {
+    __syncwarp();
+    if (threadIdx.x < 18)
+      reinterpret_cast<unsigned long long*>(out)[threadIdx.x] =
+          reinterpret_cast<const unsigned long long*>(&r)[threadIdx.x];
+  }
 }
 
-// Per-CTA state: quantised position (FP64, threads 0-2 one axis each) and the velocity
-// as an FP32 pair (threads 3-5).
-struct CtaState {
-  long long P[3];
-  float v[3];     // RN32(xdot)
-  float vl[3];    // RN32(xdot - v)
-  float xf[3];
-  int bad[3];
-};
-
-// Component i of (x, xdot): from device memory, or, with a null pointer, from the copy the
-// launch carries in its constants (selected with constant offsets, no local-memory array).
-__device__ __forceinline__ double state_at(const double* state, const EvalConsts& k, int i) {
-  if (state) return state[i];
-  double v = k.x0[0];
-#pragma unroll
-  for (int j = 1; j < 6; ++j) v = i == j ? k.x0[j] : v;
-  return v;
-}
+static_assert(offsetof(rmp_result_t, Af) == offsetof(rmp_result_t, A) + 48 &&
+                  offsetof(rmp_result_t, n_active) == offsetof(rmp_result_t, n_hits) + 4,
+              "the finish writes these as arrays");
 
 // Which state component (0-2 x, 3-5 xdot) thread t sets up, or -1: x on threads 0-2 and
 // xdot on threads 32-34, two warps, so that the FP64 work of each runs in parallel.
@@ -1491,9 +1491,9 @@ __global__ void __launch_bounds__(256) raycast_rmp_kernel(DevMap m, EvalConsts k
                                                           float* per_ray) {
   __shared__ CtaState cs;
   // state component of this thread: x on threads 0-2, xdot on threads 32-34 (another warp,
-  // so the two FP64 chains below run side by side instead of one after the other)
+  // so the two FP64 chains below run side by side instead of one after the other); a synchronous
+  // call's state comes quantised in the launch (its FP64 chain took 1200 cycles here)
   const int comp = state_component(threadIdx.x);
-  double sv = comp >= 0 && !state ? state_at(state, k, comp) : 0.0;
   typename BlockReduce<RED>::Acc acc;
   BlockReduce<RED>::init(acc);
   unsigned n_hit = 0, n_act = 0;
@@ -1507,8 +1507,10 @@ __global__ void __launch_bounds__(256) raycast_rmp_kernel(DevMap m, EvalConsts k
                                  k.perm_Q, k.perm_R);
   Ray ray = make_ray<false>(ray_idx + k.halton_offset);
   wait_previous();
-  if (comp >= 0 && state) sv = state_at(state, k, comp);
-  if (comp >= 0 && comp < 3) {
+  if (!state) {                                     // the launch carries the state, quantised
+    if (threadIdx.x == 0) cs = k.cs0;
+  } else if (comp >= 0 && comp < 3) {
+    const double sv = state[comp];
     const double o = KIND != RMP_MAP_DENSE_U8 ? 0.0
                      : (comp == 0 ? m.origin[0] : (comp == 1 ? m.origin[1] : m.origin[2]));
     const double q = __dmul_rn(__ddiv_rn(__dsub_rn(sv, o), m.vs), 65536.0);
@@ -1517,7 +1519,7 @@ __global__ void __launch_bounds__(256) raycast_rmp_kernel(DevMap m, EvalConsts k
     cs.bad[comp] = bad;
     cs.P[comp] = bad ? 0 : __double2ll_rn(q);
   } else if (comp >= 3) {
-    split_velocity(sv, cs, comp - 3);
+    split_velocity(state[comp], cs, comp - 3);
   }
   __syncthreads();                                  // state ready
   const bool bad = (cs.bad[0] | cs.bad[1] | cs.bad[2]) != 0;
@@ -1547,7 +1549,7 @@ __global__ void __launch_bounds__(256) raycast_rmp_kernel(DevMap m, EvalConsts k
   }
   launch_next();
   __shared__ CtaSums sums;
-  BlockReduce<RED>::reduce(acc, added, n_hit, n_act, sums);
+  BlockReduce<RED>::reduce(acc, added, n_hit, n_act, sums, gridDim.x == 1);
   grid_finish<RED>(sums, ws, parts, out, k.n_rays,
                    (cs.bad[0] | cs.bad[1] | cs.bad[2]) ? RMP_ERR_INVALID_ARG : RMP_OK);
 }
@@ -2524,8 +2526,13 @@ __global__ void __launch_bounds__(256) scan_rmp_kernel(const float* __restrict__
   const int comp = state_component(threadIdx.x);
   wait_previous();
   launch_next();                                    // two CTAs an SM, with room for two more
-  if (comp >= 0 && comp < 3) cs.xf[comp] = __double2float_rn(state_at(state, k, comp));
-  else if (comp >= 3) split_velocity(state_at(state, k, comp), cs, comp - 3);
+  if (!state) {
+    if (threadIdx.x == 0) cs = k.cs0;
+  } else if (comp >= 0 && comp < 3) {
+    cs.xf[comp] = __double2float_rn(state[comp]);
+  } else if (comp >= 3) {
+    split_velocity(state[comp], cs, comp - 3);
+  }
   __syncthreads();
   typename BlockReduce<RED>::Acc acc;
   BlockReduce<RED>::init(acc);
@@ -2567,7 +2574,7 @@ __global__ void __launch_bounds__(256) scan_rmp_kernel(const float* __restrict__
                  rows[threadIdx.x >> 5]);
   }
   __shared__ CtaSums sums;
-  BlockReduce<RED>::reduce(acc, added, n_hit, n_act, sums);
+  BlockReduce<RED>::reduce(acc, added, n_hit, n_act, sums, gridDim.x == 1);
   grid_finish<RED>(sums, ws, parts, out, k.n_rays, RMP_OK);
 }
 
