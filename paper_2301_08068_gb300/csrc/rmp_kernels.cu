@@ -1483,12 +1483,15 @@ __device__ __forceinline__ bool ray_outputs(const DevMap& m, const EvalConsts& k
 // ray sit in adjacent lanes, and the ray's result is the first segment (lowest index) that
 // hit or left the map, else the last one -- found with a warp ballot and moved to the
 // ray's first lane by shuffles.  That lane evaluates the policy and writes the outputs.
-template <int KIND, int LAYOUT, int RED, bool BOXES>
-__global__ void __launch_bounds__(256) raycast_rmp_kernel(DevMap m, EvalConsts k,
-                                                          const double* __restrict__ state,
-                                                          WsHeader* ws, CtaPartial* parts,
-                                                          rmp_result_t* out, rmp_ray_hit_t* hits,
-                                                          float* per_ray) {
+//
+// BLOCK, CTAS: the register budget.  256 x 2 where the launch is one wave of 256-thread CTAs: its
+// slowest warps decide, and more registers serve them better (65536 rays 15.2 us; held to 85
+// registers 17.4, to 64 18.8).  128 x 6 (85 registers, 24 warps an SM) for the 128-thread CTAs of
+// larger launches, which keep every SM busy: 262144 rays on the 100 m map 30.0 -> 27.7 us.
+template <int KIND, int LAYOUT, int RED, bool BOXES, int BLOCK, int CTAS>
+__global__ void __launch_bounds__(BLOCK, CTAS) raycast_rmp_kernel(
+    DevMap m, EvalConsts k, const double* __restrict__ state, WsHeader* ws, CtaPartial* parts,
+    rmp_result_t* out, rmp_ray_hit_t* hits, float* per_ray) {
   __shared__ CtaState cs;
   // state component of this thread: x on threads 0-2, xdot on threads 32-34 (another warp,
   // so the two FP64 chains below run side by side instead of one after the other); a synchronous
@@ -3096,7 +3099,7 @@ int raycast_occupancy(const DevMap& m, int reduce_mode, int block) {
   cudaError_t e = cudaSuccess;
   for_map(m, reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &n, raycast_rmp_kernel<kind.value, layout.value, red.value, boxes.value != 0>, block, 0);
+        &n, raycast_rmp_kernel<kind.value, layout.value, red.value, boxes.value != 0, 256, 2>, block, 0);
   });
   return e == cudaSuccess ? n : -1;
 }
@@ -3109,8 +3112,12 @@ cudaError_t launch_raycast(const DevMap& m, const EvalConsts& k, const double* s
   WsHeader* hdr = (WsHeader*)ws;
   CtaPartial* parts = (CtaPartial*)((char*)ws + kWsHeaderBytes);
   for_map(m, k.reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
-    launch_after(raycast_rmp_kernel<kind.value, layout.value, red.value, boxes.value != 0>, grid,
-                 block, stream, m, k, state_dev, hdr, parts, out_dev, hits, per_ray);
+    if (block == 256)
+      launch_after(raycast_rmp_kernel<kind.value, layout.value, red.value, boxes.value != 0, 256, 2>,
+                   grid, block, stream, m, k, state_dev, hdr, parts, out_dev, hits, per_ray);
+    else
+      launch_after(raycast_rmp_kernel<kind.value, layout.value, red.value, boxes.value != 0, 128, 6>,
+                   grid, block, stream, m, k, state_dev, hdr, parts, out_dev, hits, per_ray);
   });
   return cudaGetLastError();
 }
