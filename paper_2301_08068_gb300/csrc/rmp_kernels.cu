@@ -1821,8 +1821,8 @@ __device__ __forceinline__ void warp_sum_partial(double (&v)[9], unsigned& h, un
 // component a in lane a (0-2).  Called by all lanes of a warp, so that the root, the exponential
 // and the division are one warp instruction stream (an FP64 instruction holds the pipe about
 // 64 cycles whatever the lanes).
-__device__ __forceinline__ double attractor(const EvalConsts& k, const double* st,
-                                            const double* goal) {
+__device__ __noinline__ double attractor(const EvalConsts& k, const double* st,
+                                         const double* goal) {
   const uint32_t lane = threadIdx.x & 31, a = lane < 3 ? lane : 0;
   const double va = goal[a] - st[a];
   const double v0 = __shfl_sync(0xffffffffu, va, 0), v1 = __shfl_sync(0xffffffffu, va, 1),
@@ -1970,7 +1970,8 @@ __device__ __noinline__ void batch_group_finish(const DevMap& m, const EvalConst
                                                 const RolloutArgs& step, CtaPartial* cparts,
                                                 CtaPartial* gparts, uint32_t* sticket,
                                                 uint32_t part0, uint32_t gi, uint32_t gsz,
-                                                uint32_t n_parts, uint32_t group0, uint32_t b,
+                                                uint32_t n_parts, uint32_t chunks, uint32_t group0,
+                                                uint32_t b,
                                                 uint32_t n_b, const double* states,
                                                 const double* goals, rmp_result_t* out) {
   const uint32_t lane = threadIdx.x & 31;
@@ -2010,7 +2011,9 @@ __device__ __noinline__ void batch_group_finish(const DevMap& m, const EvalConst
   double att = 0.0;
   if (goals) {
     if (k.att_mean) mine = mine / (double)n_b;
-    att = attractor(k, states + 6 * (size_t)b, goals + 3 * (size_t)b);
+    // the first of several chunks has left it in the record
+    att = chunks > 1 ? __ldcg(&out[b].f[lane < 3 ? lane : 0])
+                     : attractor(k, states + 6 * (size_t)b, goals + 3 * (size_t)b);
   }
   // every lane gets all terms back from the lanes that hold them (warp_terms(0))
   constexpr int kHolder[9] = {0, 2, 4, 8, 10, 16, 18, 20, 24};
@@ -2159,6 +2162,14 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
       part->n_hits = cnt & 0xffffu;
       part->n_active = cnt >> 16;
     }
+    // the warp of a state's first chunk forms its attractor as well, beside the others' marches
+    // (6000 cycles of FP64 that would otherwise follow the last chunk), and leaves it in the
+    // result's record until the state is resolved; its ticket orders it before that
+    const uint32_t chunks = ((n_b << lgs) + 31) / 32;
+    if (goals && q == 0 && chunks > 1) {
+      const double att = attractor(k, states + 6 * (size_t)b, goals + 3 * (size_t)b);
+      if (lane < 3) out[b].f[lane] = att;
+    }
     const uint32_t gi = first / kBatchGroup;
     const uint32_t gsz = min(kBatchGroup, n_parts - gi * kBatchGroup);
     const uint32_t stored = min(1u << lgW, n_parts - first);
@@ -2168,8 +2179,8 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
     if (lane == 0) stage = atomicAdd(&gticket[group0 + gi], stored) + stored == gsz ? 1u : 0u;
     stage = __shfl_sync(0xffffffffu, stage, 0);
     if (stage)
-      batch_group_finish<KIND, LAYOUT, RED>(m, k, step, cparts, gparts, sticket, part0, gi, gsz, n_parts, group0, b, n_b,
-                              states, goals, out);
+      batch_group_finish<KIND, LAYOUT, RED>(m, k, step, cparts, gparts, sticket, part0, gi, gsz,
+                                            n_parts, chunks, group0, b, n_b, states, goals, out);
     c = __shfl_sync(0xffffffffu, cn, 0);
   }
 }
