@@ -2295,8 +2295,8 @@ __device__ __forceinline__ float key_float(uint32_t k) {
   return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xffffffffu));
 }
 
-// The ESDF policy, G states (8 or 32) a CTA.  An FP64 instruction holds a scheduler's pipe about
-// 64 cycles whatever its active lanes, so the exact arithmetic runs with a state per lane:
+// The ESDF policy, G states (8, 16 or 32) a CTA.  An FP64 instruction holds a scheduler's pipe
+// about 64 cycles whatever its active lanes, so the exact arithmetic runs with a state per lane:
 //   1. a warp per state finds the nearest primitive (lane i: i, i + 32, ...) from FP32 distances
 //      and their error bounds: it is decided when only one primitive's lower bound lies below
 //      the smallest upper bound; otherwise (ties, or closer than FP32 can tell) those primitives
@@ -2306,9 +2306,11 @@ __device__ __forceinline__ float key_float(uint32_t k) {
 //   3. one warp runs the Jacobi sweeps, another the adjugate solve; three warps take one
 //      Rayleigh quotient each; the first sorts, decides the rank and writes the results.
 // The warps of the serial parts rotate with the CTA and with its turn on an SM (152 of them), so
-// that an SM's CTAs use different schedulers' pipes.  Bound by the FP64 chain of steps 2 and 3.  16384 states, 200 primitives:
-// 51 us (one warp per state, every distance in FP64, policy in one lane: 638 us); 128 states 18.5 (51).
-__global__ void __launch_bounds__(256) esdf_eval_kernel(const rmp_primitive_t* __restrict__ prims,
+// that an SM's CTAs use different schedulers' pipes.  Bound by the FP64 chain of steps 2 and 3;
+// four CTAs an SM (64 registers), so that 16384 states are one wave (three: 48 us).  16384 states,
+// 200 primitives: 33.6 us (one warp per state, every distance in FP64, policy in one lane: 638);
+// 128 states 16 (51).
+__global__ void __launch_bounds__(256, 4) esdf_eval_kernel(const rmp_primitive_t* __restrict__ prims,
                                                         const float4* __restrict__ prims32,
                                                         uint32_t n_prims, EsdfConsts k,
                                                         const double* __restrict__ states,
@@ -2327,12 +2329,14 @@ __global__ void __launch_bounds__(256) esdf_eval_kernel(const rmp_primitive_t* _
   for (uint32_t base = blockIdx.x * G; base < n_states; base += gridDim.x * G) {
     for (uint32_t s = warp; s < G && base + s < n_states; s += 8) {
       const double* st = states + 6 * (size_t)(base + s);
-      const bool bad = __any_sync(0xffffffffu, lane < 6 && !isfinite(st[lane < 6 ? lane : 0]));
+      // one component a lane: a single FP64 conversion for all of them
+      const double comp = st[lane < 6 ? lane : 0];
+      const float cf = __double2float_rn(comp);
+      const bool bad = __any_sync(0xffffffffu, (__double2hiint(comp) & 0x7ff00000) == 0x7ff00000);
       uint32_t bi = kNone;
       if (!bad) {
-        const double x[3] = {st[0], st[1], st[2]};
-        const float xf[3] = {__double2float_rn(x[0]), __double2float_rn(x[1]),
-                             __double2float_rn(x[2])};
+        const float xf[3] = {__shfl_sync(0xffffffffu, cf, 0), __shfl_sync(0xffffffffu, cf, 1),
+                             __shfl_sync(0xffffffffu, cf, 2)};
         const float x_sum = fabsf(xf[0]) + fabsf(xf[1]) + fabsf(xf[2]);
         // smallest upper bound; the two smallest lower bounds and the first one's primitive
         float up = INFINITY, lo1 = INFINITY, lo2 = INFINITY;
@@ -2359,6 +2363,7 @@ __global__ void __launch_bounds__(256) esdf_eval_kernel(const rmp_primitive_t* _
         if (__popc(cand) == 1 && !more) {
           bi = __shfl_sync(0xffffffffu, i1, __ffs(cand) - 1);
         } else {
+          const double x[3] = {st[0], st[1], st[2]};
           double best = INFINITY;
           for (uint32_t i = lane; i < n_prims; i += 32) {
             float err;
@@ -3193,9 +3198,10 @@ cudaError_t launch_esdf_eval(const rmp_primitive_t* prims, const float4* prims32
                              const double* goals, uint32_t n_states, rmp_result_t* out,
                              double* query, cudaStream_t stream) {
   if (n_states == 0) return cudaSuccess;
-  // 8 states a CTA (a warp each for the search) while that leaves no more than two CTAs an SM:
-  // few states wait for latency; 32 beyond, where the FP64 steps should fill their lanes
-  const uint32_t G = n_states <= 8u * 304u ? 8u : 32u;
+  // as few states a CTA as give one CTA an SM: few states wait for latency; beyond, 32, where the
+  // FP64 steps fill their lanes (1217 states: 8 a CTA 20.1 us, 16 18.0, 32 20.5; 2432 states:
+  // 22.3, 18.2, 20.5)
+  const uint32_t G = n_states <= 8u * 152u ? 8u : (n_states <= 16u * 152u ? 16u : 32u);
   uint32_t grid = (n_states + G - 1) / G;
   if (grid > 65535) grid = 65535;                   // CTA-stride beyond
   launch_after(esdf_eval_kernel, grid, 256, stream, prims, prims32, n_prims, k, states, goals,

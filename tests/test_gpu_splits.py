@@ -1,0 +1,136 @@
+"""The cuts of the work over CTAs, warps and lanes where they change: ESDF states on both sides
+of 8, 16 and 32 states a CTA, ties and distances that FP32 cannot tell apart, coordinates past
+FP32; batches with more states than one run of the set-up kernel takes and with total loads on
+both sides of the march's segment cuts; scans whose last warp is ragged, with the per-point rows."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2301_08068_gb300 import rmp as R
+from paper_2301_08068_gb300 import workloads as W
+
+from gpu_helpers import (assert_hits_exact, assert_per_ray_close, assert_result_close,
+                         scan_abs_term, torch_cuda)
+from test_gpu_batch import run_batch
+from test_gpu_esdf import check_states, run_esdf, scene
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    torch_cuda()
+    c = R.Context(0)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("n", [1, 8, 9, 1216, 1217, 2432, 2433])
+def test_esdf_states_per_cta(ctx, n):
+    _, prims = scene(40)
+    rng = np.random.default_rng(n)
+    states = np.concatenate([rng.uniform(-1.0, 11.0, (n, 3)), rng.normal(0.0, 1.0, (n, 3))], 1)
+    goals = rng.uniform(0.0, 10.0, (n, 3))
+    eid = R.rmp_esdf_upload(ctx.handle, prims)
+    try:
+        check_states(ctx, eid, O.prims_array(prims), states, goals, W.PARAMS_STATIC_MAP)
+    finally:
+        R.rmp_esdf_release(ctx.handle, eid)
+
+
+@pytest.mark.parametrize("gap", [0.0, 1e-13, 1e-9, 1e-7])
+@pytest.mark.parametrize("n", [2, 33, 97])
+def test_esdf_ties(ctx, gap, n):
+    """n spheres and boxes at the same distance of a state but for the gap, which FP32 cannot
+    tell: the first minimum of a sequential scan wins, here in every lane and every turn."""
+    rng = np.random.default_rng(n)
+    sign = np.sign(rng.normal(size=(n, 3)))
+    # both 0.5 sqrt(3) away: the sphere 2 sqrt(3) less its radius, the box from its corner
+    prims = [W.Primitive("sphere", 5.0 + 2.0 * sign[i], np.array([1.5 * np.sqrt(3.0)])) if i % 3
+             else W.Primitive("box", 5.0 + 2.0 * sign[i], np.full(3, 1.5)) for i in range(n)]
+    for i, p in enumerate(prims):
+        p.center[0] += gap * ((7 * i) % n) * sign[i, 0]
+    pr = O.prims_array(prims)
+    states = np.zeros((20, 6))
+    states[:, :3] = 5.0
+    states[1:, :3] += rng.normal(0.0, 1e-13, (19, 3))
+    states[:, 3:] = rng.normal(0.0, 1.0, (20, 3))
+    eid = R.rmp_esdf_upload(ctx.handle, prims)
+    try:
+        check_states(ctx, eid, pr, states, None, W.PARAMS_STATIC_MAP)
+    finally:
+        R.rmp_esdf_release(ctx.handle, eid)
+
+
+def test_esdf_beyond_fp32(ctx):
+    """Primitives and states so far away that FP32 holds neither the squares nor the coordinates:
+    the query equals the oracle's bit for bit."""
+    far = [W.Primitive("sphere", np.array([1e20, -3e19, 2.0]), np.array([4e18])),
+           W.Primitive("box", np.array([-1e60, 0.0, 1e59]), np.array([1e40, 2.0, 1e30])),
+           W.Primitive("sphere", np.array([1.0, 2.0, 3.0]), np.array([0.5]))]
+    pr = O.prims_array(far)
+    x = np.array([[0.0, 0.0, 0.0], [1e17, -1e18, 2.0], [3e19, 1e19, -1e19], [-1e59, 1e58, 0.0],
+                  [-9.9e59, 1.0, 1e59], [1.2, 2.1, 3.3], [1e20, 0.0, 0.0]])
+    states = np.concatenate([x, np.full((len(x), 3), -0.25)], 1)
+    eid = R.rmp_esdf_upload(ctx.handle, far)
+    try:
+        _, q = run_esdf(ctx, eid, states, None, R.make_params(W.PARAMS_STATIC_MAP, 10.0))
+        po = O.make_params(W.PARAMS_STATIC_MAP, 10.0)
+        for i, s in enumerate(states):
+            assert np.array_equal(q[i], O.esdf_eval(pr, s[:3], s[3:], po)[1]), i
+    finally:
+        R.rmp_esdf_release(ctx.handle, eid)
+
+
+@pytest.mark.parametrize("n_states,total", [(1216, 9000), (1217, 19000), (2500, 40000),
+                                            (2500, 90000), (1217, 200000)])
+def test_batch_many_states(ctx, n_states, total):
+    """Set-up runs of 8 and of more states a CTA, states without rays and invalid ones among
+    them, 1, 2 and 4 segments marched: a state's result is bitwise the one it has alone."""
+    wl = W.hashed_workload(n_states=8, state_seed_index=21)
+    mid, om = ctx.upload(wl.map), O.OracleMap(wl.map)
+    rng = np.random.default_rng(total)
+    counts = rng.multinomial(total, rng.dirichlet(np.full(n_states, 0.3))).astype(np.uint32)
+    states = np.stack([np.concatenate([wl.states[b % 8].x, wl.states[b % 8].xdot])
+                       for b in range(n_states)])
+    bad = rng.choice(n_states, 9, replace=False)
+    counts[bad] = 100
+    states[bad, rng.integers(0, 6, 9)] = np.nan
+    pg, po = R.make_params(wl.params, wl.max_range), O.make_params(wl.params, wl.max_range)
+    try:
+        res, h, _, _ = run_batch(ctx, mid, states, counts, pg)
+        for b in range(n_states):
+            if b in bad:                # a position is checked; a velocity only ends in the sums
+                at_x = np.isnan(states[b, :3]).any()
+                assert res[b]["status"] == (R.RMP_ERR_INVALID_ARG if at_x else 0)
+            elif counts[b] == 0:
+                assert res[b]["status"] == 0 and res[b]["n_rays"] == 0
+                assert np.all(res[b]["f"] == 0.0)
+        good = np.setdiff1d(np.flatnonzero(counts), bad)
+        for b in [*good[:3], *good[-3:], *rng.choice(good, 14), int(np.argmax(counts))]:
+            ro, ho, por = O.raycast_eval(om, states[b, :3], states[b, 3:], int(counts[b]), po)
+            assert_hits_exact(h[b, :counts[b]], ho)
+            assert_result_close(res[b], ro, por)
+            alone = run_batch(ctx, mid, states[b:b + 1], counts[b:b + 1], pg, want=False)[0][0]
+            for key in ("f", "sumA", "sumAf", "eig"):
+                assert np.array_equal(alone[key], res[b][key]), (b, key)
+    finally:
+        R.rmp_map_release(ctx.handle, mid)
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 1023, 4097, 77825])
+def test_scan_rows_ragged(ctx, n):
+    """The per-point rows, which a warp writes together: against the oracle, and nothing is
+    written past the last point."""
+    sw = W.lidar_workload()
+    pts = sw.points[np.random.default_rng(n).integers(0, len(sw.points), n)]
+    torch = torch_cuda()
+    per = torch.full(((n + 7) * 9,), -7.5, dtype=torch.float32, device="cuda")
+    rg = R.rmp_scan_eval(ctx.handle, torch.from_numpy(pts).cuda(), sw.x, sw.xdot,
+                         R.make_params(sw.params, sw.max_range), per_ray=per[:9 * n])
+    got = per.cpu().numpy().reshape(-1, 9).astype(np.float64)
+    assert np.all(got[n:] == -7.5)
+    ro, por = O.scan_eval(pts, sw.x, sw.xdot, O.make_params(sw.params, sw.max_range))
+    at = scan_abs_term(pts, sw.x, sw.xdot, sw.params)
+    assert_per_ray_close(got[:n], por, at)
+    assert_result_close(rg, ro, por, at)
