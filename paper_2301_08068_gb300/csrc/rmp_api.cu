@@ -771,6 +771,16 @@ int batch_setup(rmp_ctx* c, uint32_t map_id, uint32_t n_states, uint32_t max_ray
 
 namespace {
 
+bool attractor_ok(double alpha, double beta) {
+  return std::isfinite(alpha) && alpha >= 0.0 && std::isfinite(beta) && beta >= 0.0;
+}
+
+void set_attractor(double alpha, double beta, int metric_mean, EvalConsts* k) {
+  k->att_alpha = alpha;
+  k->att_beta = beta;
+  k->att_mean = metric_mean ? 1 : 0;
+}
+
 int batch_async_impl(rmp_ctx* c, uint32_t map_id, const double* states_dev,
                      const uint32_t* n_rays_dev, uint32_t n_states, uint32_t max_rays,
                      const rmp_params_t* params, void* ws, size_t ws_bytes, rmp_stream_t stream,
@@ -781,8 +791,7 @@ int batch_async_impl(rmp_ctx* c, uint32_t map_id, const double* states_dev,
   if (n_states == 0 || n_states > kMaxBatchStates || max_rays == 0 ||
       ws_bytes < batch_layout(n_states, max_rays).total)
     return RMP_ERR_INVALID_ARG;
-  if (goals_dev && !(std::isfinite(alpha) && alpha >= 0.0 && std::isfinite(beta) && beta >= 0.0))
-    return RMP_ERR_INVALID_ARG;
+  if (goals_dev && !attractor_ok(alpha, beta)) return RMP_ERR_INVALID_ARG;
   DeviceGuard g(c->device);
   if (!g.ok()) return RMP_ERR_CUDA;
   DevMap dm;
@@ -790,9 +799,7 @@ int batch_async_impl(rmp_ctx* c, uint32_t map_id, const double* states_dev,
   int block, grid;
   int st = batch_setup(c, map_id, n_states, max_rays, params, &dm, &k, &block, &grid);
   if (st != RMP_OK) return st;
-  k.att_alpha = alpha;
-  k.att_beta = beta;
-  k.att_mean = metric_mean ? 1 : 0;
+  set_attractor(alpha, beta, metric_mean, &k);
   RMP_CUDA(launch_batch(dm, k, states_dev, n_rays_dev, n_states, max_rays, ws, out_dev, hits_dev,
                         per_ray_dev, block, grid, (cudaStream_t)stream, goals_dev, step));
   return RMP_OK;
@@ -821,8 +828,7 @@ int make_esdf_consts(const rmp_params_t* p, double alpha, double beta, EsdfConst
   EvalConsts e;
   const int st = make_consts(p, 1.0, 1, true, &e);
   if (st != RMP_OK) return st;
-  if (!(std::isfinite(alpha) && alpha >= 0.0 && std::isfinite(beta) && beta >= 0.0))
-    return RMP_ERR_INVALID_ARG;
+  if (!attractor_ok(alpha, beta)) return RMP_ERR_INVALID_ARG;
   std::memset(k, 0, sizeof(*k));
   k->eta_rep = p->eta_rep;
   k->nu_rep = p->nu_rep;
@@ -861,7 +867,17 @@ int rollout_impl(rmp_ctx* c, uint32_t map_id, const EsdfRec* esdf, const double*
   DeviceGuard g(c->device);
   if (!g.ok()) return RMP_ERR_CUDA;
   cudaStream_t s = (cudaStream_t)stream;
-  const size_t wsb = esdf ? 0 : batch_layout(n, rp->n_rays).total;
+  // a CTA per robot for all steps, or an evaluation of all robots per step
+  const bool resident = !esdf && rollout_resident(n, rp->n_rays);
+  EvalConsts k;
+  if (resident) {
+    if (!attractor_ok(rp->alpha, rp->beta)) return RMP_ERR_INVALID_ARG;
+    int block, grid;
+    const int st = batch_setup(c, map_id, n, rp->n_rays, params, &dm, &k, &block, &grid);
+    if (st != RMP_OK) return st;
+    set_attractor(rp->alpha, rp->beta, (int)rp->metric_mean, &k);
+  }
+  const size_t wsb = esdf || resident ? 0 : batch_layout(n, rp->n_rays).total;
   const size_t o_st = 0, o_goal = align256(48 * (size_t)n), o_nr = o_goal + align256(24 * (size_t)n),
                o_res = o_nr + align256(4 * (size_t)n),
                o_rs = o_res + align256(sizeof(rmp_result_t) * n),
@@ -890,6 +906,7 @@ int rollout_impl(rmp_ctx* c, uint32_t map_id, const EsdfRec* esdf, const double*
   args.rc.max_steps = rp->max_steps;
   args.rc.seg_steps = rp->seg_steps;
   args.rc.n_rays = rp->n_rays;
+  args.rc.inv_rays = 1.0 / (double)std::max(rp->n_rays, 1u);
   args.rc.pad = 0;
   args.rs = d_rs;
   args.states = d_st;
@@ -901,13 +918,20 @@ int rollout_impl(rmp_ctx* c, uint32_t map_id, const EsdfRec* esdf, const double*
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_nr, nr.data(), 4 * (size_t)n, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_rs, rs.data(), sizeof(RolloutDev) * n, cudaMemcpyHostToDevice, s);
-  // steps in rounds of 32; after each round the running count decides whether to go on
-  const uint32_t kRound = 32;
+  // steps in rounds; after each round the running count decides whether to go on (long ones where
+  // a round is one launch and every robot has an SM: its own end is then all that ends a CTA)
+  const uint32_t kRound = resident && n <= 304 ? 256 : 32;
   uint32_t running = n;
   for (uint32_t step = 0; e == cudaSuccess && status == RMP_OK && running > 0 &&
                           step < rp->max_steps;) {
     e = cudaMemsetAsync(d_cnt, 0, 4, s);
-    for (uint32_t i = 0; i < kRound && step < rp->max_steps && e == cudaSuccess; ++i, ++step) {
+    if (resident && e == cudaSuccess) {
+      const uint32_t most = std::min(kRound, rp->max_steps - step);
+      args.running = d_cnt;
+      e = launch_rollout(dm, k, args, n, most, s);
+      step += most;
+    }
+    for (uint32_t i = 0; !resident && i < kRound && step < rp->max_steps && e == cudaSuccess; ++i, ++step) {
       args.running = i + 1 == kRound || step + 1 == rp->max_steps ? d_cnt : nullptr;
       if (esdf) {
         e = launch_esdf_eval(esdf->prims, esdf->prims32, esdf->n, ek, d_st, d_goal, n, d_res, nullptr,

@@ -104,7 +104,7 @@ struct RolloutDev {
 };
 
 struct RolloutConsts {
-  double dt, goal_tol;
+  double dt, goal_tol, inv_rays;            // inv_rays: 1 / n_rays, exact for powers of two
   uint32_t max_steps, seg_steps, n_rays, pad;
 };
 
@@ -173,6 +173,18 @@ struct BatchHeader {        // 128 bytes
   uint32_t pad[29];
 };
 
+// Rollouts with a CTA per robot for all its steps (see rollout_kernel): up to 1024 rays, or as many
+// as its shared memory holds where the robots fill the SMs but once; more rays of few robots are
+// spread over all SMs instead, robots of many rays packed (us a step with its share of the call,
+// CTA per robot / evaluated together: 8 robots of 1024 rays 23 / 34, of 4096 70 / 37; 32 of 2048
+// 40 / 45; 128 of 1024 38 / 68, of 4096 77 / 121; 304 of 4096 186 / 207, 608 361 / 347; 1216 of
+// 256 175 / 227, of 1024 258 / 318).
+constexpr uint32_t kRolloutRays = 4096, kRolloutGroups = kRolloutRays * kMaxBatchSegs / (32 * 32);
+inline bool rollout_resident(uint32_t n_robots, uint32_t n_rays) {
+  return n_rays <= 1024 ||
+         (n_rays <= kRolloutRays && n_rays <= 64 * n_robots && n_robots <= 304);
+}
+
 struct BatchLayout {
   size_t states, sticket, gticket, cparts, gparts, total;
   uint64_t chunks_per_state, groups_per_state;
@@ -235,6 +247,9 @@ cudaError_t launch_esdf_eval(const rmp_primitive_t* prims, const float4* prims32
                              uint32_t n_prims, const EsdfConsts& k, const double* states,
                              const double* goals, uint32_t n_states, rmp_result_t* out,
                              double* query, cudaStream_t stream);
+// Up to `steps` control steps of the rollouts, a CTA per robot (see rollout_resident).
+cudaError_t launch_rollout(const DevMap& m, const EvalConsts& k, const RolloutArgs& g, uint32_t n,
+                           uint32_t steps, cudaStream_t stream);
 // One control step of every robot from its evaluation in res.
 cudaError_t launch_rollout_step(const DevMap& m, const RolloutArgs& step, const rmp_result_t* res,
                                 uint32_t n, cudaStream_t stream);

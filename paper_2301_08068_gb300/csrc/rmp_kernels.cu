@@ -11,6 +11,7 @@
 // Bit-exact steps (Halton direction, DDA, hit distance, the FP32 decisions that gate a
 // ray) use explicitly rounded intrinsics (__fmul_rn, __fmaf_rn, ...) so that no
 // contraction or fast-math rewrite can change them.
+#include <algorithm>
 #include <climits>
 #include <cstddef>
 #include <type_traits>
@@ -1613,7 +1614,7 @@ __device__ __forceinline__ uint32_t pick_cells_warp(uint32_t n) {
 // threads the persistent launch holds at once -- a function of the ray count and the launch
 // shape alone, so a state's result does not depend on the other states of the batch or their
 // order.
-__device__ __forceinline__ uint32_t state_lg_segs(const EvalConsts& k, uint32_t n) {
+__host__ __device__ __forceinline__ uint32_t state_lg_segs(const EvalConsts& k, uint32_t n) {
   if (k.lg_segs <= 2u) return k.lg_segs;
   if (k.seg_threads == 0u) return n <= 4096u ? 2u : (n <= 16384u ? 1u : 0u);
   uint32_t lg = 2u;
@@ -1772,6 +1773,17 @@ __global__ void __launch_bounds__(256) batch_prep_kernel(
   for (uint32_t i = first_g + tid; i < before_g; i += 256) gticket[i] = 0;
 }
 
+// s + c of an FP32 pair in FP64.  A normal value is widened by integer instructions (an FP64
+// conversion holds the pipe about 64 cycles); the rare others by the conversion.
+__device__ __forceinline__ double pair_sum(float s, float c) {
+  auto plain = [](float f) {                        // zero or normal
+    const uint32_t b = __float_as_uint(f) << 1;
+    return b == 0u || (b >= 0x01000000u && b < 0xff000000u);
+  };
+  if (plain(s) && plain(c)) return widen(s) + widen(c);
+  return (double)s + (double)c;
+}
+
 // Lane i's terms and counts of a chunk partial (FP32 pairs for the compensated reduction, as
 // CtaPartial32) or of a group partial (FP64), read past L1: another SM wrote it.
 template <bool PAIR>
@@ -1790,7 +1802,7 @@ __device__ __forceinline__ void load_partial(const CtaPartial* p, double v[9], u
     }
 #pragma unroll
     for (int i = 0; i < 9; ++i)
-      v[i] = (double)__uint_as_float(w[i]) + (double)__uint_as_float(w[9 + i]);
+      v[i] = pair_sum(__uint_as_float(w[i]), __uint_as_float(w[9 + i]));
     h = w[18];
     a = w[19];
   } else {
@@ -1859,17 +1871,42 @@ __device__ __forceinline__ bool voxel_occupied(const DevMap& m, int kx, int ky, 
   return (__ldg(reinterpret_cast<const uint32_t*>(m.bricks) + 16 * at + (p >> 5)) >> (p & 31u)) & 1u;
 }
 
-// One control step of point robot b (Sec. IV-A closed loop): the combined policy's
-// acceleration f is integrated by semi-implicit Euler in FP64, xdot' = xdot + f dt,
-// x' = x + xdot' dt; then, in this order: outside a dense grid -> LEFT_MAP; the voxel of x'
-// occupied -> COLLIDED; |x' - goal| < goal_tol -> REACHED; steps == max_steps -> TIMEOUT.  Every
-// seg_steps steps the displacement since the last segment end is a segment, and consecutive
-// segments A, B add 1 - acos(cos(A, B)) / pi to the smoothness sum.  A robot that stops running
-// gets 0 rays from then on.  Called by a warp for a running robot, axis a in lane a (0-2; an FP64
-// instruction costs the same for one lane or three), f_a in those lanes.
+// One control step of a point robot (Sec. IV-A closed loop): the combined policy's acceleration f
+// is integrated by semi-implicit Euler in FP64, xdot' = xdot + f dt, x' = x + xdot' dt; then, in
+// this order: outside a dense grid -> LEFT_MAP; the voxel of x' occupied -> COLLIDED; |x' - goal| <
+// goal_tol -> REACHED; steps == max_steps -> TIMEOUT.  Every seg_steps steps the displacement since
+// the last segment end is a segment, and consecutive segments A, B add 1 - acos(cos(A, B)) / pi to
+// the smoothness sum.  In two parts, called by a warp with axis a in lane a (0-2; an FP64
+// instruction costs the same for one lane or three): what the next evaluation waits for, and the
+// rest.
+struct RolloutMove {
+  double x, xn, v;          // position before and after, new velocity
+  long long fx;             // the new position, quantised
+  bool far;                 // it is beyond the fixed-point range
+};
+
+template <int KIND>
+__device__ __forceinline__ RolloutMove rollout_move(const DevMap& m, const RolloutConsts& rc,
+                                                    double x, double v, double f) {
+  const uint32_t lane = threadIdx.x & 31;
+  RolloutMove w;
+  w.x = x;
+  w.v = __fma_rn(f, rc.dt, v);
+  w.xn = __fma_rn(w.v, rc.dt, x);
+  const double o = KIND == RMP_MAP_DENSE_U8
+                       ? (lane == 1 ? m.origin[1] : (lane == 2 ? m.origin[2] : m.origin[0]))
+                       : 0.0;
+  const double q = __dmul_rn(__ddiv_rn(__dsub_rn(w.xn, o), m.vs), 65536.0);
+  w.far = __any_sync(0xffffffffu, lane < 3 && !(fabs(q) < 274877906944.0));
+  w.fx = w.far ? 0 : __double2ll_rn(q);
+  return w;
+}
+
+// The step's path, segment and ending into the robot's record r.  Returns the status in lane 0.
 template <int KIND, int LAYOUT>
-__device__ __noinline__ void rollout_step(const DevMap& m, const RolloutArgs& g, uint32_t b,
-                                          double f) {
+__device__ __noinline__ uint32_t rollout_book(const DevMap& m, const RolloutConsts& rc,
+                                              RolloutDev& r, double x, double xn, double goal,
+                                              long long fx, bool far) {
   const uint32_t lane = threadIdx.x & 31, a = lane < 3 ? lane : 0;
   auto of = [](double v, int i) { return __shfl_sync(0xffffffffu, v, i); };
   // (v0 w0 + v1 w1) + v2 w2 of two vectors that lie across the lanes, in every lane
@@ -1877,19 +1914,10 @@ __device__ __noinline__ void rollout_step(const DevMap& m, const RolloutArgs& g,
     const double p = __dmul_rn(of(v, 0), of(w, 0));
     return __fma_rn(of(v, 2), of(w, 2), __fma_rn(of(v, 1), of(w, 1), p));
   };
-  RolloutDev& r = g.rs[b];
-  double* st = g.states + 6 * (size_t)b;
-  const double x = st[a], goal = g.goals[3 * (size_t)b + a];
   const double path = r.path_length;
   const uint32_t steps = r.steps + 1;
-  const double vd = __fma_rn(f, g.rc.dt, st[3 + a]);
-  const double xn = __fma_rn(vd, g.rc.dt, x);
   const double dl = dot3(xn - x, xn - x);
-  if (lane < 3) {
-    st[3 + a] = vd;
-    st[a] = xn;
-  }
-  if (g.rc.seg_steps && steps % g.rc.seg_steps == 0) {
+  if (rc.seg_steps && steps % rc.seg_steps == 0) {
     const double seg = xn - r.seg_start[a], prev = r.prev_seg[a];
     const bool have = r.have_prev != 0;
     if (have) {
@@ -1910,25 +1938,39 @@ __device__ __noinline__ void rollout_step(const DevMap& m, const RolloutArgs& g,
     }
     if (lane == 0) r.have_prev = 1;
   }
-  const double o = KIND == RMP_MAP_DENSE_U8 ? (a == 0 ? m.origin[0] : (a == 1 ? m.origin[1] : m.origin[2]))
-                                            : 0.0;
-  const double q = __dmul_rn(__ddiv_rn(__dsub_rn(xn, o), m.vs), 65536.0);
-  const bool far = __any_sync(0xffffffffu, !(fabs(q) < 274877906944.0));
-  const int ka = far ? 0 : (int)(__double2ll_rn(q) >> 16);
+  const int ka = (int)(fx >> 16);
   const int k[3] = {__shfl_sync(0xffffffffu, ka, 0), __shfl_sync(0xffffffffu, ka, 1),
                     __shfl_sync(0xffffffffu, ka, 2)};
   const double dg = dot3(xn - goal, xn - goal);
   const double len = sqrt(lane == 1 ? dg : dl);    // lane 0: the step's, lane 1: to the goal
   const double to_goal = of(len, 1);
-  if (lane != 0) return;
+  if (lane != 0) return 0;
   uint32_t status = RMP_ROLLOUT_RUNNING;
   if (far || (KIND == RMP_MAP_DENSE_U8 && outside<KIND>(m, k))) status = RMP_ROLLOUT_LEFT_MAP;
   else if (voxel_occupied<LAYOUT>(m, k[0], k[1], k[2])) status = RMP_ROLLOUT_COLLIDED;
-  else if (to_goal < g.rc.goal_tol) status = RMP_ROLLOUT_REACHED;
-  else if (steps >= g.rc.max_steps) status = RMP_ROLLOUT_TIMEOUT;
+  else if (to_goal < rc.goal_tol) status = RMP_ROLLOUT_REACHED;
+  else if (steps >= rc.max_steps) status = RMP_ROLLOUT_TIMEOUT;
   r.path_length = path + len;
   r.steps = steps;
   r.status = status;
+  return status;
+}
+
+// Running robot b's control step in device memory, f_a in lane a.  A robot that stops gets 0 rays
+// from then on.
+template <int KIND, int LAYOUT>
+__device__ __forceinline__ void rollout_step(const DevMap& m, const RolloutArgs& g, uint32_t b,
+                                             double f) {
+  const uint32_t lane = threadIdx.x & 31, a = lane < 3 ? lane : 0;
+  double* st = g.states + 6 * (size_t)b;
+  const RolloutMove w = rollout_move<KIND>(m, g.rc, st[a], st[3 + a], f);
+  if (lane < 3) {
+    st[3 + a] = w.v;
+    st[a] = w.xn;
+  }
+  const uint32_t status = rollout_book<KIND, LAYOUT>(m, g.rc, g.rs[b], w.x, w.xn,
+                                                     g.goals[3 * (size_t)b + a], w.fx, w.far);
+  if (lane != 0) return;
   if (status != RMP_ROLLOUT_RUNNING) g.n_rays[b] = 0;
   else if (g.running) atomicAdd(g.running, 1u);
 }
@@ -2182,6 +2224,230 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
       batch_group_finish<KIND, LAYOUT, RED>(m, k, step, cparts, gparts, sticket, part0, gi, gsz,
                                             n_parts, chunks, group0, b, n_b, states, goals, out);
     c = __shfl_sync(0xffffffffu, cn, 0);
+  }
+}
+
+// ------------------------------------------------------------------ resident rollouts
+// A robot's control steps depend on its own steps alone, so one CTA takes one robot through all its
+// steps: no launch, set-up, ticket or fence between steps, the robot, its ray directions (the same
+// at every step) and the partials in shared memory, and a robot waits for its own slowest warp
+// instead of the launch's (where this is taken: rollout_resident).  Every sum is cut and ordered as
+// in raycast_batch_kernel (see state_lg_segs, batch_group_finish).
+// A step: the warps march the chunks, 32 / s rays each; the last two, which have no chunk where the
+// CTA has room, form the attractor and book the step before (whose ending so only decides after
+// the march whether it counts); a warp per group of 32 partials sums it; warp 0 sums the groups,
+// solves and moves the robot.
+// Bound by that chain: the slowest of a robot's marches (13 us of 1024 rays, their mean 6) and
+// the FP64 after it.
+// 128 robots of 1024 rays, 48 steps: 1380 us, of which the call itself about 450 (set-up and
+// evaluation launched per step: 2690); 16 robots of 64 rays 555 (1455).
+struct RolloutShared {
+  RolloutDev r;
+  double st[6], x0[3], goal[3], att[3], S[9];       // x0: the position before the last step
+  double gsum[kRolloutGroups][9];
+  long long P[3];
+  float v[3], vl[3];
+  rmp_result_t res;
+  uint32_t cells;
+  int go, far;
+};
+constexpr uint32_t kPartWords = 18;                 // a partial: 9 FP32 pairs or 9 doubles
+
+// Named barriers (the groups' sums meet at 2; arrival only for the warps that go on).
+__device__ __forceinline__ void bar_arrive(int id, uint32_t threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_sync(int id, uint32_t threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+template <int KIND, int LAYOUT, int RED, bool BOXES>
+__global__ void __launch_bounds__(1024, 1) rollout_kernel(const __grid_constant__ DevMap m,
+                                                          const __grid_constant__ EvalConsts k,
+                                                          const __grid_constant__ RolloutArgs g,
+                                                          uint32_t n, uint32_t lg, uint32_t lgs,
+                                                          uint32_t steps) {
+  extern __shared__ __align__(16) float dyn[];      // directions [6][n], then the partials
+  __shared__ RolloutShared sh;
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const uint32_t b = blockIdx.x;
+  const uint32_t n_parts = ((n << lg) + 31) / 32, chunks = ((n << lgs) + 31) / 32;
+  const uint32_t n_groups = (n_parts + kBatchGroup - 1) / kBatchGroup;
+  const uint32_t S = 1u << lgs, lgW = lg - lgs;
+  float* parts = dyn + ((6 * n + 3) & ~3u);
+  wait_previous();
+  if (g.rs[b].status != RMP_ROLLOUT_RUNNING) return;
+  if (warp == 0) {
+    if (lane < sizeof(RolloutDev) / 8)
+      reinterpret_cast<unsigned long long*>(&sh.r)[lane] =
+          reinterpret_cast<const unsigned long long*>(g.rs + b)[lane];
+    bool bad = false;
+    if (lane < 6) {
+      const double x = g.states[6 * (size_t)b + lane];
+      sh.st[lane] = x;
+      if (lane < 3) {
+        sh.goal[lane] = g.goals[3 * (size_t)b + lane];
+        const double o = KIND != RMP_MAP_DENSE_U8 ? 0.0
+                         : (lane == 0 ? m.origin[0] : (lane == 1 ? m.origin[1] : m.origin[2]));
+        const double q = __dmul_rn(__ddiv_rn(__dsub_rn(x, o), m.vs), 65536.0);
+        bad = !(fabs(q) < 274877906944.0);
+        sh.P[lane] = bad ? 0 : __double2ll_rn(q);
+      } else {
+        sh.v[lane - 3] = __double2float_rn(x);
+        sh.vl[lane - 3] = __double2float_rn(__dsub_rn(x, (double)sh.v[lane - 3]));
+      }
+    }
+    bad = __any_sync(0xffffffffu, bad);
+    if (bad && lane == 0) g.rs[b].status = RMP_ROLLOUT_FAILED;
+    const uint32_t M = n >= 32 ? pick_cells_warp(n) : 1u;
+    if (lane == 0) {
+      sh.cells = M;
+      sh.go = bad ? 0 : 1;
+    }
+  }
+  __syncthreads();
+  if (!sh.go) return;
+  for (uint32_t slot = threadIdx.x; slot < n; slot += blockDim.x) {
+    const uint32_t M = sh.cells, Q = n / M;
+    const Ray ray = make_ray<true>(ray_of_slot(slot, M, Q, n - Q * M) + k.halton_offset);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      dyn[a * n + slot] = ray.dir[a];
+      dyn[(3 + a) * n + slot] = __int_as_float(ray.D[a]);
+    }
+  }
+  for (uint32_t step = 0;; ++step) {
+    __syncthreads();                                // the state; first: the directions
+    const bool last = step == steps;
+    for (uint32_t q = warp; q < chunks && !last; q += nw) {
+      const uint32_t gl = q * 32 + lane, seg = gl & (S - 1);
+      const bool active = (gl >> lgs) < n;
+      const uint32_t slot = active ? gl >> lgs : 0;
+      Ray ray;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        ray.dir[a] = dyn[a * n + slot];
+        ray.D[a] = __float_as_int(dyn[(3 + a) * n + slot]);
+      }
+      const long long P[3] = {sh.P[0], sh.P[1], sh.P[2]};
+      uint32_t en, ea;
+      const int mstat = march_ray<KIND, LAYOUT, BOXES>(m, k, P, ray, seg, lgs, active, en, ea,
+                                                       nullptr);
+      const float v[3] = {sh.v[0], sh.v[1], sh.v[2]}, vl[3] = {sh.vl[0], sh.vl[1], sh.vl[2]};
+      float vals[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      unsigned nh = 0, na = 0;
+      bool adds = false;
+      if (active && seg == 0)
+        adds = ray_outputs(m, k, ray, mstat, en, ea, v, vl, quiet_state(k, v), nullptr, vals, nh, na);
+      const bool any = __any_sync(0xffffffffu, adds);
+      if (!any)
+#pragma unroll
+        for (int i = 0; i < 9; ++i) vals[i] = 0.0f;
+      const uint32_t mine = (q << lgW) + (lane >> (5 - lgW));
+      const WarpTerms t = warp_terms(lgW);
+      float* part = parts + kPartWords * mine;
+      if (RED == RMP_REDUCE_FP64) {
+        double pv[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) pv[i] = any ? (double)vals[i] : 0.0;
+        if (any) warp_reduce_terms<double, false>(pv, pv, lgW);
+        double* pd = reinterpret_cast<double*>(part);
+        if (mine < n_parts) {
+          if (t.n > 0) pd[t.first] = pv[0];
+          if (t.n > 1) pd[t.first + 1] = pv[1];
+        }
+      } else {
+        float cv[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (any) warp_reduce_terms<float, true>(vals, cv, lgW);
+        if (mine < n_parts) {
+          if (t.n > 0) {
+            part[t.first] = vals[0];
+            part[9 + t.first] = cv[0];
+          }
+          if (t.n > 1) {
+            part[t.first + 1] = vals[1];
+            part[9 + t.first + 1] = cv[1];
+          }
+        }
+      }
+    }
+    if (warp == nw - 1 && step > 0) {
+      const uint32_t a = lane < 3 ? lane : 0;
+      const uint32_t status = rollout_book<KIND, LAYOUT>(m, g.rc, sh.r, sh.x0[a], sh.st[a],
+                                                         sh.goal[a], sh.P[a], sh.far != 0);
+      if (lane == 0) sh.go = status == RMP_ROLLOUT_RUNNING;
+    }
+    if (warp == nw - 2 && !last) {
+      const double att = attractor(k, sh.st, sh.goal);
+      if (lane < 3) sh.att[lane] = att;
+    }
+    __syncthreads();                                // the partials, the attractor, the booking
+    if (last || !sh.go) break;
+    for (uint32_t gi = warp; gi < n_groups; gi += nw) {
+      const uint32_t at = gi * kBatchGroup + lane;
+      const float* part = parts + kPartWords * at;
+      double v[9];
+#pragma unroll
+      for (int i = 0; i < 9; ++i)
+        v[i] = at >= n_parts ? 0.0
+               : RED == RMP_REDUCE_FP64 ? reinterpret_cast<const double*>(part)[i]
+                                        : pair_sum(part[i], part[9 + i]);
+      warp_reduce_terms<double, false>(v, v, 0);
+      const WarpTerms t = warp_terms(0);
+      if (t.n > 0) sh.gsum[gi][t.first] = v[0];
+    }
+    const uint32_t group_warps = min(n_groups, nw);
+    if (warp > 0 && warp < group_warps) bar_arrive(2, 32 * group_warps);
+    if (warp == 0) {
+      if (group_warps > 1) bar_sync(2, 32 * group_warps);
+      else __syncwarp();
+      if (lane < 9) {
+        // term `lane` of the groups, in the order of a tree over lanes
+        double v[kRolloutGroups];
+#pragma unroll
+        for (uint32_t i = 0; i < kRolloutGroups; ++i) v[i] = i < n_groups ? sh.gsum[i][lane] : 0.0;
+#pragma unroll
+        for (uint32_t off = kRolloutGroups / 2; off > 0; off >>= 1)
+          if (n_groups > off)
+#pragma unroll
+            for (uint32_t i = 0; i < off; ++i) v[i] += v[i + off];
+        double mine = v[0];
+        if (k.att_mean) mine = (n & (n - 1)) == 0 ? mine * g.rc.inv_rays : mine / (double)n;
+        sh.S[lane] = lane == 0 || lane == 3 || lane == 5 ? mine + 1.0
+                     : lane >= 6 ? mine + sh.att[lane - 6] : mine;
+      }
+      __syncwarp();
+      // A metric I + sum A_i with entries below 1e5 has full rank beyond doubt: its eigenvalues
+      // are at least 1 less the FP32 roundings of A_i (1e-6 of the entries), the threshold is 1e-12
+      // of the largest.  f is then the adjugate's solution.
+      int ok;
+      double f = adjugate_solve_warp(sh.S, sh.S + 6, ok);
+      if (!__all_sync(0xffffffffu, ok && fabs(sh.S[lane < 6 ? lane : 0]) < 1e5)) {
+        resolve_pinv(sh.S, sh.S + 6, sh.res);
+        __syncwarp();
+        f = sh.res.f[lane < 3 ? lane : 0];
+      }
+      const uint32_t a = lane < 3 ? lane : 0;
+      const RolloutMove w = rollout_move<KIND>(m, g.rc, sh.st[a], sh.st[3 + a], f);
+      __syncwarp();
+      if (lane < 3) {
+        sh.x0[a] = w.x;
+        sh.st[a] = w.xn;
+        sh.st[3 + a] = w.v;
+        sh.P[a] = w.fx;
+        const float vh = __double2float_rn(w.v);
+        sh.v[a] = vh;
+        sh.vl[a] = __double2float_rn(__dsub_rn(w.v, (double)vh));
+      }
+      if (lane == 0) sh.far = w.far ? 1 : 0;
+    }
+  }
+  if (warp == 0) {
+    if (lane < sizeof(RolloutDev) / 8)
+      reinterpret_cast<unsigned long long*>(g.rs + b)[lane] =
+          reinterpret_cast<const unsigned long long*>(&sh.r)[lane];
+    if (lane < 6) g.states[6 * (size_t)b + lane] = sh.st[lane];
+    if (lane == 0 && sh.go) atomicAdd(g.running, 1u);
   }
 }
 
@@ -3171,6 +3437,28 @@ cudaError_t launch_batch(const DevMap& m, const EvalConsts& k, const double* sta
                  per_ray, max_rays, states_dev, goals_dev, step);
   });
   return cudaGetLastError();
+}
+
+cudaError_t launch_rollout(const DevMap& m, const EvalConsts& k, const RolloutArgs& g, uint32_t n,
+                           uint32_t steps, cudaStream_t stream) {
+  // at most 32 warps a CTA; 16 where two robots share an SM and hide each other's serial steps
+  const uint32_t rays = g.rc.n_rays, most = n <= 152u ? 32u : 16u;
+  const uint32_t lg = state_lg_segs(k, rays), parts = ((rays << lg) + 31) / 32;
+  // the most segments marched per ray whose chunks the warps hold at once beside the two of the
+  // attractor and the booking (8 robots of 256 rays: 4 segments, both on marching warps 18.3 us a
+  // step, 2 segments 15.8)
+  uint32_t lgs = lg;
+  while (lgs > 0 && ((rays << lgs) + 31) / 32 + 2 > most) --lgs;
+  const uint32_t groups = (parts + kBatchGroup - 1) / kBatchGroup;
+  const uint32_t warps = std::min(std::max(((rays << lgs) + 31) / 32 + 2, groups), most);   // >= 3
+  const size_t dyn = 4 * (size_t)(((6 * rays + 3) & ~3u) + kPartWords * parts);
+  cudaError_t e = cudaSuccess;
+  for_map(m, k.reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
+    const auto f = rollout_kernel<kind.value, layout.value, red.value, boxes.value != 0>;
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    if (e == cudaSuccess) f<<<n, 32 * warps, dyn, stream>>>(m, k, g, rays, lg, lgs, steps);
+  });
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_rollout_step(const DevMap& m, const RolloutArgs& step, const rmp_result_t* res,

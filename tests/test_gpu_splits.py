@@ -1,7 +1,10 @@
 """The cuts of the work over CTAs, warps and lanes where they change: ESDF states on both sides
 of 8, 16 and 32 states a CTA, ties and distances that FP32 cannot tell apart, coordinates past
 FP32; batches with more states than one run of the set-up kernel takes and with total loads on
-both sides of the march's segment cuts; scans whose last warp is ragged, with the per-point rows."""
+both sides of the march's segment cuts; scans whose last warp is ragged, with the per-point rows;
+rollouts with a CTA per robot."""
+from fractions import Fraction as F
+
 import numpy as np
 import pytest
 
@@ -134,3 +137,63 @@ def test_scan_rows_ragged(ctx, n):
     at = scan_abs_term(pts, sw.x, sw.xdot, sw.params)
     assert_per_ray_close(got[:n], por, at)
     assert_result_close(rg, ro, por, at)
+
+
+def fma(a, b, c):
+    """a b + c rounded once, elementwise."""
+    return np.array([float(F(x) * F(y) + F(z)) for x, y, z in zip(a, b, c)])
+
+
+@pytest.mark.parametrize("rays,mean,red,lgs,steps", [
+    (1, False, 0, -1, 40), (31, True, 0, -1, 40), (64, True, 1, -1, 12), (257, True, 0, 1, 12),
+    (300, False, 1, 0, 12), (1000, True, 0, -1, 12), (1024, False, 0, -1, 300),
+    (1025, True, 0, -1, 8), (4096, True, 0, -1, 4), (4097, True, 0, -1, 3)])
+@pytest.mark.parametrize("dense", [True, False])
+def test_rollout_cta_per_robot(ctx, dense, rays, mean, red, lgs, steps):
+    """Every number of robots and so of warps a CTA, and rollouts evaluated together per step,
+    give a robot the same bits; the path is that of combined evaluations and Euler steps.  Among
+    the robots: one at its goal, a fast one that hits or leaves, one too far away, NaN."""
+    wl = W.dense_box_workload(n_states=6, jitter=True) if dense \
+        else W.hashed_workload(n_states=6, state_seed_index=52)
+    mid = ctx.upload(wl.map)
+    torch = torch_cuda()
+    rng = np.random.default_rng(rays)
+    robots = np.array([np.concatenate([s.x, s.xdot, s.x + rng.uniform(-3, 3, 3)]) for s in wl.states])
+    robots = np.concatenate([robots, robots[:5]])
+    robots[6, 6:] = robots[6, :3] + 1e-4
+    robots[7, 3:6] = [60.0, -80.0, 10.0]
+    robots[8, :3] = 1e9
+    robots[9, 3:6] = np.nan
+    robots[10, :3] = np.nan
+    many = np.tile(robots, (28, 1))                       # 308 robots
+    p = R.make_params(dict(wl.params, reduce_mode=red), wl.max_range)
+    rp = R.rollout_params(10.0, 15.0, 0.01, 0.05, steps, 3, rays, metric_mean=mean)
+    R.rmp_tune_set(ctx.handle, R.RMP_TUNE_LG_SEGMENTS, lgs)
+    try:
+        ref = R.rmp_rollout(ctx.handle, mid, robots, p, rp)
+        for n in (1, 152, 153, 305):
+            got = R.rmp_rollout(ctx.handle, mid, many[:n], p, rp)
+            for b in range(n):
+                for key, want in ref[b % 11].items():
+                    assert np.array_equal(got[b][key], want, equal_nan=True), (n, b, key)
+        x, v, goal = robots[:8, :3].copy(), robots[:8, 3:6].copy(), robots[:8, 6:]
+        nr = torch.full((8,), rays, dtype=torch.int32, device="cuda")
+        ws = torch.empty(R.rmp_batch_workspace_bytes(8, rays), dtype=torch.uint8, device="cuda")
+        out = torch.empty((8, R.RESULT_BYTES), dtype=torch.uint8, device="cuda")
+        gl = torch.tensor(goal, device="cuda")
+        for step in range(max(r["steps"] for r in ref[:8])):
+            st = torch.tensor(np.concatenate([x, v], 1), device="cuda")
+            R.rmp_combined_eval_batch_async(ctx.handle, mid, st, nr, 8, rays, p, gl, 10.0, 15.0, ws,
+                                            out, metric_mean=mean)
+            o = out.cpu().numpy()
+            for b in range(8):
+                if step < ref[b]["steps"]:
+                    v[b] = fma(R.result_from_bytes(o[b].tobytes())["f"], [0.01] * 3, v[b])
+                    x[b] = fma(v[b], [0.01] * 3, x[b])
+        for b in range(8):
+            assert np.array_equal(ref[b]["x"], x[b]) and np.array_equal(ref[b]["xdot"], v[b]), b
+        assert ref[6]["status"] == R.RMP_ROLLOUT_REACHED and ref[8]["status"] == R.RMP_ROLLOUT_FAILED
+        assert ref[10]["status"] == R.RMP_ROLLOUT_FAILED
+    finally:
+        R.rmp_tune_set(ctx.handle, R.RMP_TUNE_LG_SEGMENTS, -1)
+        R.rmp_map_release(ctx.handle, mid)
