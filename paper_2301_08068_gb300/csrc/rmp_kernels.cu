@@ -1773,17 +1773,6 @@ __global__ void __launch_bounds__(256) batch_prep_kernel(
   for (uint32_t i = first_g + tid; i < before_g; i += 256) gticket[i] = 0;
 }
 
-// s + c of an FP32 pair in FP64.  A normal value is widened by integer instructions (an FP64
-// conversion holds the pipe about 64 cycles); the rare others by the conversion.
-__device__ __forceinline__ double pair_sum(float s, float c) {
-  auto plain = [](float f) {                        // zero or normal
-    const uint32_t b = __float_as_uint(f) << 1;
-    return b == 0u || (b >= 0x01000000u && b < 0xff000000u);
-  };
-  if (plain(s) && plain(c)) return widen(s) + widen(c);
-  return (double)s + (double)c;
-}
-
 // Lane i's terms and counts of a chunk partial (FP32 pairs for the compensated reduction, as
 // CtaPartial32) or of a group partial (FP64), read past L1: another SM wrote it.
 template <bool PAIR>
@@ -1802,7 +1791,7 @@ __device__ __forceinline__ void load_partial(const CtaPartial* p, double v[9], u
     }
 #pragma unroll
     for (int i = 0; i < 9; ++i)
-      v[i] = pair_sum(__uint_as_float(w[i]), __uint_as_float(w[9 + i]));
+      v[i] = (double)__uint_as_float(w[i]) + (double)__uint_as_float(w[9 + i]);
     h = w[18];
     a = w[19];
   } else {
@@ -2227,6 +2216,254 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
   }
 }
 
+// ------------------------------------------------------------------ one CTA per state
+// Where states have few rays (state_per_cta, rollout_resident) a CTA evaluates one by itself: its
+// partials lie in shared memory, so there is no set-up launch, ticket or fence, and a state waits
+// for its own slowest warp.  Every sum is cut and ordered as in raycast_batch_kernel.
+constexpr uint32_t kPartWords = 18;                 // a partial: 9 FP32 pairs or 9 doubles
+
+// Named barriers 1 (in resolve_pinv_cta) to 4; arrival only for the warps that go on.
+__device__ __forceinline__ void bar_arrive(int id, uint32_t threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_sync(int id, uint32_t threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// Chunk q of a state (a warp): its rays' segments marched and evaluated, its partials stored.
+template <int KIND, int LAYOUT, int RED, bool BOXES>
+__device__ __forceinline__ void state_chunk(const DevMap& m, const EvalConsts& k,
+                                            const long long* Ps, const float* vs, const float* vls,
+                                            const Ray& ray, uint32_t q, uint32_t n, uint32_t lg,
+                                            uint32_t lgs, float* parts, rmp_ray_hit_t* hit,
+                                            float* per, unsigned& nh, unsigned& na) {
+  const uint32_t lane = threadIdx.x & 31, gl = q * 32 + lane, seg = gl & ((1u << lgs) - 1);
+  const uint32_t lgW = lg - lgs, n_parts = ((n << lg) + 31) / 32;
+  const bool active = (gl >> lgs) < n;
+  const long long P[3] = {Ps[0], Ps[1], Ps[2]};
+  uint32_t en, ea;
+  const int mstat = march_ray<KIND, LAYOUT, BOXES>(m, k, P, ray, seg, lgs, active, en, ea, hit);
+  const float v[3] = {vs[0], vs[1], vs[2]}, vl[3] = {vls[0], vls[1], vls[2]};
+  float vals[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  bool adds = false;
+  if (active && seg == 0)
+    adds = ray_outputs(m, k, ray, mstat, en, ea, v, vl, quiet_state(k, v), per, vals, nh, na);
+  const bool any = __any_sync(0xffffffffu, adds);
+  if (!any)
+#pragma unroll
+    for (int i = 0; i < 9; ++i) vals[i] = 0.0f;
+  const uint32_t mine = (q << lgW) + (lane >> (5 - lgW));
+  const WarpTerms t = warp_terms(lgW);
+  float* part = parts + kPartWords * mine;
+  if (RED == RMP_REDUCE_FP64) {
+    double pv[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) pv[i] = any ? (double)vals[i] : 0.0;
+    if (any) warp_reduce_terms<double, false>(pv, pv, lgW);
+    double* pd = reinterpret_cast<double*>(part);
+    if (mine < n_parts) {
+      if (t.n > 0) pd[t.first] = pv[0];
+      if (t.n > 1) pd[t.first + 1] = pv[1];
+    }
+  } else {
+    float cv[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (any) warp_reduce_terms<float, true>(vals, cv, lgW);
+    if (mine < n_parts) {
+      if (t.n > 0) {
+        part[t.first] = vals[0];
+        part[9 + t.first] = cv[0];
+      }
+      if (t.n > 1) {
+        part[t.first + 1] = vals[1];
+        part[9 + t.first + 1] = cv[1];
+      }
+    }
+  }
+}
+
+// s + c of an FP32 pair in FP64.  A normal value is widened by integer instructions (an FP64
+// conversion holds the pipe about 64 cycles); the rare others by the conversion.  For a CTA whose
+// other warps wait; where they march the integers cost more (batches of 64 x 4096 rays 72 -> 73.5 us).
+__device__ __forceinline__ double pair_sum(float s, float c) {
+  auto plain = [](float f) {                        // zero or normal
+    const uint32_t b = __float_as_uint(f) << 1;
+    return b == 0u || (b >= 0x01000000u && b < 0xff000000u);
+  };
+  if (plain(s) && plain(c)) return widen(s) + widen(c);
+  return (double)s + (double)c;
+}
+
+// The sums of a state from its partials, called by all warps after a barrier: a warp per group,
+// then term `lane` (0-8) of the groups in those lanes of warp 0, in the order of a tree over lanes.
+template <int RED>
+__device__ __forceinline__ double state_sum(const float* parts, uint32_t n_parts,
+                                            double (*gsum)[9]) {
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const uint32_t n_groups = (n_parts + kBatchGroup - 1) / kBatchGroup;
+  for (uint32_t gi = warp; gi < n_groups; gi += nw) {
+    const uint32_t at = gi * kBatchGroup + lane;
+    const float* part = parts + kPartWords * at;
+    double v[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+      v[i] = at >= n_parts ? 0.0
+             : RED == RMP_REDUCE_FP64 ? reinterpret_cast<const double*>(part)[i]
+                                      : pair_sum(part[i], part[9 + i]);
+    warp_reduce_terms<double, false>(v, v, 0);
+    const WarpTerms t = warp_terms(0);
+    if (t.n > 0) gsum[gi][t.first] = v[0];
+  }
+  const uint32_t group_warps = min(n_groups, nw);
+  if (warp > 0 && warp < group_warps) bar_arrive(2, 32 * group_warps);
+  if (warp > 0) return 0.0;
+  if (group_warps > 1) bar_sync(2, 32 * group_warps);
+  else __syncwarp();
+  double v[kStateGroups];
+#pragma unroll
+  for (uint32_t i = 0; i < kStateGroups; ++i) v[i] = lane < 9 && i < n_groups ? gsum[i][lane] : 0.0;
+#pragma unroll
+  for (uint32_t off = kStateGroups / 2; off > 0; off >>= 1)
+    if (n_groups > off)
+#pragma unroll
+      for (uint32_t i = 0; i < off; ++i) v[i] += v[i + off];
+  return v[0];
+}
+
+// A state quantised by warp 0, a component a lane (0-5); returns whether the position is unusable.
+template <int KIND>
+__device__ __forceinline__ bool quantise_state(const DevMap& m, double x, long long* P, float* v,
+                                               float* vl) {
+  const uint32_t lane = threadIdx.x & 31;
+  bool bad = false;
+  if (lane < 3) {
+    const double o = KIND != RMP_MAP_DENSE_U8 ? 0.0
+                     : (lane == 0 ? m.origin[0] : (lane == 1 ? m.origin[1] : m.origin[2]));
+    const double q = __dmul_rn(__ddiv_rn(__dsub_rn(x, o), m.vs), 65536.0);
+    bad = !(fabs(q) < 274877906944.0);
+    P[lane] = bad ? 0 : __double2ll_rn(q);
+  } else if (lane < 6) {
+    const float vh = __double2float_rn(x);
+    v[lane - 3] = vh;
+    vl[lane - 3] = __double2float_rn(__dsub_rn(x, (double)vh));
+  }
+  return __any_sync(0xffffffffu, bad);
+}
+
+// Segments marched per ray (log2): a tuned launch's, else the most whose chunks `warps` warps hold
+// at once, at most the summation's lg.
+__host__ __device__ __forceinline__ uint32_t cta_lg_segs(const EvalConsts& k, uint32_t n,
+                                                         uint32_t lg, uint32_t warps) {
+  if (k.lg_segs <= 2u) return lg;
+  while (lg > 0 && ((n << lg) + 31) / 32 > warps) --lg;
+  return lg;
+}
+
+// A batch of few-ray states, a CTA each (see state_per_cta): set up, marched, summed and resolved
+// in one launch; the last warp forms the attractor after its chunks.  Bound by that chain.
+// 128 states of 256 rays with the attractor: 17.8 us (set-up and persistent grid 30); 304 of 1024:
+// 43 (77).
+struct StateShared {
+  double S[9], att[3];
+  double gsum[kStateGroups][9];
+  long long P[3];
+  float v[3], vl[3];
+  rmp_result_t res;
+  uint32_t n, cells;
+  unsigned hits, active;
+  int bad;
+};
+
+template <int KIND, int LAYOUT, int RED, bool BOXES>
+__global__ void __launch_bounds__(1024, 1) raycast_state_kernel(
+    const __grid_constant__ DevMap m, const __grid_constant__ EvalConsts k,
+    const double* __restrict__ states, const uint32_t* __restrict__ n_rays, uint32_t max_rays,
+    rmp_result_t* out, rmp_ray_hit_t* hits, float* per_ray, const double* goals, uint32_t most) {
+  extern __shared__ __align__(16) float parts[];
+  __shared__ StateShared sh;
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const uint32_t b = blockIdx.x;
+  wait_previous();
+  const double* st = states + 6 * (size_t)b;
+  if (warp == 0) {
+    const bool bad = quantise_state<KIND>(m, lane < 6 ? st[lane] : 0.0, sh.P, sh.v, sh.vl);
+    if (lane == 0) {
+      sh.bad = bad;
+      sh.hits = sh.active = 0;
+    }
+  } else if (warp == 1) {
+    const uint32_t n = n_rays[b], M = n >= 32 ? pick_cells_warp(n) : 1u;
+    if (lane == 0) {
+      sh.n = n;
+      sh.cells = M;
+    }
+  }
+  __syncthreads();
+  const uint32_t n = sh.n;
+  const bool bad = sh.bad || n > max_rays;
+  if (bad || n == 0) {                              // 18 8-byte words of result
+    const unsigned long long w =
+        lane == 15 ? (unsigned long long)n
+                   : (lane == 17 && bad ? (unsigned long long)RMP_ERR_INVALID_ARG : 0ull);
+    if (threadIdx.x < 18) reinterpret_cast<unsigned long long*>(out + b)[threadIdx.x] = w;
+    launch_next();
+    return;
+  }
+  const uint32_t lg = state_lg_segs(k, n), lgs = cta_lg_segs(k, n, lg, most);
+  const uint32_t n_parts = ((n << lg) + 31) / 32, chunks = ((n << lgs) + 31) / 32;
+  const uint32_t M = sh.cells, Q = n / M;
+  unsigned nh = 0, na = 0;
+  for (uint32_t q = warp; q < chunks; q += nw) {
+    const uint32_t slot = (q * 32 + lane) >> lgs;
+    const uint32_t ray_idx = ray_of_slot(slot < n ? slot : 0, M, Q, n - Q * M);
+    const Ray ray = make_ray<true>(ray_idx + k.halton_offset);
+    const size_t ro = (size_t)b * max_rays + ray_idx;
+    state_chunk<KIND, LAYOUT, RED, BOXES>(m, k, sh.P, sh.v, sh.vl, ray, q, n, lg, lgs, parts,
+                                          hits ? hits + ro : nullptr,
+                                          per_ray ? per_ray + 9 * ro : nullptr, nh, na);
+  }
+  launch_next();
+  nh = __reduce_add_sync(0xffffffffu, nh);
+  na = __reduce_add_sync(0xffffffffu, na);
+  if (lane == 0 && nh) {
+    atomicAdd(&sh.hits, nh);
+    atomicAdd(&sh.active, na);
+  }
+  if (goals && warp == nw - 1) {
+    const double att = attractor(k, st, goals + 3 * (size_t)b);
+    if (lane < 3) sh.att[lane] = att;
+  }
+  __syncthreads();                                  // partials, counts, attractor
+  double mine = state_sum<RED>(parts, n_parts, sh.gsum);
+  if (warp == 0) {
+    if (lane < 9) {
+      if (goals) {
+        if (k.att_mean) mine = mine / (double)n;
+        if (lane == 0 || lane == 3 || lane == 5) mine += 1.0;
+        if (lane >= 6) mine += sh.att[lane - 6];
+      }
+      sh.S[lane] = mine;
+    }
+    __syncwarp();
+  }
+  if (warp >= 2) return;
+  bar_sync(4, 64);
+  resolve_pinv_cta(sh.S, sh.S + 6, sh.res);
+  if (warp == 1) return;
+  if (lane < 6) sh.res.A[lane] = sh.S[lane];
+  else if (lane < 9) sh.res.Af[lane - 6] = sh.S[lane];
+  else if (lane == 9) {
+    sh.res.n_rays = n;
+    sh.res.n_hits = sh.hits;
+    sh.res.n_active = sh.active;
+    sh.res.status = RMP_OK;
+    sh.res.reserved = 0;
+  }
+  __syncwarp();
+  if (lane < 18)
+    reinterpret_cast<unsigned long long*>(out + b)[lane] =
+        reinterpret_cast<const unsigned long long*>(&sh.res)[lane];
+}
+
 // ------------------------------------------------------------------ resident rollouts
 // A robot's control steps depend on its own steps alone, so one CTA takes one robot through all its
 // steps: no launch, set-up, ticket or fence between steps, the robot, its ray directions (the same
@@ -2244,22 +2481,13 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
 struct RolloutShared {
   RolloutDev r;
   double st[6], x0[3], goal[3], att[3], S[9];       // x0: the position before the last step
-  double gsum[kRolloutGroups][9];
+  double gsum[kStateGroups][9];
   long long P[3];
   float v[3], vl[3];
   rmp_result_t res;
   uint32_t cells;
   int go, far;
 };
-constexpr uint32_t kPartWords = 18;                 // a partial: 9 FP32 pairs or 9 doubles
-
-// Named barriers (the groups' sums meet at 2; arrival only for the warps that go on).
-__device__ __forceinline__ void bar_arrive(int id, uint32_t threads) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-__device__ __forceinline__ void bar_sync(int id, uint32_t threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
 
 template <int KIND, int LAYOUT, int RED, bool BOXES>
 __global__ void __launch_bounds__(1024, 1) rollout_kernel(const __grid_constant__ DevMap m,
@@ -2272,8 +2500,6 @@ __global__ void __launch_bounds__(1024, 1) rollout_kernel(const __grid_constant_
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const uint32_t b = blockIdx.x;
   const uint32_t n_parts = ((n << lg) + 31) / 32, chunks = ((n << lgs) + 31) / 32;
-  const uint32_t n_groups = (n_parts + kBatchGroup - 1) / kBatchGroup;
-  const uint32_t S = 1u << lgs, lgW = lg - lgs;
   float* parts = dyn + ((6 * n + 3) & ~3u);
   wait_previous();
   if (g.rs[b].status != RMP_ROLLOUT_RUNNING) return;
@@ -2281,23 +2507,10 @@ __global__ void __launch_bounds__(1024, 1) rollout_kernel(const __grid_constant_
     if (lane < sizeof(RolloutDev) / 8)
       reinterpret_cast<unsigned long long*>(&sh.r)[lane] =
           reinterpret_cast<const unsigned long long*>(g.rs + b)[lane];
-    bool bad = false;
-    if (lane < 6) {
-      const double x = g.states[6 * (size_t)b + lane];
-      sh.st[lane] = x;
-      if (lane < 3) {
-        sh.goal[lane] = g.goals[3 * (size_t)b + lane];
-        const double o = KIND != RMP_MAP_DENSE_U8 ? 0.0
-                         : (lane == 0 ? m.origin[0] : (lane == 1 ? m.origin[1] : m.origin[2]));
-        const double q = __dmul_rn(__ddiv_rn(__dsub_rn(x, o), m.vs), 65536.0);
-        bad = !(fabs(q) < 274877906944.0);
-        sh.P[lane] = bad ? 0 : __double2ll_rn(q);
-      } else {
-        sh.v[lane - 3] = __double2float_rn(x);
-        sh.vl[lane - 3] = __double2float_rn(__dsub_rn(x, (double)sh.v[lane - 3]));
-      }
-    }
-    bad = __any_sync(0xffffffffu, bad);
+    const double x = lane < 6 ? g.states[6 * (size_t)b + lane] : 0.0;
+    if (lane < 6) sh.st[lane] = x;
+    if (lane < 3) sh.goal[lane] = g.goals[3 * (size_t)b + lane];
+    const bool bad = quantise_state<KIND>(m, x, sh.P, sh.v, sh.vl);
     if (bad && lane == 0) g.rs[b].status = RMP_ROLLOUT_FAILED;
     const uint32_t M = n >= 32 ? pick_cells_warp(n) : 1u;
     if (lane == 0) {
@@ -2320,56 +2533,16 @@ __global__ void __launch_bounds__(1024, 1) rollout_kernel(const __grid_constant_
     __syncthreads();                                // the state; first: the directions
     const bool last = step == steps;
     for (uint32_t q = warp; q < chunks && !last; q += nw) {
-      const uint32_t gl = q * 32 + lane, seg = gl & (S - 1);
-      const bool active = (gl >> lgs) < n;
-      const uint32_t slot = active ? gl >> lgs : 0;
+      const uint32_t at = (q * 32 + lane) >> lgs, slot = at < n ? at : 0;
       Ray ray;
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         ray.dir[a] = dyn[a * n + slot];
         ray.D[a] = __float_as_int(dyn[(3 + a) * n + slot]);
       }
-      const long long P[3] = {sh.P[0], sh.P[1], sh.P[2]};
-      uint32_t en, ea;
-      const int mstat = march_ray<KIND, LAYOUT, BOXES>(m, k, P, ray, seg, lgs, active, en, ea,
-                                                       nullptr);
-      const float v[3] = {sh.v[0], sh.v[1], sh.v[2]}, vl[3] = {sh.vl[0], sh.vl[1], sh.vl[2]};
-      float vals[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       unsigned nh = 0, na = 0;
-      bool adds = false;
-      if (active && seg == 0)
-        adds = ray_outputs(m, k, ray, mstat, en, ea, v, vl, quiet_state(k, v), nullptr, vals, nh, na);
-      const bool any = __any_sync(0xffffffffu, adds);
-      if (!any)
-#pragma unroll
-        for (int i = 0; i < 9; ++i) vals[i] = 0.0f;
-      const uint32_t mine = (q << lgW) + (lane >> (5 - lgW));
-      const WarpTerms t = warp_terms(lgW);
-      float* part = parts + kPartWords * mine;
-      if (RED == RMP_REDUCE_FP64) {
-        double pv[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) pv[i] = any ? (double)vals[i] : 0.0;
-        if (any) warp_reduce_terms<double, false>(pv, pv, lgW);
-        double* pd = reinterpret_cast<double*>(part);
-        if (mine < n_parts) {
-          if (t.n > 0) pd[t.first] = pv[0];
-          if (t.n > 1) pd[t.first + 1] = pv[1];
-        }
-      } else {
-        float cv[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (any) warp_reduce_terms<float, true>(vals, cv, lgW);
-        if (mine < n_parts) {
-          if (t.n > 0) {
-            part[t.first] = vals[0];
-            part[9 + t.first] = cv[0];
-          }
-          if (t.n > 1) {
-            part[t.first + 1] = vals[1];
-            part[9 + t.first + 1] = cv[1];
-          }
-        }
-      }
+      state_chunk<KIND, LAYOUT, RED, BOXES>(m, k, sh.P, sh.v, sh.vl, ray, q, n, lg, lgs, parts,
+                                            nullptr, nullptr, nh, na);
     }
     if (warp == nw - 1 && step > 0) {
       const uint32_t a = lane < 3 ? lane : 0;
@@ -2383,38 +2556,13 @@ __global__ void __launch_bounds__(1024, 1) rollout_kernel(const __grid_constant_
     }
     __syncthreads();                                // the partials, the attractor, the booking
     if (last || !sh.go) break;
-    for (uint32_t gi = warp; gi < n_groups; gi += nw) {
-      const uint32_t at = gi * kBatchGroup + lane;
-      const float* part = parts + kPartWords * at;
-      double v[9];
-#pragma unroll
-      for (int i = 0; i < 9; ++i)
-        v[i] = at >= n_parts ? 0.0
-               : RED == RMP_REDUCE_FP64 ? reinterpret_cast<const double*>(part)[i]
-                                        : pair_sum(part[i], part[9 + i]);
-      warp_reduce_terms<double, false>(v, v, 0);
-      const WarpTerms t = warp_terms(0);
-      if (t.n > 0) sh.gsum[gi][t.first] = v[0];
-    }
-    const uint32_t group_warps = min(n_groups, nw);
-    if (warp > 0 && warp < group_warps) bar_arrive(2, 32 * group_warps);
+    double mine = state_sum<RED>(parts, n_parts, sh.gsum);
     if (warp == 0) {
-      if (group_warps > 1) bar_sync(2, 32 * group_warps);
-      else __syncwarp();
       if (lane < 9) {
-        // term `lane` of the groups, in the order of a tree over lanes
-        double v[kRolloutGroups];
-#pragma unroll
-        for (uint32_t i = 0; i < kRolloutGroups; ++i) v[i] = i < n_groups ? sh.gsum[i][lane] : 0.0;
-#pragma unroll
-        for (uint32_t off = kRolloutGroups / 2; off > 0; off >>= 1)
-          if (n_groups > off)
-#pragma unroll
-            for (uint32_t i = 0; i < off; ++i) v[i] += v[i + off];
-        double mine = v[0];
         if (k.att_mean) mine = (n & (n - 1)) == 0 ? mine * g.rc.inv_rays : mine / (double)n;
-        sh.S[lane] = lane == 0 || lane == 3 || lane == 5 ? mine + 1.0
-                     : lane >= 6 ? mine + sh.att[lane - 6] : mine;
+        if (lane == 0 || lane == 3 || lane == 5) mine += 1.0;
+        if (lane >= 6) mine += sh.att[lane - 6];
+        sh.S[lane] = mine;
       }
       __syncwarp();
       // A metric I + sum A_i with entries below 1e5 has full rank beyond doubt: its eigenvalues
@@ -3339,18 +3487,24 @@ __global__ void hash_build_kernel(const int32_t* __restrict__ keys, uint32_t n_b
 // A launch with programmatic serialisation (see wait_previous, which every kernel launched like
 // this calls).
 template <class... P, class... A>
-static cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned block,
-                                cudaStream_t stream, A... args) {
+static cudaError_t launch_after_shared(void (*kernel)(P...), unsigned grid, unsigned block,
+                                       size_t shared, cudaStream_t stream, A... args) {
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t c = {};
   c.gridDim = dim3(grid);
   c.blockDim = dim3(block);
+  c.dynamicSmemBytes = shared;
   c.stream = stream;
   c.attrs = &attr;
   c.numAttrs = 1;
   return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+template <class... P, class... A>
+static cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned block,
+                                cudaStream_t stream, A... args) {
+  return launch_after_shared(kernel, grid, block, 0, stream, args...);
 }
 
 // Every kernel variant of a map and reduction: f is called with <kind, layout, reduction, box
@@ -3419,6 +3573,23 @@ cudaError_t launch_batch(const DevMap& m, const EvalConsts& k, const double* sta
                          void* ws, rmp_result_t* out_dev, rmp_ray_hit_t* hits, float* per_ray,
                          int block, int grid, cudaStream_t stream, const double* goals_dev,
                          const RolloutArgs& step) {
+  if (!step.rs && state_per_cta(n_states, max_rays)) {
+    // warps a CTA: all of an SM's 32 for one state, fewer where CTAs share it and hide each
+    // other's serial steps; segments only while every state has its place (5000 states of 64 rays:
+    // 4 segments 149 us, 1 86), one warp left for the attractor (128 of 256 rays 19.9 -> 17.8)
+    const uint32_t most = n_states <= 152u ? 32u : (n_states <= 304u ? 16u : 8u);
+    const uint32_t lg = state_lg_segs(k, max_rays), parts = ((max_rays << 2) + 31) / 32;
+    const uint32_t hold = n_states <= 304u ? most - (goals_dev ? 1u : 0u) : 1u;
+    const uint32_t chunks = ((max_rays << cta_lg_segs(k, max_rays, lg, hold)) + 31) / 32;
+    const uint32_t warps = std::min(std::max(chunks + (goals_dev ? 1u : 0u), 2u), most);
+    for_map(m, k.reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
+      launch_after_shared(
+          raycast_state_kernel<kind.value, layout.value, red.value, boxes.value != 0>, n_states,
+          32 * warps, 4 * kPartWords * parts, stream, m, k, states_dev, n_rays_dev, max_rays,
+          out_dev, hits, per_ray, goals_dev, hold);
+    });
+    return cudaGetLastError();
+  }
   const BatchLayout L = batch_layout(n_states, max_rays);
   char* w = (char*)ws;
   BatchHeader* hdr = (BatchHeader*)w;
@@ -3444,11 +3615,9 @@ cudaError_t launch_rollout(const DevMap& m, const EvalConsts& k, const RolloutAr
   // at most 32 warps a CTA; 16 where two robots share an SM and hide each other's serial steps
   const uint32_t rays = g.rc.n_rays, most = n <= 152u ? 32u : 16u;
   const uint32_t lg = state_lg_segs(k, rays), parts = ((rays << lg) + 31) / 32;
-  // the most segments marched per ray whose chunks the warps hold at once beside the two of the
-  // attractor and the booking (8 robots of 256 rays: 4 segments, both on marching warps 18.3 us a
-  // step, 2 segments 15.8)
-  uint32_t lgs = lg;
-  while (lgs > 0 && ((rays << lgs) + 31) / 32 + 2 > most) --lgs;
+  // two warps left for the attractor and the booking where the chunks allow (8 robots of 256 rays:
+  // 4 segments, both on marching warps 18.3 us a step, 2 segments 15.8)
+  const uint32_t lgs = cta_lg_segs(k, rays, lg, most - 2);
   const uint32_t groups = (parts + kBatchGroup - 1) / kBatchGroup;
   const uint32_t warps = std::min(std::max(((rays << lgs) + 31) / 32 + 2, groups), most);   // >= 3
   const size_t dyn = 4 * (size_t)(((6 * rays + 3) & ~3u) + kPartWords * parts);

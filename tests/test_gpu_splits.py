@@ -2,7 +2,7 @@
 of 8, 16 and 32 states a CTA, ties and distances that FP32 cannot tell apart, coordinates past
 FP32; batches with more states than one run of the set-up kernel takes and with total loads on
 both sides of the march's segment cuts; scans whose last warp is ragged, with the per-point rows;
-rollouts with a CTA per robot."""
+batches with a CTA per state, rollouts with a CTA per robot."""
 from fractions import Fraction as F
 
 import numpy as np
@@ -137,6 +137,59 @@ def test_scan_rows_ragged(ctx, n):
     at = scan_abs_term(pts, sw.x, sw.xdot, sw.params)
     assert_per_ray_close(got[:n], por, at)
     assert_result_close(rg, ro, por, at)
+
+
+@pytest.mark.parametrize("n_states,red,lgs,cells", [(1, 0, -1, -1), (8, 1, -1, -1), (152, 0, -1, -1),
+                                                    (153, 0, 2, -1), (153, 1, 1, 0), (304, 0, 0, 0),
+                                                    (305, 0, -1, -1)])
+@pytest.mark.parametrize("dense", [True, False])
+def test_batch_cta_per_state(ctx, dense, n_states, red, lgs, cells):
+    """A CTA per state (max_rays 1024) and the packed chunks of the persistent grid (1025) give the
+    same records, rows and sums, for invalid states and states without rays too; likewise combined
+    with the attractor."""
+    torch = torch_cuda()
+    wl = W.dense_box_workload(n_states=6, jitter=True) if dense \
+        else W.hashed_workload(n_states=6, state_seed_index=52)
+    mid = ctx.upload(wl.map)
+    rng = np.random.default_rng(n_states)
+    states = np.stack([np.concatenate([wl.states[b % 6].x, wl.states[b % 6].xdot])
+                       for b in range(n_states)])
+    counts = rng.choice([0, 1, 2, 31, 32, 33, 64, 100, 255, 256, 257, 511, 777, 1023, 1024], n_states)
+    counts[0] = 1024
+    if n_states > 8:
+        states[3, 1], states[4, 0], states[5, 4] = np.nan, 1e9, np.nan
+        counts[6] = 1500                                  # more rays than max_rays
+    counts = counts.astype(np.uint32)
+    p = R.make_params(dict(wl.params, reduce_mode=red), wl.max_range)
+    R.rmp_tune_set(ctx.handle, R.RMP_TUNE_LG_SEGMENTS, lgs)
+    R.rmp_tune_set(ctx.handle, R.RMP_TUNE_CELL_SKIP, cells)
+    try:
+        a, ha, pa, _ = run_batch(ctx, mid, states, counts, p, max_rays=1024)
+        o, ho, po, _ = run_batch(ctx, mid, states, counts, p, max_rays=1025)
+        assert np.array_equal(ha, ho[:, :1024])
+        assert np.array_equal(pa, po[:, :1024], equal_nan=True)
+        for b in range(n_states):
+            for key, want in o[b].items():
+                assert np.array_equal(a[b][key], want, equal_nan=True), (b, key)
+        st, nr = torch.tensor(states, device="cuda"), torch.tensor(counts.astype(np.int32)).cuda()
+        gl = torch.tensor(states[:, :3] + rng.normal(size=(n_states, 3)), device="cuda")
+        for mean in (False, True):
+            got = []
+            for mr in (1024, 1025):
+                ws = torch.empty(R.rmp_batch_workspace_bytes(n_states, mr), dtype=torch.uint8,
+                                 device="cuda")
+                out = torch.empty((n_states, R.RESULT_BYTES), dtype=torch.uint8, device="cuda")
+                R.rmp_combined_eval_batch_async(ctx.handle, mid, st, nr, n_states, mr, p, gl, 10.0,
+                                                15.0, ws, out, metric_mean=mean)
+                got.append(out.cpu().numpy())
+            for b in range(n_states):
+                a, o = (R.result_from_bytes(g[b].tobytes()) for g in got)
+                for key, want in o.items():
+                    assert np.array_equal(a[key], want, equal_nan=True), (b, key)
+    finally:
+        R.rmp_tune_set(ctx.handle, R.RMP_TUNE_LG_SEGMENTS, -1)
+        R.rmp_tune_set(ctx.handle, R.RMP_TUNE_CELL_SKIP, -1)
+        R.rmp_map_release(ctx.handle, mid)
 
 
 def fma(a, b, c):
