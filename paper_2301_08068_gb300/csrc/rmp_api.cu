@@ -919,31 +919,32 @@ int rollout_impl(rmp_ctx* c, uint32_t map_id, const EsdfRec* esdf, const double*
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_rs, rs.data(), sizeof(RolloutDev) * n, cudaMemcpyHostToDevice, s);
   // steps in rounds; after each round the running count decides whether to go on (long ones where
-  // a round is one launch and every robot has an SM: its own end is then all that ends a CTA)
-  const uint32_t kRound = resident && n <= 304 ? 256 : 32;
+  // a round is one launch and the robots fill the SMs at most about once: a CTA then ends with its
+  // robots)
+  const bool fused = esdf || resident;
+  const uint32_t kRound = fused && n <= (esdf ? 1216u : 304u) ? 256 : 32;
   uint32_t running = n;
   for (uint32_t step = 0; e == cudaSuccess && status == RMP_OK && running > 0 &&
                           step < rp->max_steps;) {
+    const uint32_t most = std::min(kRound, rp->max_steps - step);
     e = cudaMemsetAsync(d_cnt, 0, 4, s);
-    if (resident && e == cudaSuccess) {
-      const uint32_t most = std::min(kRound, rp->max_steps - step);
+    if (e != cudaSuccess) break;
+    if (esdf) {
+      args.running = nullptr;
+      e = launch_esdf_rollout(esdf->prims, esdf->prims32, esdf->n, ek, dm, args, n, most, d_res,
+                              d_cnt, s);
+    } else if (resident) {
       args.running = d_cnt;
       e = launch_rollout(dm, k, args, n, most, s);
-      step += most;
     }
-    for (uint32_t i = 0; !resident && i < kRound && step < rp->max_steps && e == cudaSuccess; ++i, ++step) {
-      args.running = i + 1 == kRound || step + 1 == rp->max_steps ? d_cnt : nullptr;
-      if (esdf) {
-        e = launch_esdf_eval(esdf->prims, esdf->prims32, esdf->n, ek, d_st, d_goal, n, d_res, nullptr,
-                             s);
-        if (e == cudaSuccess) e = launch_rollout_step(dm, args, d_res, n, s);
-      } else {                                      // the evaluation takes the step as well
-        status = batch_async_impl(c, map_id, d_st, d_nr, n, rp->n_rays, params, buf + o_ws, wsb,
-                                  stream, d_res, nullptr, nullptr, d_goal, rp->alpha, rp->beta,
-                                  (int)rp->metric_mean, args);
-        if (status != RMP_OK) break;
-      }
+    for (uint32_t i = 0; !fused && i < most && e == cudaSuccess; ++i) {
+      args.running = i + 1 == most ? d_cnt : nullptr;
+      status = batch_async_impl(c, map_id, d_st, d_nr, n, rp->n_rays, params, buf + o_ws, wsb,
+                                stream, d_res, nullptr, nullptr, d_goal, rp->alpha, rp->beta,
+                                (int)rp->metric_mean, args);
+      if (status != RMP_OK) break;
     }
+    step += most;
     if (e == cudaSuccess && status == RMP_OK) {
       e = cudaMemcpyAsync(&running, d_cnt, 4, cudaMemcpyDeviceToHost, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);

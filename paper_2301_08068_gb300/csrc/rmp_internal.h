@@ -259,9 +259,11 @@ cudaError_t launch_esdf_eval(const rmp_primitive_t* prims, const float4* prims32
 // Up to `steps` control steps of the rollouts, a CTA per robot (see rollout_resident).
 cudaError_t launch_rollout(const DevMap& m, const EvalConsts& k, const RolloutArgs& g, uint32_t n,
                            uint32_t steps, cudaStream_t stream);
-// One control step of every robot from its evaluation in res.
-cudaError_t launch_rollout_step(const DevMap& m, const RolloutArgs& step, const rmp_result_t* res,
-                                uint32_t n, cudaStream_t stream);
+// Up to `steps` control steps with the ESDF policy; `running` counts the robots that still run.
+cudaError_t launch_esdf_rollout(const rmp_primitive_t* prims, const float4* prims32,
+                                uint32_t n_prims, const EsdfConsts& k, const DevMap& m,
+                                const RolloutArgs& g, uint32_t n, uint32_t steps,
+                                rmp_result_t* res, uint32_t* running, cudaStream_t stream);
 cudaError_t launch_scan(const float* pts, const EvalConsts& k, const double* state_dev,
                         void* ws, rmp_result_t* out_dev, float* per_ray, int block, int grid,
                         cudaStream_t stream);

@@ -1970,24 +1970,6 @@ __device__ __forceinline__ void rollout_fail(const RolloutArgs& g, uint32_t b) {
   g.n_rays[b] = 0;
 }
 
-// The control steps as a launch of their own (the ESDF policy's closed loop), a warp per robot.
-template <int KIND, int LAYOUT>
-__global__ void __launch_bounds__(256) rollout_step_kernel(
-    const __grid_constant__ DevMap m, const __grid_constant__ RolloutArgs g,
-    const rmp_result_t* __restrict__ res, uint32_t n) {
-  const uint32_t b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  wait_previous();
-  launch_next();
-  if (b >= n) return;
-  if (g.rs[b].status != RMP_ROLLOUT_RUNNING) {
-    if (lane == 0) g.n_rays[b] = 0;
-  } else if (res[b].status != RMP_OK) {
-    if (lane == 0) rollout_fail(g, b);
-  } else {
-    rollout_step<KIND, LAYOUT>(m, g, b, res[b].f[lane < 3 ? lane : 0]);
-  }
-}
-
 // The last chunk of a group sums the group's partials into a group partial; the last group
 // of a state sums the state's groups, adds the attractor (combined evaluations) and
 // resolves.  Called by all 32 lanes of the warp whose chunk completed the group.  Kept
@@ -2724,13 +2706,18 @@ __device__ __forceinline__ float key_float(uint32_t k) {
 // four CTAs an SM (64 registers), so that 16384 states are one wave (three: 48 us).  16384 states,
 // 200 primitives: 33.6 us (one warp per state, every distance in FP64, policy in one lane: 638);
 // 128 states 16 (51).
-__global__ void __launch_bounds__(256, 4) esdf_eval_kernel(const rmp_primitive_t* __restrict__ prims,
-                                                        const float4* __restrict__ prims32,
-                                                        uint32_t n_prims, EsdfConsts k,
-                                                        const double* __restrict__ states,
-                                                        const double* __restrict__ goals,
-                                                        uint32_t n_states, uint32_t G,
-                                                        rmp_result_t* out, double* query) {
+//
+// ROLL: a closed loop.  The CTA takes its robots (g, in place of states and goals) through `steps`
+// control steps on map m, one evaluation and a warp per robot for the step each time, while any of
+// them runs; `running` counts those that still do.  128 robots, 24 steps, the call: 797 us (two launches a
+// step: 917).
+template <bool ROLL, int KIND, int LAYOUT>
+__global__ void __launch_bounds__(256, 4) esdf_eval_kernel(
+    const rmp_primitive_t* __restrict__ prims, const float4* __restrict__ prims32, uint32_t n_prims,
+    EsdfConsts k, const double* __restrict__ states_in, const double* __restrict__ goals_in,
+    uint32_t n_states, uint32_t G, rmp_result_t* out, double* query,
+    const __grid_constant__ DevMap m, const __grid_constant__ RolloutArgs g_roll, uint32_t steps,
+    uint32_t* running) {
   __shared__ uint32_t near_sh[32], act_sh[32];
   __shared__ bool bad_sh[32];
   __shared__ double P[7][32], att[3][32], fa[3][32], lam_sh[3][32];
@@ -2739,8 +2726,11 @@ __global__ void __launch_bounds__(256, 4) esdf_eval_kernel(const rmp_primitive_t
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t role = (warp + blockIdx.x + blockIdx.x / 152u) & 7u;
   constexpr uint32_t kNone = 0xffffffffu;
+  // a rollout's states change from step to step
+  const double* states = ROLL ? g_roll.states : states_in;
+  const double* goals = ROLL ? g_roll.goals : goals_in;
   wait_previous();
-  for (uint32_t base = blockIdx.x * G; base < n_states; base += gridDim.x * G) {
+  for (uint32_t base = blockIdx.x * G, step = 0; base < n_states;) {
     for (uint32_t s = warp; s < G && base + s < n_states; s += 8) {
       const double* st = states + 6 * (size_t)(base + s);
       // one component a lane: a single FP64 conversion for all of them
@@ -2867,7 +2857,7 @@ __global__ void __launch_bounds__(256, 4) esdf_eval_kernel(const rmp_primitive_t
       att[2][lane] = k.alpha * (e2 / hh) - k.beta * st[5];
     }
     __syncthreads();
-    if (base + gridDim.x * G >= n_states) launch_next();   // the CTA's last states
+    if (!ROLL && base + gridDim.x * G >= n_states) launch_next();   // the CTA's last states
     // the sums, in the warps that need them: A = w sc^2 r r^T, f = (f_rep + z) r
     double tv[9];
     const bool bad = mine && bad_sh[lane];
@@ -2944,6 +2934,25 @@ __global__ void __launch_bounds__(256, 4) esdf_eval_kernel(const rmp_primitive_t
       out[b] = r;
     }
     __syncthreads();                                       // the next tile reuses the arrays
+    if constexpr (!ROLL) {
+      base += gridDim.x * G;
+    } else {
+      bool runs = false;
+      for (uint32_t s = warp; s < G && base + s < n_states; s += 8) {
+        const uint32_t r = base + s;
+        if (g_roll.rs[r].status != RMP_ROLLOUT_RUNNING) continue;
+        if (out[r].status != RMP_OK) {
+          if (lane == 0) rollout_fail(g_roll, r);
+        } else {
+          rollout_step<KIND, LAYOUT>(m, g_roll, r, out[r].f[lane < 3 ? lane : 0]);
+        }
+        __syncwarp();
+        const bool goes = g_roll.rs[r].status == RMP_ROLLOUT_RUNNING;
+        runs = runs || goes;
+        if (step + 1 == steps && goes && lane == 0) atomicAdd(running, 1u);
+      }
+      if (!__syncthreads_or(runs) || ++step == steps) break;
+    }
   }
 }
 
@@ -3630,24 +3639,17 @@ cudaError_t launch_rollout(const DevMap& m, const EvalConsts& k, const RolloutAr
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_rollout_step(const DevMap& m, const RolloutArgs& step, const rmp_result_t* res,
-                                uint32_t n, cudaStream_t stream) {
-  const unsigned grid = (n + 7) / 8;
-  if (m.kind == RMP_MAP_DENSE_U8)
-    launch_after(rollout_step_kernel<RMP_MAP_DENSE_U8, kLayoutGrid>, grid, 256, stream, m, step, res, n);
-  else if (m.layout == kLayoutGrid)
-    launch_after(rollout_step_kernel<RMP_MAP_HASHED_TSDF, kLayoutGrid>, grid, 256, stream, m, step,
-                 res, n);
-  else
-    launch_after(rollout_step_kernel<RMP_MAP_HASHED_TSDF, kLayoutHash>, grid, 256, stream, m, step,
-                 res, n);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_probe_l2(const uint4* buf, size_t n16, uint32_t passes, int grid,
                             uint64_t* checksum, cudaStream_t stream) {
   probe_l2_kernel<<<grid, 512, 0, stream>>>(buf, n16, passes, checksum);
   return cudaGetLastError();
+}
+
+// As few states a CTA as give one CTA an SM: few states wait for latency; beyond, 32, where the
+// FP64 steps fill their lanes (1217 states: 8 a CTA 20.1 us, 16 18.0, 32 20.5; 2432 states: 22.3,
+// 18.2, 20.5).
+static uint32_t esdf_states_per_cta(uint32_t n) {
+  return n <= 8u * 152u ? 8u : (n <= 16u * 152u ? 16u : 32u);
 }
 
 cudaError_t launch_esdf_eval(const rmp_primitive_t* prims, const float4* prims32,
@@ -3655,14 +3657,28 @@ cudaError_t launch_esdf_eval(const rmp_primitive_t* prims, const float4* prims32
                              const double* goals, uint32_t n_states, rmp_result_t* out,
                              double* query, cudaStream_t stream) {
   if (n_states == 0) return cudaSuccess;
-  // as few states a CTA as give one CTA an SM: few states wait for latency; beyond, 32, where the
-  // FP64 steps fill their lanes (1217 states: 8 a CTA 20.1 us, 16 18.0, 32 20.5; 2432 states:
-  // 22.3, 18.2, 20.5)
-  const uint32_t G = n_states <= 8u * 152u ? 8u : (n_states <= 16u * 152u ? 16u : 32u);
+  const uint32_t G = esdf_states_per_cta(n_states);
   uint32_t grid = (n_states + G - 1) / G;
   if (grid > 65535) grid = 65535;                   // CTA-stride beyond
-  launch_after(esdf_eval_kernel, grid, 256, stream, prims, prims32, n_prims, k, states, goals,
-               n_states, G, out, query);
+  launch_after(esdf_eval_kernel<false, 0, 0>, grid, 256, stream, prims, prims32, n_prims, k, states,
+               goals, n_states, G, out, query, DevMap(), RolloutArgs(), 0u, (uint32_t*)nullptr);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_esdf_rollout(const rmp_primitive_t* prims, const float4* prims32,
+                                uint32_t n_prims, const EsdfConsts& k, const DevMap& m,
+                                const RolloutArgs& g, uint32_t n, uint32_t steps,
+                                rmp_result_t* res, uint32_t* running, cudaStream_t stream) {
+  const uint32_t G = esdf_states_per_cta(n), grid = (n + G - 1) / G;
+  const double* none = nullptr;
+  double* query = nullptr;
+  auto run = [&](auto kernel) {
+    launch_after(kernel, grid, 256, stream, prims, prims32, n_prims, k, none, none, n, G, res, query,
+                 m, g, steps, running);
+  };
+  if (m.kind == RMP_MAP_DENSE_U8) run(esdf_eval_kernel<true, RMP_MAP_DENSE_U8, kLayoutGrid>);
+  else if (m.layout == kLayoutGrid) run(esdf_eval_kernel<true, RMP_MAP_HASHED_TSDF, kLayoutGrid>);
+  else run(esdf_eval_kernel<true, RMP_MAP_HASHED_TSDF, kLayoutHash>);
   return cudaGetLastError();
 }
 

@@ -250,3 +250,29 @@ def test_rollout_cta_per_robot(ctx, dense, rays, mean, red, lgs, steps):
     finally:
         R.rmp_tune_set(ctx.handle, R.RMP_TUNE_LG_SEGMENTS, -1)
         R.rmp_map_release(ctx.handle, mid)
+
+
+@pytest.mark.parametrize("n", [1, 9, 1217, 2433])
+def test_esdf_rollout_states_per_cta(ctx, n):
+    """8, 16 and 32 robots a CTA: each robot's path is the one it has among few, robots that stop
+    early and an invalid one beside it."""
+    wl = W.hashed_workload(n_states=6, state_seed_index=52)
+    _, prims = scene(40)
+    rng = np.random.default_rng(5)
+    robots = np.concatenate([rng.uniform(0.5, 9.5, (12, 3)), rng.normal(0.0, 1.0, (12, 3)),
+                             rng.uniform(0.5, 9.5, (12, 3))], 1)
+    robots[1, 6:] = robots[1, :3] + 1e-4                  # at its goal
+    robots[2, 0] = np.nan
+    mid, eid = ctx.upload(wl.map), R.rmp_esdf_upload(ctx.handle, prims)
+    p = R.make_params(wl.params, wl.max_range)
+    rp = R.rollout_params(10.0, 15.0, 0.01, 0.05, 45, 4, 1)
+    try:
+        one = [R.rmp_rollout_esdf(ctx.handle, mid, eid, robots[b:b + 1], p, rp)[0] for b in range(12)]
+        got = R.rmp_rollout_esdf(ctx.handle, mid, eid, np.tile(robots, (n // 12 + 1, 1))[:n], p, rp)
+        for b in range(n):
+            for key, want in one[b % 12].items():
+                assert np.array_equal(got[b][key], want, equal_nan=True), (b, key)
+        assert one[1]["steps"] == 1 and one[2]["status"] == R.RMP_ROLLOUT_FAILED
+    finally:
+        R.rmp_map_release(ctx.handle, mid)
+        R.rmp_esdf_release(ctx.handle, eid)
