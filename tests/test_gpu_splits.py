@@ -276,3 +276,39 @@ def test_esdf_rollout_states_per_cta(ctx, n):
     finally:
         R.rmp_map_release(ctx.handle, mid)
         R.rmp_esdf_release(ctx.handle, eid)
+
+
+def test_map_memory_reused(ctx):
+    """Maps uploaded and released in turn by several threads, each on a stream of its own: the
+    memory one gives back serves another, and every evaluation is the one of a fresh context."""
+    import threading
+    torch = torch_cuda()
+    wls = [W.dense_box_workload(n_states=1, jitter=True), W.hashed_workload(n_states=1, state_seed_index=52)]
+    want = []
+    for wl in wls:
+        c = R.Context(0)
+        s = wl.states[0]
+        want.append(R.rmp_raycast_eval(c.handle, c.upload(wl.map), s.x, s.xdot, 2000,
+                                       R.make_params(wl.params, wl.max_range)))
+        c.close()
+    bad = []
+
+    def work(i):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            for j in range(6):
+                wl, w = wls[(i + j) % 2], want[(i + j) % 2]
+                mid = ctx.upload(wl.map)
+                s = wl.states[0]
+                got = R.rmp_raycast_eval(ctx.handle, mid, s.x, s.xdot, 2000,
+                                         R.make_params(wl.params, wl.max_range))
+                R.rmp_map_release(ctx.handle, mid)
+                if any(not np.array_equal(got[k], w[k]) for k in w):
+                    bad.append((i, j))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
