@@ -370,8 +370,8 @@ __device__ __forceinline__ uint32_t block_entry(const DevMap& m, const uint32_t*
 // exit axis by exact 64-bit comparisons, the crossing counts of the other two axes) with two
 // dependent loads; the field's lines stay in L1, which holds all of the SM's 228 KB since
 // nothing is staged in shared memory.  Measured against a march over symmetric free boxes of
-// blocks with a voxel walk inside occupied blocks: 65536 rays on the 40 m map 54 -> 20 us,
-// 262144 rays on the 100 m map 101.6 -> 33 us.
+// blocks with a voxel walk inside occupied blocks: 65536 rays on the 40 m map 54 -> 15.2 us,
+// 262144 rays on the 100 m map 101.6 -> 27.7 us (whole evaluations, later changes included).
 template <int KIND, int LAYOUT, bool BOXES>
 __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const RayFx& r,
                                          const uint32_t L[3], int at_limit, bool work) {
@@ -1625,8 +1625,8 @@ __host__ __device__ __forceinline__ uint32_t state_lg_segs(const EvalConsts& k, 
 // Segments marched per ray (log2), at most the summation's: a tuned launch marches those, the
 // default the most whose threads fill half of the persistent launch over the whole batch of
 // `total` rays -- beyond that, the extra segments' set-up costs more than their shorter chains
-// save (256 states, 5.3 M rays: 1 / 2 / 4 segments 458 / 745 / 1252 us; 16 states, 50 k rays: 36 /
-// 38 / 50; one state of 16384: 44 / 37 / 35).
+// save (256 states of 20000 rays: 1 / 2 / 4 segments 365 / 598 / 1006 us; 16 of 3125: 29.8 / 28.7 /
+// 40.6; one of 16384: 25.1 / 23.5 / 24.2).
 __device__ __forceinline__ uint32_t march_lg_segs(const EvalConsts& k, uint32_t lg_sum,
                                                   unsigned long long total) {
   if (k.lg_segs <= 2u) return lg_sum;
@@ -2265,7 +2265,8 @@ __device__ __forceinline__ void state_chunk(const DevMap& m, const EvalConsts& k
 
 // s + c of an FP32 pair in FP64.  A normal value is widened by integer instructions (an FP64
 // conversion holds the pipe about 64 cycles); the rare others by the conversion.  For a CTA whose
-// other warps wait; where they march the integers cost more (batches of 64 x 4096 rays 72 -> 73.5 us).
+// other warps wait; where they march the integers cost more (64 states of 4096 rays packed 72 ->
+// 73.5 us).
 __device__ __forceinline__ double pair_sum(float s, float c) {
   auto plain = [](float f) {                        // zero or normal
     const uint32_t b = __float_as_uint(f) << 1;
@@ -2709,8 +2710,8 @@ __device__ __forceinline__ float key_float(uint32_t k) {
 //
 // ROLL: a closed loop.  The CTA takes its robots (g, in place of states and goals) through `steps`
 // control steps on map m, one evaluation and a warp per robot for the step each time, while any of
-// them runs; `running` counts those that still do.  128 robots, 24 steps, the call: 797 us (two launches a
-// step: 917).
+// them runs; `running` counts those that still do.  128 robots, 24 steps, the call: 797 us (two
+// launches a step: 917).
 template <bool ROLL, int KIND, int LAYOUT>
 __global__ void __launch_bounds__(256, 4) esdf_eval_kernel(
     const rmp_primitive_t* __restrict__ prims, const float4* __restrict__ prims32, uint32_t n_prims,

@@ -46,11 +46,12 @@ inline void pick_ray_cells(uint32_t n, EvalConsts* k) {
 // Segments per ray of a single-state evaluation left to the library: as many (up to 32,
 // kMaxSingleLgSegs) as keep the launch within one wave of 256-thread CTAs (`wave256`
 // threads), since the evaluation lasts as long as its longest ray's serial march and
-// segments shorten it while the extra threads still find free SMs (measured, L2 flushed:
-// hashed map 1024 rays 33.0 / 26.6 / 22.0 / 19.9 us with 4 / 8 / 16 / 32 segments, 4096
-// rays 33.5 / 26.7 / 23.7; dense 1024 rays 26.4 / 21.8 / 19.3 / 18.3; 16384 rays 54.3 us with 2 segments,
-// 47.1 with 4; 32768 rays 65.5 with 1, 57.2 with 2; 65536 rays best with 1).  Without a
-// wave size (0) the ray-count rule of make_consts stays.
+// segments shorten it while the extra threads still find free SMs (measured, device time, hashed
+// 40 m map: 1024 rays 14.3 / 11.2 / 10.1 / 9.4 / 9.3 us with 1 / 4 / 8 / 16 / 32 segments, 4096
+// rays 14.6 / 11.1 / 10.6 / 10.1 with 1 / 4 / 8 / 16, 16384 rays 13.9 / 13.0 / 12.1 with 1 / 2 / 4,
+// 32768 rays 14.4 / 13.7 with 1 / 2, 65536 rays, past one wave with 2, 15.0 / 19.3; dense 64^3 map
+// 1024 rays 11.0 / 9.8 / 9.4 / 8.9 / 9.1).  Without a wave size (0) the ray-count rule of
+// make_consts stays.
 constexpr uint32_t kMaxSingleLgSegs = 5;
 inline void auto_segments(const Tuning& t, uint32_t n, uint64_t wave256, EvalConsts* k) {
   if (t.lg_segs >= 0 || wave256 == 0) return;
@@ -68,9 +69,10 @@ inline void single_state_cells(int tune_cells, const EvalConsts& k, DevMap* dm) 
 }
 
 // n_threads: rays (or points) times segments per ray.  Threads per CTA: the tuned value, or
-// (automatic) 256 when the whole launch fits in one wave of 256-thread CTAs (`wave256`
-// threads; fewer CTAs stage the radius field and store partials: 65536 rays 69.7 -> 68.1 us
-// hashed, 46.3 -> 43.8 us dense) and 128 otherwise (262144 rays: 132 against 135 us).
+// (automatic) 256 when the whole launch fits in one wave of 256-thread CTAs (`wave256` threads:
+// fewer CTA partials, and more registers for its slowest warps: 65536 rays 15.0 us, 17.3 with
+// 128) and 128 otherwise, held to fewer registers so that more warps fit an SM (262144 rays on the
+// 40 m map 27.8 us, 31.2 with 256; on the 100 m map 28.0 and 31.8).
 inline void launch_shape(const Tuning& t, uint64_t n_threads, uint64_t wave256, int* block,
                   int* grid) {
   int b = t.block;
@@ -84,8 +86,8 @@ inline void launch_shape(const Tuning& t, uint64_t n_threads, uint64_t wave256, 
 
 // Scans: threads per CTA the tuned value or (automatic) 256, and at most 512 threads per
 // SM, each thread striding over several points, so that large scans are reduced from few
-// CTA partials (measured, L2 flushed: 4096 / 65536 / 262144 points 16.4 / 20.5 / 24.3 us
-// with 128-thread CTAs and 4 per SM, 14.4 / 18.5 / 21.0 us with 256 and 2 per SM).
+// CTA partials (measured, device time: 4096 / 65536 / 262144 points 5.7 / 8.1 / 9.7 us with
+// 128-thread CTAs and 4 per SM, 5.7 / 6.3 / 8.1 us with 256 and 2 per SM).
 inline void scan_shape(const Tuning& t, int sm_count, uint64_t n, int* block, int* grid) {
   const int b = t.block != 0 ? t.block : 256;
   const uint64_t cap = (uint64_t)(512 / b) * (uint64_t)(sm_count > 0 ? sm_count : 1);
