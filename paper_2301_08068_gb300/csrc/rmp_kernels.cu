@@ -381,7 +381,9 @@ __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const 
   const float rA[3] = {recip_fast(__uint2float_rn(A[0])), recip_fast(__uint2float_rn(A[1])),
                        recip_fast(__uint2float_rn(A[2]))};
   int hi[3];                                        // first voxel beyond the map / the grid
-  uint32_t H[3];                                    // dense: N of the map's far faces
+  // dense: N of the map's far faces, or, for a face farther than any range, of a voxel in between
+  // that no crossing within L reaches (L is at most 2^30, H stays below 2^32)
+  uint32_t H[3];
   int step[4] = {0, 0, 0, 0};                       // signed brick strides and the first brick
   const uint32_t* top = m.top;
   int status = at_limit;
@@ -392,7 +394,7 @@ __device__ __forceinline__ int march_run(const DevMap& m, MarchState& st, const 
     for (int a = 0; a < 3; ++a) {
       const bool up = (r.up >> a) & 1u;
       hi[a] = (KIND == RMP_MAP_DENSE_U8 && up) ? m.dims[a] : 8 * m.gdim[a];
-      H[a] = N[a] + ((uint32_t)(hi[a] - 1 - q[a]) << 16);
+      H[a] = N[a] + ((uint32_t)min(hi[a] - 1 - q[a], 2 * kMaxRangeVoxels - 1) << 16);
       step[a] = up ? str[a] : -str[a];
       step[3] += up ? 0 : (m.gdim[a] - 1) * str[a];
       // a dense map: a piece that starts outside has left the map

@@ -75,3 +75,22 @@ def test_empty_hashed_map(ctx):
     keys = np.array([[0, 0, 0], [3, -2, 1]], np.int32)
     tsdf = np.full((2, 512), 0.2, np.float32)
     check(ctx, W.HashedMap(keys, tsdf, VS), [np.zeros(3), np.array([5.0, -5.0, 5.0])], 100, 20.0)
+
+
+@pytest.mark.parametrize("axis,size", [(0, 66000), (1, 65600), (2, 70001)])
+def test_dense_long_axis(ctx, axis, size):
+    """More than 65535 voxels ahead on one axis, where the far face's crossing no longer fits 32
+    bits (2^16 a voxel): states near both ends and 65535 to 65540 voxels before either face, among
+    obstacles a few voxels away."""
+    dims = [9, 10, 9]
+    dims[axis] = size
+    rng = np.random.default_rng(size)
+    occ = (rng.uniform(size=dims[::-1]) < 0.01).astype(np.uint8)
+    xs = []
+    for k in (2, 65536, 65537, 65539, 65541, size - 1 - 65535, size - 1 - 65536, size - 1 - 65539,
+              size - 3):
+        c = np.array([4, 4, 4])
+        c[axis] = min(max(k, 0), size - 1)
+        occ[tuple(c[::-1])] = 0
+        xs.append((c + 0.5) * VS)
+    check(ctx, W.DenseMap(occ, VS, np.zeros(3)), xs, 333, 4.0)
