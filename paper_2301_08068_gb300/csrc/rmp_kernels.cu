@@ -3622,6 +3622,11 @@ cudaError_t launch_batch(const DevMap& m, const EvalConsts& k, const double* sta
   return cudaGetLastError();
 }
 
+// Shared memory of a resident rollout: directions and partials.
+static size_t rollout_shared(uint32_t rays, uint32_t parts) {
+  return 4 * (size_t)(((6 * rays + 3) & ~3u) + kPartWords * parts);
+}
+
 cudaError_t launch_rollout(const DevMap& m, const EvalConsts& k, const RolloutArgs& g, uint32_t n,
                            uint32_t steps, cudaStream_t stream) {
   // at most 32 warps a CTA; 16 where two robots share an SM and hide each other's serial steps
@@ -3632,11 +3637,14 @@ cudaError_t launch_rollout(const DevMap& m, const EvalConsts& k, const RolloutAr
   const uint32_t lgs = cta_lg_segs(k, rays, lg, most - 2);
   const uint32_t groups = (parts + kBatchGroup - 1) / kBatchGroup;
   const uint32_t warps = std::min(std::max(((rays << lgs) + 31) / 32 + 2, groups), most);   // >= 3
-  const size_t dyn = 4 * (size_t)(((6 * rays + 3) & ~3u) + kPartWords * parts);
+  const size_t dyn = rollout_shared(rays, parts);
+  // the limit belongs to the kernel, whichever thread or context launches it: every call sets the
+  // same one, the most that any may want, so that none lowers it under another's launch
+  const int limit = (int)rollout_shared(kStateRays, kStateGroups * kBatchGroup);
   cudaError_t e = cudaSuccess;
   for_map(m, k.reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
     const auto f = rollout_kernel<kind.value, layout.value, red.value, boxes.value != 0>;
-    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
     if (e == cudaSuccess) f<<<n, 32 * warps, dyn, stream>>>(m, k, g, rays, lg, lgs, steps);
   });
   return e != cudaSuccess ? e : cudaGetLastError();

@@ -312,3 +312,50 @@ def test_map_memory_reused(ctx):
     for t in threads:
         t.join()
     assert not bad
+
+
+@pytest.mark.parametrize("contexts", [1, 2])
+def test_rollouts_from_several_threads(ctx, contexts):
+    """Rollouts of 2000 rays, whose CTAs want 66 KB of shared memory, while three other threads keep
+    asking for rollouts of 16 rays, on one context and on two: every call succeeds and gives
+    what it gives alone."""
+    import ctypes as C
+    import threading
+    wl = W.hashed_workload(n_states=32, state_seed_index=52)
+    p = R.make_params(wl.params, wl.max_range)
+    robots = np.stack([np.concatenate([s.x, s.xdot, s.x + 3.0]) for s in wl.states])
+    other = R.Context(0) if contexts == 2 else ctx
+    rp = [R.rollout_params(10.0, 15.0, 0.01, 0.05, 1, 1, rays) for rays in (2000, 16)]
+    jobs = [(ctx, ctx.upload(wl.map), 32, rp[0]), (other, other.upload(wl.map), 1, rp[1])]
+    fn = R.lib().rmp_rollout
+
+    def call(i):
+        c, mid, n, r = jobs[i]
+        out = (R.rmp_rollout_result_t * n)()
+        st = fn(c.handle, mid, robots.ctypes.data, n, C.byref(p), C.byref(r), None, out)
+        return st, bytes(out)
+
+    want = [call(0), call(1)]
+    assert want[0][0] == 0 and want[1][0] == 0
+    bad, done = [], threading.Event()
+
+    def work(i):
+        if i == 0:
+            bad.extend(g[0] for g in (call(0) for _ in range(1500)) if g != want[0])
+            done.set()
+        else:
+            while not done.is_set():
+                g = call(1)
+                if g != want[1]:
+                    bad.append(g[0])
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for c, mid, _, _ in jobs:
+        R.rmp_map_release(c.handle, mid)
+    if contexts == 2:
+        other.close()
+    assert not bad, (len(bad), bad[:3])
