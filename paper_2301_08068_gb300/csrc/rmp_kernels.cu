@@ -161,6 +161,11 @@ __device__ __forceinline__ Ray make_ray(uint32_t i) {
 // call at the start the ESDF policy of 4096 states took 27 us for 23).  The order of effects is
 // the stream's; what overlaps is the launch itself and work on parameters alone: back to back,
 // 1024 rays 12.4 -> 9.8 us, a batch of one state 26.5 -> 21.7 us.
+// Such a kernel is resident while its predecessor still writes, so what a launch can write --
+// states, counts, points, set-up records -- is read by plain loads only: the read-only path
+// (__ldg, const __restrict__ parameters) is for data that does not change while the kernel runs,
+// and its loads may be moved above the wait.  Maps and primitives stay on it: an upload is
+// complete before any launch that uses it.
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void launch_next() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1493,7 +1498,7 @@ __device__ __forceinline__ bool ray_outputs(const DevMap& m, const EvalConsts& k
 // larger launches, which keep every SM busy: 262144 rays on the 100 m map 30.0 -> 27.7 us.
 template <int KIND, int LAYOUT, int RED, bool BOXES, int BLOCK, int CTAS>
 __global__ void __launch_bounds__(BLOCK, CTAS) raycast_rmp_kernel(
-    DevMap m, EvalConsts k, const double* __restrict__ state, WsHeader* ws, CtaPartial* parts,
+    DevMap m, EvalConsts k, const double* state, WsHeader* ws, CtaPartial* parts,
     rmp_result_t* out, rmp_ray_hit_t* hits, float* per_ray) {
   __shared__ CtaState cs;
   // state component of this thread: x on threads 0-2, xdot on threads 32-34 (another warp,
@@ -1658,7 +1663,7 @@ __device__ __forceinline__ uint32_t block_sum256(uint32_t x, uint32_t* sh) {
 // Bound by one state's latency: 7.3 us for 256 states (one CTA with 8 states a warp, and cells
 // picked with divisions: 46 us).
 __global__ void __launch_bounds__(256) batch_prep_kernel(
-    const double* __restrict__ states, const uint32_t* __restrict__ n_rays, uint32_t n_states,
+    const double* states, const uint32_t* n_rays, uint32_t n_states,
     uint32_t max_rays, DevMap m, EvalConsts k, BatchHeader* hdr, BatchState* bs,
     uint32_t* sticket, uint32_t* gticket, rmp_result_t* out) {
   __shared__ uint32_t sh[8], scan[3][8];
@@ -2074,7 +2079,7 @@ __device__ __noinline__ void batch_group_finish(const DevMap& m, const EvalConst
 // per-state values used only after the march are read after it.
 template <int KIND, int LAYOUT, int RED, bool BOXES>
 __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
-    const __grid_constant__ DevMap m, const __grid_constant__ EvalConsts k, BatchHeader* hdr, const BatchState* __restrict__ bs,
+    const __grid_constant__ DevMap m, const __grid_constant__ EvalConsts k, BatchHeader* hdr, const BatchState* bs,
     uint32_t* sticket, uint32_t* gticket, CtaPartial* cparts, CtaPartial* gparts,
     rmp_result_t* out, rmp_ray_hit_t* hits, float* per_ray, uint32_t max_rays,
     const double* states, const double* goals, const __grid_constant__ RolloutArgs step) {
@@ -2096,26 +2101,26 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
     uint32_t lo = 0, len = nst;
     while (len > 1) {
       const uint32_t by = (len + 31) / 32, at = lo + lane * by;
-      const bool le = lane * by < len && __ldg(&bs[at].work0) <= c;   // true for lane 0
+      const bool le = lane * by < len && bs[at].work0 <= c;   // true for lane 0
       const uint32_t last = 31 - __clz(__ballot_sync(0xffffffffu, le));
       lo += last * by;
       len = min(by, len - last * by);
     }
     const uint32_t b = lo;
     const BatchState* sp = bs + b;
-    if (__ldg(&sp->status) != RMP_OK) {              // its result is the prep kernel's
-      if (step.rs && lane == 0 && c == __ldg(&sp->work0)) rollout_fail(step, b);
+    if (sp->status != RMP_OK) {              // its result is the prep kernel's
+      if (step.rs && lane == 0 && c == sp->work0) rollout_fail(step, b);
       c = __shfl_sync(0xffffffffu, cn, 0);
       continue;
     }
-    const long long P[3] = {__ldg(&sp->P[0]), __ldg(&sp->P[1]), __ldg(&sp->P[2])};
-    const uint32_t n_b = __ldg(&sp->n_rays);
-    const uint32_t q = c - __ldg(&sp->work0);
-    const uint32_t lgs = __ldg(&sp->lg_segs) >> 8, S = 1u << lgs;
+    const long long P[3] = {sp->P[0], sp->P[1], sp->P[2]};
+    const uint32_t n_b = sp->n_rays;
+    const uint32_t q = c - sp->work0;
+    const uint32_t lgs = sp->lg_segs >> 8, S = 1u << lgs;
     const uint32_t g = q * 32 + lane;
     const uint32_t slot = g >> lgs, seg = g & (S - 1);
     const bool active = slot < n_b;
-    const uint32_t pM = __ldg(&sp->perm_M), pQ = __ldg(&sp->perm_Q);
+    const uint32_t pM = sp->perm_M, pQ = sp->perm_Q;
     const uint32_t ray_idx = ray_of_slot(active ? slot : 0, pM, pQ, n_b - pQ * pM);
     const Ray ray = make_ray<true>(ray_idx + k.halton_offset);
     const size_t ro = (size_t)b * max_rays + ray_idx;
@@ -2123,10 +2128,10 @@ __global__ void __launch_bounds__(256, 4) raycast_batch_kernel(
     const int mstat = march_ray<KIND, LAYOUT, BOXES>(m, k, P, ray, seg, lgs, active, en, ea,
                                               hits ? hits + ro : nullptr);
     // read after the march, so that they are not held in registers across it
-    const float v[3] = {__ldg(&sp->v[0]), __ldg(&sp->v[1]), __ldg(&sp->v[2])};
-    const float vl[3] = {__ldg(&sp->vl[0]), __ldg(&sp->vl[1]), __ldg(&sp->vl[2])};
-    const uint32_t part0 = __ldg(&sp->part0), group0 = __ldg(&sp->group0);
-    const uint32_t lg = __ldg(&sp->lg_segs) & 255u, lgW = lg - lgs;
+    const float v[3] = {sp->v[0], sp->v[1], sp->v[2]};
+    const float vl[3] = {sp->vl[0], sp->vl[1], sp->vl[2]};
+    const uint32_t part0 = sp->part0, group0 = sp->group0;
+    const uint32_t lg = sp->lg_segs & 255u, lgW = lg - lgs;
     float vals[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     unsigned nh = 0, na = 0;
     bool adds = false;
@@ -2361,7 +2366,7 @@ struct StateShared {
 template <int KIND, int LAYOUT, int RED, bool BOXES>
 __global__ void __launch_bounds__(1024, 1) raycast_state_kernel(
     const __grid_constant__ DevMap m, const __grid_constant__ EvalConsts k,
-    const double* __restrict__ states, const uint32_t* __restrict__ n_rays, uint32_t max_rays,
+    const double* states, const uint32_t* n_rays, uint32_t max_rays,
     rmp_result_t* out, rmp_ray_hit_t* hits, float* per_ray, const double* goals, uint32_t most) {
   extern __shared__ __align__(16) float parts[];
   __shared__ StateShared sh;
@@ -2717,7 +2722,7 @@ __device__ __forceinline__ float key_float(uint32_t k) {
 template <bool ROLL, int KIND, int LAYOUT>
 __global__ void __launch_bounds__(256, 4) esdf_eval_kernel(
     const rmp_primitive_t* __restrict__ prims, const float4* __restrict__ prims32, uint32_t n_prims,
-    EsdfConsts k, const double* __restrict__ states_in, const double* __restrict__ goals_in,
+    EsdfConsts k, const double* states_in, const double* goals_in,
     uint32_t n_states, uint32_t G, rmp_result_t* out, double* query,
     const __grid_constant__ DevMap m, const __grid_constant__ RolloutArgs g_roll, uint32_t steps,
     uint32_t* running) {
@@ -2961,9 +2966,8 @@ __global__ void __launch_bounds__(256, 4) esdf_eval_kernel(
 
 // ------------------------------------------------------------------ LiDAR scan kernel (Sec. III-G)
 template <int RED>
-__global__ void __launch_bounds__(256) scan_rmp_kernel(const float* __restrict__ pts,
-                                                       EvalConsts k,
-                                                       const double* __restrict__ state,
+__global__ void __launch_bounds__(256) scan_rmp_kernel(const float* pts, EvalConsts k,
+                                                       const double* state,
                                                        WsHeader* ws, CtaPartial* parts,
                                                        rmp_result_t* out, float* per_ray) {
   __shared__ CtaState cs;
@@ -2993,7 +2997,7 @@ __global__ void __launch_bounds__(256) scan_rmp_kernel(const float* __restrict__
     const bool in = j < k.n_rays;
     float q[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) q[a] = in ? __fsub_rn(__ldg(pts + 3 * (size_t)j + a), cs.xf[a]) : 0.0f;
+    for (int a = 0; a < 3; ++a) q[a] = in ? __fsub_rn(pts[3 * (size_t)j + a], cs.xf[a]) : 0.0f;
     float f[3] = {0.f, 0.f, 0.f}, vals[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     bool valid = isfinite(q[0]) && isfinite(q[1]) && isfinite(q[2]);
     float d = 0.0f;
