@@ -637,9 +637,10 @@ int rmp_eval_launch_info(rmp_ctx* c, uint32_t map_id, uint32_t n_rays, const rmp
   std::lock_guard<std::mutex> lk(c->mu);
   auto it = c->maps.find(map_id);
   if (it == c->maps.end()) return RMP_ERR_UNKNOWN_MAP;
-  const DevMap dm = it->second.dm;
+  DevMap dm = it->second.dm;
   EvalConsts k;
   const Tuning t = tuning_of(c);
+  if (t.cells == 0) dm.cells = nullptr;             // as launch_single
   int st = make_consts(params, dm.vs, n_rays, false, &k, t);
   if (st != RMP_OK) return st;
   DeviceGuard g(c->device);

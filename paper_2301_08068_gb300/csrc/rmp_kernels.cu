@@ -3546,12 +3546,17 @@ static void for_map(const DevMap& m, int reduce_mode, F f) {
   else for_reduction<RMP_MAP_HASHED_TSDF, kLayoutHash>(m, reduce_mode, f);
 }
 
+// CTAs per SM of the variant that launch_raycast runs at this CTA size.
 int raycast_occupancy(const DevMap& m, int reduce_mode, int block) {
   int n = 0;
   cudaError_t e = cudaSuccess;
   for_map(m, reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &n, raycast_rmp_kernel<kind.value, layout.value, red.value, boxes.value != 0, 256, 2>, block, 0);
+    if (block == 256)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &n, raycast_rmp_kernel<kind.value, layout.value, red.value, boxes.value != 0, 256, 2>, block, 0);
+    else
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &n, raycast_rmp_kernel<kind.value, layout.value, red.value, boxes.value != 0, 128, 6>, block, 0);
   });
   return e == cudaSuccess ? n : -1;
 }

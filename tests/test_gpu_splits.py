@@ -359,3 +359,23 @@ def test_rollouts_from_several_threads(ctx, contexts):
     if contexts == 2:
         other.close()
     assert not bad, (len(bad), bad[:3])
+
+
+@pytest.mark.parametrize("cells", [-1, 0])
+@pytest.mark.parametrize("block,least", [(64, 12), (128, 6), (256, 2)])
+def test_launch_info_of_the_kernel_that_runs(ctx, block, least, cells):
+    """Resident CTAs per SM are those of the variant launched at this CTA size: 64- and 128-thread
+    CTAs run one that is bounded to 768 threads an SM (85 registers), 256-thread ones one bounded
+    to 512."""
+    wl = W.hashed_workload(n_states=1, state_seed_index=52)
+    mid = ctx.upload(wl.map)
+    p = R.make_params(wl.params, wl.max_range)
+    R.rmp_tune_set(ctx.handle, R.RMP_TUNE_BLOCK, block)
+    R.rmp_tune_set(ctx.handle, R.RMP_TUNE_CELL_SKIP, cells)
+    try:
+        info = R.rmp_eval_launch_info(ctx.handle, mid, 262144, p)
+        assert info["block"] == block and info["ctas_per_sm"] >= least, info
+    finally:
+        R.rmp_tune_set(ctx.handle, R.RMP_TUNE_BLOCK, 0)
+        R.rmp_tune_set(ctx.handle, R.RMP_TUNE_CELL_SKIP, -1)
+        R.rmp_map_release(ctx.handle, mid)
