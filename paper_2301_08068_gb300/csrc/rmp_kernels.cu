@@ -2492,7 +2492,6 @@ __global__ void __launch_bounds__(1024, 1) rollout_kernel(const __grid_constant_
   const uint32_t n_parts = ((n << lg) + 31) / 32, chunks = ((n << lgs) + 31) / 32;
   float* parts = dyn + ((6 * n + 3) & ~3u);
   wait_previous();
-  if (g.rs[b].status != RMP_ROLLOUT_RUNNING) return;
   if (warp == 0) {
     if (lane < sizeof(RolloutDev) / 8)
       reinterpret_cast<unsigned long long*>(&sh.r)[lane] =
@@ -2501,11 +2500,13 @@ __global__ void __launch_bounds__(1024, 1) rollout_kernel(const __grid_constant_
     if (lane < 6) sh.st[lane] = x;
     if (lane < 3) sh.goal[lane] = g.goals[3 * (size_t)b + lane];
     const bool bad = quantise_state<KIND>(m, x, sh.P, sh.v, sh.vl);
-    if (bad && lane == 0) g.rs[b].status = RMP_ROLLOUT_FAILED;
     const uint32_t M = n >= 32 ? pick_cells_warp(n) : 1u;
-    if (lane == 0) {
+    __syncwarp();
+    if (lane == 0) {                                // the other warps learn of a stopped robot by go
+      const bool runs = sh.r.status == RMP_ROLLOUT_RUNNING;
+      if (runs && bad) g.rs[b].status = RMP_ROLLOUT_FAILED;
       sh.cells = M;
-      sh.go = bad ? 0 : 1;
+      sh.go = runs && !bad ? 1 : 0;
     }
   }
   __syncthreads();
