@@ -1916,6 +1916,7 @@ __device__ __noinline__ uint32_t rollout_book(const DevMap& m, const RolloutCons
   if (rc.seg_steps && steps % rc.seg_steps == 0) {
     const double seg = xn - r.seg_start[a], prev = r.prev_seg[a];
     const bool have = r.have_prev != 0;
+    __syncwarp();                                   // every lane has read what lanes 0-2 write below
     if (have) {
       const double dot = dot3(prev, seg), na = dot3(prev, prev), nb = dot3(seg, seg);
       if (na > 0.0 && nb > 0.0) {
@@ -2949,7 +2950,9 @@ __global__ void __launch_bounds__(256, 4) esdf_eval_kernel(
       bool runs = false;
       for (uint32_t s = warp; s < G && base + s < n_states; s += 8) {
         const uint32_t r = base + s;
-        if (g_roll.rs[r].status != RMP_ROLLOUT_RUNNING) continue;
+        const uint32_t before = g_roll.rs[r].status;
+        __syncwarp();                               // every lane has read what lane 0 may write
+        if (before != RMP_ROLLOUT_RUNNING) continue;
         if (out[r].status != RMP_OK) {
           if (lane == 0) rollout_fail(g_roll, r);
         } else {
