@@ -163,7 +163,13 @@ int rmp_params_preset(int preset, rmp_params_t* out);
 
 /* Upload a map (Sec. III-F: the map lives in GPU memory, shared by all evaluations).
  * Work is enqueued on `stream` and completed before return.  *map_id receives a
- * context-local id.  INVALID_ARG on bad dims, keys out of range or duplicate keys. */
+ * context-local id.  INVALID_ARG on bad dims, keys out of range or duplicate keys.
+ * Device memory: 64 bytes per 8^3 block, 32 more per block in the grid layout (all blocks of the
+ * bounding box) or at least 64 in the hash layout, and the box field: 4 KB per block that holds an
+ * occupied voxel (the 40 m map of 0.1 m voxels: 3 MB and 32 MB; rmp_map_info tells).  The field
+ * makes evaluations 1.2 to 3 times faster and takes about 9 ns per such block to build.  A map
+ * gets none if RMP_TUNE_CELL_SKIP is 0 at the upload, or if the field would exceed 32 GiB or
+ * leave less than a sixteenth of the device's memory free; results are the same without it. */
 int rmp_map_upload(rmp_ctx* ctx, const rmp_map_desc_t* desc, rmp_stream_t stream,
                    uint32_t* map_id);
 
@@ -525,8 +531,9 @@ int rmp_probe_l2_read(rmp_ctx* ctx, const void* buf_dev, size_t bytes, uint32_t 
  *  RMP_TUNE_SPLIT_BUDGET accepted (-1..65536) and read back, without effect: rays are marched
  *                        box by box, which leaves no long pieces to split over a warp
  *  RMP_TUNE_CELL_SKIP    free boxes of voxels inside occupied blocks crossed in one step: 1
- *                        or -1 (default) always, 0 never (voxel by voxel there; slower, for
- *                        comparison) */
+ *                        or -1 (default) wherever the map has a box field, 0 never (voxel by
+ *                        voxel there, slower).  At an upload: 0 leaves the map without a field,
+ *                        for good, where its memory or its time counts more */
 #define RMP_TUNE_BLOCK 1
 #define RMP_TUNE_LG_SEGMENTS 2
 #define RMP_TUNE_RAY_ORDER 3

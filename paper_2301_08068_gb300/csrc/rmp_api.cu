@@ -253,11 +253,23 @@ void free_map(rmp_ctx* c, MapRec& r) {
   r.bricks = r.table = r.top = r.boxes = nullptr;
 }
 
+// Whether the pool may give a box field of `bytes` (see box_field_fits).
+bool field_fits(rmp_ctx* c, uint64_t bytes) {
+  uint64_t reserved = 0, used = 0;
+  if (cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
+      cudaMemPoolGetAttribute(c->pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess)
+    return false;
+  const uint64_t room = reserved - std::min(used, reserved);
+  size_t free_bytes = 0, total = 0;
+  if (bytes > room && cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) return false;
+  return box_field_fits(bytes, room, free_bytes, total);
+}
+
 // The box field of a map whose bricks (and hash table) are in r: n bricks, of which `occupied`
 // hold an occupied voxel (at most, if not `counted`).  keys: hash layout, the blocks' keys.  A
-// field that is too large or does not fit is left out: occupied blocks are then marched
-// voxel by voxel.
-int build_boxes(rmp_ctx* c, MapRec& r, uint32_t n, uint32_t occupied, bool counted,
+// field that is not wanted (RMP_TUNE_CELL_SKIP 0), too large or does not fit is left out: occupied
+// blocks are then marched voxel by voxel.
+int build_boxes(rmp_ctx* c, MapRec& r, bool wanted, uint32_t n, uint32_t occupied, bool counted,
                 const int32_t* keys, cudaStream_t s) {
   const bool grid = r.dm.layout == kLayoutGrid;
   uint32_t* scratch = nullptr;                  // count, slots, list
@@ -268,12 +280,12 @@ int build_boxes(rmp_ctx* c, MapRec& r, uint32_t n, uint32_t occupied, bool count
   if (e == cudaSuccess)
     e = launch_block_slots((const uint32_t*)r.bricks, n, keys, r.dm, (HashEntry*)r.table,
                            scratch + at_slots, scratch + at_list, scratch, s);
-  uint32_t count = occupied;
+  uint32_t count = wanted ? occupied : 0;
   if (e == cudaSuccess && !counted && count * kBoxBytes > (64ull << 20)) {   // too loose to allocate
     e = cudaMemcpyAsync(&count, scratch, 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
-  if (e == cudaSuccess && count > 0 && count * kBoxBytes <= kMaxBoxFieldBytes) {
+  if (e == cudaSuccess && count > 0 && field_fits(c, count * kBoxBytes)) {
     if (pool_alloc(c, &r.boxes, count * kBoxBytes) == cudaSuccess) {
       r.dm.cells = (const uint32_t*)r.boxes;
       r.bytes += count * kBoxBytes;
@@ -394,6 +406,11 @@ int rmp_map_upload(rmp_ctx* c, const rmp_map_desc_t* d, rmp_stream_t stream, uin
   cudaStream_t s = (cudaStream_t)stream;
   DeviceGuard g(c->device);
   if (!g.ok()) return RMP_ERR_CUDA;
+  bool boxes;
+  {
+    std::lock_guard<std::mutex> lk(c->mu);
+    boxes = c->tune_cells != 0;
+  }
   MapRec r;
   std::memset(&r.dm, 0, sizeof(r.dm));
   r.dm.kind = d->kind;
@@ -444,7 +461,7 @@ int rmp_map_upload(rmp_ctx* c, const rmp_map_desc_t* d, rmp_stream_t stream, uin
     if (e == cudaSuccess) e = launch_dense_bricks(occ, r.dm.dims, r.dm.gdim, (uint32_t*)r.bricks, s);
     if (e != cudaSuccess) return fail(cuda_status(e));
     r.bytes = nbr * 64;
-    const int rs = build_boxes(c, r, (uint32_t)nbr, (uint32_t)nbr, false, nullptr, s);
+    const int rs = build_boxes(c, r, boxes, (uint32_t)nbr, (uint32_t)nbr, false, nullptr, s);
     if (rs != RMP_OK) return fail(rs);
   } else if (d->kind == RMP_MAP_HASHED_TSDF) {
     const uint32_t n = d->n_blocks;
@@ -522,7 +539,7 @@ int rmp_map_upload(rmp_ctx* c, const rmp_map_desc_t* d, rmp_stream_t stream, uin
         e = launch_grid_scatter(keys, (const uint32_t*)compact, n, r.dm, (uint32_t*)r.bricks, s);
       if (e != cudaSuccess) return fail(cuda_status(e));
       r.bytes = grid_bytes;
-      const int rs = build_boxes(c, r, (uint32_t)gprod, occupied, true, nullptr, s);
+      const int rs = build_boxes(c, r, boxes, (uint32_t)gprod, occupied, true, nullptr, s);
       if (rs != RMP_OK) return fail(rs);
     } else {
       r.dm.layout = kLayoutHash;
@@ -534,7 +551,7 @@ int rmp_map_upload(rmp_ctx* c, const rmp_map_desc_t* d, rmp_stream_t stream, uin
       r.bytes = (uint64_t)cap * sizeof(HashEntry) + (uint64_t)n * 64;
       r.dm.bricks = (const uint4*)r.bricks;
       r.dm.table = (const HashEntry*)r.table;
-      const int rs = build_boxes(c, r, n, occupied, true, keys, s);
+      const int rs = build_boxes(c, r, boxes, n, occupied, true, keys, s);
       if (rs != RMP_OK) return fail(rs);
     }
   } else {

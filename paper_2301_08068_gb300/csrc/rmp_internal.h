@@ -43,8 +43,8 @@ struct HashEntry {
 constexpr int kLayoutGrid = 0;
 constexpr int kLayoutHash = 1;
 constexpr uint64_t kBoxBytes = 4096;                  // box field of one occupied block
-// Largest box field (8 M occupied blocks); a map beyond it, or one whose field does not fit the
-// device's memory, is marched voxel by voxel inside occupied blocks
+// Largest box field (8 M occupied blocks); a map beyond it, or one whose field does not fit (see
+// box_field_fits), is marched voxel by voxel inside occupied blocks
 constexpr uint64_t kMaxBoxFieldBytes = 32ull << 30;
 constexpr int kCellDistCap = 4;                       // cell free distances are capped here
 constexpr uint64_t kMaxCellBytes = 256ull << 20;      // cell distances given up to this size

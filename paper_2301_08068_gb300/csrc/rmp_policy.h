@@ -84,6 +84,17 @@ inline void launch_shape(const Tuning& t, uint64_t n_threads, uint64_t wave256, 
   *grid = (int)g;
 }
 
+// Whether a map gets a box field of `bytes`: up to kMaxBoxFieldBytes, from memory the context's
+// pool holds already (`room`) or while a sixteenth of the device's memory stays free beside it.  At
+// 4 KB per occupied block the field is by far the largest part of a map, and one that a map can
+// do without (65536 rays on the 40 m map 15.5 us with it, 44 without, 52 by the voxel walk before
+// it): it is never the reason why another map, or another library, finds no memory.
+inline bool box_field_fits(uint64_t bytes, uint64_t room, uint64_t free_bytes,
+                           uint64_t total_bytes) {
+  if (bytes > kMaxBoxFieldBytes) return false;
+  return bytes <= room || (free_bytes >= bytes && free_bytes - bytes >= total_bytes / 16);
+}
+
 // Scans: threads per CTA the tuned value or (automatic) 256, and at most 512 threads per
 // SM, each thread striding over several points, so that large scans are reduced from few
 // CTA partials (measured, device time: 4096 / 65536 / 262144 points 5.7 / 8.1 / 9.7 us with

@@ -94,3 +94,36 @@ def test_dense_long_axis(ctx, axis, size):
         occ[tuple(c[::-1])] = 0
         xs.append((c + 0.5) * VS)
     check(ctx, W.DenseMap(occ, VS, np.zeros(3)), xs, 333, 4.0)
+
+
+@pytest.mark.parametrize("kind", ["dense", "grid", "hash"])
+def test_uploaded_without_box_field(ctx, kind):
+    """RMP_TUNE_CELL_SKIP 0 at the upload leaves the box field out, 4 KB per occupied block;
+    evaluations give the oracle's records whatever the knob says then."""
+    rng = np.random.default_rng(11)
+    if kind == "dense":
+        occ = (rng.uniform(size=(40, 33, 70)) < 0.02).astype(np.uint8)
+        m, xs, r = W.DenseMap(occ, VS, np.zeros(3)), [np.array([3.0, 1.6, 2.0]), np.zeros(3) + 0.01], 4.0
+        occupied = 9 * 5 * 5
+    else:
+        keys = np.unique(rng.integers(-4, 5, (60, 3)), axis=0).astype(np.int32)
+        if kind == "hash":
+            keys = np.concatenate([keys, [[9000, -7000, 800]]]).astype(np.int32)
+        tsdf = np.where(rng.uniform(size=(len(keys), 512)) < 0.05, -0.1, 0.2).astype(np.float32)
+        tsdf[:, 7] = -0.1
+        m, xs, r = W.HashedMap(keys, tsdf, VS), [np.array([0.05, -0.05, 0.15]), np.array([4.1, 4.1, 4.1])], 20.0
+        occupied = len(keys)
+    size = []
+    for knob in (-1, 0):
+        R.rmp_tune_set(ctx.handle, R.RMP_TUNE_CELL_SKIP, knob)
+        mid = ctx.upload(m)
+        size.append(R.rmp_map_info(ctx.handle, mid)["device_bytes"])
+        R.rmp_map_release(ctx.handle, mid)
+    assert size[0] - size[1] == 4096 * occupied, size
+    upload = ctx.upload
+    try:                                            # as check does, on a map without a field
+        ctx.upload = lambda mm: (R.rmp_tune_set(ctx.handle, R.RMP_TUNE_CELL_SKIP, 0), upload(mm))[1]
+        check(ctx, m, xs, 500, r)
+    finally:
+        del ctx.upload
+        R.rmp_tune_set(ctx.handle, R.RMP_TUNE_CELL_SKIP, -1)
