@@ -26,6 +26,7 @@ struct MapRec {
   uint32_t n_bricks = 0;
   uint32_t cap = 0;
   uint64_t bytes = 0;
+  uint64_t pool_bytes = 0;        // of them from the context's pool
   uint64_t wave256[2] = {0, 0};   // threads of one wave of 256-thread CTAs, per reduction
 };
 
@@ -57,6 +58,8 @@ struct rmp_ctx {
   rmp_result_t* result_map = nullptr;   // its device address
   cudaMemPool_t pool = nullptr;         // box fields (see pool_create)
   cudaStream_t pool_stream = nullptr;
+  std::mutex pool_mu;
+  uint64_t pool_live = 0, pool_largest = 0, pool_threshold = 0;   // see pool_note
 };
 
 namespace {
@@ -210,23 +213,18 @@ cudaError_t launch_single(const MapRec& mr, const Tuning& t, EvalConsts k,
   return launch_raycast(dm, k, state_dev, ws, out, hits, per_ray, block, grid, s);
 }
 
-// Memory of a map's box field, from the context's pool: a cudaMalloc and a cudaFree of the field's
-// megabytes map and unmap pages on every upload and release of a map (refresh of a 128^3 map with
-// an evaluation 260 us, 88 from the pool; of the 40 m map 527 and 358).  The pool keeps at most
-// kPoolKeepBytes of what is given back, until the context is destroyed.  All of it is allocated
-// and freed on one stream of its own, idle otherwise, so that what one map gives back the next
-// one gets.
-constexpr uint64_t kPoolKeepBytes = 64ull << 20;
-
+// Memory of a map's box field, its planes and the scratch of an upload, from the context's pool: a
+// cudaMalloc and a cudaFree of these megabytes map and unmap pages on every upload and release of a
+// map (refresh of a 128^3 map with an evaluation 260 us, 88 from the pool; of the 40 m map 527 and
+// 380).  All of it is allocated and freed on one stream of its own, idle otherwise, so that what
+// one map gives back the next one gets.
 cudaError_t pool_create(rmp_ctx* c) {
   cudaMemPoolProps props;
   std::memset(&props, 0, sizeof(props));
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = c->device;
-  uint64_t keep = kPoolKeepBytes;
   cudaError_t e = cudaMemPoolCreate(&c->pool, &props);
-  if (e == cudaSuccess) e = cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->pool_stream, cudaStreamNonBlocking);
   return e;
 }
@@ -240,6 +238,18 @@ cudaError_t pool_alloc(rmp_ctx* c, void** p, size_t bytes) {
   return cudaStreamSynchronize(c->pool_stream);   // for use on any stream
 }
 
+// The maps hold `more` bytes of the pool than before, after an upload that took `peak` with its
+// scratch (0: a release); sets what the pool keeps (see pool_keep) before anything goes back.
+void pool_note(rmp_ctx* c, int64_t more, uint64_t peak) {
+  std::lock_guard<std::mutex> lk(c->pool_mu);
+  c->pool_live += (uint64_t)more;
+  c->pool_largest = std::max(c->pool_largest, peak);
+  uint64_t keep = pool_keep(c->pool_live, c->pool_largest);
+  if (keep != c->pool_threshold &&
+      cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+    c->pool_threshold = keep;
+}
+
 // Nothing on the device uses p any more.
 void pool_free(rmp_ctx* c, void* p) {
   if (p) cudaFreeAsync(p, c->pool_stream);
@@ -250,6 +260,8 @@ void free_map(rmp_ctx* c, MapRec& r) {
   if (r.table) cudaFree(r.table);
   pool_free(c, r.top);
   pool_free(c, r.boxes);
+  if (r.pool_bytes) pool_note(c, -(int64_t)r.pool_bytes, 0);
+  r.pool_bytes = 0;
   r.bricks = r.table = r.top = r.boxes = nullptr;
 }
 
@@ -273,9 +285,10 @@ int build_boxes(rmp_ctx* c, MapRec& r, bool wanted, uint32_t n, uint32_t occupie
                 const int32_t* keys, cudaStream_t s) {
   const bool grid = r.dm.layout == kLayoutGrid;
   uint32_t* scratch = nullptr;                  // count, slots, list
-  const size_t at_slots = 64, at_list = at_slots + (grid ? n : 0);
-  cudaError_t e = pool_alloc(c, (void**)&scratch, (at_list + n) * 4);
-  if (e == cudaSuccess && grid) e = pool_alloc(c, &r.top, (size_t)n * 32);
+  const size_t at_slots = 64, at_list = at_slots + (grid ? n : 0), scratch_bytes = (at_list + n) * 4;
+  uint64_t held = grid ? (uint64_t)n * 32 : 0;
+  cudaError_t e = pool_alloc(c, (void**)&scratch, scratch_bytes);
+  if (e == cudaSuccess && grid) e = pool_alloc(c, &r.top, held);
   if (e == cudaSuccess) e = cudaMemsetAsync(scratch, 0, 4, s);
   if (e == cudaSuccess)
     e = launch_block_slots((const uint32_t*)r.bricks, n, keys, r.dm, (HashEntry*)r.table,
@@ -288,7 +301,7 @@ int build_boxes(rmp_ctx* c, MapRec& r, bool wanted, uint32_t n, uint32_t occupie
   if (e == cudaSuccess && count > 0 && field_fits(c, count * kBoxBytes)) {
     if (pool_alloc(c, &r.boxes, count * kBoxBytes) == cudaSuccess) {
       r.dm.cells = (const uint32_t*)r.boxes;
-      r.bytes += count * kBoxBytes;
+      held += count * kBoxBytes;
     } else {
       cudaGetLastError();
       r.boxes = nullptr;
@@ -300,8 +313,12 @@ int build_boxes(rmp_ctx* c, MapRec& r, bool wanted, uint32_t n, uint32_t occupie
                          c->sm_count, s);
   const cudaError_t done = cudaStreamSynchronize(s);   // the scratch and the field are used on s
   if (e == cudaSuccess) e = done;
+  if (e == cudaSuccess) {
+    r.bytes += held;
+    r.pool_bytes = held;
+    pool_note(c, (int64_t)held, held + scratch_bytes);
+  }
   pool_free(c, scratch);
-  r.bytes += grid ? (uint64_t)n * 32 : 0;
   return e == cudaSuccess ? RMP_OK : cuda_status(e);
 }
 

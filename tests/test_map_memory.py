@@ -41,3 +41,12 @@ def policy(tmp_path_factory):
 ])
 def test_box_field_leaves_memory(policy, field, room, free, fits):
     assert policy(["fits %d %d %d %d" % (field, room, free, TOTAL)]) == [int(fits)]
+
+
+@pytest.mark.parametrize("live,largest,free", [
+    (0, 0, 0), (500 << 20, 1, 1),
+    (0, 90 << 20, 90 << 20), (3 * GB, 90 << 20, 90 << 20),   # one more map of the largest size
+    (0, 5 * GB, 2 * GB), (7 * GB, 5 * GB, 2 * GB),  # the most
+])
+def test_pool_keeps_one_map(policy, live, largest, free):
+    assert policy(["keep %d %d" % (live, largest)]) == [live + free + (64 << 20)]
