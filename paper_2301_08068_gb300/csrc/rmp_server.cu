@@ -5,10 +5,11 @@
 // worker thread keeps up to `slots` batches in flight, each on its own CUDA stream: as
 // soon as a slot is free it admits the oldest pending request and every later pending
 // request with the same map and parameters (FIFO order, up to max_batch_states), as long
-// as the batch's device memory (workspace, states, counts, results) fits in what is left
-// of the server's budget, and launches one rmp_raycast_eval_batch_async.  Batches on
-// different streams overlap on the device; a finished batch (event) returns its memory
-// and completes its requests, which frees room for the requests that arrived meanwhile.
+// as the batch's device memory (its workspace) fits in what is left of the server's budget,
+// and launches one rmp_raycast_eval_batch_async; states, ray counts and results lie in the
+// slot's pinned host memory, which the kernels read and write.  Batches on different streams
+// overlap on the device; a finished batch (event) returns its memory and completes its
+// requests, which frees room for the requests that arrived meanwhile.
 // A request whose batch alone would exceed the budget is completed with
 // RMP_ERR_NO_MEMORY; a CUDA error completes the batch's requests with RMP_ERR_CUDA.
 // The worker sleeps whenever it can launch nothing: a host function enqueued after each
@@ -68,18 +69,9 @@ bool same_key(const Request& a, const Request& b) {
   return a.map_id == b.map_id && std::memcmp(&a.params, &b.params, sizeof(rmp_params_t)) == 0;
 }
 
-struct BatchBytes {
-  size_t ws, states, counts, out, total;
-};
-
-BatchBytes batch_bytes(uint32_t n, uint32_t max_rays) {
-  BatchBytes b;
-  b.ws = batch_layout(n, max_rays).total;
-  b.states = Arena::round(6 * sizeof(double) * n);
-  b.counts = Arena::round(4 * (size_t)n);
-  b.out = Arena::round(sizeof(rmp_result_t) * n);
-  b.total = b.ws + b.states + b.counts + b.out;
-  return b;
+// Device memory of a batch of n states.
+size_t batch_bytes(uint32_t n, uint32_t max_rays) {
+  return Arena::round(batch_layout(n, max_rays).total);
 }
 
 rmp_result_t failed_result(uint32_t n_rays, int status) {
@@ -153,7 +145,7 @@ void wake_worker(rmp_server* s) {
   s->wake_cv.notify_all();
 }
 
-// Host function enqueued after a batch's result copy: marks the slot finished and wakes the
+// Host function enqueued after a batch's kernels: marks the slot finished and wakes the
 // worker.  It calls no CUDA function and takes only the wake-up mutex.
 void CUDART_CB batch_done(void* arg) {
   Slot* sl = static_cast<Slot*>(arg);
@@ -167,18 +159,20 @@ void CUDART_CB batch_done(void* arg) {
 // do not wait for launches.  States and counts are read from, and results written to, the
 // slot's pinned host memory by the kernels themselves: 48 bytes in and 144 out per request,
 // where three copies cost the stream and the worker more than the transfers (a burst of 96
-// requests over three maps: 1.93 -> 1.72 ms together).
+// requests over three maps: 1.93 -> 1.72 ms together; one batch of 256 requests 97 us, with copies
+// 114, of 2433 82 / 86; only past about 3000 requests in a batch, whose set-up reads all counts in
+// every CTA, would copies be faster: 4096 119 / 112, 65536 865 / 637).
 bool launch_batch_on(rmp_server* s, Slot& sl, std::unique_lock<std::mutex>& lk) {
   const Request first = s->pending.front();
   const uint32_t cap = s->cfg.max_batch_states;
-  BatchBytes need = batch_bytes(1, first.n_rays);
-  if (need.total > s->arena->size()) {           // can never fit: fail it, keep going
+  size_t need = batch_bytes(1, first.n_rays);
+  if (need > s->arena->size()) {           // can never fit: fail it, keep going
     s->pending.pop_front();
     complete_now(s, first, RMP_ERR_NO_MEMORY);
     return true;
   }
   const size_t room = s->arena->largest_free();
-  if (need.total > room) return false;
+  if (need > room) return false;
   // members: the oldest request, then later ones with the same key while the batch fits
   std::vector<size_t> take{0};
   uint32_t max_rays = first.n_rays;
@@ -187,17 +181,17 @@ bool launch_batch_on(rmp_server* s, Slot& sl, std::unique_lock<std::mutex>& lk) 
     const Request& r = s->pending[i];
     if (!same_key(r, first)) continue;
     const uint32_t mr = r.n_rays > max_rays ? r.n_rays : max_rays;
-    const BatchBytes nb = batch_bytes((uint32_t)take.size() + 1, mr);
-    if (nb.total > room) break;
+    const size_t nb = batch_bytes((uint32_t)take.size() + 1, mr);
+    if (nb > room) break;
     take.push_back(i);
     max_rays = mr;
     need = nb;
   }
   const uint32_t n = (uint32_t)take.size();
-  const size_t off = s->arena->alloc(need.total);
+  const size_t off = s->arena->alloc(need);
   if (off == Arena::kFail) return false;
   sl.off = off;
-  sl.bytes = need.total;
+  sl.bytes = need;
   sl.ids.resize(n);
   sl.t_submit.resize(n);
   for (uint32_t j = 0; j < n; ++j) {
@@ -224,7 +218,7 @@ bool launch_batch_on(rmp_server* s, Slot& sl, std::unique_lock<std::mutex>& lk) 
   lk.unlock();
   sl.finished.store(false, std::memory_order_relaxed);
   int st = rmp_raycast_eval_batch_async(s->ctx, first.map_id, sl.h_states, sl.h_counts, n, max_rays,
-                                        &first.params, s->arena_dev + off, need.ws, sl.stream,
+                                        &first.params, s->arena_dev + off, need, sl.stream,
                                         sl.h_out, nullptr, nullptr);
   if (st == RMP_OK && cudaEventRecord(sl.done, sl.stream) != cudaSuccess) st = RMP_ERR_CUDA;
   if (st == RMP_OK && cudaLaunchHostFunc(sl.stream, batch_done, &sl) != cudaSuccess)

@@ -123,6 +123,18 @@ def test_server_memory_budget_admission(env):
     assert st["rejected"] == 1
 
 
+@pytest.mark.parametrize("n_rays", [1000, 30000])       # a CTA for the state, the persistent grid
+def test_server_budget_is_the_workspace(env, n_rays):
+    """Device memory is taken for a batch's workspace alone (states, counts and results lie in
+    pinned memory): a budget of just that serves a request, 256 bytes less refuse it."""
+    ctx, maps = env
+    need = (R.rmp_batch_workspace_bytes(1, n_rays) + 255) // 256 * 256
+    for budget, status in ((need, 0), (need - 256, R.STATUS_CODES["RMP_ERR_NO_MEMORY"])):
+        with R.Server(ctx, slots=2, mem_budget_bytes=budget, max_rays=262144) as srv:
+            res, _ = srv.wait(submit(srv, maps["hashed"], 0, n_rays))
+            assert res["status"] == status and srv.stats()["mem_high_water"] <= budget
+
+
 def test_server_errors(env):
     ctx, maps = env
     wl, mid, om = maps["hashed"]
