@@ -842,6 +842,7 @@ int batch_setup(rmp_ctx* c, uint32_t map_id, uint32_t n_states, uint32_t max_ray
   const int occ = batch_occupancy(*dm, k->reduce_mode, *block);
   if (occ <= 0) return RMP_ERR_CUDA;
   *grid = c->sm_count * occ;
+  k->sms = (uint32_t)c->sm_count;
   k->seg_threads = (uint32_t)*grid * (uint32_t)*block;
   return RMP_OK;
 }
@@ -903,7 +904,8 @@ int rmp_combined_eval_batch_async(rmp_ctx* c, uint32_t map_id, const double* sta
 namespace {
 
 // Constants of the ESDF policy from rmp_params_t (validated as for the ray policy).
-int make_esdf_consts(const rmp_params_t* p, double alpha, double beta, EsdfConsts* k) {
+int make_esdf_consts(const rmp_ctx* c, const rmp_params_t* p, double alpha, double beta,
+                     EsdfConsts* k) {
   EvalConsts e;
   const int st = make_consts(p, 1.0, 1, true, &e);
   if (st != RMP_OK) return st;
@@ -919,6 +921,7 @@ int make_esdf_consts(const rmp_params_t* p, double alpha, double beta, EsdfConst
   k->alpha = alpha;
   k->beta = beta;
   k->w_mode = (int)p->w_mode;
+  k->sms = (uint32_t)c->sm_count;
   return RMP_OK;
 }
 
@@ -933,7 +936,7 @@ int rollout_impl(rmp_ctx* c, uint32_t map_id, const EsdfRec* esdf, const double*
     return RMP_ERR_INVALID_ARG;
   EsdfConsts ek;
   if (esdf) {
-    const int st = make_esdf_consts(params, rp->alpha, rp->beta, &ek);
+    const int st = make_esdf_consts(c, params, rp->alpha, rp->beta, &ek);
     if (st != RMP_OK) return st;
   }
   DevMap dm;
@@ -947,7 +950,7 @@ int rollout_impl(rmp_ctx* c, uint32_t map_id, const EsdfRec* esdf, const double*
   if (!g.ok()) return RMP_ERR_CUDA;
   cudaStream_t s = (cudaStream_t)stream;
   // a CTA per robot for all steps, or an evaluation of all robots per step
-  const bool resident = !esdf && rollout_resident(n, rp->n_rays);
+  const bool resident = !esdf && rollout_resident(n, rp->n_rays, (uint32_t)c->sm_count);
   EvalConsts k;
   if (resident) {
     if (!attractor_ok(rp->alpha, rp->beta)) return RMP_ERR_INVALID_ARG;
@@ -1001,7 +1004,7 @@ int rollout_impl(rmp_ctx* c, uint32_t map_id, const EsdfRec* esdf, const double*
   // a round is one launch and the robots fill the SMs at most about once: a CTA then ends with its
   // robots)
   const bool fused = esdf || resident;
-  const uint32_t kRound = fused && n <= (esdf ? 1216u : 304u) ? 256 : 32;
+  const uint32_t kRound = fused && n <= (esdf ? 8u : 2u) * (uint32_t)c->sm_count ? 256 : 32;
   uint32_t running = n;
   for (uint32_t step = 0; e == cudaSuccess && status == RMP_OK && running > 0 &&
                           step < rp->max_steps;) {
@@ -1146,7 +1149,7 @@ int rmp_esdf_eval_async(rmp_ctx* c, uint32_t esdf_id, const double* states_dev,
                         double* query_dev) {
   if (!c || !states_dev || !out_dev || n_states == 0) return RMP_ERR_INVALID_ARG;
   EsdfConsts k;
-  const int st = make_esdf_consts(params, alpha, beta, &k);
+  const int st = make_esdf_consts(c, params, alpha, beta, &k);
   if (st != RMP_OK) return st;
   EsdfRec r;
   {

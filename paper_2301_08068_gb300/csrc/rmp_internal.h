@@ -92,6 +92,7 @@ struct EvalConsts {
   double att_alpha, att_beta;        // attractor gain and damping (combined evaluations)
   int att_mean;                      // combined: ray sums divided by the ray count first
   uint32_t seg_threads;              // batches: threads of the persistent launch (segments)
+  uint32_t sms;                      // batches and rollouts: SMs of the device
   CtaState cs0;                      // the state carried in the launch itself, read when the
                                      // kernel's state pointer is null (synchronous calls)
 };
@@ -176,22 +177,25 @@ struct BatchHeader {        // 128 bytes
 // States and robots evaluated by one CTA each have their partials in shared memory.
 constexpr uint32_t kStateRays = 4096, kStateGroups = kStateRays * kMaxBatchSegs / (32 * 32);
 // Batches with a CTA per state (see raycast_state_kernel): where a CTA's 32 warps hold a state's
-// rays, and up to 2432 states (16 of the smallest CTAs an SM), beyond which the packed chunks of the
-// persistent grid gain as much as the set-up costs (us, CTA per state / packed: 128 states of 16 to
-// 256 rays 13.5 / 25, 17.8 / 30; 304 of 1024 43 / 77; 1216 of 32 to 1024 71 / 74; 2432 of 64 to 256
-// 73 / 82; 5000 of 64 to 256 142 / 137; above 1024 rays 64 states of 512 to 4096 55 / 34).
-inline bool state_per_cta(uint32_t n_states, uint32_t max_rays) {
-  return max_rays <= 1024 && n_states <= 2432;
+// rays, and up to 16 states an SM (of the smallest CTAs), beyond which the packed chunks of the
+// persistent grid gain as much as the set-up costs (us on 152 SMs, CTA per state / packed: 128
+// states of 16 to 256 rays 13.5 / 25, 17.8 / 30; 304 of 1024 43 / 77; 1216 of 32 to 1024 71 / 74;
+// 2432 of 64 to 256 73 / 82; 5000 of 64 to 256 142 / 137; above 1024 rays 64 states of 512 to 4096
+// 55 / 34).
+inline bool state_per_cta(uint32_t n_states, uint32_t max_rays, uint32_t sms) {
+  return max_rays <= 1024 && n_states <= 16 * sms;
 }
 // Rollouts with a CTA per robot for all its steps (see rollout_kernel): up to 1024 rays, or as many
-// as its shared memory holds where the robots fill the SMs but once; more rays of few robots are
+// as its shared memory holds where two robots an SM take them all; more rays of few robots are
 // spread over all SMs instead, robots of many rays packed (us a step with its share of the call,
 // CTA per robot / evaluated together: 8 robots of 1024 rays 23 / 34, of 4096 70 / 37; 32 of 2048
 // 40 / 45; 128 of 1024 38 / 68, of 4096 77 / 121; 304 of 4096 186 / 207, 608 361 / 347; 1216 of
-// 256 175 / 227, of 1024 258 / 318).
-inline bool rollout_resident(uint32_t n_robots, uint32_t n_rays) {
+// 256 175 / 227, of 1024 258 / 318).  Few-ray robots have no upper bound: 16 steps of 65536 robots
+// take 11.7 ms with 16 rays each and 25.7 with 64, 4096 robots of 1024 6.6 (set-up and evaluation
+// launched per step, before: 197, 245 and 63).
+inline bool rollout_resident(uint32_t n_robots, uint32_t n_rays, uint32_t sms) {
   return n_rays <= 1024 ||
-         (n_rays <= kStateRays && n_rays <= 64 * n_robots && n_robots <= 304);
+         (n_rays <= kStateRays && n_rays <= 64 * n_robots && n_robots <= 2 * sms);
 }
 
 struct BatchLayout {
@@ -227,7 +231,7 @@ struct EsdfConsts {
   double eta_rep, nu_rep, eta_damp, nu_damp, r, c, eps;
   double alpha, beta;       // attractor (with goals)
   int w_mode;
-  int pad;
+  uint32_t sms;             // SMs of the device
 };
 
 // Launchers (rmp_kernels.cu).  All enqueue on `stream` and return cudaGetLastError().

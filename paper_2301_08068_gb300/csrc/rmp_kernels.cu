@@ -2711,7 +2711,7 @@ __device__ __forceinline__ float key_float(uint32_t k) {
 //      one its repulsion and weight, one the attractor;
 //   3. one warp runs the Jacobi sweeps, another the adjugate solve; three warps take one
 //      Rayleigh quotient each; the first sorts, decides the rank and writes the results.
-// The warps of the serial parts rotate with the CTA and with its turn on an SM (152 of them), so
+// The warps of the serial parts rotate with the CTA and with its turn on an SM, so
 // that an SM's CTAs use different schedulers' pipes.  Bound by the FP64 chain of steps 2 and 3;
 // four CTAs an SM (64 registers), so that 16384 states are one wave (three: 48 us).  16384 states,
 // 200 primitives: 33.6 us (one warp per state, every distance in FP64, policy in one lane: 638);
@@ -2734,7 +2734,7 @@ __global__ void __launch_bounds__(256, 4) esdf_eval_kernel(
   __shared__ float W[9][32], dv_sh[3][32];
   __shared__ int ok_sh[32];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t role = (warp + blockIdx.x + blockIdx.x / 152u) & 7u;
+  const uint32_t role = (warp + blockIdx.x + blockIdx.x / k.sms) & 7u;
   constexpr uint32_t kNone = 0xffffffffu;
   // a rollout's states change from step to step
   const double* states = ROLL ? g_roll.states : states_in;
@@ -3598,13 +3598,14 @@ cudaError_t launch_batch(const DevMap& m, const EvalConsts& k, const double* sta
                          void* ws, rmp_result_t* out_dev, rmp_ray_hit_t* hits, float* per_ray,
                          int block, int grid, cudaStream_t stream, const double* goals_dev,
                          const RolloutArgs& step) {
-  if (!step.rs && state_per_cta(n_states, max_rays)) {
+  const uint32_t sms = k.sms;
+  if (!step.rs && state_per_cta(n_states, max_rays, sms)) {
     // warps a CTA: all of an SM's 32 for one state, fewer where CTAs share it and hide each
     // other's serial steps; segments only while every state has its place (5000 states of 64 rays:
     // 4 segments 149 us, 1 86), one warp left for the attractor (128 of 256 rays 19.9 -> 17.8)
-    const uint32_t most = n_states <= 152u ? 32u : (n_states <= 304u ? 16u : 8u);
+    const uint32_t most = n_states <= sms ? 32u : (n_states <= 2 * sms ? 16u : 8u);
     const uint32_t lg = state_lg_segs(k, max_rays), parts = ((max_rays << 2) + 31) / 32;
-    const uint32_t hold = n_states <= 304u ? most - (goals_dev ? 1u : 0u) : 1u;
+    const uint32_t hold = n_states <= 2 * sms ? most - (goals_dev ? 1u : 0u) : 1u;
     const uint32_t chunks = ((max_rays << cta_lg_segs(k, max_rays, lg, hold)) + 31) / 32;
     const uint32_t warps = std::min(std::max(chunks + (goals_dev ? 1u : 0u), 2u), most);
     for_map(m, k.reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
@@ -3624,7 +3625,7 @@ cudaError_t launch_batch(const DevMap& m, const EvalConsts& k, const double* sta
   CtaPartial* cparts = (CtaPartial*)(w + L.cparts);
   CtaPartial* gparts = (CtaPartial*)(w + L.gparts);
   // 8 states a CTA (a warp each) as far as the SMs go; longer runs beyond
-  const unsigned prep = n_states < 8u * 152u ? (n_states + 7u) / 8u : 152u;
+  const unsigned prep = n_states < 8u * sms ? (n_states + 7u) / 8u : sms;
   launch_after(batch_prep_kernel, prep, 256, stream, states_dev, n_rays_dev, n_states, max_rays, m,
                k, hdr, bs, sticket, gticket, out_dev);
   for_map(m, k.reduce_mode, [&](auto kind, auto layout, auto red, auto boxes) {
@@ -3643,7 +3644,7 @@ static size_t rollout_shared(uint32_t rays, uint32_t parts) {
 cudaError_t launch_rollout(const DevMap& m, const EvalConsts& k, const RolloutArgs& g, uint32_t n,
                            uint32_t steps, cudaStream_t stream) {
   // at most 32 warps a CTA; 16 where two robots share an SM and hide each other's serial steps
-  const uint32_t rays = g.rc.n_rays, most = n <= 152u ? 32u : 16u;
+  const uint32_t rays = g.rc.n_rays, most = n <= k.sms ? 32u : 16u;
   const uint32_t lg = state_lg_segs(k, rays), parts = ((rays << lg) + 31) / 32;
   // two warps left for the attractor and the booking where the chunks allow (8 robots of 256 rays:
   // 4 segments, both on marching warps 18.3 us a step, 2 segments 15.8)
@@ -3670,10 +3671,10 @@ cudaError_t launch_probe_l2(const uint4* buf, size_t n16, uint32_t passes, int g
 }
 
 // As few states a CTA as give one CTA an SM: few states wait for latency; beyond, 32, where the
-// FP64 steps fill their lanes (1217 states: 8 a CTA 20.1 us, 16 18.0, 32 20.5; 2432 states: 22.3,
-// 18.2, 20.5).
-static uint32_t esdf_states_per_cta(uint32_t n) {
-  return n <= 8u * 152u ? 8u : (n <= 16u * 152u ? 16u : 32u);
+// FP64 steps fill their lanes (152 SMs, 1217 states: 8 a CTA 20.1 us, 16 18.0, 32 20.5; 2432 states:
+// 22.3, 18.2, 20.5).
+static uint32_t esdf_states_per_cta(uint32_t n, uint32_t sms) {
+  return n <= 8u * sms ? 8u : (n <= 16u * sms ? 16u : 32u);
 }
 
 cudaError_t launch_esdf_eval(const rmp_primitive_t* prims, const float4* prims32,
@@ -3681,7 +3682,7 @@ cudaError_t launch_esdf_eval(const rmp_primitive_t* prims, const float4* prims32
                              const double* goals, uint32_t n_states, rmp_result_t* out,
                              double* query, cudaStream_t stream) {
   if (n_states == 0) return cudaSuccess;
-  const uint32_t G = esdf_states_per_cta(n_states);
+  const uint32_t G = esdf_states_per_cta(n_states, k.sms);
   uint32_t grid = (n_states + G - 1) / G;
   if (grid > 65535) grid = 65535;                   // CTA-stride beyond
   launch_after(esdf_eval_kernel<false, 0, 0>, grid, 256, stream, prims, prims32, n_prims, k, states,
@@ -3693,7 +3694,7 @@ cudaError_t launch_esdf_rollout(const rmp_primitive_t* prims, const float4* prim
                                 uint32_t n_prims, const EsdfConsts& k, const DevMap& m,
                                 const RolloutArgs& g, uint32_t n, uint32_t steps,
                                 rmp_result_t* res, uint32_t* running, cudaStream_t stream) {
-  const uint32_t G = esdf_states_per_cta(n), grid = (n + G - 1) / G;
+  const uint32_t G = esdf_states_per_cta(n, k.sms), grid = (n + G - 1) / G;
   const double* none = nullptr;
   double* query = nullptr;
   auto run = [&](auto kernel) {
