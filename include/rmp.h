@@ -249,7 +249,9 @@ int rmp_scan_eval_async(rmp_ctx* ctx, const float* points_dev, uint32_t n,
  * order of the floating-point reduction.  The paper evaluates one state per call; the
  * batch is this library's throughput form of the same computation (candidate states of
  * a planner, or many robots).  Work is cut into chunks of 32 threads that a persistent
- * grid takes from a counter, so states of any ray counts share the device evenly.
+ * grid takes from a counter, so states of any ray counts share the device evenly; a batch of
+ * few-ray states (max_rays up to 1024, up to 16 states per SM) takes a CTA per state instead,
+ * with the same results to the bit.
  *
  * Capacity: n_states in [1, 65536]; every n_rays_dev[b] <= max_rays, max_rays +
  * halton_offset <= 2^24.  A state with n_b > max_rays or an invalid position gets
@@ -263,8 +265,8 @@ int rmp_scan_eval_async(rmp_ctx* ctx, const float* points_dev, uint32_t n,
  * resets what it uses. */
 size_t rmp_batch_workspace_bytes(uint32_t n_states, uint32_t max_rays);
 
-/* Enqueues two kernels on `stream` (per-state set-up, then the persistent evaluation);
- * no host synchronisation and no allocation, so the call may be captured in a CUDA graph
+/* Enqueues one kernel on `stream` (a CTA per state, see above) or two (per-state set-up, then
+ * the persistent evaluation); no host synchronisation and no allocation, so the call may be captured in a CUDA graph
  * and the graph replayed with new contents of states_dev / n_rays_dev.  The workspace
  * must not be shared by batches that may run concurrently. */
 int rmp_raycast_eval_batch_async(rmp_ctx* ctx, uint32_t map_id, const double* states_dev,
@@ -284,7 +286,8 @@ int rmp_raycast_eval_batch(rmp_ctx* ctx, uint32_t map_id, const double* states,
  * 256} and segments per ray 2^{0,1,2} (rays per thread 1, 1/2, 1/4) on this batch (one
  * untimed launch, then the median of `reps` timed launches, CUDA events on `stream`;
  * synchronises), and leaves the fastest in the context's knobs.  times_ms (nullable,
- * n_times entries) receives the 9 medians in the order block-major, then segments.  The
+ * n_times entries) receives the 9 medians in the order block-major, then segments.  A batch
+ * that takes a CTA per state has no use for the CTA size: its three sizes time the same launch.  The
  * workspace must be sized for the batch (rmp_batch_workspace_bytes). */
 int rmp_batch_autotune(rmp_ctx* ctx, uint32_t map_id, const double* states_dev,
                        const uint32_t* n_rays_dev, uint32_t n_states, uint32_t max_rays,
@@ -300,8 +303,8 @@ int rmp_batch_autotune(rmp_ctx* ctx, uint32_t map_id, const double* states_dev,
  * has no bounded latency).  Per-ray outputs are not offered.
  * Limit: batches whose workspace (rmp_batch_workspace_bytes(n_states, max_rays)) exceeds
  * 4 MiB are rejected with RMP_ERR_NO_MEMORY (one state of up to 406016 rays, or up to six
- * states of 65536).  Nothing in the array has to start at zero: each call's set-up kernel clears
- * what it uses.  The first call on a device looks up the array's address with that device
+ * states of 65536).  Nothing in the array has to start at zero: each call clears what it
+ * uses.  The first call on a device looks up the array's address with that device
  * current (which can load module data), so make one call before any stream capture.
  * The address is kept for the life of the process: do not use this entry point after a
  * cudaDeviceReset of its device (the kept address would then be stale).
@@ -331,8 +334,10 @@ int rmp_combined_eval_batch_async(rmp_ctx* ctx, uint32_t map_id, const double* s
                                   rmp_result_t* out_dev);
 
 /* Closed-loop rollout of point robots (the map-based experiment of Sec. IV-A): every control
- * step evaluates f_c for all running robots in one batched launch and integrates it by
- * semi-implicit Euler in FP64 (xdot' = xdot + f_c dt, x' = x + xdot' dt).  A robot stops
+ * step evaluates f_c for each running robot and integrates it by semi-implicit Euler in FP64
+ * (xdot' = xdot + f_c dt, x' = x + xdot' dt).  Robots of few rays are taken through up to 256
+ * steps by one launch, a CTA each; robots of many rays are evaluated together, a batched
+ * evaluation per step.  A robot stops
  * when, in this order, it leaves a dense grid (LEFT_MAP), the voxel holding it is occupied
  * (COLLIDED), it is within goal_tol of its goal (REACHED), or it has taken max_steps steps
  * (TIMEOUT); an evaluation error stops it with FAILED.  Smoothness is the mean over
@@ -417,7 +422,8 @@ typedef struct {
   uint32_t max_batch_states;   /* requests per batch, 1..65536 */
   uint32_t max_rays;           /* largest accepted request */
   uint32_t reserved;
-  uint64_t mem_budget_bytes;   /* device memory for all batches in flight (allocated once) */
+  uint64_t mem_budget_bytes;   /* device memory for all batches in flight (allocated once);
+                                  a batch takes its workspace of it */
 } rmp_server_config_t;
 
 typedef struct {
@@ -488,8 +494,8 @@ int rmp_esdf_release(rmp_ctx* ctx, uint32_t esdf_id);
  * without goals out.f = A_obs^+ A_obs f_obs.  out.n_rays = 1, n_hits = 1 if the ESDF has a
  * primitive, n_active = 1 if the policy is active and in radius; a state with a non-finite
  * component gets RMP_ERR_INVALID_ARG in its status.  query_dev (nullable): d and the
- * gradient per state (4 doubles; d = +inf with no primitive).  One warp per state, one
- * kernel on `stream`, no allocation; the result is written to out_dev[n_states]. */
+ * gradient per state (4 doubles; d = +inf with no primitive).  One kernel on
+ * `stream`, no allocation; the result is written to out_dev[n_states]. */
 int rmp_esdf_eval_async(rmp_ctx* ctx, uint32_t esdf_id, const double* states_dev,
                         const double* goals_dev, uint32_t n_states, const rmp_params_t* params,
                         double alpha, double beta, rmp_stream_t stream, rmp_result_t* out_dev,
@@ -519,7 +525,8 @@ int rmp_probe_l2_read(rmp_ctx* ctx, const void* buf_dev, size_t bytes, uint32_t 
  * the floating-point reduction, hit records are identical.
  *  RMP_TUNE_BLOCK        threads per CTA: 64, 128 or 256, or 0 (default) automatic: for
  *                        one state, 256 when the launch fits in one wave of 256-thread CTAs,
- *                        else 128; scans 256; batches 128
+ *                        else 128; scans 256; batches 128.  Without effect where a CTA takes a
+ *                        state or a robot by itself (few-ray batches and rollouts)
  *  RMP_TUNE_LG_SEGMENTS  log2 of the segments each ray is split into and marched by that
  *                        many threads (0..5; batches use at most 2, a larger value counts
  *                        as 2 there), or -1 (default) to choose: one state, the most (up

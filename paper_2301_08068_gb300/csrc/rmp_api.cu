@@ -147,7 +147,8 @@ int make_consts(const rmp_params_t* p, double vs, uint32_t n, bool scan, EvalCon
   k->r_hi = (float)p->r;
   k->r_lo = (float)(p->r - (double)k->r_hi);
   // the policy's z = eta_damp / (d / nu_damp + eps) |xdot . r|^2 stays below 1e37 for |xdot|^2 below
-  // this, and its other factors are finite and its divisors nonzero in FP32
+  // this, and its other factors are finite and its divisors nonzero in FP32 (but eta_damp / eps,
+  // which may overflow at d = 0: a hit not approached then adds its exact value, zero, not 0 x inf)
   k->quiet_v2 = (p->eta_rep < 1e37 && p->eta_damp < 1e37 && p->eps > 1e-30 && p->eps < 1e30 &&
                  p->c > 1e-30 && p->c < 1e30 && p->nu_rep > 1e-30 && p->nu_damp > 1e-30 && p->r > 1e-30)
                     ? (float)std::min(1e30, 1e36 * p->eps / std::max(p->eta_damp, 1e-6))
