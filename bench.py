@@ -19,6 +19,8 @@ Printed JSON line (rank 0):
             bandwidth; traffic from the committed ncu capture when it matches this kernel;
   cpu_baseline  the C oracle on a bounded sample: one evaluation per host thread at once,
             on every core of this host (and, beside it, on one core).
+The sections with long lists (served sweep, closed loops, the oracle per configuration) go to
+stderr as a second JSON line, so that the line on stdout stays below 8 KB.
 --impl reference times the oracle instead (rank 0 only, every host core).
 """
 from __future__ import annotations
@@ -272,6 +274,21 @@ def strict_json(obj):
     if isinstance(obj, (list, tuple)):
         return [strict_json(v) for v in obj]
     return obj
+
+
+DETAIL_SECTIONS = ("served", "rollout", "per_ray_outputs_on", "lidar_stream_os0")
+
+
+def split_details(line: dict):
+    """(line, details): the result line without its long sections, and those sections."""
+    short, details = dict(line), {}
+    for key in DETAIL_SECTIONS:
+        if key in short:
+            details[key] = short.pop(key)
+    if "configs" in (short.get("cpu_baseline") or {}):
+        short["cpu_baseline"] = dict(short["cpu_baseline"])
+        details["cpu_configs"] = short["cpu_baseline"].pop("configs")
+    return short, details
 
 
 def stratified_order(costs) -> list:
@@ -1123,6 +1140,8 @@ def main():
                               "note": "65536 rays at up to 3 kHz (abstract), unnamed GPU of "
                                       "Jetson NX / MX150 / Titan Xp, different map"},
         }
+        line, details = split_details(line)
+        print("details " + json.dumps(strict_json(details), allow_nan=False), file=sys.stderr, flush=True)
         print(json.dumps(strict_json(line), allow_nan=False), flush=True)
     ctx.close()
     if world > 1:

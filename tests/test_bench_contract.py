@@ -76,3 +76,18 @@ def test_strict_json_and_stratified_order():
     assert [ranks.index(i) for i in order] == [0, 4, 2, 6, 1, 5, 3, 7]
     with pytest.raises(AssertionError):
         bench.stratified_order([1.0, 2.0, 3.0])
+
+
+def test_result_line_stays_short():
+    """The sections with long lists leave the line for stderr; nothing is lost, and what remains
+    keeps the keys of the contract and fits 8 KB."""
+    many = [{"rays": 16, "success": 0.4375, "wall_s": 0.05277670400001}] * 60
+    line = {"metric": bench.METRIC, "value": 2.7, "cpu_baseline": {"value": 1.0, "configs": {"c1": many}},
+            "e2e": {"value": 1.9}, "served": {"sweep": many}, "rollout": {"a": many},
+            "lidar_stream_os0": {"p50_ms": 0.06}, "per_ray_outputs_on": {"us": 25.0}}
+    short, details = bench.split_details(line)
+    assert len(json.dumps(line)) > 8192 > len(json.dumps(short))
+    assert set(short) == {"metric", "value", "cpu_baseline", "e2e"} and short["cpu_baseline"] == {"value": 1.0}
+    assert details["cpu_configs"] == {"c1": many} and details["served"] == line["served"]
+    assert set(details) == {"cpu_configs", *bench.DETAIL_SECTIONS} and "configs" in line["cpu_baseline"]
+    assert bench.split_details(short) == (short, {})
