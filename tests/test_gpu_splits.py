@@ -379,3 +379,48 @@ def test_launch_info_of_the_kernel_that_runs(ctx, block, least, cells):
         R.rmp_tune_set(ctx.handle, R.RMP_TUNE_BLOCK, 0)
         R.rmp_tune_set(ctx.handle, R.RMP_TUNE_CELL_SKIP, -1)
         R.rmp_map_release(ctx.handle, mid)
+
+
+@pytest.mark.parametrize("n_states,max_rays", [(40, 1100), (3000, 40), (300, 500)])
+def test_batches_back_to_back_on_one_workspace(ctx, n_states, max_rays):
+    """Batches of other states and counts follow one another on one workspace without a wait, each
+    resident beside its predecessor: every result is the one the batch has on its own.  The
+    packed grid with few and with many states, and a CTA per state; single evaluations between
+    them."""
+    torch = torch_cuda()
+    wl = W.hashed_workload(n_states=64, state_seed_index=23)
+    mid = ctx.upload(wl.map)
+    pg = R.make_params(wl.params, wl.max_range)
+    rng = np.random.default_rng(n_states)
+    sets = []
+    for i in range(3):
+        pick = rng.integers(0, 64, n_states)
+        st = np.stack([np.concatenate([wl.states[b].x, wl.states[b].xdot]) for b in pick])
+        counts = rng.integers(0, max_rays + 1, n_states).astype(np.int32)
+        sets.append((torch.tensor(st, device="cuda"), torch.tensor(counts, device="cuda")))
+    ws = torch.empty(R.rmp_batch_workspace_bytes(n_states, max_rays), dtype=torch.uint8, device="cuda")
+    one = torch.empty(R.rmp_workspace_bytes(), dtype=torch.uint8, device="cuda")
+    R.rmp_workspace_init(one)
+
+    def batch(i, out):
+        R.rmp_raycast_eval_batch_async(ctx.handle, mid, *sets[i], n_states, max_rays, pg, ws, out)
+
+    def buffer():
+        return torch.zeros((n_states, R.RESULT_BYTES), dtype=torch.uint8, device="cuda")
+
+    want, single = [buffer() for _ in sets], torch.zeros(R.RESULT_BYTES, dtype=torch.uint8, device="cuda")
+    for i, out in enumerate(want):
+        batch(i, out)
+        torch.cuda.synchronize()
+    R.rmp_raycast_eval_async(ctx.handle, mid, sets[0][0][0], 700, pg, one, single)
+    got, alone = [buffer() for _ in range(24)], torch.zeros_like(single)
+    torch.cuda.synchronize()
+    for j, out in enumerate(got):
+        batch(j % 3, out)
+        if j % 5 == 4:
+            R.rmp_raycast_eval_async(ctx.handle, mid, sets[0][0][0], 700, pg, one, alone)
+    torch.cuda.synchronize()
+    assert torch.equal(single, alone)
+    for j, out in enumerate(got):
+        assert torch.equal(out, want[j % 3]), j
+    R.rmp_map_release(ctx.handle, mid)
